@@ -1,35 +1,38 @@
-// Threshold select and compaction kernels of surgeon_prune_compact, and surgeon_decompress.
+// Threshold select and compaction of surgeon_prune_compact, and surgeon_decompress.
 //
 // Algorithm 1, prune step: the kept set of a layer is its n_keep largest-magnitude elements, ties
 // at the threshold broken by lowest flat index.  Its decompose step / Section 4.2: the pruned
 // activation is cached as the vector of kept elements plus one index bit per element.
 //
-// The tensor is read twice: once to find the threshold, once to emit the store.  No CTA of the
-// emitting pass waits on another: everything it needs to place a chunk's output (how many
-// elements before the chunk are kept, how many ties precede it) is counted during the first read.
-// Both reads are persistent kernels fed by TMA into a shared-memory ring, in which every lane owns
-// 128 consecutive bytes, so bitmap words are built without cross-lane traffic.
+// One cooperative kernel does the whole call: every CTA owns a contiguous range of 4 KB chunks
+// (the unit one warp works on, fetched by TMA into a ring of its own), and the CTAs meet at two or
+// three grid-wide exchanges, at which CTA 0 collects, decides and answers:
 //
-//   sample   : a strided sample (about 1/32 of the tensor) gives a bracket [lo_key, hi_key] of
-//              keys that contains the threshold with overwhelming probability and holds 1-3 %
-//              of the elements.
-//   classify : the first read.  Per 4 KB chunk: the number of keys above the bracket, the number
-//              inside, and the keys inside themselves (the chunk's slot).  Its last CTA decides
-//              where the threshold lies and, for bf16, which key it is.
-//   count    : fp32 resolves the threshold among the listed keys with two histogram levels;
-//              then the listed keys above / equal to the threshold complete the per-chunk counts,
-//              and an exclusive scan over chunks follows (cooperative launch, grid barriers).
-//              The one chunk inside which the tie quota ends is emitted here, by the CTA that
-//              finds it, with its ties ranked by flat index.
-//   compact  : the second read.  A chunk's warp starts from its entry of the scan and skips
-//              that one chunk.
+//   sample    a scattered sample gives a bracket [lo, hi] of keys that contains the threshold with
+//             overwhelming probability (1-4 % of the elements)
+//   classify  first pass over the CTA's chunks: keys above the bracket are counted per chunk, the
+//             keys inside are listed and counted in a histogram of 512 bins over the bracket
+//   exchange  the summed histogram gives the threshold's bin: one key for bf16, whose brackets are
+//             narrower than 512 keys, some thousands of keys for fp32, of which few occur
+//   exchange  every CTA reports its count above the bin and the keys it has inside; CTA 0 finds the
+//             threshold among them and gives every CTA its place in the packed vector
+//   emit      the lists complete the per-chunk counts, a scan turns them into places, and a second
+//             pass over the chunks, last one first, writes the store
 //
-// If the threshold falls outside the bracket, a slot overflows (massive ties at a non-zero
-// value) or the tensor is below kStreamMinBytes, the count kernel runs an exact radix select
-// over the tensor and counts the chunks from the tensor (a small tensor is then emitted by
-// compact_small_kernel).  The result is exact and unique either way.
-// Every count fits 32 bits because n <= SURGEON_MAX_N < 2^31.
+// Why one kernel: as four kernels behind a memset a call took 45-60 us whatever the tensor's size,
+// most of it launches, drained pipelines and grids that started empty; an exchange costs about 2 us.
+// A tensor of at most 48 chunks per SM (29 MB) stays in shared memory between the passes, so it is
+// read from memory once; of a larger one the end of each CTA's range stays, and the second pass
+// starts there and goes backwards, where the L2 cache still holds most of what it needs.
+//
+// When the sample misleads (the bracket misses, or holds more equal keys than a list takes) the
+// first pass is repeated with the bracket the counts prove; the result is exact and unique
+// either way.  Every count fits 32 bits because n <= SURGEON_MAX_N < 2^31.
 #include <cuda.h>
+
+#include <atomic>
+#include <chrono>
+#include <random>
 
 #include "surgeon_internal.cuh"
 #include "tc_common.cuh"
@@ -40,230 +43,104 @@ namespace {
 
 using tc::smem_u32;
 
-constexpr int kSelThreads = 1024;
 constexpr uint32_t kFull = 0xFFFFFFFFu;
-constexpr int kHistWords = kBuckets + 32;   // + one private bin per lane that swallows zeros
-__device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-  return v;
-}
 
-// dst[0 .. kBuckets) = src[0 .. kBuckets) with all loads of a thread in flight together
-// (1024 threads; src is global memory written by other CTAs, dst shared memory).
-__device__ __forceinline__ void load_hist_to_smem(const uint32_t* __restrict__ src, uint32_t* dst) {
-  constexpr int kPer = kBuckets / 4 / kSelThreads;   // 8 vectors per thread
-  uint4 v[kPer];
-#pragma unroll
-  for (int i = 0; i < kPer; ++i)
-    v[i] = __ldcg(reinterpret_cast<const uint4*>(src) + i * kSelThreads + threadIdx.x);
-#pragma unroll
-  for (int i = 0; i < kPer; ++i)
-    reinterpret_cast<uint4*>(dst)[i * kSelThreads + threadIdx.x] = v[i];
-}
-__device__ __forceinline__ void zero_hist_smem(uint32_t* dst) {
-#pragma unroll
-  for (int i = 0; i < kBuckets / 4 / kSelThreads; ++i)
-    reinterpret_cast<uint4*>(dst)[i * kSelThreads + threadIdx.x] = make_uint4(0, 0, 0, 0);
-}
-// Adds the non-zero bins of a CTA's shared-memory histogram to the global one.
-__device__ __forceinline__ void flush_hist(const uint32_t* hist, uint32_t* __restrict__ ghist) {
-#pragma unroll 4
-  for (int i = 0; i < kBuckets / 4 / kSelThreads; ++i) {
-    const int v = i * kSelThreads + threadIdx.x;
-    const uint4 h = reinterpret_cast<const uint4*>(hist)[v];
-    if (h.x) atomicAdd(&ghist[4 * v + 0], h.x);
-    if (h.y) atomicAdd(&ghist[4 * v + 1], h.y);
-    if (h.z) atomicAdd(&ghist[4 * v + 2], h.z);
-    if (h.w) atomicAdd(&ghist[4 * v + 3], h.w);
-  }
-}
+// ---- geometry -----------------------------------------------------------------------------------
+// A chunk is 32 rows of 128 bytes (128-byte swizzle, so that 32 lanes can each read their own row
+// without bank conflicts): each LANE owns one row, i.e. 32 (fp32) or 64 (bf16) consecutive
+// elements, and bitmap words are built without cross-lane traffic.
+constexpr int kWarps = 16;                       // one CTA per SM; 128 registers a thread
+constexpr int kThreads = kWarps * 32;
+constexpr int kSlotsPerWarp = 3;                 // chunks in flight per warp: 192 KB per SM
+constexpr int kChunkBytes = 4096;
+constexpr int kRingBytes = kWarps * kSlotsPerWarp * kChunkBytes;
+constexpr int kResidentChunks = kWarps * kSlotsPerWarp;
+// The rest of the shared memory.  Slots: the listed keys, room for 1/16 of every chunk.
+constexpr int kMaxLocalChunks = 512;             // per-chunk counts in shared memory up to here
+constexpr int kSlotBytes = 256;
+constexpr int kAuxSlots = 8192;                  // (histograms before it)
+constexpr int kAuxCnt = kAuxSlots + kResidentChunks * kSlotBytes;
+constexpr int kAuxPrefix = kAuxCnt + kMaxLocalChunks * 4;
+constexpr int kSampleBinsLog2 = 14;              // top 14 key bits: 64 bins per octave; 16-bit counters here
+constexpr int kSampleBytes = 2 << kSampleBinsLog2;
+static_assert((1 << kSampleBinsLog2) == kSampleBins, "bins of the sample");
+constexpr int kAuxBytes = kAuxPrefix + kMaxLocalChunks * 8 > kSampleBytes ? kAuxPrefix + kMaxLocalChunks * 8 : kSampleBytes;
+// emit: per-warp staging of the kept values of a sparse chunk, in the place of histogram and slots
+constexpr int kStageBytes = (kAuxCnt / kWarps) & ~15;
+constexpr size_t kPruneSmem = static_cast<size_t>(kRingBytes) + kAuxBytes + 1024;
+static_assert(kChunkBytes == kTileVecs * 16, "chunk size");
+constexpr int kMaxKeys = 64;                     // keys one CTA reports at the last exchange
+constexpr int kKeysPerThread = 8;                // and CTA 0 takes in
+constexpr int kKeysAtOnce = kKeysPerThread * kThreads;
 
-// Cooperative search from the top of a histogram of NB bins (NB a multiple of 1024) by a CTA of
-// 1024 threads: finds the bin b with  #(bins above b) < rank <= #(bins >= b)  and writes
-// res[0] = b, res[1] = count in the bins above b.  `ld(i)` returns bin i.  rank >= 1 and the
-// histogram holds at least `rank` entries.  scratch: 32 words of shared memory.
-template <int NB, typename Load>
-__device__ void find_from_top(Load ld, uint32_t rank, uint32_t* scratch, uint32_t* res) {
-  constexpr int PER_WARP = NB / 32;
-  constexpr int PER_LANE = PER_WARP / 32;
-  const int warp = threadIdx.x >> 5;
-  const uint32_t lane = lane_id();
-  // level 1: warp w owns the PER_WARP bins below NB - w*PER_WARP
-  const int top = NB - warp * PER_WARP;   // exclusive upper end
-  uint32_t s = 0;
-#pragma unroll 8
-  for (int i = lane; i < PER_WARP; i += 32) s += ld(top - 1 - i);
-  s = warp_sum(s);
-  if (lane == 0) scratch[warp] = s;
-  __syncthreads();
-  uint32_t acc = 0;
-  int W = 0;
-  for (; W < 31; ++W) {
-    const uint32_t t = scratch[W];
-    if (acc + t >= rank) break;
-    acc += t;
-  }
-  if (warp == W) {
-    // level 2: lane L owns the PER_LANE bins below top - L*PER_LANE
-    const int ltop = top - static_cast<int>(lane) * PER_LANE;
-    uint32_t ls = 0;
-#pragma unroll 8
-    for (int i = 0; i < PER_LANE; ++i) ls += ld(ltop - 1 - ((i + lane) % PER_LANE));
-    const uint32_t excl = warp_excl_scan(ls);
-    const uint32_t want = rank - acc;
-    if (excl < want && want <= excl + ls) {
-      uint32_t a = excl;
-      int b = ltop - 1;
-      for (int i = 0; i < PER_LANE - 1; ++i, --b) {
-        const uint32_t c = ld(b);
-        if (a + c >= want) break;
-        a += c;
-      }
-      res[0] = static_cast<uint32_t>(b);
-      res[1] = acc + a;
-    }
-  }
-  __syncthreads();
-}
+struct PruneArgs {
+  const void* x;
+  long long n, n_rows_full;      // elements; whole 128-byte rows (what the tensor map covers)
+  uint32_t k;
+  int n_chunks;                  // chunks in all
+  int drop_zeros, stall;
+  unsigned long long token;      // unlike any other call's
+  surgeon_header* hdr;
+  uint32_t* bitmap;
+  void* values;
+  uint32_t* offsets;
+  ulonglong2* arrive;            // [kSelPhases][kSelMaxCtas]: {token, what the CTA reports}
+  ulonglong2* answer;            // [kSelPhases][kSelMaxCtas + 2]: {token, what CTA 0 answers}
+  uint32_t* keys;                // [kSelMaxCtas][kMaxKeys]
+  uint32_t* hist;                // [kSelHists][kSelBins]
+  uint32_t* cnt;                 // per chunk (used when a CTA has more than kMaxLocalChunks)
+  unsigned long long* prefix;    // likewise
+  void* slots;                   // per chunk, listed keys of ranges that are not resident
+};
 
 __device__ __forceinline__ uint32_t hash_u32(uint32_t v) {
   v ^= v >> 16; v *= 0x7FEB352Du; v ^= v >> 15; v *= 0x846CA68Bu; v ^= v >> 16;
   return v;
 }
 
-// ---- bracket of buckets around the threshold, predicted from a strided sample ------------------
-template <int DT>
-__global__ void __launch_bounds__(kSelThreads, 1)
-sample_kernel(const uint4* __restrict__ xq, long long n, uint32_t k, uint32_t n_seg,
-              uint32_t seg_stride, SelectState* __restrict__ st, uint32_t* __restrict__ shist) {
-  constexpr uint32_t kMask = Elem<DT>::kKeyMask;
-  constexpr int EPV = (DT == 0) ? 4 : 8;
-  extern __shared__ __align__(128) uint32_t hist[];   // kHistWords
-  __shared__ uint32_t scratch[32];
-  __shared__ uint32_t res[2];
-  __shared__ bool s_last;
-  const int tid = threadIdx.x;
-  const uint32_t lane = lane_id();
-  zero_hist_smem(hist);
-  __syncthreads();
-  uint32_t zero_cnt = 0;
-#pragma unroll 4
-  for (uint32_t seg = blockIdx.x * 32 + (tid >> 5); seg < n_seg; seg += gridDim.x * 32) {
-    // one segment = 32 lanes x 16 bytes, at a hashed position inside its stride
-    const unsigned long long pos =
-        static_cast<unsigned long long>(seg) * seg_stride + hash_u32(seg) % seg_stride;
-    const uint4 q = __ldg(xq + pos * 32 + lane);
-    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-    for (int e = 0; e < EPV; ++e) {
-      const uint32_t bits = (DT == 0) ? w[e % 4] : (w[e >> 1] >> (16 * (e & 1)));
-      const uint32_t key = bits & kMask;
-      const bool isz = key == 0;
-      zero_cnt += isz ? 1u : 0u;
-      // zeros (half of post-ReLU data) go to a bin private to the lane: no conflicts, no branch
-      atomicAdd(&hist[isz ? kBuckets + lane : (DT == 0 ? key >> 16 : key)], 1u);
+// ---- grid-wide exchange ----------------------------------------------------------------------------
+// A CTA reports by storing {token, 8 bytes} in its own word of the phase; CTA 0 polls these words,
+// one thread per CTA, and answers by storing {token, 8 bytes} in words that the others poll.  (Every
+// CTA polling the words of all others took 4-6 us on 148 SMs: the same L2 lines, 148 times over.)
+// No counter has to start at zero, so the call needs no memset: the token differs from call to
+// call.  For a captured graph, whose replays carry the same token, CTA 0 clears every report that it
+// has read, clears a phase's answers before it answers the phase before it, and clears the first
+// answer (phase 0) after the reports of phase 1.  All CTAs are resident (cooperative launch); polls
+// are bounded.
+__device__ __forceinline__ void word_store(ulonglong2* p, unsigned long long token, unsigned long long v) {
+  asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}"
+               ::"l"(p), "l"(token), "l"(v) : "memory");
+}
+__device__ __forceinline__ ulonglong2 word_load(const ulonglong2* p) {
+  ulonglong2 v;
+  asm volatile("{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}"
+               : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+// One thread waits for a word of this call (what it announces apart from its own 8 bytes is visible
+// after a fence).  `stall` is the diagnostic of SURGEON_DEBUG_STALL_BARRIER: a value nobody ever
+// stores, and a cap of 1024 polls.
+__device__ __forceinline__ bool word_wait(const ulonglong2* p, unsigned long long token, unsigned long long* v,
+                                          bool stall = false) {
+  const uint32_t cap = stall ? 1024u : (1u << 22);
+  for (uint32_t spins = 0; spins <= cap; ++spins) {
+    const ulonglong2 w = word_load(p);
+    if (w.x == (stall ? ~token : token)) {
+      *v = w.y;
+      return true;
     }
+    if (spins > 64u) __nanosleep(20);
   }
-  zero_cnt = warp_sum(zero_cnt);
-  if (lane == 0 && zero_cnt) atomicAdd(&hist[0], zero_cnt);
-  __syncthreads();
-  flush_hist(hist, shist);
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) s_last = (atomicAdd(&st->ticket_sample, 1u) == gridDim.x - 1);
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  load_hist_to_smem(shist, hist);
-  __syncthreads();
-  // rank of the threshold inside the sample, +- 5 standard deviations of a binomial count
-  // (single precision, one thread: double-precision arithmetic is slow on this GPU)
-  __shared__ uint32_t s_rank[2];
-  if (tid == 0) {
-    const float S = static_cast<float>(32 * EPV) * static_cast<float>(n_seg);
-    const float q = static_cast<float>(static_cast<double>(k) / static_cast<double>(n));
-    const float r = q * S;
-    const float delta = 5.0f * sqrtf(S * q * (1.0f - q)) + 16.0f;
-    s_rank[0] = (r - delta >= 1.0f) ? static_cast<uint32_t>(r - delta) : 0u;           // 0: none
-    s_rank[1] = (r + delta <= S - 1.0f) ? static_cast<uint32_t>(r + delta) + 1u : 0u;  // 0: none
-  }
-  __syncthreads();
-  uint32_t bhi = kBuckets - 1, blo = 0;
-  auto ld = [&](int i) { return hist[i]; };
-  if (s_rank[0]) {
-    find_from_top<kBuckets>(ld, s_rank[0], scratch, res);
-    bhi = res[0];
-    __syncthreads();
-  }
-  if (s_rank[1]) {
-    find_from_top<kBuckets>(ld, s_rank[1], scratch, res);
-    blo = res[0];
-  }
-  if (tid == 0) {
-    st->blo = blo;
-    st->bhi = bhi;
-    // the bracket as keys; key 0 (exact zeros) is never a candidate
-    const uint32_t lo = (DT == 0) ? (blo << 16) : blo;
-    st->lo_key = lo < 1u ? 1u : lo;
-    const uint32_t hi = (DT == 0) ? ((bhi << 16) | 0xFFFFu) : bhi;
-    st->hi_key = hi;                                            // hi < lo_key: the bracket is {0}
-    const int range_bits = hi >= st->lo_key ? 32 - __clz(hi - st->lo_key) : 0;   // widest relative key
-    st->shiftA = range_bits > 9 ? static_cast<uint32_t>(range_bits - 9) : 0u;
-  }
+  return false;
 }
 
-// ---- geometry shared by the two streaming kernels -----------------------------------------------
-// Persistent CTAs.  One producer thread keeps a ring of 32 KB stages full with 2-D TMA loads of
-// [256 rows x 128 bytes] (128-byte swizzle, so that 32 lanes can each read their own row without
-// bank conflicts).  Each of the 8 consumer warps owns one 4 KB chunk of a stage; each LANE owns
-// one 128-byte row of it, i.e. 32 (fp32) or 64 (bf16) consecutive elements.
-constexpr int kCsWarps = 8;
-constexpr int kCsThreads = (kCsWarps + 1) * 32;
-constexpr int kCsStageRows = kCsWarps * 32;
-constexpr int kCsStageBytes = kCsStageRows * 128;
-constexpr int kCsStages = 3;
-// The ring starts on a 4 KB boundary: every warp's 4 KB part of a stage is then 4 KB-aligned, which
-// the compaction's gather uses to swizzle full shared-memory addresses.
-constexpr uintptr_t kCsAlign = 4096;
-constexpr int kMinTilesPerCta = 4;
-constexpr size_t kCsSmem = static_cast<size_t>(kCsStages) * kCsStageBytes + kCsAlign;
-static_assert(kCsStageRows * 128 / 16 == kCsWarps * kTileVecs, "a warp's 32 rows are one chunk");
-
-// This lane's row (8 vectors) out of the swizzled stage; the ragged last row of the tensor, which
-// the tensor map does not cover, comes from global memory.  Returns the row's valid element count.
-template <int DT>
-__device__ __forceinline__ int load_row(const unsigned char* region, const typename Elem<DT>::type* x,
-                                        long long n, long long n_rows_full, long long grow,
-                                        uint4 (&q)[8]) {
-  constexpr int EPR = 128 / sizeof(typename Elem<DT>::type);
-  const uint32_t lane = lane_id();
-  const unsigned char* row = region + lane * 128;
-#pragma unroll
-  for (int j = 0; j < 8; ++j)
-    q[j] = *reinterpret_cast<const uint4*>(row + ((j ^ (lane & 7)) << 4));
-  const long long e0 = grow * EPR;
-  long long nv = n - e0;
-  nv = nv < 0 ? 0 : (nv > EPR ? EPR : nv);
-  if (grow >= n_rows_full && nv > 0) {
-    uint32_t t[64];
-#pragma unroll
-    for (int i = 0; i < 64; ++i) t[i] = (i < EPR && i < nv) ? static_cast<uint32_t>(x[e0 + i]) : 0u;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      if (DT == 0) q[j] = make_uint4(t[4 * j], t[4 * j + 1], t[4 * j + 2], t[4 * j + 3]);
-      else q[j] = make_uint4(t[8 * j] | (t[8 * j + 1] << 16), t[8 * j + 2] | (t[8 * j + 3] << 16),
-                             t[8 * j + 4] | (t[8 * j + 5] << 16), t[8 * j + 6] | (t[8 * j + 7] << 16));
-    }
-  }
-  return static_cast<int>(nv);
-}
 // bf16 keys are compared two at a time inside their 32-bit word: a key is at most 0x7FFF, so
 // key + (0x8000 - t) carries into bit 15 of its half exactly when key >= t, and never into the
 // other half.  The flag bits of the 16 words of a group of 32 elements are collected in one mask,
 // word i shifted right by i: bit (15 - i) is element 2i, bit (31 - i) element 2i + 1.
 __device__ __forceinline__ uint32_t ge_const(uint32_t t) {       // t in [0, 0x8000]
-  return (0x8000u - t) * 0x10001u;
+  return (0x8000u - (t > 0x8000u ? 0x8000u : t)) * 0x10001u;
 }
 __device__ __forceinline__ uint32_t pair_flags(uint32_t keys2, uint32_t c, int i) {
   return ((keys2 + c) >> i) & (0x80008000u >> i);
@@ -285,694 +162,78 @@ __device__ __forceinline__ uint32_t valid_mask(int nv, int w) {
   return left >= 32 ? 0xFFFFFFFFu : (left <= 0 ? 0u : ((1u << left) - 1u));
 }
 
-// The chunk's keys inside the bracket (flagged in cw0 / cw1, `c_tot` of them in the warp) if they
-// all are one key, else 0 (no candidate key is 0).  Called for chunks whose slot overflows only,
-// and kept out of line so that the classify kernel's registers are those of its common path; it
-// reads the lane's row again, a piece at a time.
-template <int DT>
-__device__ __noinline__ uint32_t one_key_of_chunk(const unsigned char* region,
-                                                  const typename Elem<DT>::type* x, long long n,
-                                                  long long n_rows_full, long long grow,
-                                                  uint32_t cw0, uint32_t cw1, uint32_t c_tot) {
-  using E = typename Elem<DT>::type;
-  constexpr uint32_t kMask = Elem<DT>::kKeyMask;
-  constexpr int EPR = 128 / sizeof(E);
+// This lane's row (8 vectors) out of the swizzled chunk.
+__device__ __forceinline__ void load_row(const unsigned char* region, uint4 (&q)[8]) {
   const uint32_t lane = lane_id();
-  const bool ragged = grow >= n_rows_full;
+  const unsigned char* row = region + lane * 128;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) q[j] = *reinterpret_cast<const uint4*>(row + ((j ^ (lane & 7)) << 4));
+}
+// Element e of this lane's row.
+template <int DT>
+__device__ __forceinline__ uint32_t row_elem(const unsigned char* region, int e) {
+  using E = typename Elem<DT>::type;
+  const uint32_t lane = lane_id();
+  const int byte = e * static_cast<int>(sizeof(E));
+  return static_cast<uint32_t>(*reinterpret_cast<const E*>(region + lane * 128 + (((byte >> 4) ^ (lane & 7)) << 4) + (byte & 15)));
+}
+
+// Masks of the elements with key >= t, bit e = element e, elements past nv cleared.  fp32 keys are
+// below 2^31, so the sign bit of (key - t) says key < t; a funnel shift collects it (two
+// instructions per element), element e in bit 31 - e, and one bit reversal puts it back.
+template <int DT, int WPL>
+__device__ __forceinline__ void mask_ge(const uint4 (&q)[8], int nv, uint32_t t, uint32_t (&m)[WPL]) {
+  const uint32_t c_t = ge_const(t);
+#pragma unroll
+  for (int w = 0; w < WPL; ++w) m[w] = 0;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const uint32_t c[4] = {q[j].x, q[j].y, q[j].z, q[j].w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int pw = 4 * j + i;
+      if (DT == 0) m[0] = __funnelshift_l((c[i] & Elem<DT>::kKeyMask) - t, m[0], 1);
+      else m[(pw >> 4) % WPL] |= pair_flags(c[i] & 0x7FFF7FFFu, c_t, pw & 15);
+    }
+  }
+#pragma unroll
+  for (int w = 0; w < WPL; ++w)
+    m[w] = (DT == 0 ? ~__brev(m[w]) : pairs_to_element_order(m[w])) & valid_mask(nv, w);
+}
+
+// The chunk's keys inside the bracket (flagged in cw0 / cw1, `c_tot` of them in the warp) if they
+// all are one key, else 0 (no key inside a bracket is 0).  Called where massive ties overflow a
+// list, and kept out of line so that the first pass's registers are those of its common path.
+template <int DT>
+__device__ __noinline__ uint32_t one_key_of_chunk(const unsigned char* region, uint32_t cw0, uint32_t cw1,
+                                                  uint32_t c_tot) {
+  constexpr uint32_t kMask = Elem<DT>::kKeyMask;
+  const uint32_t lane = lane_id();
   const unsigned char* row = region + lane * 128;
   const int src = __ffs(__ballot_sync(kFull, (cw0 | cw1) != 0u)) - 1;
   uint32_t k0 = 0;
-  if (static_cast<int>(lane) == src) {
-    const int e = cw0 ? __ffs(cw0) - 1 : 32 + __ffs(cw1) - 1;      // (fp32: cw1 is cw0)
-    if (ragged) {
-      k0 = static_cast<uint32_t>(x[grow * EPR + e]) & kMask;
-    } else {
-      const int byte = e * static_cast<int>(sizeof(E));
-      k0 = static_cast<uint32_t>(*reinterpret_cast<const E*>(row + (((byte >> 4) ^ (lane & 7)) << 4) + (byte & 15))) & kMask;
-    }
-  }
+  if (static_cast<int>(lane) == src)                                   // (fp32: cw1 is cw0)
+    k0 = row_elem<DT>(region, cw0 ? __ffs(cw0) - 1 : 32 + __ffs(cw1) - 1) & kMask;
   k0 = __shfl_sync(kFull, k0, src);
   uint32_t eq = 0;
-  if (ragged) {                                  // the tensor's last, partial row: element by element
-    for (int e = 0; e < EPR; ++e)
-      if (grow * EPR + e < n) eq += (static_cast<uint32_t>(x[grow * EPR + e]) & kMask) == k0 ? 1u : 0u;
-  } else {
-    const uint32_t c_ge = ge_const(k0 & 0x7FFFu), c_gt = ge_const((k0 & 0x7FFFu) + 1u);   // bf16: k0 <= 0x7FFF
+  const uint32_t c_ge = ge_const(k0), c_gt = ge_const(k0 + 1u);
 #pragma unroll 1
-    for (int j = 0; j < 8; ++j) {                // one 16-byte piece at a time: few registers
-      const uint4 v = *reinterpret_cast<const uint4*>(row + ((j ^ (lane & 7)) << 4));
-      const uint32_t c[4] = {v.x, v.y, v.z, v.w};
+  for (int j = 0; j < 8; ++j) {                  // one 16-byte piece at a time: few registers
+    const uint4 v = *reinterpret_cast<const uint4*>(row + ((j ^ (lane & 7)) << 4));
+    const uint32_t c[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if (DT == 0) {
-          eq += (c[i] & kMask) == k0 ? 1u : 0u;
-        } else {
-          const uint32_t keys2 = c[i] & 0x7FFF7FFFu;
-          eq += __popc(((keys2 + c_ge) & ~(keys2 + c_gt)) & 0x80008000u);
-        }
+    for (int i = 0; i < 4; ++i) {
+      if (DT == 0) {
+        eq += (c[i] & kMask) == k0 ? 1u : 0u;
+      } else {
+        const uint32_t keys2 = c[i] & 0x7FFF7FFFu;
+        eq += __popc(((keys2 + c_ge) & ~(keys2 + c_gt)) & 0x80008000u);
       }
     }
   }
-  // (a ragged row's fill is key 0, never a candidate)
+  // (rows past the tensor's end hold key 0)
   return __reduce_add_sync(kFull, eq) == c_tot ? k0 : 0u;
 }
-
-// ---- the select's read of the tensor ---------------------------------------------------------
-// Per chunk: how many keys lie above the bracket, how many inside; the keys inside go to the
-// chunk's slot.  A level-A histogram of the keys inside (relative to lo_key) is kept per CTA.
-// The last CTA places the threshold: above the bracket or a full slot -> fall back; inside ->
-// bin of level A (bf16: the threshold itself); below, with lo_key == 1 -> the threshold is 0.
-template <int DT>
-__global__ void __launch_bounds__(kCsThreads, 2)
-classify_kernel(const __grid_constant__ CUtensorMap xmap, const void* __restrict__ xv, long long n,
-                long long n_rows_full, uint32_t k, SelectState* __restrict__ st,
-                uint32_t* __restrict__ hist_a, uint32_t* __restrict__ cnt_gt,
-                uint32_t* __restrict__ cand_cnt, void* __restrict__ slots_v,
-                surgeon_header* __restrict__ hdr, int n_chunks, int n_stage_tiles,
-                int drop_zeros) {
-  using E = typename Elem<DT>::type;
-  constexpr uint32_t kMask = Elem<DT>::kKeyMask;
-  constexpr int EPR = 128 / sizeof(E);
-  constexpr int WPL = EPR / 32;
-  constexpr int kSlot = (DT == 0) ? 64 : 128;
-  extern __shared__ __align__(1024) unsigned char cs_smem_raw[];
-  unsigned char* ring = reinterpret_cast<unsigned char*>(
-      (reinterpret_cast<uintptr_t>(cs_smem_raw) + kCsAlign - 1) & ~(kCsAlign - 1));
-  __shared__ __align__(8) unsigned long long bars[2 * kCsStages];
-  __shared__ uint32_t s_hist[kBinsA];
-  __shared__ uint32_t s_tot[4];        // keys above / inside the bracket, largest key inside, largest ~key inside
-  __shared__ bool s_last;
-  const E* __restrict__ x = reinterpret_cast<const E*>(xv);
-  E* __restrict__ slots = reinterpret_cast<E*>(slots_v);   // fp32: 32-bit keys, bf16: 16-bit keys
-  const int tid = threadIdx.x;
-  const int warp = tid >> 5;
-  const uint32_t lane = lane_id();
-  if (st->mode == 1u) return;          // the sample found no usable bracket
-  const uint32_t lo_key = st->lo_key, hi_key = st->hi_key;
-  const uint32_t shiftA = st->shiftA;
-  // bf16: the two comparisons as additions on packed pairs of keys (hi_key <= 0x7FFF there)
-  const uint32_t c_above = ge_const(hi_key >= 0x7FFFu ? 0x8000u : hi_key + 1u);
-  const uint32_t c_lo = hi_key >= lo_key ? ge_const(lo_key > 0x8000u ? 0x8000u : lo_key) : 0u;
-  const uint32_t full_bar = smem_u32(bars);
-  const uint32_t empty_bar = smem_u32(bars + kCsStages);
-  if (tid == 0) {
-    tc::tma_prefetch_desc(&xmap);
-    for (int s = 0; s < kCsStages; ++s) {
-      tc::mbar_init(full_bar + 8 * s, 1);
-      tc::mbar_init(empty_bar + 8 * s, kCsWarps);
-    }
-    tc::fence_barrier_init();
-    s_tot[0] = 0;
-    s_tot[1] = 0;
-    s_tot[2] = 0;
-    s_tot[3] = 0;
-  }
-  for (int i = tid; i < kBinsA; i += kCsThreads) s_hist[i] = 0;
-  __syncthreads();
-  const int first = blockIdx.x;
-  const int n_it = first < n_stage_tiles ? (n_stage_tiles - 1 - first) / static_cast<int>(gridDim.x) + 1 : 0;
-
-  if (warp == kCsWarps) {
-    // ---- producer ----
-    if (lane == 0) {
-      for (int it = 0; it < n_it; ++it) {
-        const int s = it % kCsStages;
-        if (it >= kCsStages && !tc::mbar_wait(empty_bar + 8 * s, ((it / kCsStages) - 1) & 1, 20)) {
-          atomicMax(&st->error, static_cast<uint32_t>(SURGEON_ERR_TIMEOUT));
-          break;
-        }
-        const int t = first + it * static_cast<int>(gridDim.x);
-        tc::mbar_arrive_expect_tx(full_bar + 8 * s, kCsStageBytes);
-        tc::tma_load_2d(smem_u32(ring + s * kCsStageBytes), &xmap, 0, t * kCsStageRows,
-                        full_bar + 8 * s);
-      }
-    }
-  } else {
-    // ---- consumers ----
-    uint32_t w_above = 0, w_cand = 0;
-    uint32_t w_kmax = 0, w_kinv = 0;     // largest key inside the bracket seen by this lane, and largest ~key
-    for (int it = 0; it < n_it; ++it) {
-      const int s = it % kCsStages;
-      const int chunk = (first + it * static_cast<int>(gridDim.x)) * kCsWarps + warp;
-      if (!tc::mbar_wait(full_bar + 8 * s, (it / kCsStages) & 1, 20)) {
-        if (lane == 0) atomicMax(&st->error, static_cast<uint32_t>(SURGEON_ERR_TIMEOUT));
-        break;
-      }
-      const unsigned char* region = ring + s * kCsStageBytes + warp * 4096;
-      if (chunk < n_chunks) {
-        uint4 q[8];
-        const long long grow = static_cast<long long>(chunk) * 32 + lane;
-        const int nv = load_row<DT>(region, x, n, n_rows_full, grow, q);
-        uint32_t cw[WPL];
-        uint32_t ac = 0, cc = 0;
-        if (DT == 0) {
-          // Keys are below 2^31, so the sign bit of (hi_key - key) says key > hi_key and that of
-          // (key - lo) says key < lo; a funnel shift collects it: two instructions per element
-          // and comparison.  Element e ends up in bit 31 - e, one bit reversal per word puts it back.
-          uint32_t aw = 0, lw = 0;
-          const uint32_t lo_cmp = hi_key >= lo_key ? lo_key : 0x7FFFFFFFu;   // bracket {0}: nothing is a candidate
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const uint32_t c[4] = {q[j].x, q[j].y, q[j].z, q[j].w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const uint32_t key = c[i] & kMask;
-              aw = __funnelshift_l(hi_key - key, aw, 1);
-              lw = __funnelshift_l(key - lo_cmp, lw, 1);
-            }
-          }
-          const uint32_t vm = valid_mask(nv, 0);
-          aw = __brev(aw) & vm;
-          cw[0] = ~__brev(lw) & ~aw & vm;
-          if (hi_key < lo_key) cw[0] = 0u;
-          ac = __popc(aw);
-        } else {
-          // above: key >= hi_key + 1; inside the bracket: key >= lo_key and not above
-          uint32_t ga[WPL], gl[WPL];
-#pragma unroll
-          for (int w = 0; w < WPL; ++w) { ga[w] = 0; gl[w] = 0; }
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const uint32_t c[4] = {q[j].x, q[j].y, q[j].z, q[j].w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const int pw = 4 * j + i;           // packed word of the row: elements 2pw, 2pw + 1
-              const uint32_t keys2 = c[i] & 0x7FFF7FFFu;
-              ga[(pw >> 4) % WPL] |= pair_flags(keys2, c_above, pw & 15);
-              gl[(pw >> 4) % WPL] |= pair_flags(keys2, c_lo, pw & 15);
-            }
-          }
-#pragma unroll
-          for (int w = 0; w < WPL; ++w) {
-            ac += __popc(ga[w]);        // zeros that fill a ragged row are never above
-            const uint32_t in = gl[w] & ~ga[w];
-            cw[w] = in ? (pairs_to_element_order(in) & valid_mask(nv, w)) : 0u;
-          }
-        }
-#pragma unroll
-        for (int w = 0; w < WPL; ++w) cc += __popc(cw[w]);
-        const uint32_t a_tot = __reduce_add_sync(kFull, ac);
-        const uint32_t c_tot = __reduce_add_sync(kFull, cc);
-        if (lane == 0) { cnt_gt[chunk] = a_tot; cand_cnt[chunk] = c_tot; }
-        w_above += a_tot;
-        w_cand += c_tot;
-        const bool ragged = grow >= n_rows_full;
-        const unsigned char* row = region + lane * 128;
-        auto key_at = [&](int e) -> uint32_t {        // key of element e of this lane's row
-          if (ragged) return static_cast<uint32_t>(x[grow * EPR + e]) & kMask;
-          const int byte = e * static_cast<int>(sizeof(E));
-          return static_cast<uint32_t>(*reinterpret_cast<const E*>(
-                     row + (((byte >> 4) ^ (lane & 7)) << 4) + (byte & 15))) & kMask;
-        };
-        if (c_tot > static_cast<uint32_t>(kSlot)) {
-          if (lane == 0) st->list_overflow = 1u;
-          // Too many keys inside the bracket for the slot: massive ties.  If they all are one and the
-          // same key - here and in every other chunk - that key is the threshold and the counts
-          // above are all the count kernel needs; the last CTA checks that through the extremes.
-          const uint32_t k1 = one_key_of_chunk<DT>(region, x, n, n_rows_full, grow, cw[0], cw[WPL - 1], c_tot);
-          w_kmax = k1 ? max(w_kmax, k1) : 0xFFFFFFFFu;
-          w_kinv = k1 ? max(w_kinv, ~k1) : 0xFFFFFFFFu;
-        } else if (c_tot) {
-          // keys inside the bracket -> the chunk's slot (order does not matter)
-          uint32_t pos = warp_excl_scan(cc);
-          E* slot = slots + static_cast<long long>(chunk) * kSlot;
-#pragma unroll
-          for (int w = 0; w < WPL; ++w) {
-            uint32_t m = cw[w];
-            while (m) {
-              const int e = 32 * w + __ffs(m) - 1;
-              m &= m - 1;
-              const uint32_t key = key_at(e);
-              slot[pos++] = static_cast<E>(key);
-              atomicAdd(&s_hist[(key - lo_key) >> shiftA], 1u);
-              w_kmax = max(w_kmax, key);
-              w_kinv = max(w_kinv, ~key);
-            }
-          }
-        }
-      }
-      __syncwarp();
-      if (lane == 0) tc::mbar_arrive(empty_bar + 8 * s);
-    }
-    w_kmax = __reduce_max_sync(kFull, w_kmax);
-    w_kinv = __reduce_max_sync(kFull, w_kinv);
-    if (lane == 0) {
-      if (w_above) atomicAdd(&s_tot[0], w_above);
-      if (w_cand) atomicAdd(&s_tot[1], w_cand);
-      if (w_kmax) atomicMax(&s_tot[2], w_kmax);
-      if (w_kinv) atomicMax(&s_tot[3], w_kinv);
-    }
-  }
-  __syncthreads();
-  for (int i = tid; i < kBinsA; i += kCsThreads)
-    if (s_hist[i]) atomicAdd(&hist_a[i], s_hist[i]);
-  if (tid == 0) {
-    if (s_tot[0]) atomicAdd(&st->above_total, s_tot[0]);
-    if (s_tot[1]) atomicAdd(&st->cand_total, s_tot[1]);
-    if (s_tot[2]) atomicMax(&st->cand_key_max, s_tot[2]);
-    if (s_tot[3]) atomicMax(&st->cand_keyinv_max, s_tot[3]);
-  }
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) s_last = (atomicAdd(&st->ticket_classify, 1u) == gridDim.x - 1);
-  __syncthreads();
-  if (!s_last || warp != 0) return;
-
-  // ---- last CTA, one warp: where does the threshold lie? ----
-  __threadfence();
-  const uint32_t above_total = __ldcg(&st->above_total);
-  const uint32_t n_cand = __ldcg(&st->cand_total);
-  const bool overflow = __ldcg(&st->list_overflow) != 0;
-  const long long r = static_cast<long long>(k) - above_total;     // rank among the rest
-  const long long zeros = (lo_key == 1u) ? n - above_total - n_cand : 0;
-  uint32_t mode, tau = 0, n_greater = 0;
-  if (overflow && r >= 1 && r <= n_cand &&
-      __ldcg(&st->cand_key_max) == ~__ldcg(&st->cand_keyinv_max)) {
-    // every key inside the bracket is the same one: it is the threshold, all candidates are ties
-    mode = 4;
-    tau = __ldcg(&st->cand_key_max);
-    n_greater = above_total;
-  } else if (overflow || r < 1) {
-    mode = 1;
-  } else if (r <= n_cand) {
-    // level A from the top: lane L owns bins [kBinsA - 16(L+1), kBinsA - 16L)
-    constexpr int kPerLane = kBinsA / 32;
-    const int ltop = kBinsA - static_cast<int>(lane) * kPerLane;
-    uint32_t ls = 0;
-#pragma unroll
-    for (int i = 0; i < kPerLane; ++i) ls += __ldcg(hist_a + ltop - 1 - i);
-    const uint32_t excl = warp_excl_scan(ls);
-    const uint32_t want = static_cast<uint32_t>(r);
-    uint32_t bin = 0, aboveA = 0;
-    if (excl < want && want <= excl + ls) {
-      uint32_t a = excl;
-      int b = ltop - 1;
-      for (int i = 0; i < kPerLane - 1; ++i, --b) {
-        const uint32_t c = __ldcg(hist_a + b);
-        if (a + c >= want) break;
-        a += c;
-      }
-      bin = static_cast<uint32_t>(b);
-      aboveA = a;
-    }
-    const uint32_t owner = __ffs(__ballot_sync(kFull, excl < want && want <= excl + ls)) - 1;
-    bin = __shfl_sync(kFull, bin, owner);
-    aboveA = __shfl_sync(kFull, aboveA, owner);
-    if (lane == 0) {
-      st->binA = bin;
-      st->aboveA = aboveA;
-      st->rankA = want - aboveA;
-    }
-    mode = shiftA ? 0u : 2u;
-    tau = lo_key + bin;                       // shiftA == 0: level A is exact
-    n_greater = above_total + aboveA;
-  } else if (lo_key == 1u && r <= n_cand + zeros) {
-    mode = 2;
-    tau = 0;
-    n_greater = above_total + n_cand;
-  } else {
-    mode = 1;
-  }
-  if (lane == 0) {
-    if (mode == 2 || mode == 4) {
-      // store variant without kept zeros: a threshold of key 0 keeps the non-zero elements only
-      const bool nz = drop_zeros && tau == 0u;
-      hdr->threshold_key = tau;
-      hdr->status = __ldcg(&st->error);
-      hdr->n_keep = nz ? static_cast<long long>(n_greater) : static_cast<long long>(k);
-      hdr->n_greater = n_greater;
-      hdr->tie_quota = nz ? 0 : static_cast<long long>(k) - n_greater;
-    }
-    st->mode = mode;
-    __threadfence();
-  }
-}
-
-// n_keep == 0 (ratio 1, or an empty tensor): nothing to select.
-__global__ void header_empty_kernel(surgeon_header* hdr, uint32_t sentinel, uint32_t* offsets,
-                                    long long n_blocks) {
-  if (n_blocks > 0) offsets[n_blocks] = 0u;      // the sentinel entry of the block offsets
-  hdr->threshold_key = sentinel;
-  hdr->status = SURGEON_OK;
-  hdr->n_keep = 0;
-  hdr->n_greater = 0;
-  hdr->tie_quota = 0;
-}
-
-constexpr unsigned long long kCountMask = 0x7FFFFFFFull;
-constexpr int kRows = 4;                 // rows of 32 lanes x 16 bytes per warp
-constexpr int kTileWarps = kTileVecs / (kRows * 32);   // warps of the generic per-tile kernels
-static_assert(kTileWarps * kRows * 32 == kTileVecs, "compaction tile");
-constexpr int kCompactThreads = kTileWarps * 32;
-
-// Defined with the compaction kernels below; the count kernel emits the boundary tile itself.
-template <int DT, bool SLOW>
-__device__ __forceinline__ void compact_tile(const typename Elem<DT>::type* __restrict__ x,
-                                             long long n, const uint4 (&q)[kRows], int tile,
-                                             uint32_t tau, long long quota, bool ties,
-                                             long long gt_tile_before, long long eq_tile_before,
-                                             surgeon_header* __restrict__ hdr,
-                                             uint32_t* __restrict__ bitmap,
-                                             typename Elem<DT>::type* __restrict__ values,
-                                             uint32_t* __restrict__ offsets);
-template <int DT>
-__device__ __forceinline__ void load_tile(const typename Elem<DT>::type* __restrict__ x,
-                                          long long n, int tile, uint4 (&q)[kRows]);
-
-// ---- threshold (where still open), per-chunk counts, exclusive scan ------------------------------
-// Launched cooperatively (all CTAs resident), so that the steps can be separated by grid-wide
-// barriers: a counter every CTA increments and then polls, with a bounded number of polls.
-// Returns false when the wait gave up (uniform over the CTA); the caller then leaves the kernel.
-// `stall` is the diagnostic of SURGEON_DEBUG_STALL_BARRIER: the arrival target is one more than
-// the CTAs that exist and the poll cap is 1024, so the wait is certain to run out, quickly.
-__device__ __forceinline__ bool grid_barrier(SelectState* st, uint32_t& epoch, bool stall = false) {
-  __shared__ uint32_t s_ok;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(&st->barrier_count, 1u);
-    ++epoch;
-    const uint32_t target = epoch * gridDim.x + (stall ? 1u : 0u);
-    const uint32_t cap = stall ? 1024u : (1u << 22);
-    uint32_t spins = 0, ok = 1;
-    while (*reinterpret_cast<volatile uint32_t*>(&st->barrier_count) < target) {
-      if (++spins > cap) { atomicMax(&st->error, static_cast<uint32_t>(SURGEON_ERR_TIMEOUT)); ok = 0; break; }
-      __nanosleep(40);
-    }
-    __threadfence();
-    s_ok = ok;
-  }
-  __syncthreads();
-  return s_ok != 0u;
-}
-
-// Calls f(key) for the first `cc` keys of chunk c's slot; one thread, 16-byte loads, four in flight.
-template <int DT, typename F>
-__device__ __forceinline__ void for_slot_keys(const typename Elem<DT>::type* __restrict__ slots,
-                                              int c, uint32_t cc, F f) {
-  constexpr int kSlot = (DT == 0) ? 64 : 128;
-  constexpr int EPV = (DT == 0) ? 4 : 8;
-  const uint4* __restrict__ p = reinterpret_cast<const uint4*>(slots + static_cast<long long>(c) * kSlot);
-  const int nv = static_cast<int>((cc + EPV - 1) / EPV);
-  for (int v0 = 0; v0 < nv; v0 += 4) {
-    uint4 q[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) q[u] = (v0 + u < nv) ? __ldg(p + v0 + u) : make_uint4(0, 0, 0, 0);
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const uint32_t w[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
-#pragma unroll
-      for (int e = 0; e < EPV; ++e) {
-        const uint32_t idx = static_cast<uint32_t>((v0 + u) * EPV + e);
-        const uint32_t key = (DT == 0) ? w[e % 4] : ((w[e >> 1] >> (16 * (e & 1))) & 0xFFFFu);
-        if (idx < cc) f(key);
-      }
-    }
-  }
-}
-
-// prefix[c] = (elements kept for sure before chunk c) << 31 | (ties at the threshold before it),
-// c = 0 .. chunks (the last entry holds the totals).
-// The fp32 instance is held to 32 registers (a few spills), so that a CTA fits on an SM beside one
-// CTA of another stream's streaming kernel instead of waiting for an empty SM (those kernels are
-// memory-bound in fp32 and lose nothing to the neighbour).  The bf16 streaming kernels are bound
-// by instruction issue: sharing their SM cost the ViT-shaped stack 6 % even with the spills moved
-// out of the way, so that instance keeps a whole SM.
-template <int DT>
-__global__ void __launch_bounds__(kSelThreads, DT == 0 ? 2 : 1)
-count_kernel(const void* __restrict__ xv, long long n, uint32_t k, SelectState* __restrict__ st,
-             surgeon_header* __restrict__ hdr, uint32_t* __restrict__ hist_b,
-             uint32_t* __restrict__ hist_fb, const uint32_t* __restrict__ cnt_gt,
-             const uint32_t* __restrict__ cand_cnt, const void* __restrict__ slots_v,
-             unsigned long long* __restrict__ val, unsigned long long* __restrict__ prefix,
-             unsigned long long* __restrict__ partial, int tiles,
-             uint32_t* __restrict__ bitmap, void* __restrict__ values_v,
-             uint32_t* __restrict__ offsets, int drop_zeros, int stall) {
-  using E = typename Elem<DT>::type;
-  constexpr uint32_t kMask = Elem<DT>::kKeyMask;
-  constexpr int EPV = 16 / sizeof(E);
-  constexpr long long kChunkElems = static_cast<long long>(kTileVecs) * EPV;
-  __shared__ uint32_t s_hist[kBinsB];          // level B / fall-back digit histogram
-  __shared__ int s_bnd;                        // the chunk inside which the tie quota ends, if this CTA owns it
-  __shared__ uint32_t s_err;                   // a bounded wait of this call has given up
-  __shared__ unsigned long long s_bnd_prefix;
-  __shared__ uint32_t scratch[32];
-  __shared__ uint32_t res[2];
-  __shared__ unsigned long long s_tot[32];
-  const E* __restrict__ x = reinterpret_cast<const E*>(xv);
-  const E* __restrict__ slots = reinterpret_cast<const E*>(slots_v);
-  const int tid = threadIdx.x;
-  const int warp = tid >> 5;
-  const uint32_t lane = lane_id();
-  uint32_t epoch = 0;
-  const uint32_t mode = __ldcg(&st->mode);
-  uint32_t tau = 0, n_greater = 0;
-  if (tid == 0) s_bnd = -1;                    // read after several barriers below
-  // A barrier that gave up: the CTA reports it and leaves before it stores anything to the
-  // outputs (the CTAs still waiting for it run out of polls in turn).
-  auto leave = [&]() { if (tid == 0) atomicMax(&hdr->status, static_cast<uint32_t>(SURGEON_ERR_TIMEOUT)); };
-
-  if (mode == 1u) {
-    // ---- fall-back: exact radix select over the tensor itself, one digit per round ----
-    constexpr int kRounds = (DT == 0) ? 3 : 2;
-    const int shifts[3] = {DT == 0 ? 20 : 7, DT == 0 ? 10 : 0, 0};
-    const int bits[3] = {DT == 0 ? 11 : 8, DT == 0 ? 10 : 7, 10};
-    uint32_t fixed = 0, rank = k, above = 0;
-    const long long nvec = n / EPV;
-    const uint4* __restrict__ xq = reinterpret_cast<const uint4*>(xv);
-    for (int round = 0; round < kRounds; ++round) {
-      const int sh = shifts[round], nb = 1 << bits[round], hi = sh + bits[round];
-      for (int i = tid; i < kFbBins; i += kSelThreads) s_hist[i] = 0;
-      __syncthreads();
-      uint32_t zero_cnt = 0;     // digit 0 in a register (half of post-ReLU data)
-      auto add = [&](uint32_t key) {
-        const bool match = hi >= 31 || (key >> hi) == (fixed >> hi);
-        if (match) {
-          const uint32_t d = (key >> sh) & (nb - 1);
-          if (d == 0) ++zero_cnt;
-          else atomicAdd(&s_hist[d], 1u);
-        }
-      };
-      for (long long v = static_cast<long long>(blockIdx.x) * kSelThreads + tid; v < nvec;
-           v += static_cast<long long>(gridDim.x) * kSelThreads) {
-        const uint4 q = __ldg(xq + v);
-        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-        for (int i = 0; i < EPV; ++i)
-          add(((DT == 0) ? w[i % 4] : (w[i >> 1] >> (16 * (i & 1)))) & kMask);
-      }
-      if (blockIdx.x == 0)
-        for (long long j = nvec * EPV + tid; j < n; j += kSelThreads)
-          add(static_cast<uint32_t>(x[j]) & kMask);
-      zero_cnt = warp_sum(zero_cnt);
-      if (lane == 0 && zero_cnt) atomicAdd(&s_hist[0], zero_cnt);
-      __syncthreads();
-      uint32_t* gh = hist_fb + round * kFbBins;
-      for (int i = tid; i < kFbBins; i += kSelThreads)
-        if (s_hist[i]) atomicAdd(&gh[i], s_hist[i]);
-      if (!grid_barrier(st, epoch, stall != 0)) { leave(); return; }
-      for (int i = tid; i < kFbBins; i += kSelThreads) s_hist[i] = __ldcg(gh + i);
-      __syncthreads();
-      find_from_top<kFbBins>([&](int i) { return s_hist[i]; }, rank, scratch, res);
-      fixed |= res[0] << sh;
-      above += res[1];
-      rank -= res[1];
-      __syncthreads();
-    }
-    tau = fixed;
-    n_greater = above;
-  } else if (mode == 0u) {
-    // ---- further levels of at most 11 bits over the candidates that match so far ----
-    const uint32_t lo_key = __ldcg(&st->lo_key);
-    uint32_t shift = __ldcg(&st->shiftA), pre = __ldcg(&st->binA), rank = __ldcg(&st->rankA);
-    uint32_t above_c = __ldcg(&st->aboveA);
-    for (int level = 0; shift > 0; ++level) {
-      const uint32_t nb = shift < 11u ? shift : 11u, ns = shift - nb;
-      uint32_t* gh = hist_b + level * kFbBins;
-      for (int c = blockIdx.x * kSelThreads + tid; c < tiles; c += gridDim.x * kSelThreads) {
-        for_slot_keys<DT>(slots, c, __ldg(cand_cnt + c), [&](uint32_t key) {
-          const uint32_t rel = key - lo_key;
-          if ((rel >> shift) == pre) atomicAdd(&gh[(rel >> ns) & ((1u << nb) - 1u)], 1u);
-        });
-      }
-      if (!grid_barrier(st, epoch, stall != 0)) { leave(); return; }
-      for (int i = tid; i < kFbBins; i += kSelThreads) s_hist[i] = __ldcg(gh + i);
-      __syncthreads();
-      find_from_top<kFbBins>([&](int i) { return s_hist[i]; }, rank, scratch, res);
-      pre = (pre << nb) | res[0];
-      above_c += res[1];
-      rank -= res[1];
-      shift = ns;
-      __syncthreads();
-    }
-    tau = lo_key + pre;
-    n_greater = __ldcg(&st->above_total) + above_c;
-  } else {
-    tau = hdr->threshold_key;
-  }
-  const bool nz = drop_zeros && tau == 0u;       // store variant without kept zeros (see classify_kernel)
-  const bool hdr_final = mode == 2u || mode == 4u;   // the classify pass has written the header
-  if (!hdr_final && blockIdx.x == 0 && tid == 0) {
-    hdr->threshold_key = tau;
-    hdr->status = __ldcg(&st->error);
-    hdr->n_keep = nz ? static_cast<long long>(n_greater) : static_cast<long long>(k);
-    hdr->n_greater = n_greater;
-    hdr->tie_quota = nz ? 0 : static_cast<long long>(k) - n_greater;
-  }
-
-  const long long quota = hdr_final ? hdr->tie_quota : (nz ? 0 : static_cast<long long>(k) - n_greater);
-
-  // ---- per-chunk values; CTA b owns the chunks [b*per, (b+1)*per) ----
-  const int per = (tiles + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x);
-  const int c_begin = blockIdx.x * per < tiles ? blockIdx.x * per : tiles;
-  const int c_end = c_begin + per < tiles ? c_begin + per : tiles;
-  unsigned long long acc = 0;
-  if (mode == 4u) {
-    // every key inside the bracket equals the threshold (the slots may have overflowed): the
-    // classify pass's counts are the answer
-    for (int c = c_begin + tid; c < c_end; c += kSelThreads) {
-      const unsigned long long v = (static_cast<unsigned long long>(__ldg(cnt_gt + c)) << 31) | __ldg(cand_cnt + c);
-      val[c] = v;
-      acc += v;
-    }
-  } else if (mode != 1u) {
-    // one thread per chunk: the listed keys above / equal to the threshold complete the counts
-    for (int c = c_begin + tid; c < c_end; c += kSelThreads) {
-      const uint32_t cc = __ldg(cand_cnt + c), cg = __ldg(cnt_gt + c);
-      uint32_t g = cg, q = 0;
-      for_slot_keys<DT>(slots, c, cc, [&](uint32_t key) {
-        g += key > tau ? 1u : 0u;
-        q += key == tau ? 1u : 0u;
-      });
-      if (tau == 0) {         // lo_key == 1: whatever is neither above nor inside the bracket is 0
-        const long long left = n - static_cast<long long>(c) * kChunkElems;
-        q += static_cast<uint32_t>(left < kChunkElems ? left : kChunkElems) - cg - cc;
-      }
-      const unsigned long long v = (static_cast<unsigned long long>(g) << 31) | q;
-      val[c] = v;
-      acc += v;
-    }
-  } else {
-   for (int c = c_begin + warp; c < c_end; c += 32) {
-    uint32_t g = 0, q = 0;
-    {
-#pragma unroll
-      for (int u = 0; u < kTileVecs / 32; ++u) {
-        const long long base = (static_cast<long long>(c) * kTileVecs + u * 32 + lane) * EPV;
-        if (base + EPV <= n) {
-          const uint4 v = __ldg(reinterpret_cast<const uint4*>(x + base));
-          const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-          for (int i = 0; i < EPV; ++i) {
-            const uint32_t key = ((DT == 0) ? w[i % 4] : (w[i >> 1] >> (16 * (i & 1)))) & kMask;
-            g += key > tau ? 1u : 0u;
-            q += key == tau ? 1u : 0u;
-          }
-        } else {
-          for (int i = 0; i < EPV; ++i) {
-            if (base + i < n) {
-              const uint32_t key = static_cast<uint32_t>(x[base + i]) & kMask;
-              g += key > tau ? 1u : 0u;
-              q += key == tau ? 1u : 0u;
-            }
-          }
-        }
-      }
-      g = __reduce_add_sync(kFull, g);
-      q = __reduce_add_sync(kFull, q);
-    }
-    const unsigned long long v = (static_cast<unsigned long long>(g) << 31) | q;
-    if (lane == 0) { val[c] = v; acc += v; }
-   }
-  }
-  acc = warp_sum_u64(acc);
-  if (lane == 0) s_tot[warp] = acc;
-  __syncthreads();
-  if (tid == 0) {
-    unsigned long long t = 0;
-    for (int w = 0; w < 32; ++w) t += s_tot[w];
-    partial[blockIdx.x] = t;
-  }
-  if (!grid_barrier(st, epoch, stall != 0)) { leave(); return; }
-
-  // ---- exclusive scan: carry from the CTAs before, then warp w scans a sub-range ----
-  unsigned long long carry = 0;
-  {
-    unsigned long long p = 0;
-    for (int b = tid; b < static_cast<int>(blockIdx.x); b += kSelThreads) p += __ldcg(partial + b);
-    p = warp_sum_u64(p);
-    if (lane == 0) s_tot[warp] = p;
-    __syncthreads();
-    for (int w = 0; w < 32; ++w) carry += s_tot[w];
-    __syncthreads();
-  }
-  const int sub = ((per + 31) / 32 + 31) & ~31;
-  const int begin = c_begin + warp * sub < c_end ? c_begin + warp * sub : c_end;
-  const int end = begin + sub < c_end ? begin + sub : c_end;
-  unsigned long long wsum = 0;
-#pragma unroll 4
-  for (int c = begin + lane; c < end; c += 32) wsum += __ldcg(val + c);
-  wsum = warp_sum_u64(wsum);
-  if (lane == 0) s_tot[warp] = wsum;
-  __syncthreads();
-  for (int w = 0; w < warp; ++w) carry += s_tot[w];
-  for (int c0 = begin; c0 < end; c0 += 32) {
-    const int c = c0 + lane;
-    const unsigned long long v = c < end ? __ldcg(val + c) : 0ull;
-    unsigned long long incl = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned long long up = __shfl_up_sync(kFull, incl, o);
-      if (lane >= static_cast<uint32_t>(o)) incl += up;
-    }
-    if (c < end) {
-      const unsigned long long ex = carry + incl - v;
-      prefix[c] = ex;
-      const long long eq_b = static_cast<long long>(ex & 0x7FFFFFFFull);
-      const long long eq_e = static_cast<long long>((ex + v) & 0x7FFFFFFFull);
-      if (eq_b < quota && eq_e > quota) { s_bnd = c; s_bnd_prefix = ex; }
-    }
-    carry += __shfl_sync(kFull, incl, 31);
-  }
-  // The chunk inside which the tie quota ends is emitted here, with its ties ranked by index, by
-  // the first two warps of the CTA that owns it; the compaction kernels skip that chunk.
-  // Nothing is stored to the outputs once a bounded wait has given up anywhere in this call (the
-  // counts the offsets come from may then be incomplete).
-  if (tid == 0) s_err = *reinterpret_cast<volatile uint32_t*>(&st->error);
-  __syncthreads();
-  if (s_err == 0u && s_bnd >= 0 && warp < kTileWarps) {
-    const unsigned long long pb = s_bnd_prefix;
-    uint4 q[kRows];
-    load_tile<DT>(x, n, s_bnd, q);
-    compact_tile<DT, true>(x, n, q, s_bnd, tau, quota, false, static_cast<long long>(pb >> 31),
-                           static_cast<long long>(pb & kCountMask), hdr, bitmap,
-                           reinterpret_cast<E*>(values_v), offsets);
-  }
-  if (c_end == tiles && c_begin < tiles) {
-    // the CTA that owns the last chunk also writes the totals and checks them
-    __syncthreads();
-    if (tid == 0) {
-      // the sentinel entry of the block offsets = the number of stored values
-      offsets[(n + SURGEON_BLOCK - 1) >> kBlockShift] =
-          nz ? static_cast<uint32_t>(hdr_final ? hdr->n_greater : n_greater) : k;
-      unsigned long long total = 0;
-      for (int b = 0; b <= static_cast<int>(blockIdx.x); ++b) total += __ldcg(partial + b);
-      prefix[tiles] = total;
-      const long long gt_all = static_cast<long long>(total >> 31);
-      const long long eq_all = static_cast<long long>(total & 0x7FFFFFFFull);
-      const long long ng = hdr_final ? hdr->n_greater : static_cast<long long>(n_greater);
-      const long long want = nz ? ng : static_cast<long long>(k);
-      const long long kept = gt_all + (eq_all < quota ? eq_all : quota);
-      // every mode and every barrier of this kernel is behind us: whatever gave up shows now
-      const uint32_t err = *reinterpret_cast<volatile uint32_t*>(&st->error);
-      if (err) atomicMax(&hdr->status, err);
-      else if (gt_all != ng || kept != want)
-        atomicMax(&hdr->status, static_cast<uint32_t>(SURGEON_ERR_INTERNAL));
-    }
-  }
-}
-
-// ---- compaction -----------------------------------------------------------------------------
 
 // Keep only the lowest `allowed` set bits of `m`.
 __device__ __forceinline__ uint32_t lowest_set_bits(uint32_t m, long long allowed) {
@@ -985,484 +246,1105 @@ __device__ __forceinline__ uint32_t lowest_set_bits(uint32_t m, long long allowe
   return m;
 }
 
-// Emits one tile.  SLOW = false: every tie of the tile is kept, or none is (`ties`), so one
-// decision per element suffices.  SLOW = true: the tie quota ends inside this tile; ties are
-// ranked by flat index.  Nothing is exchanged between CTAs.
-template <int DT, bool SLOW>
-__device__ __forceinline__ void compact_tile(const typename Elem<DT>::type* __restrict__ x,
-                                             long long n, const uint4 (&q)[kRows], int tile,
-                                             uint32_t tau, long long quota, bool ties,
-                                             long long gt_tile_before, long long eq_tile_before,
-                                             surgeon_header* __restrict__ hdr,
-                                             uint32_t* __restrict__ bitmap,
-                                             typename Elem<DT>::type* __restrict__ values,
-                                             uint32_t* __restrict__ offsets) {
-  using E = typename Elem<DT>::type;
-  constexpr uint32_t kMask = Elem<DT>::kKeyMask;
-  constexpr int EPV = 16 / sizeof(E);          // elements per lane and row: 4 (fp32) / 8 (bf16)
-  constexpr int ROW = 32 * EPV;                // elements per row: 128 / 256
-  constexpr int WPR = ROW / 32;                // bitmap words per row: 4 / 8
-  constexpr int LPW = 32 / EPV;                // lanes per bitmap word: 8 / 4
-  constexpr int BPR = ROW / SURGEON_BLOCK;     // offset blocks per row: 1 / 2
-  constexpr uint32_t kEMask = (1u << EPV) - 1u;
-  __shared__ uint32_t s_gt[kTileWarps], s_eq[kTileWarps];
+__device__ __forceinline__ unsigned long long warp_incl_u64(unsigned long long v) {
   const uint32_t lane = lane_id();
-  const int warp = threadIdx.x >> 5;
-  const long long n_blocks = (n + SURGEON_BLOCK - 1) >> kBlockShift;
-  const long long n_words = (n + 31) / 32;
-  const int my_word = lane / LPW;
-  const int my_shift = EPV * (lane % LPW);
-  const long long row0 = (static_cast<long long>(tile) * kTileWarps + warp) * kRows;
-
-  // per row and lane EPV decisions: g = kept for sure, e = tie at the threshold (SLOW only)
-  uint32_t g_all = 0, e_all = 0;      // kRows fields of EPV bits
 #pragma unroll
-  for (int r = 0; r < kRows; ++r) {
-    const long long base = (row0 + r) * ROW + static_cast<long long>(lane) * EPV;
-    const uint32_t w[4] = {q[r].x, q[r].y, q[r].z, q[r].w};
-    uint32_t g = 0, e = 0;
-#pragma unroll
-    for (int i = 0; i < EPV; ++i) {
-      const uint32_t bits = (DT == 0) ? w[i % 4] : (w[i >> 1] >> (16 * (i & 1)));
-      const uint32_t key = bits & kMask;
-      const bool valid = base + i < n;
-      if (SLOW) {
-        g |= (valid && key > tau) ? (1u << i) : 0u;
-        e |= (valid && key == tau) ? (1u << i) : 0u;
-      } else {
-        g |= (valid && (key > tau || (ties && key == tau))) ? (1u << i) : 0u;
-      }
-    }
-    g_all |= g << (EPV * r);
-    e_all |= e << (EPV * r);
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long up = __shfl_up_sync(kFull, v, o);
+    if (lane >= static_cast<uint32_t>(o)) v += up;
   }
-  const uint32_t gt_warp = __reduce_add_sync(kFull, __popc(g_all));
-  const uint32_t eq_warp = SLOW ? __reduce_add_sync(kFull, __popc(e_all)) : 0u;
-  if (lane == 0) { s_gt[warp] = gt_warp; s_eq[warp] = eq_warp; }
-  asm volatile("bar.sync 1, %0;" ::"n"(kCompactThreads) : "memory");   // the tile's two warps only
-
-  long long gt_before = gt_tile_before, eq_before = eq_tile_before;
-#pragma unroll
-  for (int w = 0; w < kTileWarps; ++w) {
-    if (w < warp) { gt_before += s_gt[w]; eq_before += s_eq[w]; }
-  }
-  // kept before = all greater + the ties that fit the quota.  In the fast path the kept ties of
-  // this tile are already inside the "greater" counts and eq_before stays the tile's value.
-  long long kept_before = gt_before + (eq_before < quota ? eq_before : quota);
-
-  uint32_t my_words[WPR];      // lane r keeps the bitmap words of row r
-  uint32_t my_off[BPR];        // and the offsets of its blocks
-  uint32_t my_cnt[BPR];
-#pragma unroll
-  for (int j = 0; j < WPR; ++j) my_words[j] = 0;
-#pragma unroll
-  for (int j = 0; j < BPR; ++j) { my_off[j] = 0; my_cnt[j] = 0; }
-
-  if (row0 * ROW < n) {
-#pragma unroll
-    for (int r = 0; r < kRows; ++r) {
-      uint32_t keep = (g_all >> (EPV * r)) & kEMask;
-      if (SLOW) {
-        const uint32_t e = (e_all >> (EPV * r)) & kEMask;
-        const uint32_t ec = __popc(e);
-        const uint32_t before = warp_excl_scan(ec);      // ties of this row in lower lanes
-        keep |= lowest_set_bits(e, quota - eq_before - before);
-        eq_before += warp_sum(ec);
-      }
-      // bitmap words of the row, known to every lane
-      const uint32_t shifted = keep << my_shift;
-      uint32_t words[WPR];
-#pragma unroll
-      for (int j = 0; j < WPR; ++j)
-        words[j] = __reduce_or_sync(kFull, my_word == j ? shifted : 0u);
-      uint32_t pre = 0, total = 0, half = 0;
-#pragma unroll
-      for (int j = 0; j < WPR; ++j) {
-        const uint32_t pc = __popc(words[j]);
-        if (j < my_word) pre += pc;
-        if (j == my_word) pre += __popc(words[j] & ((1u << my_shift) - 1u));
-        if (j < WPR / 2) half += pc;
-        total += pc;
-      }
-      if (static_cast<int>(lane) == r) {
-#pragma unroll
-        for (int j = 0; j < WPR; ++j) my_words[j] = words[j];
-        my_off[0] = static_cast<uint32_t>(kept_before);
-        if (BPR == 2) {
-          my_off[BPR - 1] = static_cast<uint32_t>(kept_before) + half;
-          my_cnt[0] = half;
-          my_cnt[BPR - 1] = total - half;
-        } else {
-          my_cnt[0] = total;
-        }
-      }
-      // packed values: consecutive kept elements go to consecutive addresses
-      E* dst = values + kept_before + pre;
-      const uint32_t w[4] = {q[r].x, q[r].y, q[r].z, q[r].w};
-#pragma unroll
-      for (int i = 0; i < EPV; ++i) {
-        if ((keep >> i) & 1u) {
-          if (SURGEON_IN_BOUNDS(dst - values, hdr->n_keep, &hdr->status))
-            *dst = (DT == 0) ? static_cast<E>(w[i % 4])
-                             : static_cast<E>((w[i >> 1] >> (16 * (i & 1))) & 0xFFFFu);
-          ++dst;
-        }
-      }
-      kept_before += total;
-    }
-    // lanes 0..kRows-1 store the words and offsets of their rows: contiguous 16-byte pieces
-    if (lane < kRows) {
-      const long long row = row0 + lane;
-      const long long w0 = row * WPR;
-      if (w0 + WPR <= n_words) {
-#pragma unroll
-        for (int j = 0; j < WPR; j += 4)
-          *reinterpret_cast<uint4*>(bitmap + w0 + j) =
-              make_uint4(my_words[j], my_words[j + 1], my_words[j + 2], my_words[j + 3]);
-      } else {
-#pragma unroll
-        for (int j = 0; j < WPR; ++j)
-          if (w0 + j < n_words) bitmap[w0 + j] = my_words[j];
-      }
-#pragma unroll
-      for (int j = 0; j < BPR; ++j) {
-        const long long blk = row * BPR + j;
-        if (blk < n_blocks) {
-          offsets[blk] = my_off[j];
-          if (blk == n_blocks - 1) {
-            const long long total = static_cast<long long>(my_off[j]) + my_cnt[j];
-            offsets[n_blocks] = static_cast<uint32_t>(total);
-            if (total != hdr->n_keep)
-              atomicMax(&hdr->status, static_cast<uint32_t>(SURGEON_ERR_INTERNAL));
-          }
-        }
-      }
-    }
-  }
+  return v;
 }
 
+// ---- emit one chunk -------------------------------------------------------------------------------
+// before = (elements above the threshold before the chunk) << 32 | (ties before it); n_eq = its ties.
+// True when the chunk's place in the ring has been written to.
 template <int DT>
-__device__ __forceinline__ void load_tile(const typename Elem<DT>::type* __restrict__ x,
-                                          long long n, int tile, uint4 (&q)[kRows]) {
-  constexpr int EPV = 16 / sizeof(typename Elem<DT>::type);
-  constexpr int ROW = 32 * EPV;
-  const long long row0 = (static_cast<long long>(tile) * kTileWarps + (threadIdx.x >> 5)) * kRows;
-#pragma unroll
-  for (int r = 0; r < kRows; ++r) {
-    const long long base = (row0 + r) * ROW + static_cast<long long>(lane_id()) * EPV;
-    if (base + EPV <= n) {
-      q[r] = __ldg(reinterpret_cast<const uint4*>(x + base));
-    } else {
-      uint32_t t[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-        t[i] = (i < EPV && base + i < n) ? static_cast<uint32_t>(x[base + i]) : 0u;
-      if (DT == 0) q[r] = make_uint4(t[0], t[1], t[2], t[3]);
-      else q[r] = make_uint4(t[0] | (t[1] << 16), t[2] | (t[3] << 16), t[4] | (t[5] << 16),
-                             t[6] | (t[7] << 16));
-    }
-  }
-}
-
-// True when a bounded wait of the select gave up or a self-check failed (uniform over the CTA); the
-// status reaches the header, and the caller stores nothing: offsets taken from incomplete counts
-// could point past the end of `values`.
-__device__ __forceinline__ bool gave_up(surgeon_header* __restrict__ hdr, const uint32_t* __restrict__ err) {
-  const uint32_t e = __ldcg(err);
-  const uint32_t s = *reinterpret_cast<volatile uint32_t*>(&hdr->status);
-  if (e && threadIdx.x == 0) atomicMax(&hdr->status, e);
-  return (e | s) != 0u;
-}
-
-// One small CTA per tile: used for tensors too small for the streaming kernel.  The one tile
-// inside which the tie quota ends (if any) is left to the count kernel.
-template <int DT>
-__global__ void __launch_bounds__(kCompactThreads)
-compact_small_kernel(const void* __restrict__ xv, long long n, surgeon_header* __restrict__ hdr,
-               uint32_t* __restrict__ bitmap, void* __restrict__ values_v,
-               uint32_t* __restrict__ offsets, const unsigned long long* __restrict__ prefix,
-               const uint32_t* __restrict__ err) {
+__device__ __forceinline__ bool emit_chunk(const PruneArgs& a, unsigned char* region, unsigned char* stage,
+                                           int chunk, uint32_t tau, long long quota,
+                                           unsigned long long before, uint32_t n_eq, long long n_stored) {
   using E = typename Elem<DT>::type;
-  const E* __restrict__ x = reinterpret_cast<const E*>(xv);
-  const int tile = blockIdx.x;
-  uint4 q[kRows];
-  load_tile<DT>(x, n, tile, q);     // in flight while the header and the scan entries arrive
-  if (gave_up(hdr, err)) return;    // the scan may be incomplete: store nothing
-  const uint32_t tau = hdr->threshold_key;
-  const long long quota = hdr->tie_quota;
-  const unsigned long long pb = prefix[tile], pe = prefix[tile + 1];
-  const long long eq_b = static_cast<long long>(pb & kCountMask);
-  const long long eq_e = static_cast<long long>(pe & kCountMask);
-  if (eq_b < quota && eq_e > quota) return;            // boundary tile
-  compact_tile<DT, false>(x, n, q, tile, tau, quota, /*ties=*/eq_e <= quota,
-                          static_cast<long long>(pb >> 31), eq_b, hdr, bitmap,
-                          reinterpret_cast<E*>(values_v), offsets);
-}
-
-// ---- streaming compaction ---------------------------------------------------------------------
-// Same ring and lane-per-row layout as classify_kernel.  A lane builds the bitmap word(s) of its
-// row with no cross-lane traffic; one warp scan places the lanes' kept values; they are gathered
-// in the warp's part of the stage (in place) and leave as 16-byte vectors.
-template <int DT>
-__global__ void __launch_bounds__(kCsThreads, 2)
-compact_stream_kernel(const __grid_constant__ CUtensorMap xmap, const void* __restrict__ xv,
-                      long long n, long long n_rows_full, surgeon_header* __restrict__ hdr,
-                      uint32_t* __restrict__ bitmap, void* __restrict__ values_v,
-                      uint32_t* __restrict__ offsets, const unsigned long long* __restrict__ prefix,
-                      const uint32_t* __restrict__ err, int n_chunks, int n_stage_tiles) {
-  using E = typename Elem<DT>::type;
-  constexpr uint32_t kMask = Elem<DT>::kKeyMask;
   constexpr int EPR = 128 / sizeof(E);         // elements per row (= per lane): 32 / 64
   constexpr int EPV = 16 / sizeof(E);          // elements per 16-byte vector: 4 / 8
   constexpr int WPL = EPR / 32;                // bitmap words per lane: 1 / 2
   constexpr int BPC = 32 * EPR / SURGEON_BLOCK;   // offset blocks per chunk: 8 / 16
   constexpr int LPB = 32 / BPC;                // lanes per offset block: 4 / 2
-  extern __shared__ __align__(1024) unsigned char cs_smem_raw[];
-  unsigned char* ring = reinterpret_cast<unsigned char*>(
-      (reinterpret_cast<uintptr_t>(cs_smem_raw) + kCsAlign - 1) & ~(kCsAlign - 1));
-  __shared__ __align__(8) unsigned long long bars[2 * kCsStages];
-  const E* __restrict__ x = reinterpret_cast<const E*>(xv);
-  E* __restrict__ values = reinterpret_cast<E*>(values_v);
-  const int warp = threadIdx.x >> 5;
   const uint32_t lane = lane_id();
-  const uint32_t full_bar = smem_u32(bars);
-  const uint32_t empty_bar = smem_u32(bars + kCsStages);
-  if (gave_up(hdr, err)) return;   // before any load or store; the whole CTA takes the same way
-  if (threadIdx.x == 0) {
-    tc::tma_prefetch_desc(&xmap);
-    for (int s = 0; s < kCsStages; ++s) {
-      tc::mbar_init(full_bar + 8 * s, 1);
-      tc::mbar_init(empty_bar + 8 * s, kCsWarps);
+  E* __restrict__ values = reinterpret_cast<E*>(a.values);
+  uint4 q[8];
+  load_row(region, q);
+  const long long grow = static_cast<long long>(chunk) * 32 + lane;   // row index in the tensor
+  long long left = a.n - grow * EPR;
+  const int nv = left < 0 ? 0 : (left > EPR ? EPR : static_cast<int>(left));
+  const long long eq_b = static_cast<long long>(before & 0xFFFFFFFFull);
+  const long long eq_e = eq_b + n_eq;
+  // every tie of the chunk is kept, or none is; in the one chunk inside which the quota ends they
+  // are ranked by flat index (= lane, then bit)
+  const bool ties = eq_e <= quota;
+  uint32_t word[WPL];
+  mask_ge<DT, WPL>(q, nv, ties ? tau : tau + 1u, word);
+  if (!ties && eq_b < quota) {
+    uint32_t ge[WPL], ec = 0;
+    mask_ge<DT, WPL>(q, nv, tau, ge);
+#pragma unroll
+    for (int w = 0; w < WPL; ++w) { ge[w] &= ~word[w]; ec += __popc(ge[w]); }
+    long long allowed = quota - eq_b - warp_excl_scan(ec);
+#pragma unroll
+    for (int w = 0; w < WPL; ++w) {
+      word[w] |= lowest_set_bits(ge[w], allowed);
+      allowed -= __popc(ge[w]);
     }
-    tc::fence_barrier_init();
   }
-  __syncthreads();
-  const int first = blockIdx.x;
-  const int n_it = first < n_stage_tiles ? (n_stage_tiles - 1 - first) / static_cast<int>(gridDim.x) + 1 : 0;
-
-  if (warp == kCsWarps) {
-    // ---- producer ----
-    if (lane == 0) {
-      for (int it = 0; it < n_it; ++it) {
-        const int s = it % kCsStages;
-        if (it >= kCsStages && !tc::mbar_wait(empty_bar + 8 * s, ((it / kCsStages) - 1) & 1, 20)) {
-          atomicMax(&hdr->status, static_cast<uint32_t>(SURGEON_ERR_TIMEOUT));
-          break;
-        }
-        const int t = first + it * static_cast<int>(gridDim.x);
-        tc::mbar_arrive_expect_tx(full_bar + 8 * s, kCsStageBytes);
-        tc::tma_load_2d(smem_u32(ring + s * kCsStageBytes), &xmap, 0, t * kCsStageRows,
-                        full_bar + 8 * s);
-      }
-    }
-    return;
+  uint32_t cnt = 0;
+#pragma unroll
+  for (int w = 0; w < WPL; ++w) cnt += __popc(word[w]);
+  uint32_t incl = cnt;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t up = __shfl_up_sync(kFull, incl, o);
+    if (lane >= static_cast<uint32_t>(o)) incl += up;
   }
+  const uint32_t lane_pre = incl - cnt;
+  const uint32_t total = __shfl_sync(kFull, incl, 31);
+  const long long kept_before = static_cast<long long>(before >> 32) + (eq_b < quota ? eq_b : quota);
 
-  // ---- consumers ----
-  const uint32_t tau = hdr->threshold_key;
-  const long long quota = hdr->tie_quota;
-  const bool none = hdr->n_keep == 0;
-  const long long n_words = (n + 31) / 32;
-  const long long n_blocks = (n + SURGEON_BLOCK - 1) >> kBlockShift;
-  auto chunk_of = [&](int it) { return (first + it * static_cast<int>(gridDim.x)) * kCsWarps + warp; };
-  unsigned long long pb = 0, pe = 0;    // scan entries of this iteration's chunk, fetched one ahead
-  if (n_it > 0 && chunk_of(0) < n_chunks) { pb = prefix[chunk_of(0)]; pe = prefix[chunk_of(0) + 1]; }
-  for (int it = 0; it < n_it; ++it) {
-    const int s = it % kCsStages;
-    const int chunk = chunk_of(it);
-    unsigned long long pb_next = 0, pe_next = 0;
-    if (it + 1 < n_it && chunk_of(it + 1) < n_chunks) {
-      pb_next = prefix[chunk_of(it + 1)];
-      pe_next = prefix[chunk_of(it + 1) + 1];
-    }
-    if (!tc::mbar_wait(full_bar + 8 * s, (it / kCsStages) & 1, 20)) {
-      if (lane == 0) atomicMax(&hdr->status, static_cast<uint32_t>(SURGEON_ERR_TIMEOUT));
-      break;
-    }
-    unsigned char* region = ring + s * kCsStageBytes + warp * 4096;   // this warp's 32 rows
-    const long long eq_b = static_cast<long long>(pb & kCountMask);
-    const long long eq_e = static_cast<long long>(pe & kCountMask);
-    const bool boundary = eq_b < quota && eq_e > quota;   // left to the count kernel
-    if (chunk < n_chunks && !boundary) {
-      // ---- this lane's row: 8 vectors, un-swizzled ----
-      uint4 q[8];
-      const unsigned char* row = region + lane * 128;
-#pragma unroll
-      for (int j = 0; j < 8; ++j)
-        q[j] = *reinterpret_cast<const uint4*>(row + ((j ^ (lane & 7)) << 4));
-      const long long grow = static_cast<long long>(chunk) * 32 + lane;   // row index in the tensor
-      const long long e0 = grow * EPR;
-      long long nv = n - e0;                      // valid elements of the row
-      nv = nv < 0 ? 0 : (nv > EPR ? EPR : nv);
-      if (grow >= n_rows_full && nv > 0) {        // the ragged last row is not covered by the map
-        uint32_t t[64];
-#pragma unroll
-        for (int i = 0; i < 64; ++i) t[i] = (i < EPR && i < nv) ? static_cast<uint32_t>(x[e0 + i]) : 0u;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          if (DT == 0) q[j] = make_uint4(t[4 * j], t[4 * j + 1], t[4 * j + 2], t[4 * j + 3]);
-          else q[j] = make_uint4(t[8 * j] | (t[8 * j + 1] << 16), t[8 * j + 2] | (t[8 * j + 3] << 16),
-                                 t[8 * j + 4] | (t[8 * j + 5] << 16), t[8 * j + 6] | (t[8 * j + 7] << 16));
-        }
-      }
-      // ---- one decision per element: key >= thr ----
-      const bool ties = eq_e <= quota;            // every tie of this chunk is kept (else none is)
-      const uint32_t thr = ties ? tau : tau + 1u;
-      uint32_t word[WPL];
-#pragma unroll
-      for (int w = 0; w < WPL; ++w) word[w] = 0;
-      const uint32_t c_thr = ge_const(thr > 0x8000u ? 0x8000u : thr);   // bf16: packed pairs of keys
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const uint32_t c[4] = {q[j].x, q[j].y, q[j].z, q[j].w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          if (DT == 0) {
-            // key < thr is the sign bit of key - thr (key < 2^31, thr <= 2^31); collected by a funnel
-            // shift with element e in bit 31 - e, put back in order below
-            word[0] = __funnelshift_l((c[i] & kMask) - thr, word[0], 1);
-          } else {
-            const int pw = 4 * j + i;             // packed word of the row: elements 2pw, 2pw + 1
-            word[(pw >> 4) % WPL] |= pair_flags(c[i] & 0x7FFF7FFFu, c_thr, pw & 15);
-          }
-        }
-      }
-      if (DT != 0) {
-#pragma unroll
-        for (int w = 0; w < WPL; ++w) word[w] = pairs_to_element_order(word[w]);
-      } else {
-        word[0] = ~__brev(word[0]);
-      }
-#pragma unroll
-      for (int w = 0; w < WPL; ++w) {
-        const long long left = nv - 32 * w;
-        const uint32_t vmask = left >= 32 ? 0xFFFFFFFFu : (left <= 0 ? 0u : ((1u << left) - 1u));
-        word[w] = none ? 0u : (word[w] & vmask);
-      }
-      uint32_t cnt = 0;
-#pragma unroll
-      for (int w = 0; w < WPL; ++w) cnt += __popc(word[w]);
-      uint32_t incl = cnt;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t up = __shfl_up_sync(kFull, incl, o);
-        if (lane >= static_cast<uint32_t>(o)) incl += up;
-      }
-      const uint32_t lane_pre = incl - cnt;
-      const uint32_t total = __shfl_sync(kFull, incl, 31);
-      const long long kept_before = static_cast<long long>(pb >> 31) + (eq_b < quota ? eq_b : quota);
+  // ---- bitmap words and block offsets: coalesced ----
+  const long long n_words = (a.n + 31) / 32;
+  const long long n_blocks = (a.n + SURGEON_BLOCK - 1) >> kBlockShift;
+  const long long wi = static_cast<long long>(chunk) * 32 * WPL + lane * WPL;
+  if (WPL == 2 && wi + 1 < n_words) {
+    *reinterpret_cast<uint2*>(a.bitmap + wi) = make_uint2(word[0], word[WPL - 1]);
+  } else if (wi < n_words) {
+    a.bitmap[wi] = word[0];
+  }
+  const uint32_t off = __shfl_sync(kFull, lane_pre, (lane * LPB) & 31);
+  const long long blk = static_cast<long long>(chunk) * BPC + lane;
+  if (lane < BPC && blk < n_blocks) a.offsets[blk] = static_cast<uint32_t>(kept_before) + off;
+  if (total == 0) return false;
 
-      // ---- bitmap words and block offsets: coalesced ----
+  // ---- kept values, in packed order into shared memory, then out as 16-byte vectors ----
+  // The sequence starts `mis` elements into its place, mis = the misalignment of its destination in
+  // `values`: 16-byte vectors of the two then line up.
+  const uint32_t mis = static_cast<uint32_t>(kept_before % EPV);
+  const uint32_t most = __reduce_max_sync(kFull, cnt);
+  // Sparse rows: a loop over the set bits, which fetches each kept element from the row; its cost is
+  // that of the fullest row (about 13 instructions per element), the unrolled gather's is 5 per element
+  // of the row, kept or not.
+  const bool sparse = most <= (DT == 0 ? 12u : 26u) &&
+                      (total + mis) * sizeof(E) <= static_cast<uint32_t>(kStageBytes);
+  if (sparse) {
+    uint32_t sa = smem_u32(stage) + (lane_pre + mis) * static_cast<uint32_t>(sizeof(E));
 #pragma unroll
-      for (int w = 0; w < WPL; ++w) {
-        const long long wi = static_cast<long long>(chunk) * 32 * WPL + lane * WPL + w;
-        if (wi < n_words) bitmap[wi] = word[w];
-      }
-      const uint32_t off = __shfl_sync(kFull, lane_pre, (lane * LPB) & 31);
-      const long long blk = static_cast<long long>(chunk) * BPC + lane;
-      if (lane < BPC && blk < n_blocks) offsets[blk] = static_cast<uint32_t>(kept_before) + off;
-
-      // ---- kept values: gathered in place (packed order), then out as 16-byte vectors ----
-      __syncwarp();                                // every lane has its row in registers
-      E* outp = reinterpret_cast<E*>(region);
-      // The byte at offset a of the packed sequence lives at a ^ ((a >> 5) & 0x7C): the 32-bit word
-      // index is XORed with the index of its 128-byte row.  Without it, lanes that keep their
-      // whole row (chunks before the end of a large tie quota, e.g. the zeros of post-ReLU data at
-      // a low ratio) all start a multiple of 32 words apart and every store of the gather is a
-      // 32-way bank conflict.  The region is 4 KB-aligned, so the same expression works on the
-      // full shared-memory address.
-      auto swz = [](uint32_t p) -> uint32_t {       // the same map on element indices
-        return p ^ ((((p * static_cast<uint32_t>(sizeof(E))) >> 7) & 31u) << (DT == 0 ? 0 : 1));
-      };
-      // The sequence starts `mis` elements into the region when that fits, mis = the misalignment
-      // of its destination in `values`: 16-byte vectors of the region and of `values` then line up.
-      const uint32_t mis = static_cast<uint32_t>(kept_before % EPV);
-      const bool lined_up = total + mis <= static_cast<uint32_t>(32 * EPR);
-      const uint32_t shift = lined_up ? mis : 0u;
-      const uint32_t rbase = smem_u32(region);
-      uint32_t a = rbase + (lane_pre + shift) * static_cast<uint32_t>(sizeof(E));
-      auto put = [&](uint32_t v) {
-        const uint32_t pa = a ^ ((a >> 5) & 0x7Cu);
-        if (DT == 0) asm volatile("st.shared.u32 [%0], %1;" ::"r"(pa), "r"(v) : "memory");
-        else asm volatile("st.shared.u16 [%0], %1;" ::"r"(pa), "h"(static_cast<unsigned short>(v)) : "memory");
-        a += static_cast<uint32_t>(sizeof(E));
-      };
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const uint32_t c[4] = {q[j].x, q[j].y, q[j].z, q[j].w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          if (DT == 0) {
-            if ((word[0] >> (4 * j + i)) & 1u) put(c[i]);
-          } else {
-            const int e = 8 * j + 2 * i;
-            if ((word[(e >> 5) % WPL] >> (e & 31)) & 1u) put(c[i]);
-            if ((word[(e >> 5) % WPL] >> ((e + 1) & 31)) & 1u) put(c[i] >> 16);
-          }
-        }
-      }
-      __syncwarp();
-      if (lined_up) {
-        // slots [mis, mis + total) of the region go to gbase[mis ...]; gbase is 16-byte aligned
-        E* gbase = values + (kept_before - mis);
-        const uint32_t end = mis + total;
-        const uint32_t v_first = mis ? 1u : 0u;    // first whole vector
-        const uint32_t v_end = end / EPV;          // one past the last whole vector
-        if (mis) {
-          const uint32_t sl = mis + lane;
-          if (sl < static_cast<uint32_t>(EPV) && sl < end &&
-              SURGEON_IN_BOUNDS(kept_before - mis + sl, hdr->n_keep, &hdr->status))
-            gbase[sl] = outp[swz(sl)];
-        }
-        for (uint32_t g = v_first + lane; g < v_end; g += 32) {
-          // the four words of a vector share their row: one 16-byte load, words permuted by the XOR
-          const uint32_t la = g * 16u;
-          const uint32_t xr = (la >> 5) & 0x7Cu;
-          uint4 u = *reinterpret_cast<const uint4*>(region + (la ^ (xr & 0x70u)));
-          if (xr & 4u) { uint32_t t = u.x; u.x = u.y; u.y = t; t = u.z; u.z = u.w; u.w = t; }
-          if (xr & 8u) { uint32_t t = u.x; u.x = u.z; u.z = t; t = u.y; u.y = u.w; u.w = t; }
-          if (SURGEON_IN_BOUNDS(kept_before - mis + g * EPV + EPV - 1, hdr->n_keep, &hdr->status))
-            *reinterpret_cast<uint4*>(gbase + g * EPV) = u;
-        }
-        const uint32_t t0 = (v_end > v_first ? v_end : v_first) * EPV;
-        if (t0 + lane < end && SURGEON_IN_BOUNDS(kept_before - mis + t0 + lane, hdr->n_keep, &hdr->status))
-          gbase[t0 + lane] = outp[swz(t0 + lane)];
-      } else {
-        // a full chunk with a misaligned destination: no room for the shift, element-wise vectors
-        E* dst = values + kept_before;
-        uint32_t head = mis ? EPV - mis : 0;
-        if (head > total) head = total;
-        const uint32_t n_vec = (total - head) / EPV;
-        if (lane < head && SURGEON_IN_BOUNDS(kept_before + lane, hdr->n_keep, &hdr->status))
-          dst[lane] = outp[swz(lane)];
-        for (uint32_t v = lane; v < n_vec; v += 32) {
-          const uint32_t b = head + v * EPV;
-          uint4 o;
-          if (DT == 0) {
-            o = make_uint4(outp[swz(b)], outp[swz(b + 1)], outp[swz(b + 2)], outp[swz(b + 3)]);
-          } else {
-            o = make_uint4(outp[swz(b)] | (static_cast<uint32_t>(outp[swz(b + 1)]) << 16),
-                           outp[swz(b + 2)] | (static_cast<uint32_t>(outp[swz(b + 3)]) << 16),
-                           outp[swz(b + 4 % EPV)] | (static_cast<uint32_t>(outp[swz(b + 5 % EPV)]) << 16),
-                           outp[swz(b + 6 % EPV)] | (static_cast<uint32_t>(outp[swz(b + 7 % EPV)]) << 16));
-          }
-          if (SURGEON_IN_BOUNDS(kept_before + head + v * EPV + EPV - 1, hdr->n_keep, &hdr->status))
-            *reinterpret_cast<uint4*>(dst + head + v * EPV) = o;
-        }
-        const uint32_t done = head + n_vec * EPV;
-        if (lane < total - done && SURGEON_IN_BOUNDS(kept_before + done + lane, hdr->n_keep, &hdr->status))
-          dst[done + lane] = outp[swz(done + lane)];
+    for (int w = 0; w < WPL; ++w) {
+      uint32_t m = word[w];
+      while (m) {
+        const int e = 32 * w + __ffs(m) - 1;
+        m &= m - 1;
+        const uint32_t v = row_elem<DT>(region, e);
+        if (DT == 0) asm volatile("st.shared.u32 [%0], %1;" ::"r"(sa), "r"(v) : "memory");
+        else asm volatile("st.shared.u16 [%0], %1;" ::"r"(sa), "h"(static_cast<unsigned short>(v)) : "memory");
+        sa += static_cast<uint32_t>(sizeof(E));
       }
     }
-    tc::fence_proxy_async();     // this warp's writes to the stage precede the next TMA fill
     __syncwarp();
-    if (lane == 0) tc::mbar_arrive(empty_bar + 8 * s);
-    pb = pb_next;
-    pe = pe_next;
+    const E* outp = reinterpret_cast<const E*>(stage);
+    E* gbase = values + (kept_before - mis);
+    const uint32_t end = mis + total, v_first = mis ? 1u : 0u, v_end = end / EPV;
+    if (mis) {
+      const uint32_t sl = mis + lane;
+      if (sl < static_cast<uint32_t>(EPV) && sl < end &&
+          SURGEON_IN_BOUNDS(kept_before - mis + sl, n_stored, &a.hdr->status))
+        gbase[sl] = outp[sl];
+    }
+    for (uint32_t g = v_first + lane; g < v_end; g += 32)
+      if (SURGEON_IN_BOUNDS(kept_before - mis + g * EPV + EPV - 1, n_stored, &a.hdr->status))
+        *reinterpret_cast<uint4*>(gbase + g * EPV) = *reinterpret_cast<const uint4*>(stage + g * 16);
+    const uint32_t t0 = (v_end > v_first ? v_end : v_first) * EPV;
+    if (t0 + lane < end && SURGEON_IN_BOUNDS(kept_before - mis + t0 + lane, n_stored, &a.hdr->status))
+      gbase[t0 + lane] = outp[t0 + lane];
+    __syncwarp();                                // the staging area is this warp's next chunk's
+    return false;
+  }
+  // Dense rows: gathered in place in the chunk's own part of the ring.
+  __syncwarp();                                  // every lane has its row in registers
+  // The byte at address a of the packed sequence lives at a ^ ((a >> 5) & 0x7C): the 32-bit word
+  // index is XORed with the index of its 128-byte row.  Without it, lanes that keep their whole
+  // row (chunks before the end of a large tie quota, e.g. the zeros of post-ReLU data at a low
+  // ratio) all start a multiple of 32 words apart and every store of the gather is a 32-way
+  // bank conflict.
+  const uint32_t rbase = smem_u32(region);
+  auto swz = [](uint32_t addr) -> uint32_t { return addr ^ ((addr >> 5) & 0x7Cu); };
+  const bool lined_up = total + mis <= static_cast<uint32_t>(32 * EPR);
+  uint32_t pa = rbase + (lane_pre + (lined_up ? mis : 0u)) * static_cast<uint32_t>(sizeof(E));
+  auto put = [&](uint32_t v) {
+    if (DT == 0) asm volatile("st.shared.u32 [%0], %1;" ::"r"(swz(pa)), "r"(v) : "memory");
+    else asm volatile("st.shared.u16 [%0], %1;" ::"r"(swz(pa)), "h"(static_cast<unsigned short>(v)) : "memory");
+    pa += static_cast<uint32_t>(sizeof(E));
+  };
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const uint32_t c[4] = {q[j].x, q[j].y, q[j].z, q[j].w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (DT == 0) {
+        if ((word[0] >> (4 * j + i)) & 1u) put(c[i]);
+      } else {
+        const int e = 8 * j + 2 * i;
+        if ((word[(e >> 5) % WPL] >> (e & 31)) & 1u) put(c[i]);
+        if ((word[(e >> 5) % WPL] >> ((e + 1) & 31)) & 1u) put(c[i] >> 16);
+      }
+    }
+  }
+  __syncwarp();
+  auto elem_at = [&](uint32_t i) -> E {          // packed element i of the region
+    E v;
+    const uint32_t addr = swz(rbase + i * static_cast<uint32_t>(sizeof(E)));
+    if (DT == 0) { uint32_t u; asm volatile("ld.shared.u32 %0, [%1];" : "=r"(u) : "r"(addr) : "memory"); v = static_cast<E>(u); }
+    else { unsigned short u; asm volatile("ld.shared.u16 %0, [%1];" : "=h"(u) : "r"(addr) : "memory"); v = static_cast<E>(u); }
+    return v;
+  };
+  if (lined_up) {
+    // slots [mis, mis + total) of the region go to gbase[mis ...]; gbase is 16-byte aligned
+    E* gbase = values + (kept_before - mis);
+    const uint32_t end = mis + total;
+    const uint32_t v_first = mis ? 1u : 0u;    // first whole vector
+    const uint32_t v_end = end / EPV;          // one past the last whole vector
+    if (mis) {
+      const uint32_t sl = mis + lane;
+      if (sl < static_cast<uint32_t>(EPV) && sl < end &&
+          SURGEON_IN_BOUNDS(kept_before - mis + sl, n_stored, &a.hdr->status))
+        gbase[sl] = elem_at(sl);
+    }
+    for (uint32_t g = v_first + lane; g < v_end; g += 32) {
+      // the four words of a vector share their row: one 16-byte load, words permuted by the XOR
+      const uint32_t la = rbase + g * 16u;
+      const uint32_t xr = (la >> 5) & 0x7Cu;
+      uint4 u;
+      asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];"
+                   : "=r"(u.x), "=r"(u.y), "=r"(u.z), "=r"(u.w) : "r"(la ^ (xr & 0x70u)) : "memory");
+      if (xr & 4u) { uint32_t t = u.x; u.x = u.y; u.y = t; t = u.z; u.z = u.w; u.w = t; }
+      if (xr & 8u) { uint32_t t = u.x; u.x = u.z; u.z = t; t = u.y; u.y = u.w; u.w = t; }
+      if (SURGEON_IN_BOUNDS(kept_before - mis + g * EPV + EPV - 1, n_stored, &a.hdr->status))
+        *reinterpret_cast<uint4*>(gbase + g * EPV) = u;
+    }
+    const uint32_t t0 = (v_end > v_first ? v_end : v_first) * EPV;
+    if (t0 + lane < end && SURGEON_IN_BOUNDS(kept_before - mis + t0 + lane, n_stored, &a.hdr->status))
+      gbase[t0 + lane] = elem_at(t0 + lane);
+  } else {
+    // a full chunk with a misaligned destination: no room for the shift, element-wise vectors
+    E* dst = values + kept_before;
+    uint32_t head = mis ? EPV - mis : 0;
+    if (head > total) head = total;
+    const uint32_t n_vec = (total - head) / EPV;
+    if (lane < head && SURGEON_IN_BOUNDS(kept_before + lane, n_stored, &a.hdr->status))
+      dst[lane] = elem_at(lane);
+    for (uint32_t v = lane; v < n_vec; v += 32) {
+      const uint32_t b = head + v * EPV;
+      uint4 o;
+      if (DT == 0) {
+        o = make_uint4(elem_at(b), elem_at(b + 1), elem_at(b + 2), elem_at(b + 3));
+      } else {
+        o = make_uint4(elem_at(b) | (static_cast<uint32_t>(elem_at(b + 1)) << 16),
+                       elem_at(b + 2) | (static_cast<uint32_t>(elem_at(b + 3)) << 16),
+                       elem_at(b + 4) | (static_cast<uint32_t>(elem_at(b + 5)) << 16),
+                       elem_at(b + 6) | (static_cast<uint32_t>(elem_at(b + 7)) << 16));
+      }
+      if (SURGEON_IN_BOUNDS(kept_before + head + v * EPV + EPV - 1, n_stored, &a.hdr->status))
+        *reinterpret_cast<uint4*>(dst + head + v * EPV) = o;
+    }
+    const uint32_t done = head + n_vec * EPV;
+    if (lane < total - done && SURGEON_IN_BOUNDS(kept_before + done + lane, n_stored, &a.hdr->status))
+      dst[done + lane] = elem_at(done + lane);
+  }
+  return true;
+}
+
+// ---- searching a histogram of kSelBins bins from its top ---------------------------------------------
+// Thread t holds bin kSelBins - 1 - t (threads past the bins: 0); returns the count above its bin.
+// `total` (every thread): the sum of all bins.  One barrier inside, one due before s_warp is used again.
+__device__ __forceinline__ uint32_t count_above_mine(uint32_t b, uint32_t* s_warp, uint32_t* total) {
+  const uint32_t excl = warp_excl_scan(b);
+  const int warp = threadIdx.x >> 5;
+  if (lane_id() == 31) s_warp[warp] = excl + b;
+  __syncthreads();
+  uint32_t above = excl, all = 0;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) {
+    const uint32_t v = s_warp[w];
+    if (w < warp) above += v;
+    all += v;
+  }
+  *total = all;
+  return above;
+}
+// The bin with #(bins above) < want <= #(bins >= it): its thread stores it, the count above it and its own.
+__device__ __forceinline__ void place_rank(uint32_t b, uint32_t above, uint32_t want, uint32_t* res) {
+  if (above < want && want <= above + b) {
+    res[0] = static_cast<uint32_t>(kSelBins - 1 - static_cast<int>(threadIdx.x));
+    res[1] = above;
+    res[2] = b;
+  }
+}
+__device__ __forceinline__ uint32_t my_bin(const uint32_t* hist) {
+  return threadIdx.x < kSelBins ? hist[kSelBins - 1 - threadIdx.x] : 0u;
+}
+
+// The first n_in keys of a slot, f(key): a warp together (slots in shared memory, a few chunks per
+// warp), or one lane alone with its loads in flight together (slots in global memory, a chunk per lane).
+template <int DT, typename F>
+__device__ __forceinline__ void slot_keys_warp(const typename Elem<DT>::type* slot, uint32_t n_in, F f) {
+  for (uint32_t i = lane_id(); i < n_in; i += 32) f(static_cast<uint32_t>(slot[i]));
+}
+template <int DT, typename F>
+__device__ __forceinline__ void slot_keys_lane(const typename Elem<DT>::type* slot, uint32_t n_in, F f) {
+  constexpr uint32_t EPV = 16 / sizeof(typename Elem<DT>::type);
+  const uint4* p = reinterpret_cast<const uint4*>(slot);
+  for (uint32_t v0 = 0; v0 * EPV < n_in; v0 += 4) {
+    uint4 q[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) q[u] = (v0 + u) * EPV < n_in ? p[v0 + u] : make_uint4(0, 0, 0, 0);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const uint32_t w[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
+#pragma unroll
+      for (uint32_t e = 0; e < EPV; ++e)
+        if ((v0 + u) * EPV + e < n_in) f((DT == 0) ? w[e % 4] : (w[e >> 1] >> (16 * (e & 1))) & 0xFFFFu);
+    }
   }
 }
 
-__global__ void offsets_empty_kernel(uint32_t* offsets) { offsets[0] = 0u; }
+// ---- the kernel -----------------------------------------------------------------------------------
+// What CTA 0 answers at an exchange: the next bracket, the count of keys above it, and what to do.
+enum Step : uint32_t {
+  kRead = 0,       // count the bracket in another pass over the chunks
+  kRefine = 1,     // count it from the lists
+  kKeys = 2,       // few enough listed keys lie inside: report them
+  kZero = 3,       // the threshold is 0: whatever is neither above nor inside the last bracket is a tie
+  kOneKey = 4,     // the threshold is lo, the only key inside the last bracket: the counts stand
+  kListed = 5,     // the threshold is lo; the lists complete the counts
+  kRecount = 6,    // the threshold is lo; the lists overflowed: count once more
+};
+
+// CTA 0: the answers of a phase and the histogram of a round, before the exchange that leads to them.
+__device__ __forceinline__ void prepare_phase(const PruneArgs& a, int phase) {
+  if (phase < kSelPhases)
+    for (int i = threadIdx.x; i < kSelMaxCtas + 2; i += kThreads) a.answer[phase * (kSelMaxCtas + 2) + i].x = 0ull;
+}
+__device__ __forceinline__ void prepare_round(const PruneArgs& a, int round) {
+  if (round < kSelHists && threadIdx.x < kSelBins) a.hist[round * kSelBins + threadIdx.x] = 0u;
+}
+
+// RES: the CTA's whole range stays in the ring (at most kResidentChunks chunks per CTA).
+template <int DT, bool RES>
+__global__ void __launch_bounds__(kThreads, 1)
+prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ PruneArgs a) {
+  using E = typename Elem<DT>::type;
+  constexpr uint32_t kMask = Elem<DT>::kKeyMask;
+  constexpr uint32_t kKeyMax = kMask;
+  constexpr int EPR = 128 / sizeof(E);
+  constexpr int WPL = EPR / 32;
+  constexpr int EPV = 16 / sizeof(E);
+  constexpr int kSlot = slot_entries(DT);
+  static_assert(kSlot * sizeof(E) == kSlotBytes, "slot size");
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* ring = reinterpret_cast<unsigned char*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  unsigned char* aux = ring + kRingBytes;
+  uint32_t* hist = reinterpret_cast<uint32_t*>(aux);
+  __shared__ __align__(8) unsigned long long bars[kResidentChunks];
+  __shared__ uint32_t s_warp[kWarps];
+  __shared__ unsigned long long s_warp64[kWarps];
+  __shared__ uint32_t s_res[8];
+  __shared__ uint32_t s_tot[4];                // keys above / inside the bracket, largest key inside, largest ~key inside
+  __shared__ uint32_t s_over, s_fail, s_nkeys;
+  __shared__ unsigned long long s_ans[2];
+
+  const int tid = threadIdx.x;
+  const int warp = tid >> 5;
+  const uint32_t lane = lane_id();
+  const int G = static_cast<int>(gridDim.x);
+  const bool master = blockIdx.x == 0;
+  const int c_begin = static_cast<int>(static_cast<long long>(a.n_chunks) * blockIdx.x / G);
+  const int c_end = static_cast<int>(static_cast<long long>(a.n_chunks) * (blockIdx.x + 1) / G);
+  const int n_local = c_end - c_begin;
+  const int n_mine = warp < n_local ? (n_local - 1 - warp) / kWarps + 1 : 0;   // chunks c_begin + warp + 16 i
+  uint32_t* cnt = n_local <= kMaxLocalChunks ? reinterpret_cast<uint32_t*>(aux + kAuxCnt) : a.cnt + c_begin;
+  unsigned long long* prefix =
+      n_local <= kMaxLocalChunks ? reinterpret_cast<unsigned long long*>(aux + kAuxPrefix) : a.prefix + c_begin;
+  E* s_slots = reinterpret_cast<E*>(aux + kAuxSlots);     // RES: the chunks' slots, else a staging slot per warp
+  E* g_slots = reinterpret_cast<E*>(a.slots) + static_cast<long long>(c_begin) * kSlot;
+  const E* __restrict__ x = reinterpret_cast<const E*>(a.x);
+
+  // ---- the ring: this warp's places ----
+  unsigned char* my_ring = ring + warp * (kSlotsPerWarp * kChunkBytes);
+  const uint32_t my_bars = smem_u32(bars + warp * kSlotsPerWarp);
+  uint32_t parity = 0;                           // bit s: phase of place s's next wait
+  auto chunk_of = [&](int i) { return c_begin + warp + kWarps * i; };
+  auto issue = [&](int i) {                      // start the load of this warp's chunk i (one lane)
+    const int c = chunk_of(i), s = i % kSlotsPerWarp;
+    if (lane == 0 && static_cast<long long>(c) * 32 < a.n_rows_full) {
+      tc::mbar_arrive_expect_tx(my_bars + 8 * s, kChunkBytes);
+      tc::tma_load_2d(smem_u32(my_ring + s * kChunkBytes), &xmap, 0, c * 32, my_bars + 8 * s);
+    }
+  };
+  auto issue_first = [&]() {
+    for (int i = 0; i < n_mine && i < kSlotsPerWarp; ++i) issue(i);
+  };
+  auto arrived = [&](int i) -> bool {            // wait for it; the tensor's last, partial row is added
+    const int c = chunk_of(i), s = i % kSlotsPerWarp;
+    unsigned char* region = my_ring + s * kChunkBytes;
+    const long long row0 = static_cast<long long>(c) * 32;
+    if (row0 < a.n_rows_full) {
+      if (!tc::mbar_wait(my_bars + 8 * s, (parity >> s) & 1u)) return false;
+      parity ^= 1u << s;
+    } else {
+      for (int v = lane; v < kChunkBytes / 16; v += 32)
+        *reinterpret_cast<uint4*>(region + v * 16) = make_uint4(0, 0, 0, 0);
+      __syncwarp();
+    }
+    if (row0 + 32 > a.n_rows_full && a.n > a.n_rows_full * EPR) {
+      const int r = static_cast<int>(a.n_rows_full - row0);       // the map fills the rows past it with zeros
+      for (int e = lane; e < static_cast<int>(a.n - a.n_rows_full * EPR); e += 32) {
+        const int byte = e * static_cast<int>(sizeof(E));
+        *reinterpret_cast<E*>(region + r * 128 + (((byte >> 4) ^ (r & 7)) << 4) + (byte & 15)) =
+            x[a.n_rows_full * EPR + e];
+      }
+      __syncwarp();
+    }
+    return true;
+  };
+  // A wait for chunk i gave up: the loads behind it are waited for (with a limit) as well.
+  auto give_up = [&](int i, int step) {
+    s_fail = 1;
+    for (int u = 1; u < kSlotsPerWarp; ++u) {
+      const int j = i + u * step;
+      if (j >= 0 && j < n_mine) arrived(j);
+    }
+  };
+  // One pass over the warp's chunks in ascending order: f(i, region).
+  auto for_chunks = [&](bool loading, auto f) {
+    for (int i = 0; i < n_mine; ++i) {
+      unsigned char* region = my_ring + (i % kSlotsPerWarp) * kChunkBytes;
+      if (loading && !arrived(i)) { give_up(i, 1); break; }
+      f(i, region);
+      if (!RES && i + kSlotsPerWarp < n_mine) {
+        __syncwarp();                            // every lane has read the place
+        issue(i + kSlotsPerWarp);
+      }
+    }
+  };
+  auto drain = [&]() {                           // before leaving with the first loads under way
+    for (int i = 0; i < n_mine && i < kSlotsPerWarp; ++i) arrived(i);
+  };
+  auto quit = [&]() { if (tid == 0) atomicMax(&a.hdr->status, static_cast<uint32_t>(SURGEON_ERR_TIMEOUT)); };
+
+  // ---- set-up ----
+  if (lane == 0) {                               // a warp's barriers are its own
+    for (int s = 0; s < kSlotsPerWarp; ++s) tc::mbar_init(my_bars + 8 * s, 1);
+    tc::fence_barrier_init();
+  }
+  __syncwarp();
+  issue_first();
+  if (tid == 0) {
+    s_fail = 0;
+    s_over = 0;
+  }
+  if (tid < 4) s_tot[tid] = 0;
+  for (int i = tid; i < kSampleBytes / 16; i += kThreads) reinterpret_cast<uint4*>(aux)[i] = make_uint4(0, 0, 0, 0);
+  __syncthreads();
+
+  // ---- the sample ----
+  // A resident tensor: 2048 vectors of 32 (fp32) or 16 (bf16) bytes, one per stratum, the same for
+  // every CTA (each starts elsewhere in it, so that they do not all ask for the same lines at the
+  // same time).  More would not pay: 148 CTAs that read 8192 places took 12 us.  The margin is 4
+  // standard deviations (a miss costs a round).  A larger tensor, for which a miss is another read
+  // of it and a narrow bracket pays: every CTA takes its own 512 or 1024 strata; CTA 0's part gives
+  // a window of bins, in which the CTAs' histograms are added up (all bins together: 150 thousand
+  // additions, 4 us); the first loads are under way meanwhile.
+  uint32_t lo = 1, hi = kKeyMax;
+  int phase = 1;
+  const uint32_t n_vec = static_cast<uint32_t>(a.n / EPV);
+  constexpr int kPer = RES ? (DT == 0 ? 8 : 4) : 2;       // vectors per thread
+  constexpr int kBinShift = Elem<DT>::kKeyBits - kSampleBinsLog2;
+  constexpr float kSigmas = RES ? 4.0f : 5.0f;
+  uint4 v[kPer];
+  {
+    constexpr uint32_t kStrata = kPer * kThreads / (DT == 0 ? 2 : 1);     // of this CTA
+    const uint32_t strata = RES ? kStrata : kStrata * G;
+    const float stride = static_cast<float>(n_vec) / static_cast<float>(strata);
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      uint32_t loc = u * kThreads + tid, part = 0;
+      if (DT == 0) { part = loc & 1u; loc >>= 1; }         // two lanes share a stratum: 32 bytes
+      loc = RES ? (loc + blockIdx.x * 37u) % kStrata : blockIdx.x * kStrata + loc;
+      const float at = (static_cast<float>(loc) + static_cast<float>(hash_u32(loc) >> 8) * (1.0f / 16777216.0f)) * stride;
+      uint32_t pos = static_cast<uint32_t>(at);
+      if (DT == 0) pos = (pos & ~1u) + part;
+      v[u] = n_vec ? __ldg(reinterpret_cast<const uint4*>(a.x) + min(pos, n_vec - 1)) : make_uint4(0, 0, 0, 0);
+    }
+  }
+  if (master) {                                  // meanwhile CTA 0 prepares the exchange
+    if (tid == 0) a.hdr->status = SURGEON_OK;
+    prepare_phase(a, 1);
+    prepare_round(a, 0);
+    if (RES) {
+      __syncthreads();
+      if (tid == 0) {
+        fence_gpu();
+        word_store(a.answer, a.token, 0ull);     // phase 0: the histogram is zero, the header begun
+      }
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+    for (int e = 0; e < EPV; ++e) {
+      const uint32_t key = ((DT == 0) ? w[e % 4] : (w[e >> 1] >> (16 * (e & 1)))) & kMask;
+      const uint32_t bin = key >> kBinShift;
+      if (key) atomicAdd(&hist[bin >> 1], 1u << (16 * (bin & 1)));   // (not the zeros, half of post-ReLU data)
+    }
+  }
+  // rank of the threshold inside the sample, and a margin of some standard deviations of a binomial count
+  const float q = static_cast<float>(a.k) / static_cast<float>(a.n);
+  auto ranks = [&](float S, float sigmas, uint32_t* r_hi, uint32_t* r_lo) {
+    const float delta = sigmas * sqrtf(S * q * (1.0f - q)) + 16.0f;
+    *r_hi = (q * S - delta >= 1.0f) ? static_cast<uint32_t>(q * S - delta) : 0u;           // 0: none
+    *r_lo = (q * S + delta <= S - 1.0f) ? static_cast<uint32_t>(q * S + delta) + 1u : 0u;  // 0: none
+  };
+  constexpr float kOwn = static_cast<float>(kPer * kThreads * EPV);        // elements in this CTA's histogram
+  uint32_t r_hi, r_lo;
+  ranks(kOwn, RES ? kSigmas : 6.0f, &r_hi, &r_lo);
+  if (!RES && r_hi == 0) r_hi = 1;               // (a window: from the largest key seen)
+  if (tid < 2) s_res[tid] = tid == 0 && r_hi == 0 ? kSampleBins - 1u : 0u;
+  __syncthreads();
+  if (RES || master) {
+    // the bins of the two ranks in the CTA's own histogram
+    // thread t owns the 32 bins below 2^14 - 32 t
+    const uint4* mine = reinterpret_cast<const uint4*>(hist) + 4 * (kSampleBins / 32 - 1 - tid);
+    uint32_t sum = 0;
+    if (tid < kSampleBins / 32) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {              // (started at a lane-dependent vector: no bank conflicts)
+        const uint4 h = mine[(j + (lane >> 1)) & 3];
+        sum += (h.x & 0xFFFFu) + (h.x >> 16) + (h.y & 0xFFFFu) + (h.y >> 16) + (h.z & 0xFFFFu) + (h.z >> 16) +
+               (h.w & 0xFFFFu) + (h.w >> 16);
+      }
+    }
+    uint32_t all;
+    const uint32_t above = count_above_mine(sum, s_warp, &all);
+#pragma unroll
+    for (int which = 0; which < 2; ++which) {
+      // (a rank among the zeros lies below every counted bin: bin 0)
+      const uint32_t want = which ? r_lo : r_hi;
+      if (want && above < want && want <= above + sum) {
+        uint32_t acc = above;
+        int bin = 31;
+        for (; bin > 0; --bin) {
+          const uint32_t c = (reinterpret_cast<const uint32_t*>(mine)[bin >> 1] >> (16 * (bin & 1))) & 0xFFFFu;
+          if (acc + c >= want) break;
+          acc += c;
+        }
+        s_res[which] = static_cast<uint32_t>(kSampleBins - 32 - 32 * tid + bin);
+      }
+    }
+    __syncthreads();
+    lo = max(s_res[1] << kBinShift, 1u);
+    hi = (s_res[0] << kBinShift) | ((1u << kBinShift) - 1u);
+    if (!RES && tid == 0) {
+      fence_gpu();
+      word_store(a.answer, a.token, s_res[0]);   // phase 0 as above, and the window's top bin
+      s_ans[0] = s_res[0];
+    }
+  } else if (tid == 0) {
+    unsigned long long ans = 0;
+    if (!RES && !word_wait(a.answer, a.token, &ans)) s_fail = 1;
+    fence_gpu();
+    s_ans[0] = ans;
+  }
+  if (!RES) {
+    __syncthreads();
+    if (s_fail) { drain(); quit(); return; }
+    // the window: kSelBins bins from its top down (8 octaves; what lies lower, lies lower)
+    const int top = static_cast<int>(s_ans[0]);
+    uint32_t over_top = 0;
+    for (int i = (top >> 1) + tid; i < kSampleBins / 2; i += kThreads) {
+      const uint32_t h = hist[i];
+      over_top += (2 * i > top ? h & 0xFFFFu : 0u) + (2 * i + 1 > top ? h >> 16 : 0u);
+    }
+    over_top = warp_sum(over_top);
+    if (lane == 0 && over_top) atomicAdd(&s_tot[0], over_top);
+    if (tid < kSelBins && tid <= top) {
+      const uint32_t h = (hist[(top - tid) >> 1] >> (16 * ((top - tid) & 1))) & 0xFFFFu;
+      if (h) atomicAdd(&a.hist[kSelBins - 1 - tid], h);
+    }
+    __syncthreads();
+    if (tid == 0) {
+      fence_gpu();
+      word_store(a.arrive + phase * kSelMaxCtas + blockIdx.x, a.token, s_tot[0]);
+    }
+    if (master) {
+      int ok = 1;
+      unsigned long long n_over = 0;
+      if (tid < G) {
+        ok = word_wait(a.arrive + phase * kSelMaxCtas + tid, a.token, &n_over);
+        a.arrive[phase * kSelMaxCtas + tid].x = 0ull;
+        fence_gpu();
+      }
+      prepare_phase(a, phase + 1);
+      prepare_round(a, 1);
+      if (tid == 0) s_tot[1] = 0;
+      if (!__syncthreads_and(ok)) { drain(); quit(); return; }
+      const uint32_t w_over = __reduce_add_sync(kFull, static_cast<uint32_t>(n_over));
+      if (lane == 0 && w_over) atomicAdd(&s_tot[1], w_over);
+      const uint32_t b = tid < kSelBins ? __ldcg(a.hist + kSelBins - 1 - tid) : 0u;
+      uint32_t all;
+      ranks(kOwn * static_cast<float>(G), kSigmas, &r_hi, &r_lo);
+      const uint32_t above = count_above_mine(b, s_warp, &all) + s_tot[1];
+      if (r_hi) place_rank(b, above, r_hi, s_res);
+      if (r_lo) place_rank(b, above, r_lo, s_res + 3);
+      __syncthreads();
+      // (a rank above or below the window bounds its side of the bracket by the window's end, or not at all)
+      const int bottom = top - (kSelBins - 1);
+      const uint32_t below = s_tot[1] + all;     // ranks past this one lie below the window
+      hi = r_hi <= s_tot[1] ? kKeyMax
+           : r_hi > below   ? (static_cast<uint32_t>(max(bottom, 1)) << kBinShift) - 1u
+                            : (static_cast<uint32_t>(bottom + static_cast<int>(s_res[0])) << kBinShift) | ((1u << kBinShift) - 1u);
+      lo = r_lo == 0 || r_lo > below ? 1u
+           : r_lo <= s_tot[1]        ? static_cast<uint32_t>(top + 1) << kBinShift
+                                     : max(static_cast<uint32_t>(bottom + static_cast<int>(s_res[3])) << kBinShift, 1u);
+      if (tid == 0) {
+        fence_gpu();
+        word_store(a.answer + phase * (kSelMaxCtas + 2), a.token, lo | (static_cast<unsigned long long>(hi) << 32));
+        a.answer[0].x = 0ull;
+      }
+    } else {
+      if (tid == 0) {
+        unsigned long long ans = 0;
+        if (!word_wait(a.answer + phase * (kSelMaxCtas + 2), a.token, &ans)) s_fail = 1;
+        s_ans[1] = ans;
+      }
+      __syncthreads();
+      if (s_fail) { drain(); quit(); return; }
+      lo = static_cast<uint32_t>(s_ans[1]);
+      hi = static_cast<uint32_t>(s_ans[1] >> 32);
+    }
+    ++phase;
+  }
+
+  // ---- the threshold ----
+  // Every round counts the keys of [lo, hi] in bins of 2^shift keys, either in a pass over the chunks
+  // (kRead) or from the keys that the last such pass listed (kRefine).
+  uint32_t step = kRead, n_above = 0;            // n_above: keys above hi
+  bool listed = false, loaded = true;            // (CTA 0) the last pass's lists are complete
+  int shift = 0;
+  int round = RES ? 0 : 1;                       // (the shared sample used histogram 0)
+  uint32_t tau = 0, n_greater = 0;
+  unsigned long long before = 0;
+  for (;;) {
+  for (; step <= kRefine; ++round) {
+    const uint32_t range = hi - lo;
+    shift = max(0, 32 - __clz(range) - kSelBinsLog2);
+    __syncthreads();
+    if (tid < kSelBins) hist[tid] = 0;
+    if (step == kRead) {
+      if (tid < 4) s_tot[tid] = 0;
+      if (tid == 0) s_over = 0;
+    }
+    __syncthreads();
+    if (step == kRead) {
+      if (!RES && !loaded) {                     // the pass starts over
+        tc::fence_proxy_async();
+        __syncwarp();
+        issue_first();
+      }
+      uint32_t w_above = 0;
+      uint32_t kmax = 0, kinv = 0;               // largest key inside the bracket seen by this lane, and largest ~key
+      const uint32_t c_above = ge_const(hi + 1u), c_lo = ge_const(lo);
+      for_chunks(!RES || loaded, [&](int i, unsigned char* region) {
+        const int cl = warp + kWarps * i;        // the chunk's place in the CTA's range
+        uint4 q[8];
+        load_row(region, q);
+        // (rows and elements past the tensor's end hold key 0: below every bracket)
+        uint32_t cw[WPL], ac = 0, cc = 0;
+        if (DT == 0) {
+          // the sign bit of (hi - key) says key > hi, that of (key - lo) says key < lo (see mask_ge)
+          uint32_t aw = 0, lw = 0;
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const uint32_t w[4] = {q[j].x, q[j].y, q[j].z, q[j].w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const uint32_t key = w[e] & kMask;
+              aw = __funnelshift_l(hi - key, aw, 1);
+              lw = __funnelshift_l(key - lo, lw, 1);
+            }
+          }
+          ac = __popc(aw);
+          cw[0] = __brev(~lw & ~aw);
+        } else {
+          uint32_t ga[WPL], gl[WPL];
+#pragma unroll
+          for (int w = 0; w < WPL; ++w) { ga[w] = 0; gl[w] = 0; }
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const uint32_t w[4] = {q[j].x, q[j].y, q[j].z, q[j].w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const int pw = 4 * j + e;           // packed word of the row: elements 2pw, 2pw + 1
+              const uint32_t keys2 = w[e] & 0x7FFF7FFFu;
+              ga[(pw >> 4) % WPL] |= pair_flags(keys2, c_above, pw & 15);
+              gl[(pw >> 4) % WPL] |= pair_flags(keys2, c_lo, pw & 15);
+            }
+          }
+#pragma unroll
+          for (int w = 0; w < WPL; ++w) {
+            ac += __popc(ga[w]);
+            const uint32_t in = gl[w] & ~ga[w];
+            cw[w] = in ? pairs_to_element_order(in) : 0u;
+          }
+        }
+#pragma unroll
+        for (int w = 0; w < WPL; ++w) cc += __popc(cw[w]);
+        const uint32_t both = __reduce_add_sync(kFull, ac | (cc << 16));   // a chunk has at most 2048 elements
+        const uint32_t a_tot = both & 0xFFFFu, c_tot = both >> 16;
+        if (lane == 0) cnt[cl] = both;
+        w_above += a_tot;
+        if (c_tot > static_cast<uint32_t>(kSlot)) {
+          // Massive ties.  If the chunk's keys inside the bracket all are one key, it is counted in
+          // one go; if that holds everywhere with the same key, it is the threshold and the counts
+          // are final without a list.
+          const uint32_t k1 = one_key_of_chunk<DT>(region, cw[0], cw[WPL - 1], c_tot);
+          if (lane == 0) s_over = 1;
+          if (k1) {
+            if (lane == 0) atomicAdd(&hist[(k1 - lo) >> shift], c_tot);
+            kmax = max(kmax, k1);
+            kinv = max(kinv, ~k1);
+          } else {
+#pragma unroll
+            for (int w = 0; w < WPL; ++w) {
+              for (uint32_t m = cw[w]; m; m &= m - 1) {
+                const uint32_t key = row_elem<DT>(region, 32 * w + __ffs(m) - 1) & kMask;
+                atomicAdd(&hist[(key - lo) >> shift], 1u);
+              }
+            }
+            kmax = kinv = 0xFFFFFFFFu;
+          }
+        } else if (c_tot) {
+          // the lanes put their keys into the slot, then share the rest of the work evenly
+          E* sl = s_slots + (RES ? cl : warp) * kSlot;
+          uint32_t pos = warp_excl_scan(cc);
+#pragma unroll
+          for (int w = 0; w < WPL; ++w)
+            for (uint32_t m = cw[w]; m; m &= m - 1)
+              sl[pos++] = static_cast<E>(row_elem<DT>(region, 32 * w + __ffs(m) - 1) & kMask);
+          __syncwarp();
+          for (uint32_t t = lane; t < c_tot; t += 32) {
+            const uint32_t key = sl[t];
+            atomicAdd(&hist[(key - lo) >> shift], 1u);
+            kmax = max(kmax, key);
+            kinv = max(kinv, ~key);
+            if (!RES) g_slots[static_cast<long long>(cl) * kSlot + t] = static_cast<E>(key);
+          }
+          __syncwarp();
+        }
+      });
+      loaded = false;
+      kmax = __reduce_max_sync(kFull, kmax);
+      kinv = __reduce_max_sync(kFull, kinv);
+      if (lane == 0) {
+        if (w_above) atomicAdd(&s_tot[0], w_above);
+        if (kmax) atomicMax(&s_tot[2], kmax);
+        if (kinv) atomicMax(&s_tot[3], kinv);
+      }
+    } else {
+      auto add = [&](uint32_t key) {
+        const uint32_t rel = key - lo;           // (below lo: wraps far above the range)
+        if (rel <= range) atomicAdd(&hist[rel >> shift], 1u);
+      };
+      if (RES) {
+        for (int c = warp; c < n_local; c += kWarps) slot_keys_warp<DT>(s_slots + c * kSlot, cnt[c] >> 16, add);
+      } else {
+        for (int c = tid; c < n_local; c += kThreads)
+          slot_keys_lane<DT>(g_slots + static_cast<long long>(c) * kSlot, cnt[c] >> 16, add);
+      }
+    }
+    if (RES && round == 0 && tid == 0) {         // CTA 0 has zeroed the histograms
+      unsigned long long ignored;
+      if (!word_wait(a.answer, a.token, &ignored)) s_fail = 1;
+      fence_gpu();
+    }
+    __syncthreads();
+    if (s_fail) { quit(); return; }
+    uint32_t* gh = a.hist + round * kSelBins;
+    if (tid < kSelBins) {
+      const uint32_t h = hist[tid];
+      if (h) atomicAdd(&gh[tid], h);
+    }
+    __syncthreads();
+    if (tid == 0) {
+      // reported: keys above, whether a list overflowed, and the one key inside (0: none, ~0: several)
+      fence_gpu();
+      const uint32_t one = s_tot[2] == 0u ? 0u : (s_tot[2] == ~s_tot[3] ? s_tot[2] : 0xFFFFFFFFu);
+      word_store(a.arrive + phase * kSelMaxCtas + blockIdx.x, a.token,
+                 (static_cast<unsigned long long>(one) << 32) | s_tot[0] | (s_over << 31));
+    }
+    if (master) {
+      unsigned long long v = 0;
+      int ok = 1;
+      if (tid < G) {
+        ok = word_wait(a.arrive + phase * kSelMaxCtas + tid, a.token, &v, a.stall != 0);
+        a.arrive[phase * kSelMaxCtas + tid].x = 0ull;
+        fence_gpu();
+      }
+      prepare_phase(a, phase + 1);
+      prepare_round(a, round + 1);
+      if (!__syncthreads_and(ok)) { quit(); return; }
+      const uint32_t b = tid < kSelBins ? __ldcg(gh + kSelBins - 1 - tid) : 0u;
+      const uint32_t one = static_cast<uint32_t>(v >> 32);
+      const uint32_t w_max = __reduce_max_sync(kFull, one), w_inv = __reduce_max_sync(kFull, one ? ~one : 0u);
+      const uint32_t w_over = __any_sync(kFull, (static_cast<uint32_t>(v) >> 31) != 0u) ? 1u : 0u;
+      const uint32_t w_sum = __reduce_add_sync(kFull, static_cast<uint32_t>(v) & 0x7FFFFFFFu);
+      __shared__ uint4 s_red[kWarps];
+      if (lane == 0) s_red[warp] = make_uint4(w_sum, w_max, w_inv, w_over);
+      uint32_t n_in;
+      const uint32_t above = count_above_mine(b, s_warp, &n_in);
+      uint32_t sum = 0, key_max = 0, key_inv = 0, over = 0;
+#pragma unroll
+      for (int w = 0; w < kWarps; ++w) {
+        const uint4 u = s_red[w];
+        sum += u.x; key_max = max(key_max, u.y); key_inv = max(key_inv, u.z); over |= u.w;
+      }
+      const bool was_read = step == kRead;
+      if (was_read) { n_above = sum; listed = over == 0; }
+      const long long r = static_cast<long long>(a.k) - n_above;     // rank among the keys of [0, hi]
+      if (r < 1) {                               // the bracket lies too low: the threshold is above it
+        lo = hi + 1u; hi = kKeyMax; step = kRead;
+      } else if (r > n_in) {
+        if (lo == 1u) { step = kZero; n_above += n_in; lo = hi = 0; }   // neither above nor inside: zeros
+        else { hi = lo - 1u; lo = 1u; step = kRead; }                   // the bracket lies too high
+      } else if (was_read && key_max != 0xFFFFFFFFu && key_max == ~key_inv) {
+        step = kOneKey; lo = hi = key_max;
+      } else {
+        place_rank(b, above, static_cast<uint32_t>(r), s_res);
+        __syncthreads();
+        n_above += s_res[1];
+        lo += s_res[0] << shift;
+        hi = min(hi, lo + ((1u << shift) - 1u));
+        if (shift == 0) step = listed ? kListed : kRecount;
+        else if (!listed) step = kRead;
+        else step = s_res[2] <= static_cast<uint32_t>(kKeysAtOnce / 2) && shift <= 2 * kSelBinsLog2 ? kKeys : kRefine;
+      }
+      __syncthreads();
+      if (tid == 0) {
+        fence_gpu();                             // the cleared words and bins of what comes next
+        word_store(a.answer + phase * (kSelMaxCtas + 2), a.token, lo | (static_cast<unsigned long long>(hi) << 32));
+        word_store(a.answer + phase * (kSelMaxCtas + 2) + 1, a.token, n_above | (static_cast<unsigned long long>(step) << 32));
+        if (RES && phase == 1) a.answer[0].x = 0ull;
+      }
+    } else {
+      if (tid < 2) {
+        unsigned long long v = 0;
+        if (!word_wait(a.answer + phase * (kSelMaxCtas + 2) + tid, a.token, &v, a.stall != 0)) s_fail = 1;
+        s_ans[tid] = v;
+      }
+      __syncthreads();
+      if (s_fail) { quit(); return; }
+      lo = static_cast<uint32_t>(s_ans[0]);
+      hi = static_cast<uint32_t>(s_ans[0] >> 32);
+      n_above = static_cast<uint32_t>(s_ans[1]);
+      step = static_cast<uint32_t>(s_ans[1] >> 32);
+    }
+    ++phase;
+    if (round + 1 >= kSelHists && step <= kRefine) {   // cannot happen: a miss, three levels and a pass for ties are the most
+      if (tid == 0) atomicMax(&a.hdr->status, static_cast<uint32_t>(SURGEON_ERR_INTERNAL));
+      return;
+    }
+  }
+
+  // ---- what this CTA has above the threshold (or above its bin) and at it ----
+  if (step == kRecount) {                        // the lists overflowed: count once more from the chunks
+    __syncthreads();
+    if (!RES) {
+      tc::fence_proxy_async();
+      __syncwarp();
+      issue_first();
+    }
+    for_chunks(!RES, [&](int i, unsigned char* region) {
+      uint4 q[8];
+      load_row(region, q);
+      uint32_t ge[WPL], gt[WPL], g = 0, e = 0;   // (lo >= 1: what lies past the tensor's end is below it)
+      mask_ge<DT, WPL>(q, EPR, lo, ge);
+      mask_ge<DT, WPL>(q, EPR, lo + 1u, gt);
+#pragma unroll
+      for (int w = 0; w < WPL; ++w) { g += __popc(gt[w]); e += __popc(ge[w] & ~gt[w]); }
+      const uint32_t both = __reduce_add_sync(kFull, g | (e << 16));
+      if (lane == 0) cnt[warp + kWarps * i] = both;
+    });
+  }
+  if (tid == 0) s_nkeys = 0;
+  __syncthreads();
+  if (s_fail) { quit(); return; }
+  uint32_t n_gt = 0, n_eq = 0;
+  if (step == kListed || step == kKeys) {
+    auto report = [&](uint32_t key, uint32_t& g, uint32_t& e) {
+      if (key > hi) ++g;
+      else if (key >= lo) {
+        ++e;
+        if (step == kKeys) {
+          const uint32_t at = atomicAdd(&s_nkeys, 1u);
+          if (at < static_cast<uint32_t>(kMaxKeys)) a.keys[blockIdx.x * kMaxKeys + at] = key;
+        }
+      }
+    };
+    if (RES) {
+      for (int c = warp; c < n_local; c += kWarps) {
+        const uint32_t v = cnt[c];
+        uint32_t g = 0, e = 0;
+        slot_keys_warp<DT>(s_slots + c * kSlot, v >> 16, [&](uint32_t key) { report(key, g, e); });
+        if (lane == 0) g += v & 0xFFFFu;
+        n_gt += g;
+        n_eq += e;
+        if (step == kListed) {
+          const uint32_t both = __reduce_add_sync(kFull, g | (e << 16));
+          if (lane == 0) cnt[c] = both;
+        }
+      }
+    } else {
+      for (int c = tid; c < n_local; c += kThreads) {
+        const uint32_t v = cnt[c];
+        uint32_t g = v & 0xFFFFu, e = 0;
+        slot_keys_lane<DT>(g_slots + static_cast<long long>(c) * kSlot, v >> 16, [&](uint32_t key) { report(key, g, e); });
+        if (step == kListed) cnt[c] = g | (e << 16);
+        n_gt += g;
+        n_eq += e;
+      }
+    }
+  } else {
+    for (int c = tid; c < n_local; c += kThreads) {
+      const uint32_t v = cnt[c];
+      uint32_t g = v & 0xFFFFu, e = v >> 16;
+      if (step == kZero) {
+        const long long left = a.n - static_cast<long long>(c_begin + c) * (32 * EPR);
+        g += e;
+        e = static_cast<uint32_t>(left < 32 * EPR ? left : 32 * EPR) - g;
+        cnt[c] = g | (e << 16);
+      }
+      n_gt += g;
+      n_eq += e;
+    }
+  }
+  n_gt = warp_sum(n_gt);
+  n_eq = warp_sum(n_eq);
+  if (lane == 0) s_warp64[warp] = (static_cast<unsigned long long>(n_gt) << 32) | n_eq;
+  __syncthreads();
+  if (tid == 0) {
+    unsigned long long t = 0;
+    for (int w = 0; w < kWarps; ++w) t += s_warp64[w];
+    fence_gpu();
+    word_store(a.arrive + phase * kSelMaxCtas + blockIdx.x, a.token, t);
+  }
+
+  // ---- last exchange: the threshold, and every CTA's place ----
+  tau = lo; n_greater = n_above;
+  bool again = false;                            // a CTA has more keys than it can report: narrow the bin first
+  if (master) {
+    unsigned long long v = 0;
+    int ok = 1;
+    if (tid < G) {
+      ok = word_wait(a.arrive + phase * kSelMaxCtas + tid, a.token, &v);
+      a.arrive[phase * kSelMaxCtas + tid].x = 0ull;
+      fence_gpu();
+    }
+    prepare_phase(a, phase + 1);
+    if (step == kKeys && tid < kSelBins) hist[tid] = hist[kSelBins + tid] = 0;
+    if (!__syncthreads_and(ok)) { quit(); return; }
+    if (step == kKeys) {
+      const uint32_t n_k = tid < G ? static_cast<uint32_t>(v) : 0u;
+      uint32_t* nk = reinterpret_cast<uint32_t*>(aux + kAuxPrefix);     // [3][kSelMaxCtas]: keys, above, ties per CTA
+      if (tid < kSelMaxCtas) { nk[tid] = n_k; nk[kSelMaxCtas + tid] = 0; nk[2 * kSelMaxCtas + tid] = 0; }
+      const uint32_t w_most = __reduce_max_sync(kFull, n_k);
+      if (lane == 0) s_warp[warp] = w_most;
+      __syncthreads();
+      int most = 0;
+#pragma unroll
+      for (int w = 0; w < kWarps; ++w) most = max(most, static_cast<int>(s_warp[w]));
+      __syncthreads();
+      constexpr int kPer = kKeysPerThread;
+      again = most > kMaxKeys || most * G > kKeysAtOnce;
+      if (!again) {
+        uint32_t key[kPer];
+        int who[kPer];
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+          const int idx = u * kThreads + tid;
+          who[u] = idx / most;
+          const int i = idx - who[u] * most;
+          const bool have = who[u] < G && i < static_cast<int>(nk[min(who[u], kSelMaxCtas - 1)]);
+          key[u] = have ? __ldcg(a.keys + who[u] * kMaxKeys + i) : 0u;
+        }
+        // the rank among them: by the upper bits of key - lo, then by the rest
+        const int coarse = shift > kSelBinsLog2 ? shift - kSelBinsLog2 : 0;
+#pragma unroll
+        for (int u = 0; u < kPer; ++u)
+          if (key[u]) atomicAdd(&hist[(key[u] - lo) >> coarse], 1u);
+        __syncthreads();
+        uint32_t all;
+        uint32_t b = my_bin(hist);
+        place_rank(b, count_above_mine(b, s_warp, &all), a.k - n_above, s_res);
+        __syncthreads();
+        tau = lo + (s_res[0] << coarse);
+        n_greater = n_above + s_res[1];
+        if (coarse) {
+#pragma unroll
+          for (int u = 0; u < kPer; ++u)
+            if (key[u] >= tau && ((key[u] - tau) >> coarse) == 0u) atomicAdd(&hist[kSelBins + key[u] - tau], 1u);
+          __syncthreads();
+          b = my_bin(hist + kSelBins);
+          place_rank(b, count_above_mine(b, s_warp, &all), a.k - n_greater, s_res + 3);
+          __syncthreads();
+          tau += s_res[3];
+          n_greater += s_res[4];
+        }
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+          if (key[u] > tau) atomicAdd(&nk[kSelMaxCtas + who[u]], 1u);
+          else if (key[u] == tau) atomicAdd(&nk[2 * kSelMaxCtas + who[u]], 1u);
+        }
+        __syncthreads();
+        if (tid < G)
+          v = ((v >> 32 << 32) + (static_cast<unsigned long long>(nk[kSelMaxCtas + tid]) << 32)) | nk[2 * kSelMaxCtas + tid];
+      }
+    }
+    // exclusive scan over the CTAs
+    const unsigned long long incl = warp_incl_u64(v);
+    if (lane == 31) s_warp64[warp] = incl;
+    __syncthreads();
+    unsigned long long all = 0, base = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+      if (w < warp) base += s_warp64[w];
+      all += s_warp64[w];
+    }
+    const bool nz = a.drop_zeros && tau == 0u;   // store variant without kept zeros
+    const long long quota = nz ? 0 : static_cast<long long>(a.k) - n_greater;
+    const long long n_stored = nz ? static_cast<long long>(n_greater) : static_cast<long long>(a.k);
+    const long long eq_all = static_cast<long long>(all & 0xFFFFFFFFull);
+    // self-check: offsets taken from wrong counts could point past the end of `values`, so nothing
+    // is stored then
+    const bool sound = static_cast<long long>(all >> 32) == n_greater && quota >= 0 &&
+                       n_greater + (eq_all < quota ? eq_all : quota) == n_stored;
+    const uint32_t verdict = again ? 1u : (sound ? 0u : 2u);
+    if (step == kKeys) {                         // (the cleared words of a further round)
+      if (tid == 0) fence_gpu();
+      __syncthreads();
+    }
+    if (tid < G) word_store(a.answer + phase * (kSelMaxCtas + 2) + 2 + tid, a.token, base + incl - v);
+    if (tid == 0) {
+      word_store(a.answer + phase * (kSelMaxCtas + 2), a.token, tau | (static_cast<unsigned long long>(n_greater) << 32));
+      word_store(a.answer + phase * (kSelMaxCtas + 2) + 1, a.token, verdict);
+      if (verdict == 0u) {
+        a.hdr->threshold_key = tau;
+        a.hdr->n_keep = n_stored;
+        a.hdr->n_greater = n_greater;
+        a.hdr->tie_quota = quota;
+        a.offsets[(a.n + SURGEON_BLOCK - 1) >> kBlockShift] = static_cast<uint32_t>(n_stored);   // the sentinel entry
+      } else if (verdict == 2u) {
+        atomicMax(&a.hdr->status, static_cast<uint32_t>(SURGEON_ERR_INTERNAL));
+      }
+    }
+    before = 0;                                  // CTA 0's chunks are the first
+    if (verdict == 2u) return;
+  } else {
+    __shared__ unsigned long long s_last[3];
+    if (tid < 3) {
+      unsigned long long v = 0;
+      const int which = tid < 2 ? tid : 2 + static_cast<int>(blockIdx.x);
+      if (!word_wait(a.answer + phase * (kSelMaxCtas + 2) + which, a.token, &v)) s_fail = 1;
+      s_last[tid] = v;
+    }
+    __syncthreads();
+    if (s_fail) { quit(); return; }
+    if (s_last[1] == 2ull) return;
+    again = s_last[1] == 1ull;
+    tau = static_cast<uint32_t>(s_last[0]);
+    n_greater = static_cast<uint32_t>(s_last[0] >> 32);
+    before = s_last[2];
+  }
+  ++phase;
+  if (!again) break;
+  step = kRefine;
+  }
+  const bool nz = a.drop_zeros && tau == 0u;     // store variant without kept zeros
+  const long long quota = nz ? 0 : static_cast<long long>(a.k) - n_greater;
+  const long long n_stored = nz ? static_cast<long long>(n_greater) : static_cast<long long>(a.k);
+
+  // ---- per-chunk counts and places ----
+  if (RES && step == kKeys) {
+    for (int c = warp; c < n_local; c += kWarps) {
+      const uint32_t v = cnt[c];
+      uint32_t both = 0;
+      slot_keys_warp<DT>(s_slots + c * kSlot, v >> 16, [&](uint32_t key) { if (key >= tau) both += key > tau ? 1u : 0x10000u; });
+      both = __reduce_add_sync(kFull, both);
+      if (lane == 0) cnt[c] = (v & 0xFFFFu) + both;
+    }
+    __syncthreads();
+  }
+  unsigned long long carry = before;
+  for (int c0 = 0; c0 < n_local; c0 += kThreads) {
+    const int c = c0 + tid;
+    uint32_t v = c < n_local ? cnt[c] : 0u;
+    if (!RES && step == kKeys && c < n_local) {
+      const uint32_t n_in = v >> 16;
+      v &= 0xFFFFu;
+      slot_keys_lane<DT>(g_slots + static_cast<long long>(c) * kSlot, n_in, [&](uint32_t key) { if (key >= tau) v += key > tau ? 1u : 0x10000u; });
+      cnt[c] = v;
+    }
+    const unsigned long long val = (static_cast<unsigned long long>(v & 0xFFFFu) << 32) | (v >> 16);
+    const unsigned long long incl = warp_incl_u64(val);
+    if (lane == 31) s_warp64[warp] = incl;
+    __syncthreads();
+    unsigned long long base = carry;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+      if (w < warp) base += s_warp64[w];
+      carry += s_warp64[w];
+    }
+    if (c < n_local) prefix[c] = base + incl - val;
+    __syncthreads();
+  }
+
+  // ---- emit: the chunks still in the ring first, then backwards through the rest ----
+  unsigned char* stage = aux + warp * kStageBytes;
+  for (int i = n_mine - 1; i >= 0; --i) {
+    const int c = chunk_of(i);
+    const bool in_ring = i + kSlotsPerWarp >= n_mine;
+    if (!RES && !in_ring && !arrived(i)) {
+      atomicMax(&a.hdr->status, static_cast<uint32_t>(SURGEON_ERR_TIMEOUT));
+      give_up(i, -1);
+      break;
+    }
+    const bool written =
+        emit_chunk<DT>(a, my_ring + (i % kSlotsPerWarp) * kChunkBytes, stage, c, tau, quota,
+                   prefix[c - c_begin], cnt[c - c_begin] >> 16, n_stored);
+    if (!RES && i >= kSlotsPerWarp) {
+      if (written) tc::fence_proxy_async();      // this warp's writes to the place precede the next TMA fill
+      __syncwarp();
+      issue(i - kSlotsPerWarp);
+    }
+  }
+}
+
+// n_keep == 0 (ratio 1, or an empty tensor): nothing to select.
+__global__ void header_empty_kernel(surgeon_header* hdr, uint32_t sentinel, uint32_t* offsets,
+                                    long long n_blocks) {
+  offsets[n_blocks] = 0u;                        // the sentinel entry of the block offsets
+  hdr->threshold_key = sentinel;
+  hdr->status = SURGEON_OK;
+  hdr->n_keep = 0;
+  hdr->n_greater = 0;
+  hdr->tie_quota = 0;
+}
 
 // ---- decompress -------------------------------------------------------------------------------
 
@@ -1502,17 +1384,29 @@ using TmaEncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, 
                                  const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// The tensor as rows of 128 bytes (32 words), box = one ring stage, 128-byte swizzle.
+// The tensor as rows of 128 bytes (32 words), box = one chunk, 128-byte swizzle.
 bool make_row_map(const void* x, long long n_rows_full, CUtensorMap* map) {
   const TmaEncodeFn encode = reinterpret_cast<TmaEncodeFn>(tensor_map_encode_fn());
   if (!encode) return false;
   const cuuint64_t dims[2] = {32, static_cast<cuuint64_t>(n_rows_full)};
   const cuuint64_t strides[1] = {128};
-  const cuuint32_t box[2] = {32, static_cast<cuuint32_t>(kCsStageRows)};
+  const cuuint32_t box[2] = {32, 32};
   const cuuint32_t estr[2] = {1, 1};
   return encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, const_cast<void*>(x), dims, strides, box,
                 estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// A value that no other call of this or another process carries (see grid_arrive).
+unsigned long long next_token() {
+  static std::atomic<unsigned long long> counter{[] {
+    std::random_device rd;
+    const unsigned long long t = static_cast<unsigned long long>(
+        std::chrono::steady_clock::now().time_since_epoch().count());
+    return ((static_cast<unsigned long long>(rd()) << 32) | rd()) ^ (t << 20);
+  }()};
+  unsigned long long v = counter.fetch_add(1, std::memory_order_relaxed);
+  return v ? v : counter.fetch_add(1, std::memory_order_relaxed);
 }
 
 template <int DT>
@@ -1520,115 +1414,49 @@ cudaError_t run_prune_compact(const void* x, long long n, long long k, int drop_
                               const surgeon_compressed& out, void* workspace,
                               cudaStream_t stream) {
   using E = typename Elem<DT>::type;
-  constexpr int VEC = 16 / static_cast<int>(sizeof(E));
+  if (k == 0) {
+    const long long n_blocks = (n + SURGEON_BLOCK - 1) >> kBlockShift;
+    if (n > 0) {   // nothing is kept: an empty bitmap, and no value before any block
+      cudaError_t e = cudaMemsetAsync(out.bitmap, 0, static_cast<size_t>((n + 31) / 32) * 4, stream);
+      if (e == cudaSuccess) e = cudaMemsetAsync(out.block_offsets, 0, static_cast<size_t>(n_blocks) * 4, stream);
+      if (e != cudaSuccess) return e;
+    }
+    header_empty_kernel<<<1, 1, 0, stream>>>(out.header, Elem<DT>::kSentinel, out.block_offsets, n_blocks);
+    note_launches(1);
+    return cudaGetLastError();
+  }
   const PruneLayout L = prune_layout(n, DT);
   char* ws = static_cast<char*>(workspace);
-  SelectState* st = reinterpret_cast<SelectState*>(ws);
-  uint32_t* hist_s = reinterpret_cast<uint32_t*>(ws + L.hist_s);
-  uint32_t* hist_a = reinterpret_cast<uint32_t*>(ws + L.hist_a);
-  uint32_t* hist_b = reinterpret_cast<uint32_t*>(ws + L.hist_b);
-  uint32_t* hist_fb = reinterpret_cast<uint32_t*>(ws + L.hist_fb);
-  uint32_t* cnt_gt = reinterpret_cast<uint32_t*>(ws + L.cnt_gt);
-  uint32_t* cand_cnt = reinterpret_cast<uint32_t*>(ws + L.cand_cnt);
-  unsigned long long* val = reinterpret_cast<unsigned long long*>(ws + L.val);
-  unsigned long long* prefix = reinterpret_cast<unsigned long long*>(ws + L.prefix);
-  unsigned long long* partial = reinterpret_cast<unsigned long long*>(ws + L.partial);
-  void* slots = ws + L.slots;
-  cudaError_t e = cudaMemsetAsync(workspace, 0, L.zero_bytes, stream);
-  if (e != cudaSuccess) return e;
-  const int sms = sm_count();
-  static bool attrs_done_on[64] = {false};   // per device; a race only repeats idempotent calls
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = 0;
-  if (!attrs_done_on[dev]) {
-    e = cudaFuncSetAttribute(sample_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kHistWords * 4);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(classify_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(kCsSmem));
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(compact_stream_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(kCsSmem));
-    if (e != cudaSuccess) return e;
-    attrs_done_on[dev] = true;
-  }
-  const long long n_rows_full = n * static_cast<long long>(sizeof(E)) / 128;
-  const int n_chunks = static_cast<int>(L.tiles);
-  const int n_stage_tiles = (n_chunks + kCsWarps - 1) / kCsWarps;
-  // at least kMinTilesPerCta stages per CTA: a CTA's set-up and tail cost about two stages' time, and a
-  // small tensor then leaves SM slots to the kernels of other streams
-  const int want_ctas = (n_stage_tiles + kMinTilesPerCta - 1) / kMinTilesPerCta;
-  const int stream_grid = want_ctas < 2 * sms ? want_ctas : 2 * sms;
+  PruneArgs a;
+  a.x = x; a.n = n; a.k = static_cast<uint32_t>(k);
+  a.n_rows_full = n * static_cast<long long>(sizeof(E)) / 128;
+  a.n_chunks = static_cast<int>(L.tiles);
+  a.drop_zeros = drop_zeros; a.stall = stall;
+  a.token = next_token();
+  a.hdr = out.header; a.bitmap = out.bitmap; a.values = out.values; a.offsets = out.block_offsets;
+  a.arrive = reinterpret_cast<ulonglong2*>(ws + L.arrive);
+  a.answer = reinterpret_cast<ulonglong2*>(ws + L.answer);
+  a.keys = reinterpret_cast<uint32_t*>(ws + L.keys);
+  a.hist = reinterpret_cast<uint32_t*>(ws + L.hist);
+  a.cnt = reinterpret_cast<uint32_t*>(ws + L.cnt);
+  a.prefix = reinterpret_cast<unsigned long long*>(ws + L.prefix);
+  a.slots = ws + L.slots;
   CUtensorMap map;
-  const bool streamed = n * static_cast<long long>(sizeof(E)) >= kStreamMinBytes && make_row_map(x, n_rows_full, &map);
-
-  if (k == 0) {
-    header_empty_kernel<<<1, 1, 0, stream>>>(out.header, Elem<DT>::kSentinel, out.block_offsets,
-                                             (n + SURGEON_BLOCK - 1) >> kBlockShift);
-    note_launches(1);
-    if (n > 0) {   // nothing is kept: the scan is all zeros
-      e = cudaMemsetAsync(prefix, 0, static_cast<size_t>(L.tiles + 1) * 8, stream);
-      if (e != cudaSuccess) return e;
-    }
-  } else {
-    if (streamed) {
-      // sample: segments of 32 vectors, about 1/32 of the tensor, at most 16384 segments
-      const long long n_seg_all = (n / VEC) / 32;
-      long long n_seg = n_seg_all / 32;
-      if (n_seg < 256) n_seg = 256;
-      if (n_seg > 16384) n_seg = 16384;
-      const long long seg_stride = n_seg_all / n_seg;   // >= 1: a streamed tensor has at least 2^22 elements
-      const long long want = (n_seg + 127) / 128;
-      const int grid = static_cast<int>(want < sms ? want : sms);
-      sample_kernel<DT><<<grid, kSelThreads, kHistWords * 4, stream>>>(
-          reinterpret_cast<const uint4*>(x), n, static_cast<uint32_t>(k),
-          static_cast<uint32_t>(n_seg), static_cast<uint32_t>(seg_stride), st, hist_s);
-      classify_kernel<DT><<<stream_grid, kCsThreads, kCsSmem, stream>>>(
-          map, x, n, n_rows_full, static_cast<uint32_t>(k), st, hist_a, cnt_gt, cand_cnt, slots,
-          out.header, n_chunks, n_stage_tiles, drop_zeros);
-      note_launches(2);
-    } else {
-      // small tensor: straight to the fall-back select (mode = 1; the state is little-endian)
-      e = cudaMemsetAsync(&st->mode, 1, 1, stream);
-      if (e != cudaSuccess) return e;
-    }
-    {
-      // cooperative launch: every CTA must be resident for the grid-wide barriers
-      // list path: one thread per chunk; fall-back (known for small tensors): all SMs read x
-      const long long want = streamed ? (L.tiles + kSelThreads - 1) / kSelThreads : (L.tiles + 31) / 32;
-      const int grid = static_cast<int>(want < 1 ? 1 : (want < sms ? want : sms));
-      const void* xa = x;
-      long long na = n;
-      uint32_t ka = static_cast<uint32_t>(k);
-      surgeon_header* hdr = out.header;
-      const uint32_t* cg = cnt_gt;
-      const uint32_t* cc = cand_cnt;
-      const void* sl = slots;
-      int tiles = n_chunks;
-      uint32_t* bm = out.bitmap;
-      void* vals = out.values;
-      uint32_t* offs = out.block_offsets;
-      void* args[] = {&xa, &na, &ka, &st, &hdr, &hist_b, &hist_fb, &cg, &cc, &sl, &val, &prefix,
-                      &partial, &tiles, &bm, &vals, &offs, &drop_zeros, &stall};
-      e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(count_kernel<DT>), dim3(grid),
-                                      dim3(kSelThreads), args, 0, stream);
-      if (e != cudaSuccess) return e;
-      note_launches(1);
-    }
-  }
-  if (n == 0) {
-    offsets_empty_kernel<<<1, 1, 0, stream>>>(out.block_offsets);
-    note_launches(1);
-  } else {
-    if (streamed)
-      compact_stream_kernel<DT><<<stream_grid, kCsThreads, kCsSmem, stream>>>(
-          map, x, n, n_rows_full, out.header, out.bitmap, out.values, out.block_offsets, prefix,
-          &st->error, n_chunks, n_stage_tiles);
-    else
-      compact_small_kernel<DT><<<static_cast<unsigned>(L.tiles), kCompactThreads, 0, stream>>>(
-          x, n, out.header, out.bitmap, out.values, out.block_offsets, prefix, &st->error);
-    note_launches(1);
-  }
+  if (!make_row_map(x, a.n_rows_full > 0 ? a.n_rows_full : 1, &map)) return cudaErrorNotSupported;
+  // one chunk per warp at least: fewer CTAs make the barriers cheaper, and leave SMs to other streams
+  const int sms = sm_count() < kSelMaxCtas ? sm_count() : kSelMaxCtas;
+  const int want = (a.n_chunks + kWarps - 1) / kWarps;
+  const int grid = want < sms ? want : sms;
+  const bool resident = a.n_chunks <= grid * kResidentChunks &&
+                        (a.n_chunks + grid - 1) / grid <= kResidentChunks;
+  const void* kernel = resident ? reinterpret_cast<const void*>(prune_kernel<DT, true>)
+                                : reinterpret_cast<const void*>(prune_kernel<DT, false>);
+  cudaError_t e = allow_dynamic_smem(kernel, static_cast<int>(kPruneSmem));
+  if (e != cudaSuccess) return e;
+  void* args[] = {&map, &a};
+  e = cudaLaunchCooperativeKernel(kernel, dim3(grid), dim3(kThreads), args, kPruneSmem, stream);
+  if (e != cudaSuccess) return e;
+  note_launches(1);
   return cudaGetLastError();
 }
 

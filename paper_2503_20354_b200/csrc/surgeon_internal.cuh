@@ -29,71 +29,39 @@ constexpr int kBlockWords = SURGEON_BLOCK / 32;      // bitmap words per offset 
 static_assert((1 << kBlockShift) == SURGEON_BLOCK, "SURGEON_BLOCK must be 128");
 
 // ---- scratch of surgeon_prune_compact ---------------------------------------------------------
-// Compaction tile ("chunk") = 4 KB of input = 256 16-byte vectors: the unit one warp emits and
+// Compaction tile ("chunk") = 4 KB of input = 256 16-byte vectors: the unit one warp works on and
 // the unit of the exclusive scan that places it.
 constexpr int kTileVecs = 256;
 constexpr int64_t compact_tile_elems(int dt) { return dt == 0 ? 1024 : 2048; }
-constexpr int kBuckets = 32768;        // bins of the sample histogram (top 15 key bits)
-constexpr int kBinsA = 512;            // level A of the select among candidates: the top bits of
-                                       // (key - lo_key), shifted so that the bracket fits
-constexpr int kBinsB = 4096;           // up to two further levels of 2048 bins each
-constexpr int kFbBins = 2048;          // digit histogram of the fall-back radix select
-// Tensors below this size go straight to the fall-back select: its passes over a tensor that
-// stays in L2 finish sooner than the four dependent kernels of the sampled path.  Alone on the
-// GPU that holds up to 16-32 MB; next to other streams' kernels the fall-back's cooperative
-// grid (one CTA per 32 chunks) has to wait for them, and 4 MB is where both cases gain.
-constexpr int64_t kStreamMinBytes = 4 << 20;
+constexpr int kSelBinsLog2 = 9;        // bins of the select's histograms, over the bracket's keys
+constexpr int kSelBins = 1 << kSelBinsLog2;
+constexpr int kSelHists = 8;           // rounds of the select (2 in the common case)
+constexpr int kSampleBins = 16384;     // bins of the sample
+constexpr int kSelPhases = 12;         // grid-wide exchanges of a call (3 in the common case)
+constexpr int kSelMaxCtas = 256;
 // Candidate slots: per chunk, room for 1/16 of its elements (fp32: 32-bit keys, bf16: 16-bit).
-constexpr int slot_entries(int dt) { return dt == 0 ? 64 : 128; }
+__host__ __device__ constexpr int slot_entries(int dt) { return dt == 0 ? 64 : 128; }
 constexpr int slot_entry_bytes(int dt) { return dt == 0 ? 4 : 2; }
 
-struct SelectState {
-  uint32_t ticket_sample, ticket_classify, barrier_count, error;
-  uint32_t blo, bhi;             // bucket bracket around the threshold, predicted from the sample
-  uint32_t lo_key, hi_key;       // the same bracket as an inclusive key range (lo_key >= 1)
-  uint32_t mode;                 // 0 = threshold among the candidates, level B pending (fp32);
-                                 // 1 = bracket unusable, fall back to a radix select over x;
-                                 // 2 = threshold already final in the header;
-                                 // 4 = likewise, and every key inside the bracket equals it
-  uint32_t list_overflow;
-  uint32_t above_total, cand_total;   // keys above hi_key / inside [lo_key, hi_key]
-  uint32_t shiftA;               // level A bin of a key = (key - lo_key) >> shiftA
-  uint32_t binA, rankA, aboveA;  // level A: bin of the threshold, its rank inside, candidates above
-  uint32_t fb_prefix, fb_rank, fb_above;   // fall-back select: key bits fixed so far, rank, count above
-  uint32_t reserved0;            // (unused)
-  uint32_t cand_key_max, cand_keyinv_max;   // extremes of the keys inside the bracket: max key, max ~key
-  uint32_t pad[10];
-};
-static_assert(sizeof(SelectState) == 128, "SelectState layout");
-constexpr size_t kWsStateBytes = 256;
-
-// Byte offsets of the parts of the scratch buffer; everything in [0, zero_bytes) must be zero
-// when the first kernel starts.  Per chunk: cnt_gt = keys above the bracket, cand_cnt = keys
-// inside it (both written by the classify pass), val = (kept for sure << 31 | ties) once the
-// threshold is known, prefix = exclusive scan of val (chunks + 1 entries), slots = the keys
-// inside the bracket.  partial: one scan carry per CTA of the count kernel.
+// Byte offsets of the parts of the scratch buffer; nothing in it has to start at any value.
+// arrive / answer / keys: what the CTAs exchange; hist: the select's histograms, one per round; cnt
+// and prefix: per-chunk counts and places of CTAs with too many chunks for shared memory; slots:
+// the keys inside the bracket, per chunk.
 struct PruneLayout {
-  size_t hist_s, hist_a, hist_b, hist_fb, zero_bytes, cnt_gt, cand_cnt, val, prefix, partial,
-      slots, total;
+  size_t arrive, answer, keys, hist, cnt, prefix, slots, total;
   int64_t tiles;
 };
-constexpr size_t kMaxCountCtas = 1024;
 constexpr PruneLayout prune_layout(int64_t n, int dt) {
   PruneLayout L{};
   L.tiles = (n + compact_tile_elems(dt) - 1) / compact_tile_elems(dt);
   const size_t t = static_cast<size_t>(L.tiles);
-  size_t off = kWsStateBytes;
-  L.hist_s = off; off += static_cast<size_t>(kBuckets) * 4;
-  L.hist_a = off; off += static_cast<size_t>(kBinsA) * 4;
-  L.hist_b = off; off += static_cast<size_t>(kBinsB) * 4;
-  L.hist_fb = off; off += static_cast<size_t>(3 * kFbBins) * 4;
-  L.zero_bytes = off;
-  L.cnt_gt = off; off += t * 4;
-  L.cand_cnt = off; off += t * 4;
-  off = (off + 15) & ~static_cast<size_t>(15);
-  L.val = off; off += t * 8;
-  L.prefix = off; off += (t + 1) * 8;
-  L.partial = off; off += kMaxCountCtas * 8;
+  size_t off = 0;
+  L.arrive = off; off += static_cast<size_t>(kSelPhases) * kSelMaxCtas * 16;
+  L.answer = off; off += static_cast<size_t>(kSelPhases) * (kSelMaxCtas + 2) * 16;
+  L.keys = off; off += static_cast<size_t>(kSelMaxCtas) * 64 * 4;
+  L.hist = off; off += static_cast<size_t>(kSelHists) * kSelBins * 4;
+  L.prefix = off; off += t * 8;
+  L.cnt = off; off += t * 4;
   off = (off + 255) & ~static_cast<size_t>(255);
   L.slots = off;
   off += t * static_cast<size_t>(slot_entries(dt)) * slot_entry_bytes(dt);
