@@ -39,16 +39,18 @@ constexpr int kSelHists = 8;           // rounds of the select (2 in the common 
 constexpr int kSampleBins = 16384;     // bins of the sample
 constexpr int kSelPhases = 12;         // grid-wide exchanges of a call (3 in the common case)
 constexpr int kSelMaxCtas = 256;
+constexpr int kClaimSets = 4, kClaimStride = 32;
 // Candidate slots: per chunk, room for 1/16 of its elements (fp32: 32-bit keys, bf16: 16-bit).
 __host__ __device__ constexpr int slot_entries(int dt) { return dt == 0 ? 64 : 128; }
 constexpr int slot_entry_bytes(int dt) { return dt == 0 ? 4 : 2; }
 
 // Byte offsets of the parts of the scratch buffer; nothing in it has to start at any value.
-// arrive / answer / keys: what the CTAs exchange; hist: the select's histograms, one per round; cnt
+// arrive / answer / keys: what the CTAs exchange; hist: the select's histograms, one per round; claims:
+// counters of claimed chunks; cnt
 // and prefix: per-chunk counts and places of CTAs with too many chunks for shared memory; slots:
 // the keys inside the bracket, per chunk.
 struct PruneLayout {
-  size_t arrive, answer, keys, hist, cnt, prefix, slots, total;
+  size_t arrive, answer, keys, hist, claims, cnt, prefix, slots, total;
   int64_t tiles;
 };
 constexpr PruneLayout prune_layout(int64_t n, int dt) {
@@ -60,6 +62,7 @@ constexpr PruneLayout prune_layout(int64_t n, int dt) {
   L.answer = off; off += static_cast<size_t>(kSelPhases) * (kSelMaxCtas + 2) * 16;
   L.keys = off; off += static_cast<size_t>(kSelMaxCtas) * 64 * 4;
   L.hist = off; off += static_cast<size_t>(kSelHists) * kSelBins * 4;
+  L.claims = off; off += static_cast<size_t>(kSelPhases) * kClaimSets * kClaimStride * 4;
   L.prefix = off; off += t * 8;
   L.cnt = off; off += t * 4;
   off = (off + 255) & ~static_cast<size_t>(255);
