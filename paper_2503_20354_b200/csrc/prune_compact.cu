@@ -1478,7 +1478,7 @@ __global__ void header_empty_kernel(surgeon_header* hdr, uint32_t sentinel, uint
 // loads; a lane then puts the values of its bitmap word (a loop over the set bits, about 8
 // instructions per kept element of the fullest word) into its row of a zeroed tile, and the tile
 // leaves as 16-byte vectors.  Bound by the memory; a lane per element, with two-byte stores and two
-// shuffles and a population count each, took 2.4 times as long on 38.7 M bf16 elements (ratio 0.7).
+// shuffles and a population count each, took 53 us on 38.7 M bf16 elements (ratio 0.7), this 45.
 constexpr int kDecWarps = 8;
 constexpr int kDecElems = 1024;
 template <int DT>
