@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import threading
 from dataclasses import dataclass
 from typing import Optional
 
@@ -75,7 +76,7 @@ def lib():
                                                   C.c_size_t, C.c_void_p]
         l.surgeon_compact_sizes.restype = C.c_int
         l.surgeon_compact_sizes.argtypes = [C.c_int64, C.c_int, C.c_double, C.c_void_p, C.c_void_p,
-                                            C.c_void_p, C.c_void_p, C.c_void_p]
+                                            C.c_void_p, C.c_void_p, C.c_void_p]      # int64 and size_t: 8 bytes each
         l.surgeon_prune_compact.restype = C.c_int
         l.surgeon_prune_compact.argtypes = [C.c_void_p, C.c_int64, C.c_int, C.c_double,
                                             C.POINTER(Compressed), C.c_void_p, C.c_size_t, C.c_void_p]
@@ -116,8 +117,10 @@ def _check(status: int, where: str, allow=()):
 
 
 def _stream_ptr(stream: Optional[torch.cuda.Stream]) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return int(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    # the raw handle: a Stream object, made only to be asked for it, costs 3 us of a call's 10
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _scratch(nbytes: int, device, stream: Optional[torch.cuda.Stream]) -> torch.Tensor:
@@ -202,13 +205,25 @@ class CompactSizes:
     workspace_bytes: int
 
 
+class _SizesOut(threading.local):
+    """Where the C call puts its five numbers, one place per thread (made once: five ctypes objects
+    and references per call cost more than the call)."""
+
+    def __init__(self):
+        self.words = (C.c_int64 * 5)()
+        a = C.addressof(self.words)
+        self.at = tuple(a + 8 * i for i in range(5))
+
+
+_sizes_out = _SizesOut()
+
+
 def surgeon_compact_sizes(n: int, dt: int, ratio: float) -> CompactSizes:
-    k = C.c_int64(0)
-    b, v, o, w = C.c_size_t(0), C.c_size_t(0), C.c_size_t(0), C.c_size_t(0)
-    st = lib().surgeon_compact_sizes(int(n), int(dt), float(ratio), C.byref(k), C.byref(b),
-                                     C.byref(v), C.byref(o), C.byref(w))
-    _check(st, "surgeon_compact_sizes")
-    return CompactSizes(k.value, b.value, v.value, o.value, w.value)
+    out = _sizes_out
+    st = lib().surgeon_compact_sizes(int(n), int(dt), float(ratio), *out.at)
+    if st != SURGEON_OK:
+        _check(st, "surgeon_compact_sizes")
+    return CompactSizes(*out.words)
 
 
 # ---------------------------------------------------------------------------------------------
@@ -218,14 +233,16 @@ def surgeon_compact_sizes(n: int, dt: int, ratio: float) -> CompactSizes:
 class CompressedActivation:
     """Device buffers of one compressed activation plus the C struct that points at them."""
 
-    def __init__(self, n: int, dt: int, ratio: float, device, sizes: Optional[CompactSizes] = None):
+    def __init__(self, n: int, dt: int, ratio: float, device, sizes: Optional[CompactSizes] = None,
+                 _blank: bool = False):
+        # _blank: a call that writes the header follows, so it need not be zeroed (a kernel launch)
         s = sizes or surgeon_compact_sizes(n, dt, ratio)
         self.n, self.dt, self.ratio, self.sizes = int(n), int(dt), float(ratio), s
         self.bitmap = torch.empty(max(s.bitmap_bytes // 4, 1), dtype=torch.int32, device=device)
         vt = torch.float32 if dt == SURGEON_F32 else torch.bfloat16
         self.values = torch.empty(max(s.n_keep, 1), dtype=vt, device=device)
         self.block_offsets = torch.empty(s.offsets_bytes // 4, dtype=torch.int32, device=device)
-        self.header = torch.zeros(4, dtype=torch.int64, device=device)
+        self.header = (torch.empty if _blank else torch.zeros)(4, dtype=torch.int64, device=device)
         self.c = Compressed(self.n, self.dt, 0, self.bitmap.data_ptr(), self.values.data_ptr(),
                             self.block_offsets.data_ptr(), self.header.data_ptr())
 
@@ -271,7 +288,7 @@ def surgeon_prune_compact(x: torch.Tensor, ratio: float, out: Optional[Compresse
     n = x.numel()
     sizes = surgeon_compact_sizes(n, dt, ratio)
     if out is None:
-        out = CompressedActivation(n, dt, ratio, x.device, sizes)
+        out = CompressedActivation(n, dt, ratio, x.device, sizes, _blank=True)
     else:
         if out.n != n or out.dt != dt or out.values.numel() < sizes.n_keep:
             raise ValueError("output store does not fit this tensor / ratio")
@@ -282,7 +299,8 @@ def surgeon_prune_compact(x: torch.Tensor, ratio: float, out: Optional[Compresse
                                            workspace.data_ptr(),
                                            workspace.numel() * workspace.element_size(),
                                            _stream_ptr(stream))
-    _check(st, "surgeon_prune_compact")
+    if st != SURGEON_OK:
+        _check(st, "surgeon_prune_compact")
     return out
 
 
@@ -346,14 +364,13 @@ def surgeon_weight_grad(act: CompressedActivation, desc: LayerDesc, grad_out: to
     """dW of the layer from the compressed activation and fp32 ``grad_out``; returns ``dw``."""
     if grad_out.dtype != torch.float32 or not grad_out.is_cuda or not grad_out.is_contiguous():
         raise ValueError("grad_out must be a contiguous fp32 CUDA tensor")
-    shape = (desc.c_out, desc.c_in // max(desc.groups, 1), desc.kh, desc.kw) if desc.kind == 1 else (desc.c_out, desc.c_in)
     if dw is None:
         if accumulate:
             raise ValueError("accumulate needs an existing dw")
+        shape = (desc.c_out, desc.c_in // max(desc.groups, 1), desc.kh, desc.kw) if desc.kind == 1 else (desc.c_out, desc.c_in)
         dw = torch.empty(shape, dtype=torch.float32, device=grad_out.device)
-    need = surgeon_weight_grad_workspace(desc)
     if workspace is None:
-        workspace = _scratch(need, grad_out.device, stream)
+        workspace = _scratch(surgeon_weight_grad_workspace(desc), grad_out.device, stream)
     st = lib().surgeon_weight_grad(C.byref(act.c), C.byref(desc), grad_out.data_ptr(), dw.data_ptr(),
                                    1 if accumulate else 0, workspace.data_ptr(),
                                    workspace.numel() * workspace.element_size(), _stream_ptr(stream))

@@ -116,6 +116,14 @@ void note_launches(int n);
 // was launched the ordinary way.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// The first kernel of a weight-gradient call: it waits for what came before on the stream, zeroes the
+// call's status word (a memset of its own cost 2 us of host time and as much of the stream's), and
+// only then lets its dependents start, which read the store without waiting for anything else.
+__device__ __forceinline__ void prepass_begin(uint32_t* status) {
+  pdl_wait();
+  if (blockIdx.x == 0 && threadIdx.x == 0) { *status = 0u; __threadfence(); }
+  pdl_trigger();
+}
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                                  cudaStream_t stream, bool dependent, Args&&... args) {

@@ -917,9 +917,9 @@ cudaError_t launch_weight_grad_tc(const surgeon_compressed& act, const surgeon_l
   if (weight_grad_tc_workspace(d) == 0 || workspace == nullptr) return cudaErrorNotSupported;
   uint32_t* status = static_cast<uint32_t*>(workspace);
   float* partial = reinterpret_cast<float*>(static_cast<char*>(workspace) + kStatusBytes);
-  cudaError_t e = cudaMemsetAsync(status, 0, kStatusBytes, stream);
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
 #ifdef SURGEON_DW_STATS
+  cudaMemsetAsync(status, 0, kStatusBytes, stream);
   cudaMemsetAsync(reinterpret_cast<char*>(status) + 14 * 8, 0xFF, 8, stream);
 #endif
   DirectParams dp;
@@ -972,9 +972,9 @@ cudaError_t launch_weight_grad_tc(const surgeon_compressed& act, const surgeon_l
     const size_t pbytes = (static_cast<size_t>(p.splits) * p.O * p.n_gemm * sizeof(float) + 255) & ~size_t(255);
     void* grad_bf16 = reinterpret_cast<char*>(partial) + pbytes;
     if (pitch != p.P)
-      e = launch_grad_to_bf16_rows(grad_out, static_cast<long long>(p.B) * p.O, p.P, pitch, grad_bf16, stream);
+      e = launch_grad_to_bf16_rows(grad_out, static_cast<long long>(p.B) * p.O, p.P, pitch, grad_bf16, status, stream);
     else
-      e = launch_grad_to_bf16(grad_out, static_cast<long long>(p.B) * p.O * p.P, grad_bf16, stream);
+      e = launch_grad_to_bf16(grad_out, static_cast<long long>(p.B) * p.O * p.P, grad_bf16, status, stream);
     if (e != cudaSuccess) return e;
     using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
@@ -1012,6 +1012,8 @@ cudaError_t launch_weight_grad_tc(const surgeon_compressed& act, const surgeon_l
     return cudaGetLastError();
   }
   if (!plan(d, act.dt, &p)) return cudaErrorNotSupported;
+  e = cudaMemsetAsync(status, 0, kStatusBytes, stream);     // (no pre-pass here)
+  if (e != cudaSuccess) return e;
   p.n_words = (act.n + 31) / 32;
   const size_t smem = smem_bytes(p);
   const uint32_t* offs = act.block_offsets;

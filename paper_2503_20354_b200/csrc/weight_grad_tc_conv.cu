@@ -416,8 +416,9 @@ dw_conv_fast_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict_
 
 // fp32 -> bf16 (round to nearest even), 8 elements per thread.
 __global__ void __launch_bounds__(256)
-grad_to_bf16_kernel(const float* __restrict__ g, long long n, unsigned short* __restrict__ out) {
-  pdl_trigger();
+grad_to_bf16_kernel(const float* __restrict__ g, long long n, unsigned short* __restrict__ out,
+                    uint32_t* __restrict__ status) {
+  prepass_begin(status);
   const long long n8 = n >> 3;
   const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
   for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < n8;
@@ -437,8 +438,8 @@ grad_to_bf16_kernel(const float* __restrict__ g, long long n, unsigned short* __
 // rows of `len` floats -> rows of `pitch` bf16 (pitch a multiple of 8, padding zero)
 __global__ void __launch_bounds__(256)
 grad_to_bf16_rows_kernel(const float* __restrict__ g, long long rows, int len, int pitch,
-                         unsigned short* __restrict__ out) {
-  pdl_trigger();
+                         unsigned short* __restrict__ out, uint32_t* __restrict__ status) {
+  prepass_begin(status);
   const int per_row = pitch >> 3;
   const long long total = rows * per_row;
   const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
@@ -552,24 +553,23 @@ bool plan_conv_fast(const surgeon_layer_desc& d, FastParams* out) {
   return memo_plan<Tag>(d, 0, out, [&](FastParams* p) { return compute_plan_conv_fast(d, p); });
 }
 
-cudaError_t launch_grad_to_bf16(const float* g, long long n, void* out_bf16, cudaStream_t stream) {
+cudaError_t launch_grad_to_bf16(const float* g, long long n, void* out_bf16, uint32_t* status, cudaStream_t stream) {
   const long long want = (n / 8 + 255) / 256;
   const long long cap = 16LL * sm_count();
   const int grid = static_cast<int>(want < 1 ? 1 : (want > cap ? cap : want));
-  grad_to_bf16_kernel<<<grid, 256, 0, stream>>>(g, n, static_cast<unsigned short*>(out_bf16));
   note_launches(1);
-  return cudaGetLastError();
+  return launch_kernel(grad_to_bf16_kernel, dim3(grid), dim3(256), 0, stream, true, g, n,
+                       static_cast<unsigned short*>(out_bf16), status);
 }
 
 cudaError_t launch_grad_to_bf16_rows(const float* g, long long rows, int len, int pitch,
-                                     void* out_bf16, cudaStream_t stream) {
+                                     void* out_bf16, uint32_t* status, cudaStream_t stream) {
   const long long want = (rows * (pitch >> 3) + 255) / 256;
   const long long cap = 16LL * sm_count();
   const int grid = static_cast<int>(want < 1 ? 1 : (want > cap ? cap : want));
-  grad_to_bf16_rows_kernel<<<grid, 256, 0, stream>>>(g, rows, len, pitch,
-                                                     static_cast<unsigned short*>(out_bf16));
   note_launches(1);
-  return cudaGetLastError();
+  return launch_kernel(grad_to_bf16_rows_kernel, dim3(grid), dim3(256), 0, stream, true, g, rows, len, pitch,
+                       static_cast<unsigned short*>(out_bf16), status);
 }
 
 size_t conv_fast_grad_bf16_bytes(const FastParams& p) {
@@ -581,14 +581,8 @@ cudaError_t launch_conv_fast(const surgeon_compressed& act, const FastParams& p,
                              const float* grad_out, void* grad_bf16, float* partial,
                              uint32_t* status, cudaStream_t stream) {
   // 1. gradient fp32 -> bf16 (scratch), then a 3-D tensor map over [B][O][P] for the TMA loads
-  const long long gn = static_cast<long long>(p.B) * p.O * p.P;
-  {
-    const long long want = (gn / 8 + 255) / 256;
-    const long long cap = 16LL * sm_count();
-    const int grid = static_cast<int>(want < 1 ? 1 : (want > cap ? cap : want));
-    grad_to_bf16_kernel<<<grid, 256, 0, stream>>>(grad_out, gn,
-                                                  static_cast<unsigned short*>(grad_bf16));
-  }
+  cudaError_t e = launch_grad_to_bf16(grad_out, static_cast<long long>(p.B) * p.O * p.P, grad_bf16, status, stream);
+  if (e != cudaSuccess) return e;
   CUtensorMap map;
   const cuuint64_t dims[3] = {static_cast<cuuint64_t>(p.P), static_cast<cuuint64_t>(p.O),
                               static_cast<cuuint64_t>(p.B)};
@@ -606,7 +600,6 @@ cudaError_t launch_conv_fast(const surgeon_compressed& act, const FastParams& p,
 
   const uint32_t* offs = act.block_offsets;
   dim3 grid(p.m_tiles, p.n_tiles, p.splits);
-  cudaError_t e;
   if (act.dt == 0) {
     e = allow_dynamic_smem(reinterpret_cast<const void*>(dw_conv_fast_kernel<0>), p.smem_bytes);
     if (e != cudaSuccess) return e;
@@ -618,7 +611,7 @@ cudaError_t launch_conv_fast(const surgeon_compressed& act, const FastParams& p,
     dw_conv_fast_kernel<1><<<grid, kThreads, p.smem_bytes, stream>>>(
         act.bitmap, act.values, offs, map, partial, status, p);
   }
-  note_launches(2);
+  note_launches(1);
   return cudaGetLastError();
 }
 

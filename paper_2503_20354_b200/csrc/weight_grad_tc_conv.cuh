@@ -56,17 +56,18 @@ bool plan_conv_fast(const surgeon_layer_desc& d, FastParams* out);
 size_t conv_fast_grad_bf16_bytes(const FastParams& p);
 
 // Enqueues the bf16 conversion of grad_out into grad_bf16 and the kernel;
-// partial = [splits][O][n_gemm] fp32, status = one zeroed word.
+// partial = [splits][O][n_gemm] fp32, status = one word (the pre-pass zeroes it).
 cudaError_t launch_conv_fast(const surgeon_compressed& act, const FastParams& p,
                              const float* grad_out, void* grad_bf16, float* partial,
                              uint32_t* status, cudaStream_t stream);
 
 // fp32 -> bf16 (round to nearest even) copy of n elements, as one streaming kernel.
-cudaError_t launch_grad_to_bf16(const float* g, long long n, void* out_bf16, cudaStream_t stream);
+// As every gradient pre-pass, it also zeroes the call's status word.
+cudaError_t launch_grad_to_bf16(const float* g, long long n, void* out_bf16, uint32_t* status, cudaStream_t stream);
 // The same for `rows` rows of `len` elements, written with a row pitch of `pitch` >= len
 // elements (a multiple of 8); the padding is zero.
 cudaError_t launch_grad_to_bf16_rows(const float* g, long long rows, int len, int pitch,
-                                     void* out_bf16, cudaStream_t stream);
+                                     void* out_bf16, uint32_t* status, cudaStream_t stream);
 
 // ---- layers whose im2col operand is the activation itself (weight_grad_tc_direct.cu) ----------
 struct DirectParams {
@@ -97,14 +98,14 @@ struct DirectParams {
 };
 bool plan_direct(const surgeon_layer_desc& d, DirectParams* out);
 size_t direct_grad_bf16_bytes(const DirectParams& p);
-// partial = [splits][O][C] fp32 (O counts the stacked taps), status = one zeroed word.
+// partial = [splits][O][C] fp32 (O counts the stacked taps), status = one word (the pre-pass zeroes it).
 cudaError_t launch_direct(const surgeon_compressed& act, const DirectParams& p,
                           const float* grad_out, void* grad_bf16, float* partial,
                           uint32_t* status, cudaStream_t stream);
 // The pre-pass that writes the bf16 copy (or shifted copies) of the output gradient, and the
 // tensor map over it (conv: boxes of 64 positions x box_rows rows; linear: 64 columns x 64 rows).
 cudaError_t launch_direct_prepass(const DirectParams& p, const float* grad_out, void* grad_bf16,
-                                  cudaStream_t stream);
+                                  uint32_t* status, cudaStream_t stream);
 cudaError_t encode_direct_grad_map(const DirectParams& p, void* grad_bf16, int box_rows, CUtensorMap* out);
 
 // ---- the same layers on CTA pairs with the operand roles exchanged (weight_grad_tc_swap.cu) -----
@@ -131,7 +132,7 @@ struct SwapParams {
 bool plan_swap(const surgeon_layer_desc& d, SwapParams* out);
 int swap_resident_pairs();   // CTA pairs the device holds at once
 size_t swap_partial_bytes(const SwapParams& p);
-// partial = [splits][O][C] fp32 (O counts the stacked taps), status = one zeroed word.
+// partial = [splits][O][C] fp32 (O counts the stacked taps), status = one word (the pre-pass zeroes it).
 cudaError_t launch_swap(const surgeon_compressed& act, const SwapParams& p, const float* grad_out,
                         void* grad_bf16, float* partial, uint32_t* status, cudaStream_t stream);
 

@@ -635,8 +635,8 @@ dw_direct_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ v
 // zero where that lies outside the output map; tap = r * kw + s.  One thread writes 8 positions.
 __global__ void __launch_bounds__(256)
 grad_taps_bf16_kernel(const float* __restrict__ g, unsigned short* __restrict__ out,
-                      long long chunks, DirectParams p) {
-  pdl_trigger();
+                      long long chunks, DirectParams p, uint32_t* __restrict__ status) {
+  prepass_begin(status);
   const int per_row = p.pitch >> 3;
   for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < chunks;
        i += static_cast<long long>(gridDim.x) * blockDim.x) {
@@ -676,8 +676,8 @@ grad_taps_bf16_kernel(const float* __restrict__ g, unsigned short* __restrict__ 
 template <int KW>
 __global__ void __launch_bounds__(256)
 grad_taps_same_bf16_kernel(const float* __restrict__ g, unsigned short* __restrict__ out,
-                           long long items, DirectParams p) {
-  pdl_trigger();
+                           long long items, DirectParams p, uint32_t* __restrict__ status) {
+  prepass_begin(status);
   constexpr int H = (KW - 1) / 2;
   const int per_row = p.pitch >> 3;
   for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < items;
@@ -727,8 +727,8 @@ grad_taps_same_bf16_kernel(const float* __restrict__ g, unsigned short* __restri
 template <int KW, bool SAME>
 __global__ void __launch_bounds__(256)
 grad_cols_bf16_kernel(const float* __restrict__ g, unsigned short* __restrict__ out,
-                      long long chunks, DirectParams p) {
-  pdl_trigger();
+                      long long chunks, DirectParams p, uint32_t* __restrict__ status) {
+  prepass_begin(status);
   const int per_row = p.in_w >> 3;                     // chunks per map row
   const int per_plane = p.pitch >> 3;                  // pitch = OH * W
   for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < chunks;
@@ -923,58 +923,57 @@ size_t direct_grad_bf16_bytes(const DirectParams& p) {
 // The bf16 copy (or shifted copies) of the output gradient that the tensor maps of the direct
 // kernels read: one streaming pre-pass.
 cudaError_t launch_direct_prepass(const DirectParams& p, const float* grad_out, void* grad_bf16,
-                                  cudaStream_t stream) {
+                                  uint32_t* status, cudaStream_t stream) {
+  auto run = [&](auto kernel, int grid, long long items) -> cudaError_t {
+    note_launches(1);
+    return launch_kernel(kernel, dim3(grid), dim3(256), 0, stream, true, grad_out,
+                         static_cast<unsigned short*>(grad_bf16), items, p, status);
+  };
   cudaError_t e;
   if (p.row_shift) {
     const long long chunks = static_cast<long long>(p.imgs) * p.o_real * (p.pitch >> 3);
     const long long want = (chunks + 255) / 256;
     const long long cap = 32LL * sm_count();
     const int grid = static_cast<int>(want < 1 ? 1 : (want > cap ? cap : want));
-    unsigned short* ob = static_cast<unsigned short*>(grad_bf16);
     const bool same = (p.kw & 1) && p.pad == (p.kw - 1) / 2 && p.ow == p.in_w &&
                       (reinterpret_cast<uintptr_t>(grad_out) & 15) == 0;
     switch (p.kw) {
-      case 2: grad_cols_bf16_kernel<2, false><<<grid, 256, 0, stream>>>(grad_out, ob, chunks, p); break;
+      case 2: e = run(grad_cols_bf16_kernel<2, false>, grid, chunks); break;
       case 3:
-        if (same) grad_cols_bf16_kernel<3, true><<<grid, 256, 0, stream>>>(grad_out, ob, chunks, p);
-        else grad_cols_bf16_kernel<3, false><<<grid, 256, 0, stream>>>(grad_out, ob, chunks, p);
+        if (same) e = run(grad_cols_bf16_kernel<3, true>, grid, chunks);
+        else e = run(grad_cols_bf16_kernel<3, false>, grid, chunks);
         break;
       case 5:
-        if (same) grad_cols_bf16_kernel<5, true><<<grid, 256, 0, stream>>>(grad_out, ob, chunks, p);
-        else grad_cols_bf16_kernel<5, false><<<grid, 256, 0, stream>>>(grad_out, ob, chunks, p);
+        if (same) e = run(grad_cols_bf16_kernel<5, true>, grid, chunks);
+        else e = run(grad_cols_bf16_kernel<5, false>, grid, chunks);
         break;
       default:
-        if (same) grad_cols_bf16_kernel<7, true><<<grid, 256, 0, stream>>>(grad_out, ob, chunks, p);
-        else grad_cols_bf16_kernel<7, false><<<grid, 256, 0, stream>>>(grad_out, ob, chunks, p);
+        if (same) e = run(grad_cols_bf16_kernel<7, true>, grid, chunks);
+        else e = run(grad_cols_bf16_kernel<7, false>, grid, chunks);
         break;
     }
-    note_launches(1);
-    e = cudaGetLastError();
   } else if (p.taps > 1) {
     const long long chunks = static_cast<long long>(p.imgs) * p.O * (p.pitch >> 3);
     const long long want = (chunks + 255) / 256;
     const long long cap = 32LL * sm_count();
     const int grid = static_cast<int>(want < 1 ? 1 : (want > cap ? cap : want));
-    unsigned short* ob = static_cast<unsigned short*>(grad_bf16);
     const bool same = (p.kw & 1) && p.kh == p.kw && p.pad == (p.kw - 1) / 2 && p.ow == p.in_w &&
                       p.oh == p.in_h && (p.kw == 3 || p.kw == 5 || p.kw == 7);
     if (same) {
       const long long items = chunks / p.kw;        // one thread per row shift writes the kw column shifts
       const long long want_s = (items + 255) / 256;
       const int grid_s = static_cast<int>(want_s < 1 ? 1 : (want_s > cap ? cap : want_s));
-      if (p.kw == 3) grad_taps_same_bf16_kernel<3><<<grid_s, 256, 0, stream>>>(grad_out, ob, items, p);
-      else if (p.kw == 5) grad_taps_same_bf16_kernel<5><<<grid_s, 256, 0, stream>>>(grad_out, ob, items, p);
-      else grad_taps_same_bf16_kernel<7><<<grid_s, 256, 0, stream>>>(grad_out, ob, items, p);
+      if (p.kw == 3) e = run(grad_taps_same_bf16_kernel<3>, grid_s, items);
+      else if (p.kw == 5) e = run(grad_taps_same_bf16_kernel<5>, grid_s, items);
+      else e = run(grad_taps_same_bf16_kernel<7>, grid_s, items);
     } else {
-      grad_taps_bf16_kernel<<<grid, 256, 0, stream>>>(grad_out, ob, chunks, p);
+      e = run(grad_taps_bf16_kernel, grid, chunks);
     }
-    note_launches(1);
-    e = cudaGetLastError();
   } else if (p.mode != 0 && p.pitch != p.T)     // rows padded to a 16-byte pitch for the tensor map
     e = launch_grad_to_bf16_rows(grad_out, static_cast<long long>(p.imgs) * p.O, p.T, p.pitch,
-                                 grad_bf16, stream);
+                                 grad_bf16, status, stream);
   else
-    e = launch_grad_to_bf16(grad_out, static_cast<long long>(p.imgs) * p.O * p.T, grad_bf16, stream);
+    e = launch_grad_to_bf16(grad_out, static_cast<long long>(p.imgs) * p.O * p.T, grad_bf16, status, stream);
   return e;
 }
 
@@ -1017,7 +1016,7 @@ cudaError_t launch_direct(const surgeon_compressed& act, const DirectParams& pla
   p.n_keep_ptr = reinterpret_cast<const long long*>(reinterpret_cast<const char*>(act.header) +
                                                     offsetof(surgeon_header, n_keep));
   p.partial_blk = (act.n % SURGEON_BLOCK) ? static_cast<unsigned>(act.n / SURGEON_BLOCK) : 0xFFFFFFFFu;
-  cudaError_t e = launch_direct_prepass(p, grad_out, grad_bf16, stream);
+  cudaError_t e = launch_direct_prepass(p, grad_out, grad_bf16, status, stream);
   if (e != cudaSuccess) return e;
   CUtensorMap map;
   e = encode_direct_grad_map(p, grad_bf16, p.pair ? p.acc_n / 2 : p.acc_n, &map);

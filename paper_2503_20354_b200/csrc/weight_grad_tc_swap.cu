@@ -778,7 +778,7 @@ cudaError_t launch_swap(const surgeon_compressed& act, const SwapParams& plan, c
   p.n_keep_ptr = reinterpret_cast<const long long*>(reinterpret_cast<const char*>(act.header) +
                                                     offsetof(surgeon_header, n_keep));
   p.partial_blk = (act.n % SURGEON_BLOCK) ? static_cast<unsigned>(act.n / SURGEON_BLOCK) : 0xFFFFFFFFu;
-  cudaError_t e = launch_direct_prepass(p.d, grad_out, grad_bf16, stream);
+  cudaError_t e = launch_direct_prepass(p.d, grad_out, grad_bf16, status, stream);
   if (e != cudaSuccess) return e;
   CUtensorMap map;
   CUtensorMap rem_map;
