@@ -237,7 +237,7 @@ class CompressedActivation:
                  _blank: bool = False):
         # _blank: a call that writes the header follows, so it need not be zeroed (a kernel launch)
         s = sizes or surgeon_compact_sizes(n, dt, ratio)
-        self.n, self.dt, self.ratio, self.sizes = int(n), int(dt), float(ratio), s
+        self.n, self.dt, self.ratio, self._sizes = int(n), int(dt), float(ratio), s
         self.bitmap = torch.empty(max(s.bitmap_bytes // 4, 1), dtype=torch.int32, device=device)
         vt = torch.float32 if dt == SURGEON_F32 else torch.bfloat16
         self.values = torch.empty(max(s.n_keep, 1), dtype=vt, device=device)
@@ -245,6 +245,22 @@ class CompressedActivation:
         self.header = (torch.empty if _blank else torch.zeros)(4, dtype=torch.int64, device=device)
         self.c = Compressed(self.n, self.dt, 0, self.bitmap.data_ptr(), self.values.data_ptr(),
                             self.block_offsets.data_ptr(), self.header.data_ptr())
+
+    @property
+    def sizes(self) -> CompactSizes:
+        """Sizes at the store's present ratio (a call that changes the ratio leaves them to be asked for)."""
+        if self._sizes is None:
+            self._sizes = surgeon_compact_sizes(self.n, self.dt, self.ratio)
+        return self._sizes
+
+    def _now_at(self, ratio: float):
+        if ratio != self.ratio:
+            self.ratio, self._sizes = ratio, None
+
+    def _fits(self, ratio: float) -> bool:
+        # (a buffer for every element, as for ratios that change from batch to batch, fits any ratio)
+        room = self.values.numel()
+        return room >= self.n or room >= surgeon_compact_sizes(self.n, self.dt, ratio).n_keep
 
     @property
     def n_keep(self) -> int:
@@ -286,21 +302,20 @@ def surgeon_prune_compact(x: torch.Tensor, ratio: float, out: Optional[Compresse
         raise ValueError("x must be a contiguous CUDA tensor")
     dt = dtype_code(x.dtype)
     n = x.numel()
-    sizes = surgeon_compact_sizes(n, dt, ratio)
+    ratio = float(ratio)
     if out is None:
-        out = CompressedActivation(n, dt, ratio, x.device, sizes, _blank=True)
-    else:
-        if out.n != n or out.dt != dt or out.values.numel() < sizes.n_keep:
-            raise ValueError("output store does not fit this tensor / ratio")
-        out.ratio, out.sizes = float(ratio), sizes
+        out = CompressedActivation(n, dt, ratio, x.device, _blank=True)
+    elif out.n != n or out.dt != dt or not out._fits(ratio):
+        raise ValueError("output store does not fit this tensor / ratio")
     if workspace is None:
-        workspace = _scratch(sizes.workspace_bytes, x.device, stream)
-    st = lib().surgeon_prune_compact_flags(x.data_ptr(), n, dt, float(ratio), int(flags), C.byref(out.c),
+        workspace = _scratch(surgeon_compact_sizes(n, dt, ratio).workspace_bytes, x.device, stream)
+    st = lib().surgeon_prune_compact_flags(x.data_ptr(), n, dt, ratio, int(flags), C.byref(out.c),
                                            workspace.data_ptr(),
                                            workspace.numel() * workspace.element_size(),
                                            _stream_ptr(stream))
     if st != SURGEON_OK:
         _check(st, "surgeon_prune_compact")
+    out._now_at(ratio)
     return out
 
 
@@ -322,13 +337,13 @@ def surgeon_prune_compact_static(x: torch.Tensor, ratio: float, out: CompressedA
     if n > SURGEON_STATIC_MAX_N:
         raise SurgeonError(SURGEON_ERR_UNSUPPORTED, "surgeon_prune_compact_static: %d elements "
                            "exceed the built-in scratch (limit %d)" % (n, SURGEON_STATIC_MAX_N))
-    sizes = surgeon_compact_sizes(n, dt, ratio)
-    if out.n != n or out.dt != dt or out.values.numel() < sizes.n_keep:
+    ratio = float(ratio)
+    if out.n != n or out.dt != dt or not out._fits(ratio):
         raise ValueError("output store does not fit this tensor / ratio")
-    out.ratio, out.sizes = float(ratio), sizes
-    st = lib().surgeon_prune_compact_static(x.data_ptr(), n, dt, float(ratio), C.byref(out.c),
+    st = lib().surgeon_prune_compact_static(x.data_ptr(), n, dt, ratio, C.byref(out.c),
                                             _stream_ptr(stream))
     _check(st, "surgeon_prune_compact_static")
+    out._now_at(ratio)
     return out
 
 

@@ -1621,9 +1621,14 @@ cudaError_t run_prune_compact(const void* x, long long n, long long k, int drop_
   CUtensorMap map;
   if (!make_row_map(x, a.n_rows_full > 0 ? a.n_rows_full : 1, &map)) return cudaErrorNotSupported;
   // as many chunks per warp as a full grid would give its busiest warp, on as few CTAs as that takes: the
-  // others leave their SMs to other streams
+  // others leave their SMs to other streams.  A caller that changes streams from call to call (the
+  // prunes of several layers in flight) gets the smallest grid that keeps the tensor on chip: the
+  // kernel takes whole SMs, so grids of 148 run one after the other.
+  static std::atomic<cudaStream_t> last_stream{nullptr};
+  const bool alone = last_stream.exchange(stream, std::memory_order_relaxed) == stream;
   const int sms = sm_count() < kSelMaxCtas ? sm_count() : kSelMaxCtas;
-  const int per_cta = (a.n_chunks + sms * kWarps - 1) / (sms * kWarps) * kWarps;
+  int per_cta = (a.n_chunks + sms * kWarps - 1) / (sms * kWarps) * kWarps;
+  if (!alone && per_cta < kResidentChunks) per_cta = kResidentChunks;
   const int grid = (a.n_chunks + per_cta - 1) / per_cta;
   a.spread = a.n_chunks > grid * kMaxLocalChunks ? 1 : 0;
   const bool resident = (a.n_chunks + grid - 1) / grid <= kResidentChunks;

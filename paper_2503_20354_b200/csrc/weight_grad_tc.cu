@@ -898,6 +898,8 @@ size_t weight_grad_tc_workspace(const surgeon_layer_desc& d) {
   if (plan_swap(d, &sp)) return kStatusBytes + swap_partial_bytes(sp) + direct_grad_bf16_bytes(sp.d);
   DirectParams dp;
   if (plan_direct(d, &dp)) return kStatusBytes + direct_partial_bytes(dp) + direct_grad_bf16_bytes(dp);
+  StridedParams st;
+  if (plan_strided(d, &st)) return kStatusBytes + strided_partial_bytes(st) + strided_grad_bf16_bytes(st);
   FastParams f;
   if (plan_conv_fast(d, &f))
     return kStatusBytes + fast_partial_bytes(f) + conv_fast_grad_bf16_bytes(f);
@@ -952,6 +954,16 @@ cudaError_t launch_weight_grad_tc(const surgeon_compressed& act, const surgeon_l
 
     else
       launch_reduce_splits(partial, mn, dp.splits, dw, accumulate, status, act.header, stream);
+    note_launches(1);
+    return cudaGetLastError();
+  }
+  StridedParams strided;
+  if (plan_strided(d, &strided)) {
+    void* grad_bf16 = reinterpret_cast<char*>(partial) + strided_partial_bytes(strided);
+    e = launch_strided(act, strided, grad_out, grad_bf16, partial, status, stream);
+    if (e != cudaSuccess) return e;
+    launch_reduce_splits(partial, static_cast<long long>(strided.O) * strided.n_gemm, strided.splits, dw, accumulate,
+                         status, act.header, stream);
     note_launches(1);
     return cudaGetLastError();
   }

@@ -69,6 +69,28 @@ cudaError_t launch_grad_to_bf16(const float* g, long long n, void* out_bf16, uin
 cudaError_t launch_grad_to_bf16_rows(const float* g, long long rows, int len, int pitch,
                                      void* out_bf16, uint32_t* status, cudaStream_t stream);
 
+// ---- convolutions whose operand has to be expanded (weight_grad_tc_strided.cu) -----------------
+struct StridedParams {
+  int B, C, H, W, O, KH, KW, stride, pad, OH, OW;
+  int OWp, P;               // output row padded to a multiple of 8 positions; positions per image (OH * OWp)
+  int RS, n_gemm;           // KH * KW, C * RS
+  int acc_n, n_acc;         // columns per accumulator, accumulators per CTA (1 or 2)
+  int m_tiles, n_tiles, splits;
+  int tiles_per_img;        // K-tiles of 64 positions
+  int macro;                // K-tiles per rebuilt patch
+  int macros_per_img, total_macros, macros_per_split;
+  int patch_rows, plane;    // input rows of a patch, elements of a phase plane of one row
+  int patch_bytes, stages, tmem_cols, smem_bytes;
+  unsigned inv_stride;      // ix / stride = ix * inv_stride >> 16
+  long long n_words;        // words of the bitmap (filled by the launcher)
+};
+bool plan_strided(const surgeon_layer_desc& d, StridedParams* out);
+size_t strided_partial_bytes(const StridedParams& p);
+size_t strided_grad_bf16_bytes(const StridedParams& p);
+// partial = [splits][O][n_gemm] fp32, status = one word (the pre-pass zeroes it).
+cudaError_t launch_strided(const surgeon_compressed& act, const StridedParams& p, const float* grad_out,
+                           void* grad_bf16, float* partial, uint32_t* status, cudaStream_t stream);
+
 // ---- layers whose im2col operand is the activation itself (weight_grad_tc_direct.cu) ----------
 struct DirectParams {
   int mode;                 // 0 = linear [T, C] (MN-major operands), 1 = conv 1x1 stride 1 (K-major),

@@ -1,0 +1,504 @@
+// Tensor-core weight gradient of convolutions whose im2col operand has to be expanded: stride 2 and
+// more, and the small-channel layers the direct kernel leaves (weight_grad_tc_direct.cu).
+// Algorithm 1: Reshape and gradient steps with Eq. 2; the GEMM view of weight_grad_tc.cu:
+//   D[nn, o] = sum_k Acol[nn, k] * G[o, k],  nn = (c, r, s),  k = (b, y, x), output rows padded to OWp,
+// a multiple of 8 positions, so that a chunk of 8 positions (16 bytes of the operand) lies in one row.
+//
+// The output gradient is converted to bf16 by a pre-pass (padded rows, zeros in the padding) and
+// arrives by TMA.  The activation operand is built by two groups of 8 warps in turns, a macro of a few
+// K-tiles at a time:
+//   1. the input rows that the macro's positions touch are rebuilt from the store in a shared-memory
+//      patch, one lane per 16 elements of a row, once for all taps.  A row is kept as `stride` phase
+//      planes (column ix goes to plane ix mod stride, place ix div stride), with zeros around:
+//      what a tap reads for consecutive output positions is then consecutive, whatever the stride;
+//   2. a thread copies one chunk of 8 positions of four operand rows per K-tile: five 4-byte loads, a
+//      funnel shift where the tap's column offset is odd, one 16-byte store.
+// One group rebuilds while the other copies; the bitmap words and offsets of a macro's first pieces are
+// fetched while the macro before it is copied.  Bound by the latency of step 1's two dependent loads
+// and by the gradient tiles' traffic from L2.  The kernels before it copied element by element
+// (7x7 stride 2 on 224x224, 3 -> 64 channels, batch 64: 465 us a call) or rebuilt the rows for every
+// K-tile (3x3 stride 2 on 56x56, 128 channels: 215 us).
+// Every wait is bounded and ends in SURGEON_ERR_TIMEOUT.
+#include <cuda.h>
+
+#include "surgeon_internal.cuh"
+#include "tc_common.cuh"
+#include "weight_grad_tc_conv.cuh"
+
+namespace surgeon {
+
+namespace {
+
+using namespace tc;
+
+constexpr int kTileM = 128;
+constexpr int kTileK = 64;
+constexpr int kGroups = 2;
+constexpr int kGroupWarps = 8;
+constexpr int kGroupThreads = kGroupWarps * 32;
+constexpr int kThreads = 64 + kGroups * kGroupThreads;    // warp 0: MMA, warp 1: TMA, then the groups
+constexpr int kMaxStages = 8;
+constexpr int kATileBytes = kTileM * kTileK * 2;
+constexpr int kMaxPatchBytes = 44 * 1024;                 // per group
+constexpr int kPiece = 16;                                // elements of a row that one lane rebuilds
+constexpr int kAhead = 8;                                 // values in flight per lane
+
+__device__ __forceinline__ void group_sync(int g) {
+  asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(kGroupThreads) : "memory");
+}
+
+// What a lane fetches for its piece: the kept count before the 128-element block the piece starts in, the
+// words of the block before the piece's, its word and the one after it.
+struct PieceRaw {
+  uint32_t off, b0, b1, b2, w0, w1, sh;
+};
+
+template <int DT>
+__global__ void __launch_bounds__(kThreads, 1)
+dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ values,
+                  const uint32_t* __restrict__ offsets, const __grid_constant__ CUtensorMap grad_map,
+                  float* __restrict__ partial, uint32_t* __restrict__ status, StridedParams p) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* smem = reinterpret_cast<unsigned char*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  const int n_cols = p.acc_n * p.n_acc;
+  const int stage_bytes = kATileBytes + n_cols * 128;
+  __shared__ __align__(8) unsigned long long bars[2 * kMaxStages + 1];
+  __shared__ uint32_t tmem_slot;
+  __shared__ volatile uint32_t fail;
+
+  const int tid = threadIdx.x;
+  const int warp = tid >> 5;
+  const uint32_t lane = lane_id();
+  const int nn0 = blockIdx.x * kTileM;
+  const int o0 = blockIdx.y * n_cols;
+  const int n_acc_here = min(p.n_acc, (p.O - o0 + p.acc_n - 1) / p.acc_n);
+  const int split = blockIdx.z;
+  const int m_begin = split * p.macros_per_split;
+  const int m_end = min(m_begin + p.macros_per_split, p.total_macros);
+  // K-tiles of macro m (the last one of an image may be short)
+  auto tiles_of = [&](int m) { return min(p.macro, p.tiles_per_img - (m % p.macros_per_img) * p.macro); };
+
+  const uint32_t full_bar = smem_u32(bars);
+  const uint32_t empty_bar = smem_u32(bars + kMaxStages);
+  const uint32_t acc_bar = smem_u32(bars + 2 * kMaxStages);
+  if (tid == 0) {
+    tma_prefetch_desc(&grad_map);
+    for (int s = 0; s < p.stages; ++s) {
+      mbar_init(full_bar + 8 * s, kGroupWarps + 1);       // a group's warps + the TMA thread
+      mbar_init(empty_bar + 8 * s, 1);
+    }
+    mbar_init(acc_bar, 1);
+    fail = 0;
+    fence_barrier_init();
+  }
+  if (warp == 0) tmem_alloc(smem_u32(&tmem_slot), p.tmem_cols);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = tmem_slot;
+  pdl_trigger();                         // the split reduction may be launched; it waits for this grid
+
+  if (warp == 0) {
+    // ================= MMA issuer =================
+    if (lane == 0) {
+      const uint32_t idesc = make_idesc(kTileM, p.acc_n);
+      const uint32_t smem0 = smem_u32(smem);
+      const uint64_t a_base = make_desc(smem0), b_base = make_desc(smem0 + kATileBytes);
+      const uint64_t stage_inc = static_cast<uint64_t>(stage_bytes >> 4);
+      const uint64_t acc_inc = static_cast<uint64_t>((p.acc_n * 128) >> 4);
+      uint64_t da = a_base, db = b_base;
+      uint32_t parity = 0, accum = 0;
+      int s = 0;
+      bool ok = true;
+      for (int m = m_begin; m < m_end && ok; ++m) {
+        for (int t = tiles_of(m); t > 0; --t) {
+          ok = mbar_wait_suspend(full_bar + 8 * s, parity);
+          if (!ok) break;
+          tc_fence_after();
+          if (n_acc_here == 1) umma_ktile<1, 2>(tmem_base, p.acc_n, da, db, acc_inc, idesc, accum);
+          else umma_ktile<2, 2>(tmem_base, p.acc_n, da, db, acc_inc, idesc, accum);
+          umma_commit(empty_bar + 8 * s);
+          accum = 1;
+          if (++s == p.stages) { s = 0; parity ^= 1; da = a_base; db = b_base; }
+          else { da += stage_inc; db += stage_inc; }
+        }
+      }
+      if (!ok) { fail = 1; atomicMax(status, static_cast<uint32_t>(SURGEON_ERR_TIMEOUT)); }
+      umma_commit(acc_bar);
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    // ================= gradient tiles by TMA =================
+    if (lane == 0) {
+      pdl_wait();                                  // the bf16 gradient copy is complete
+      int s = 0;
+      uint32_t round = 0;
+      bool ok = true;
+      for (int m = m_begin; m < m_end && ok; ++m) {
+        const int img = m / p.macros_per_img;
+        const int kt0 = (m - img * p.macros_per_img) * p.macro;
+        const int n_t = tiles_of(m);
+        for (int t = 0; t < n_t; ++t) {
+          if (round > 0 && !mbar_wait_suspend(empty_bar + 8 * s, (round - 1) & 1)) {
+            fail = 1;
+            atomicMax(status, static_cast<uint32_t>(SURGEON_ERR_TIMEOUT));
+            ok = false;
+            break;
+          }
+          const uint32_t b_addr = smem_u32(smem + s * stage_bytes + kATileBytes);
+          mbar_arrive_expect_tx(full_bar + 8 * s, static_cast<uint32_t>(n_acc_here * p.acc_n) * 128u);
+          for (int a = 0; a < n_acc_here; ++a)
+            tma_load_3d(b_addr + a * p.acc_n * 128, &grad_map, (kt0 + t) * kTileK, o0 + a * p.acc_n, img,
+                        full_bar + 8 * s);
+          if (++s == p.stages) { s = 0; ++round; }
+        }
+      }
+    }
+    __syncwarp();
+  } else {
+    // ================= producers =================
+    const int g = (warp - 2) / kGroupWarps;
+    const int gtid = tid - 64 - g * kGroupThreads;
+    unsigned char* patch = smem + p.stages * stage_bytes + g * p.patch_bytes;
+    unsigned short* patch16 = reinterpret_cast<unsigned short*>(patch);
+    const uint32_t patch_addr = smem_u32(patch);
+    const int c_first = nn0 / p.RS;
+    const int c_last = min(nn0 + kTileM - 1, p.n_gemm - 1) / p.RS;
+    const int n_ch = c_last - c_first + 1;
+    const int row_len = p.stride * p.plane;        // elements of one input row in the patch
+    // this thread's four operand rows and its chunk of 8 positions
+    const int chunk = gtid & 7;
+    int row_base[4];                               // patch element of (channel, input row iy_lo, phase) and column offset
+    int row_r[4];                                  // kernel row, -1000000 past the last column
+    uint32_t dst_off[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int row = (gtid >> 3) + 32 * i;
+      const int nn = nn0 + row;
+      dst_off[i] = tile_off(row, chunk);
+      row_base[i] = 0;
+      row_r[i] = -1000000;
+      if (nn < p.n_gemm) {
+        const int c = nn / p.RS, rs = nn - c * p.RS;
+        const int r = rs / p.KW, s = rs - r * p.KW;
+        const int d = s - p.pad;
+        const int fd = d >= 0 ? d / p.stride : -((-d + p.stride - 1) / p.stride);
+        row_base[i] = (c - c_first) * p.patch_rows * row_len + (d - fd * p.stride) * p.plane + 8 + fd;
+        row_r[i] = r - p.pad;
+      }
+    }
+    // A macro's input rows and its pieces (channel, row, 16 columns).
+    struct Macro { int img, kt0, n_t, iy_lo, n_pieces, per_ch; };
+    const int per_row = (p.W + kPiece - 1) / kPiece;
+    auto geometry = [&](int m) {
+      Macro q;
+      q.img = m / p.macros_per_img;
+      q.kt0 = (m - q.img * p.macros_per_img) * p.macro;
+      q.n_t = tiles_of(m);
+      const int y_first = q.kt0 * kTileK / p.OWp;
+      const int y_last = min((q.kt0 + q.n_t) * kTileK - 1, p.P - 1) / p.OWp;
+      q.iy_lo = max(y_first * p.stride - p.pad, 0);
+      const int iy_hi = min(y_last * p.stride + p.KH - 1 - p.pad, p.H - 1);
+      q.per_ch = (iy_hi - q.iy_lo + 1) * per_row;
+      q.n_pieces = n_ch * q.per_ch;
+      return q;
+    };
+    auto place = [&](const Macro& q, int t, int* ci, int* row, int* col) {
+      *ci = t / q.per_ch;
+      const int rest = t - *ci * q.per_ch;
+      *row = rest / per_row;
+      *col = (rest - *row * per_row) * kPiece;
+    };
+    auto fetch = [&](const Macro& q, int t) {
+      PieceRaw r = {};
+      if (t < q.n_pieces) {
+        int ci, row, col;
+        place(q, t, &ci, &row, &col);
+        const long long start =
+            ((static_cast<long long>(q.img) * p.C + c_first + ci) * p.H + q.iy_lo + row) * p.W + col;
+        const long long blk = start >> kBlockShift, wi = start >> 5;
+        const int before = static_cast<int>(wi - blk * kBlockWords);
+        r.sh = static_cast<uint32_t>(start & 31);
+        r.off = __ldg(offsets + blk);
+        r.b0 = before > 0 ? __ldg(bitmap + wi - before) : 0u;
+        r.b1 = before > 1 ? __ldg(bitmap + wi - before + 1) : 0u;
+        r.b2 = before > 2 ? __ldg(bitmap + wi - before + 2) : 0u;
+        r.w0 = __ldg(bitmap + wi);
+        r.w1 = (r.sh > 32u - kPiece && wi + 1 < p.n_words) ? __ldg(bitmap + wi + 1) : 0u;
+      }
+      return r;
+    };
+    // The ring place of the next tile.  A barrier's phase is told by one bit: a macro is shorter than the
+    // ring (see the plan), so that the tile of this place two rounds ago is known to be consumed when
+    // the warp comes to wait for the last one.
+    int s = 0;
+    uint32_t round = 0;
+    auto skip_tiles = [&](int n) {                 // the other group's
+      s += n;
+      while (s >= p.stages) { s -= p.stages; ++round; }
+    };
+    if (g == 1 && m_begin < m_end) skip_tiles(tiles_of(m_begin));
+    auto wait_stage = [&]() {
+      // (once a wait has given up nothing waits any more: the warps still meet at the group's barriers,
+      // and what they write is not used)
+      if (round > 0 && lane == 0 && !fail && !mbar_wait_suspend(empty_bar + 8 * s, (round - 1) & 1)) {
+        fail = 1;
+        atomicMax(status, static_cast<uint32_t>(SURGEON_ERR_TIMEOUT));
+      }
+    };
+    PieceRaw raw[2] = {};                          // the next two pieces
+    if (m_begin + g < m_end) {
+      const Macro q = geometry(m_begin + g);
+      raw[0] = fetch(q, gtid);
+      raw[1] = fetch(q, gtid + kGroupThreads);
+    }
+    for (int m = m_begin + g; m < m_end; m += kGroups) {
+      const Macro q = geometry(m);
+      const int kt0 = q.kt0, n_t = q.n_t, iy_lo = q.iy_lo;
+      // ---- the patch ----
+      for (int v = gtid; v < p.patch_bytes / 16; v += kGroupThreads)
+        reinterpret_cast<uint4*>(patch)[v] = make_uint4(0, 0, 0, 0);
+      group_sync(g);
+      for (int t = gtid; t < q.n_pieces; t += kGroupThreads) {
+        const PieceRaw r = raw[0];
+        raw[0] = raw[1];
+        raw[1] = fetch(q, t + 2 * kGroupThreads);
+        int ci, row, col;
+        place(q, t, &ci, &row, &col);
+        uint32_t rank = r.off + __popc(r.b0) + __popc(r.b1) + __popc(r.b2) + __popc(r.w0 & ((1u << r.sh) - 1u));
+        const int len = min(kPiece, p.W - col);
+        uint32_t bits = __funnelshift_r(r.w0, r.w1, r.sh) & ((1u << len) - 1u);
+        unsigned short* dst = patch16 + (ci * p.patch_rows + row) * row_len + 8;
+        for (int left = __popc(bits); left > 0; left -= kAhead) {
+          uint32_t v[kAhead];
+#pragma unroll
+          for (int i = 0; i < kAhead; ++i) v[i] = ld_packed<DT>(values, rank + i, i < left);
+          rank += kAhead;
+#pragma unroll
+          for (int i = 0; i < kAhead; ++i) {
+            if (i < left) {
+              const uint32_t ix = col + __ffs(bits) - 1;
+              bits &= bits - 1;
+              const uint32_t qq = (ix * p.inv_stride) >> 16;       // ix / stride
+              if (qq + 8 < static_cast<uint32_t>(p.plane))         // (columns no tap reads)
+                dst[(ix - qq * p.stride) * p.plane + qq] =
+                    (DT == 0) ? to_bf16_bits(__uint_as_float(v[i])) : static_cast<unsigned short>(v[i]);
+            }
+          }
+        }
+      }
+      group_sync(g);
+      if (m + kGroups < m_end) {                   // in flight while this macro's tiles are copied
+        const Macro nx = geometry(m + kGroups);
+        raw[0] = fetch(nx, gtid);
+        raw[1] = fetch(nx, gtid + kGroupThreads);
+      }
+      // ---- the operand tiles ----
+      for (int t = 0; t < n_t; ++t) {
+        wait_stage();
+        __syncwarp();
+        unsigned char* a_tile = smem + s * stage_bytes;
+        const int pos = (kt0 + t) * kTileK + 8 * chunk;
+        const int y = pos / p.OWp, x0 = pos - y * p.OWp;
+        const int nv = pos < p.P ? p.OW - x0 : 0;          // positions of the chunk that exist
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int iy = y * p.stride + row_r[i];
+          uint4 out = make_uint4(0, 0, 0, 0);
+          if (iy >= 0 && iy < p.H && nv > 0) {
+            const uint32_t e = static_cast<uint32_t>(row_base[i] + (iy - iy_lo) * row_len + x0);
+            const uint32_t addr = patch_addr + (e & ~1u) * 2u;
+            uint32_t w[5];
+#pragma unroll
+            for (int j = 0; j < 5; ++j)
+              asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w[j]) : "r"(addr + 4 * j) : "memory");
+            const uint32_t shift = (e & 1u) * 16u;
+            out.x = __funnelshift_r(w[0], w[1], shift);
+            out.y = __funnelshift_r(w[1], w[2], shift);
+            out.z = __funnelshift_r(w[2], w[3], shift);
+            out.w = __funnelshift_r(w[3], w[4], shift);
+            if (nv < 8) {                                  // the padding at the end of the row
+              uint32_t* o = reinterpret_cast<uint32_t*>(&out);
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+                o[j] = 2 * j + 1 < nv ? o[j] : (2 * j < nv ? o[j] & 0xFFFFu : 0u);
+            }
+          }
+          *reinterpret_cast<uint4*>(a_tile + dst_off[i]) = out;
+        }
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(full_bar + 8 * s);
+        skip_tiles(1);
+      }
+      if (m + 1 < m_end) skip_tiles(tiles_of(m + 1));
+      group_sync(g);                               // the patch is read; it is zeroed next
+    }
+  }
+
+  // ================= epilogue: TMEM -> scratch partial tile =================
+  if (warp >= 2) {
+    const bool done = mbar_wait(acc_bar, 0, 64);
+    tc_fence_after();
+    if (done && !fail) {
+      const int lane_grp = warp & 3;              // TMEM lanes this warp may read
+      const int nn = nn0 + lane_grp * 32 + static_cast<int>(lane);
+      float* out = partial + static_cast<long long>(split) * p.O * p.n_gemm;
+      const int cols_here = n_acc_here * p.acc_n;
+      for (int col = 16 * ((warp - 2) >> 2); col < cols_here; col += 16 * (kGroups * kGroupWarps / 4)) {
+        uint32_t r[16];
+        tmem_ld16(tmem_base + (static_cast<uint32_t>(lane_grp * 32) << 16) + col, r);
+        if (nn < p.n_gemm) {
+#pragma unroll
+          for (int e = 0; e < 16; ++e) {
+            const int o = o0 + col + e;
+            if (o < p.O && SURGEON_IN_BOUNDS(static_cast<long long>(split) * p.O * p.n_gemm +
+                                                 static_cast<long long>(o) * p.n_gemm + nn,
+                                             static_cast<long long>(p.splits) * p.O * p.n_gemm, status))
+              out[static_cast<long long>(o) * p.n_gemm + nn] = __uint_as_float(r[e]);
+          }
+        }
+      }
+    } else if (!done && lane == 0) {
+      atomicMax(status, static_cast<uint32_t>(SURGEON_ERR_TIMEOUT));
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) tmem_dealloc(tmem_base, p.tmem_cols);
+}
+
+using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                              const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
+                              CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
+                              CUtensorMapFloatOOBfill);
+
+bool compute_plan_strided(const surgeon_layer_desc& d, StridedParams* out) {
+  if (d.kind != 1) return false;
+  StridedParams p{};
+  p.B = d.batch; p.C = d.c_in; p.H = d.h; p.W = d.w; p.O = d.c_out; p.KH = d.kh; p.KW = d.kw;
+  p.stride = d.stride; p.pad = d.pad;
+  p.OH = (d.h + 2 * d.pad - d.kh) / d.stride + 1;
+  p.OW = (d.w + 2 * d.pad - d.kw) / d.stride + 1;
+  p.OWp = (p.OW + 7) / 8 * 8;
+  p.P = p.OH * p.OWp;
+  p.RS = d.kh * d.kw;
+  p.n_gemm = d.c_in * p.RS;
+  // 8 zeros to the left of a plane: tap columns reach at most 8 places over the edge; ix / stride by a multiplication
+  if ((d.pad + d.stride - 1) / d.stride > 8 || (d.kw - 1) / d.stride > 5 || d.stride > 64 || d.w > 4096) return false;
+  p.inv_stride = (65536 + d.stride - 1) / d.stride;
+  for (int ix = 0; ix < d.w; ++ix)
+    if (static_cast<int>((static_cast<unsigned>(ix) * p.inv_stride) >> 16) != ix / d.stride) return false;
+  p.plane = p.OWp + 16;                            // elements; an odd number of words, against bank conflicts
+  if ((p.plane / 2) % 2 == 0) p.plane += 2;
+  p.m_tiles = (p.n_gemm + kTileM - 1) / kTileM;
+  const int n_ch = p.RS >= kTileM ? 2 : (p.C < (kTileM - 2) / p.RS + 2 ? p.C : (kTileM - 2) / p.RS + 2);
+  p.tiles_per_img = (p.P + kTileK - 1) / kTileK;
+  // columns: one or two accumulators of at most 256 columns, the fewest padded columns first
+  int best_waste = -1;
+  for (int c = 256; c >= 16; c -= 16) {
+    const int units = (p.O + c - 1) / c;
+    const int waste = units * c - p.O;
+    if (best_waste < 0 || waste < best_waste) { best_waste = waste; p.acc_n = c; }
+  }
+  const int units = (p.O + p.acc_n - 1) / p.acc_n;
+  // the longest macro (rows are rebuilt once per macro) whose patch fits, with three stages at least if possible
+  const int budget = 226 * 1024 - 1024 - 256;
+  bool found = false;
+  for (int want_stages = 3; want_stages >= 2 && !found; --want_stages) {
+    for (int n_acc = units >= 2 ? 2 : 1; n_acc >= 1 && !found; --n_acc) {
+      for (int macro = 8; macro >= 1 && !found; --macro) {
+        if (macro > p.tiles_per_img) continue;
+        int out_rows = (macro * kTileK + p.OWp - 2) / p.OWp + 1;
+        if (out_rows > p.OH) out_rows = p.OH;
+        int rows = (out_rows - 1) * d.stride + d.kh;
+        if (rows > d.h) rows = d.h;
+        const long long bytes = (static_cast<long long>(n_ch) * rows * d.stride * p.plane * 2 + 32 + 15) / 16 * 16;
+        if (bytes > kMaxPatchBytes) continue;
+        const int stage = kATileBytes + n_acc * p.acc_n * 128;
+        int stages = static_cast<int>((budget - kGroups * bytes) / stage);
+        if (stages > kMaxStages) stages = kMaxStages;
+        if (stages < want_stages || macro >= stages) continue;      // (macro < stages: see the producers' waits)
+        p.macro = macro; p.patch_rows = rows; p.patch_bytes = static_cast<int>(bytes); p.n_acc = n_acc;
+        p.stages = stages;
+        found = true;
+      }
+    }
+  }
+  if (!found) return false;
+  p.n_tiles = (units + p.n_acc - 1) / p.n_acc;
+  p.macros_per_img = (p.tiles_per_img + p.macro - 1) / p.macro;
+  const long long total = static_cast<long long>(d.batch) * p.macros_per_img;
+  if (total > 2147483647LL / 64) return false;
+  p.total_macros = static_cast<int>(total);
+  const int sms = sm_count();
+  const long long tiles_mn = static_cast<long long>(p.m_tiles) * p.n_tiles;
+  int best = 1;
+  double best_cost = 1e30;
+  for (int s = 1; s <= p.total_macros && s <= 160; ++s) {
+    const long long waves = (tiles_mn * s + sms - 1) / sms;
+    const int per = (p.total_macros + s - 1) / s;
+    const double cost = static_cast<double>(waves) * (per * p.macro + 10) + 0.02 * s * tiles_mn / sms;
+    if (cost < best_cost - 1e-9) { best_cost = cost; best = s; }
+  }
+  p.macros_per_split = (p.total_macros + best - 1) / best;
+  p.splits = (p.total_macros + p.macros_per_split - 1) / p.macros_per_split;
+  p.tmem_cols = 32;
+  while (p.tmem_cols < p.acc_n * p.n_acc) p.tmem_cols *= 2;
+  p.smem_bytes = p.stages * (kATileBytes + p.n_acc * p.acc_n * 128) + kGroups * p.patch_bytes + 1024;
+  *out = p;
+  return true;
+}
+
+}  // namespace
+
+bool plan_strided(const surgeon_layer_desc& d, StridedParams* out) {
+  struct Tag {};
+  return memo_plan<Tag>(d, 0, out, [&](StridedParams* p) { return compute_plan_strided(d, p); });
+}
+
+size_t strided_partial_bytes(const StridedParams& p) {
+  const size_t b = static_cast<size_t>(p.splits) * p.O * p.n_gemm * sizeof(float);
+  return (b + 255) & ~static_cast<size_t>(255);
+}
+
+size_t strided_grad_bf16_bytes(const StridedParams& p) {
+  const size_t b = static_cast<size_t>(p.B) * p.O * p.P * 2;
+  return (b + 255) & ~static_cast<size_t>(255);
+}
+
+cudaError_t launch_strided(const surgeon_compressed& act, const StridedParams& plan, const float* grad_out,
+                           void* grad_bf16, float* partial, uint32_t* status, cudaStream_t stream) {
+  StridedParams p = plan;
+  p.n_words = (act.n + 31) / 32;
+  cudaError_t e = p.OW == p.OWp
+                      ? launch_grad_to_bf16(grad_out, static_cast<long long>(p.B) * p.O * p.P, grad_bf16, status, stream)
+                      : launch_grad_to_bf16_rows(grad_out, static_cast<long long>(p.B) * p.O * p.OH, p.OW, p.OWp,
+                                                 grad_bf16, status, stream);
+  if (e != cudaSuccess) return e;
+  const EncodeFn encode = reinterpret_cast<EncodeFn>(tensor_map_encode_fn());
+  if (!encode) return cudaErrorNotSupported;
+  CUtensorMap map;
+  const cuuint64_t dims[3] = {static_cast<cuuint64_t>(p.P), static_cast<cuuint64_t>(p.O),
+                              static_cast<cuuint64_t>(p.B)};
+  const cuuint64_t strides[2] = {static_cast<cuuint64_t>(p.P) * 2, static_cast<cuuint64_t>(p.P) * p.O * 2};
+  const cuuint32_t box[3] = {static_cast<cuuint32_t>(kTileK), static_cast<cuuint32_t>(p.acc_n), 1};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  if (encode(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, grad_bf16, dims, strides, box, estr,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return cudaErrorInvalidValue;
+  const dim3 grid(p.m_tiles, p.n_tiles, p.splits);
+  auto launch = [&](auto kernel) -> cudaError_t {
+    const cudaError_t err = allow_dynamic_smem(reinterpret_cast<const void*>(kernel), p.smem_bytes);
+    if (err != cudaSuccess) return err;
+    return launch_kernel(kernel, grid, dim3(kThreads), static_cast<size_t>(p.smem_bytes), stream, true, act.bitmap,
+                         static_cast<const void*>(act.values), act.block_offsets, map, partial, status, p);
+  };
+  e = act.dt == 0 ? launch(dw_strided_kernel<0>) : launch(dw_strided_kernel<1>);
+  note_launches(1);
+  return e;
+}
+
+}  // namespace surgeon
