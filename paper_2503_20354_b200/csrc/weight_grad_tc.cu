@@ -19,6 +19,8 @@
 // the scratch status word, frees its tensor memory and returns.
 #include <cuda.h>
 
+#include <type_traits>
+
 #include "surgeon_internal.cuh"
 #include "tc_common.cuh"
 #include "weight_grad_tc_conv.cuh"
@@ -681,66 +683,102 @@ dw_conv_im2col_kernel(const uint32_t* __restrict__ bitmap, const void* __restric
   if (warp == 0) tmem_dealloc(tmem_base, p.tmem_cols);
 }
 
-// Sums the split partials in order and writes (or adds to) dw; copies the device status into
-// the activation's header when a wait timed out.
+// Sums the split partials in a fixed order and writes (or adds to) dw; copies the device status into
+// the activation's header when a wait timed out.  V elements per thread (4: mn a multiple of 4 and
+// 16-byte aligned pointers).  SP threads share an element's splits, each a contiguous part of them, and their
+// sums are added in order: with one thread per element a small weight tensor of a long reduction
+// (64 x 64 weights in 126 parts) took 25 us on four blocks, each a chain of dependent round trips.
+template <int V, int SP>
 __global__ void __launch_bounds__(256)
 reduce_splits_kernel(const float* __restrict__ partial, long long mn, int splits,
                      float* __restrict__ dw, int accumulate, const uint32_t* __restrict__ status,
                      surgeon_header* __restrict__ hdr) {
+  constexpr int TX = 256 / SP;
+  __shared__ float part[SP > 1 ? SP : 1][SP > 1 ? TX * V : 1];
   pdl_wait();                            // the partial tiles are complete
-  const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i == 0 && *status != 0 && hdr) atomicMax(&hdr->status, *status);
-  if (i >= mn) return;
-  float s = partial[i];
-  for (int z = 1; z < splits; ++z) s += partial[z * mn + i];
-  dw[i] = accumulate ? dw[i] + s : s;
-}
-
-// Four elements per thread (mn a multiple of 4, 16-byte aligned pointers).
-__global__ void __launch_bounds__(256)
-reduce_splits4_kernel(const float* __restrict__ partial, long long mn, int splits,
-                      float* __restrict__ dw, int accumulate, const uint32_t* __restrict__ status,
-                      surgeon_header* __restrict__ hdr) {
-  pdl_wait();                            // the partial tiles are complete
-  const long long i = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) * 4;
-  if (i == 0 && *status != 0 && hdr) atomicMax(&hdr->status, *status);
-  if (i >= mn) return;
-  float4 s = *reinterpret_cast<const float4*>(partial + i);
-#pragma unroll 4
-  for (int z = 1; z < splits; ++z) {
-    const float4 v = *reinterpret_cast<const float4*>(partial + z * mn + i);
-    s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
+  const long long i = (static_cast<long long>(blockIdx.x) * TX + tx) * V;
+  if (i == 0 && ty == 0 && *status != 0 && hdr) atomicMax(&hdr->status, *status);
+  const int per = (splits + SP - 1) / SP;
+  const int z0 = ty * per, z1 = min(z0 + per, splits);
+  float s[V];
+#pragma unroll
+  for (int e = 0; e < V; ++e) s[e] = 0.0f;
+  if (i < mn) {
+#pragma unroll 8
+    for (int z = z0; z < z1; ++z) {
+      const float* src = partial + z * mn + i;
+      if (V == 4) {
+        const float4 v = __ldcg(reinterpret_cast<const float4*>(src));
+        s[0] += v.x; s[1 % V] += v.y; s[2 % V] += v.z; s[3 % V] += v.w;
+      } else {
+        s[0] += __ldcg(src);
+      }
+    }
   }
-  if (accumulate) {
-    const float4 d = *reinterpret_cast<const float4*>(dw + i);
-    s.x += d.x; s.y += d.y; s.z += d.z; s.w += d.w;
+  if (SP > 1) {
+#pragma unroll
+    for (int e = 0; e < V; ++e) part[ty][tx * V + e] = s[e];
+    __syncthreads();
+    if (ty != 0) return;
+#pragma unroll
+    for (int e = 0; e < V; ++e) {
+      s[e] = part[0][tx * V + e];
+      for (int y = 1; y < SP; ++y) s[e] += part[y][tx * V + e];
+    }
   }
-  *reinterpret_cast<float4*>(dw + i) = s;
+  if (i >= mn) return;
+  if (V == 4) {
+    float4 o = make_float4(s[0], s[1 % V], s[2 % V], s[3 % V]);
+    if (accumulate) {
+      const float4 d = *reinterpret_cast<const float4*>(dw + i);
+      o.x += d.x; o.y += d.y; o.z += d.z; o.w += d.w;
+    }
+    *reinterpret_cast<float4*>(dw + i) = o;
+  } else {
+    dw[i] = accumulate ? dw[i] + s[0] : s[0];
+  }
 }
 
 static void launch_reduce_splits(const float* partial, long long mn, int splits, float* dw,
                                  int accumulate, const uint32_t* status, surgeon_header* hdr,
                                  cudaStream_t stream) {
   const bool vec = (mn & 3) == 0 && ((reinterpret_cast<uintptr_t>(partial) | reinterpret_cast<uintptr_t>(dw)) & 15) == 0;
+  const long long units = vec ? mn / 4 : mn;
+  // threads per element: until two blocks per SM are busy or a thread has four parts left
+  int sp = 1;
+  while (sp < 32 && units * sp < 512LL * sm_count() && splits > 4 * sp) sp *= 2;
   // launched as a programmatic dependent of the kernel that writes the partial tiles: it is
   // resident (or queued) when that kernel ends and starts at once
-  if (vec)
-    launch_kernel(reduce_splits4_kernel, dim3(static_cast<unsigned>((mn / 4 + 255) / 256)), dim3(256), 0, stream,
-                  true, partial, mn, splits, dw, accumulate, status, hdr);
-  else
-    launch_kernel(reduce_splits_kernel, dim3(static_cast<unsigned>((mn + 255) / 256)), dim3(256), 0, stream,
-                  true, partial, mn, splits, dw, accumulate, status, hdr);
+  auto launch = [&](auto kernel) {
+    launch_kernel(kernel, dim3(static_cast<unsigned>((units * sp + 255) / 256)), dim3(256), 0, stream, true, partial, mn,
+                  splits, dw, accumulate, status, hdr);
+  };
+  auto by_sp = [&](auto v) {
+    constexpr int V = decltype(v)::value;
+    switch (sp) {
+      case 1: launch(reduce_splits_kernel<V, 1>); break;
+      case 2: launch(reduce_splits_kernel<V, 2>); break;
+      case 4: launch(reduce_splits_kernel<V, 4>); break;
+      case 8: launch(reduce_splits_kernel<V, 8>); break;
+      case 16: launch(reduce_splits_kernel<V, 16>); break;
+      default: launch(reduce_splits_kernel<V, 32>); break;
+    }
+  };
+  if (vec) by_sp(std::integral_constant<int, 4>{});
+  else by_sp(std::integral_constant<int, 1>{});
 }
 
 // The same for a tap-stacked partial [splits][taps * O][C]: dw[o][c][tap] gets row tap * O + o.
 // One block sums `chunk` input channels of one output channel for all taps: the reads
 // run along c (contiguous in the partial, a kilobyte per warp), the writes along (c, tap)
-// (contiguous in dw), transposed through shared memory.  taps <= 49.
+// (contiguous in dw), transposed through shared memory.  taps <= 49.  `sp` threads share an element's splits (see
+// reduce_splits_kernel) where a chunk has too few elements for the block.
 __global__ void __launch_bounds__(256)
 reduce_splits_taps_kernel(const float* __restrict__ partial, int o_real, int c_in, int taps,
-                          int chunk, int splits, float* __restrict__ dw, int accumulate,
+                          int chunk, int splits, int sp, float* __restrict__ dw, int accumulate,
                           const uint32_t* __restrict__ status, surgeon_header* __restrict__ hdr) {
-  extern __shared__ __align__(16) float tile[];    // [n_c][taps]
+  extern __shared__ __align__(16) float tile[];    // [sp][chunk][taps]
   pdl_wait();                                      // the partial tiles are complete
   const int c0 = blockIdx.x * chunk;
   const int o = blockIdx.y;
@@ -753,24 +791,32 @@ reduce_splits_taps_kernel(const float* __restrict__ partial, int o_real, int c_i
     // four channels per thread: 16-byte reads of the partials, 16-byte writes of dw (c0 is a
     // multiple of 32 and n_c of 4, so both stay aligned); the split sums keep their order
     const int n_c4 = n_c >> 2;
-    for (int idx = threadIdx.x; idx < n_c4 * taps; idx += 256) {
-      const int tap = idx / n_c4, cl = (idx - tap * n_c4) * 4;
+    const int items = n_c4 * taps, per = (splits + sp - 1) / sp;
+    for (int idx = threadIdx.x; idx < items * sp; idx += 256) {
+      const int y = sp == 1 ? 0 : idx / items, it = idx - y * items;
+      const int tap = it / n_c4, cl = (it - tap * n_c4) * 4;
       const float* src = partial + (static_cast<long long>(tap) * o_real + o) * c_in + c0 + cl;
-      float4 s = *reinterpret_cast<const float4*>(src);
-#pragma unroll 4
-      for (int z = 1; z < splits; ++z) {
-        const float4 v = *reinterpret_cast<const float4*>(src + z * mn);
+      float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      const int z1 = min((y + 1) * per, splits);
+#pragma unroll 8
+      for (int z = y * per; z < z1; ++z) {
+        const float4 v = __ldcg(reinterpret_cast<const float4*>(src + z * mn));
         s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
       }
-      tile[cl * taps + tap] = s.x;
-      tile[(cl + 1) * taps + tap] = s.y;
-      tile[(cl + 2) * taps + tap] = s.z;
-      tile[(cl + 3) * taps + tap] = s.w;
+      float* t = tile + y * chunk * taps;
+      t[cl * taps + tap] = s.x;
+      t[(cl + 1) * taps + tap] = s.y;
+      t[(cl + 2) * taps + tap] = s.z;
+      t[(cl + 3) * taps + tap] = s.w;
     }
     __syncthreads();
     const int n4 = (n_c * taps) >> 2;                  // n_c is a multiple of 4
     for (int idx = threadIdx.x; idx < n4; idx += 256) {
       float4 v = *reinterpret_cast<const float4*>(tile + 4 * idx);
+      for (int y = 1; y < sp; ++y) {
+        const float4 u = *reinterpret_cast<const float4*>(tile + y * chunk * taps + 4 * idx);
+        v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
+      }
       if (accumulate) {
         const float4 d = *reinterpret_cast<const float4*>(out + 4 * idx);
         v.x += d.x; v.y += d.y; v.z += d.z; v.w += d.w;
@@ -946,9 +992,11 @@ cudaError_t launch_weight_grad_tc(const surgeon_compressed& act, const surgeon_l
       while (chunk > 32 && (static_cast<long long>(dp.o_real) * ((dp.C + chunk - 1) / chunk) < 4LL * sm_count() ||
                             chunk * dp.taps * 4 > 48 * 1024))
         chunk >>= 1;
+      int sp = 1;
+      while (dp.C % 4 == 0 && sp < 8 && chunk / 4 * dp.taps * sp < 256 && dp.splits >= 4 * sp) sp *= 2;
       launch_kernel(reduce_splits_taps_kernel, dim3((dp.C + chunk - 1) / chunk, dp.o_real), dim3(256),
-                    static_cast<size_t>(chunk) * dp.taps * sizeof(float), stream, true,
-                    static_cast<const float*>(partial), dp.o_real, dp.C, dp.taps, chunk, dp.splits, dw, accumulate,
+                    static_cast<size_t>(chunk) * dp.taps * sp * sizeof(float), stream, true,
+                    static_cast<const float*>(partial), dp.o_real, dp.C, dp.taps, chunk, dp.splits, sp, dw, accumulate,
                     static_cast<const uint32_t*>(status), act.header);
     }
 
