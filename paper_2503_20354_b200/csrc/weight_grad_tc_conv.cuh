@@ -100,6 +100,11 @@ struct DirectParams {
   int kh, kw, pad, in_h, oh;  // taps > 1: kernel and map sizes (with ow, in_w)
   int o_real;               // output channels of the layer; O = taps * o_real
   int row_shift;            // taps > 1: only the kw column shifts are stored; rows shift by TMA offset
+  int tg;                   // k x k on one transposed gradient copy: 1-5 (see weight_grad_tc_direct.cu), else 0
+  int map_rows, kpos;       // tg: whole map rows per K-tile, and their positions
+  int k_rows;               // tg: k-rows of a 64-channel slab in shared memory
+  int unit_bytes, b_bytes;  // tg: bytes of a unit's slabs, and of a stage
+  unsigned box_bytes;       // tg: bytes one box brings
   int copies;               // stacked gradient copies: taps, or kw with row_shift
   int g_len;                // conv: elements per row of the gradient copy (T, or oh * in_w)
   int upt, n_units;         // conv: accumulator units per tap (of acc_n columns), units in all
@@ -119,6 +124,7 @@ struct DirectParams {
   unsigned partial_blk;     // index of the bitmap's last block if it is partial, else 0xFFFFFFFF
 };
 bool plan_direct(const surgeon_layer_desc& d, DirectParams* out);
+bool plan_direct_copies(const surgeon_layer_desc& d, DirectParams* out);   // never a transposed gradient copy
 size_t direct_grad_bf16_bytes(const DirectParams& p);
 // partial = [splits][O][C] fp32 (O counts the stacked taps), status = one word (the pre-pass zeroes it).
 cudaError_t launch_direct(const surgeon_compressed& act, const DirectParams& p,

@@ -678,7 +678,7 @@ int swap_resident_pairs() { return resident_pairs(); }
 static bool compute_plan_swap(const surgeon_layer_desc& d, SwapParams* out) {
   SwapParams best{};
   DirectParams dp;
-  if (!plan_direct(d, &dp)) return false;
+  if (!plan_direct_copies(d, &dp)) return false;
   if (dp.mode == 2 || dp.C < 32) return false;
   if (dp.mode == 0 && (dp.C % 128) != 0) return false;      // whole 64-channel slabs per CTA
   // a TMA box of 128 gradient rows must fit the tensor of all copies

@@ -1,0 +1,169 @@
+"""Sizes at which the variants that a dispatch chooses between can go wrong: edges of tiles and remainders,
+the smallest and the largest of each range, against the oracle."""
+import numpy as np
+import pytest
+import torch
+from dataclasses import replace
+
+import oracle
+from paper_2503_20354_b200 import binding as B
+from paper_2503_20354_b200 import workloads as W
+from gpu_util import assert_store_equals_oracle, oracle_dw, rel_frobenius
+
+pytestmark = pytest.mark.gpu
+
+
+def _dw(layer, ratio, path, seed=5):
+    a, g = W.activation(layer, seed), W.grad_out(layer, seed)
+    comp, ref = assert_store_equals_oracle(a, ratio)
+    dw = B.surgeon_weight_grad(comp, B.layer_desc(layer, path), g.cuda()).cpu().numpy()
+    dense = oracle.decompress(ref["bitmap"], ref["values"], a.numel())
+    if layer.dt == W.BF16:
+        dense = dense.view(np.uint16)
+    assert comp.read_header().status == B.SURGEON_OK
+    return dw, oracle_dw(layer, dense, g.numpy())
+
+
+TRANSPOSED = [
+    # slabs (maps 16, 32, 64 wide): partial last K-tile, channels past a row tile, columns past a unit
+    W.conv("slab16", 3, 40, 16, 72, 3),
+    W.Layer("slab16_h5", 1, 5, 24, 5, 16, 48, 3, 3, 1, 1),
+    W.Layer("slab32_h3", 1, 7, 144, 3, 32, 176, 3, 3, 1, 1),
+    W.Layer("slab64_h1", 1, 9, 20, 1, 64, 64, 3, 3, 1, 1),
+    W.conv("slab64", 1, 20, 64, 328, 3),
+    # boxes with halo rows (rows a multiple of 8 wide)
+    W.conv("halo8", 9, 72, 8, 168, 3),
+    W.Layer("halo8_h3", 1, 4, 20, 3, 8, 56, 3, 3, 1, 1),
+    W.conv("halo24", 2, 20, 24, 64, 3),
+    W.conv("halo56", 1, 40, 56, 48, 3),
+    W.conv("halo16_nopad", 2, 20, 16, 64, 3, 1, 0),
+    W.Layer("halo16_2x3", 1, 2, 20, 9, 16, 48, 2, 3, 1, 1),
+    # a box per tap (other widths, other kernels)
+    W.conv("tap7", 9, 40, 7, 136, 3),
+    W.conv("tap14", 3, 24, 14, 264, 3),
+    W.conv("tap30_5x5", 2, 20, 30, 48, 5, 1, 2),
+    W.conv("tap3_7x7", 11, 24, 3, 64, 7, 1, 3),
+    W.conv("tap1", 70, 24, 1, 56, 3),
+    # just outside: wider than a K-tile, too few or unaligned output channels
+    W.conv("copies65", 1, 20, 65, 64, 3),
+    W.conv("copies72", 1, 20, 72, 56, 3),
+    W.conv("copies_o52", 2, 20, 16, 52, 3),
+]
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("layer", TRANSPOSED, ids=lambda l: l.name)
+def test_stride_one_taps(layer, bf16):
+    dw, ref = _dw(replace(layer, dt=W.BF16 if bf16 else W.F32), 0.6, B.PATH_TENSOR_CORE)
+    assert rel_frobenius(dw, ref) <= 5e-3
+
+
+STRIDED = [
+    W.conv("s2_w17", 3, 20, 17, 40, 3, 2),
+    W.conv("s2_w112_many_macros", 1, 3, 112, 16, 7, 2, 3),
+    W.conv("s2_two_units", 2, 30, 14, 520, 3, 2),
+    W.conv("s3_5x5", 2, 9, 23, 24, 5, 3, 2),
+    W.conv("s8", 2, 20, 64, 64, 8, 8, 0),
+    W.conv("s2_2x2_c70", 1, 70, 30, 24, 2, 2, 0),
+    W.conv("s1_c8", 3, 8, 33, 24, 3),
+    W.conv("s1_c16_w40", 2, 16, 40, 160, 3),
+    W.conv("s2_long_reduction", 40, 8, 20, 8, 3, 2),
+]
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("layer", STRIDED, ids=lambda l: l.name)
+def test_expanded_operand(layer, bf16):
+    dw, ref = _dw(replace(layer, dt=W.BF16 if bf16 else W.F32), 0.4, B.PATH_TENSOR_CORE)
+    assert rel_frobenius(dw, ref) <= 5e-3
+
+
+@pytest.mark.parametrize("layer", [
+    W.conv("c_stride2", 3, 9, 33, 70, 3, 2), W.conv("c_wide", 1, 5, 70, 9, 3), W.conv("c_stride5", 2, 30, 41, 65, 5, 5, 2),
+    W.conv("c_w3", 9, 20, 3, 129, 3), W.linear("l", 77, 129, 65, dt=W.F32), W.linear("l1", 1, 128, 64, dt=W.F32)],
+    ids=lambda l: l.name)
+def test_fp32_tiles(layer):
+    dw, ref = _dw(layer, 0.5, B.PATH_FP32)
+    assert rel_frobenius(dw, ref) <= 1e-5
+
+
+@pytest.mark.parametrize("batch,c_in,c_out,k", [(256, 16, 20, 1), (300, 64, 64, 1), (64, 7, 9, 1), (64, 20, 20, 3)])
+def test_reductions_of_small_weights(batch, c_in, c_out, k):
+    layer = W.conv("r", batch, c_in, 8, c_out, k)
+    dw, ref = _dw(layer, 0.5, B.PATH_TENSOR_CORE)
+    assert rel_frobenius(dw, ref) <= 5e-3
+    a, g = W.activation(layer, 5).cuda(), W.grad_out(layer, 5).cuda()
+    comp, d = B.surgeon_prune_compact(a, 0.5), B.layer_desc(layer, B.PATH_TENSOR_CORE)
+    acc = torch.ones(layer.dw_shape, device="cuda")
+    B.surgeon_weight_grad(comp, d, g, dw=acc, accumulate=True)
+    torch.testing.assert_close(acc, 1 + torch.from_numpy(dw).cuda(), rtol=1e-5, atol=1e-6)
+
+
+# prune: whole chunks and one element around them, resident and streamed ranges (a CTA's range is resident up to 48
+# chunks of 4 KB), counts in global memory (beyond 512 chunks per CTA on 148 SMs)
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("chunks,extra", [(1, 0), (16, 1), (17, -1), (48 * 148, 0), (48 * 148, 1), (512 * 148 + 1, 3)])
+def test_prune_ranges(chunks, extra, bf16):
+    n = chunks * (2048 if bf16 else 1024) + extra
+    x = W.draw("relu_normal", n, seed=4, device="cuda").cpu()
+    x = x.to(torch.bfloat16) if bf16 else x
+    for ratio in (0.3, 0.85):
+        assert_store_equals_oracle(x, ratio)
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+def test_sample_that_misleads(bf16):
+    """A short stretch holds all the large values: the strided sample sees few of them or none, so the bracket can
+    miss and the select has to start over with what its counts prove."""
+    n = 1 << 23
+    for where in (0, n // 2 + 13, n - 5000):
+        x = W.draw("normal", n, seed=9) * 1e-3
+        x[where:where + 5000] = W.draw("normal", 5000, seed=10) * 100.0
+        x = x.to(torch.bfloat16) if bf16 else x
+        for ratio in (1 - 2500 / n, 1 - 5000 / n, 1 - 5200 / n):
+            assert_store_equals_oracle(x, ratio)
+
+
+@pytest.mark.parametrize("n", [5000, (1 << 23) + 77])
+def test_captured_call_replays_and_alternating_streams(n):
+    xs = [W.draw("normal", n, seed=20 + i).cuda() for i in range(3)]
+    ref = [B.surgeon_prune_compact(x, 0.8).to_numpy()[:3] for x in xs]
+    x, out = xs[0].clone(), B.CompressedActivation(n, B.SURGEON_F32, 0.0, "cuda")
+    ws = torch.empty(out.sizes.workspace_bytes, dtype=torch.uint8, device="cuda")
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        B.surgeon_prune_compact(x, 0.8, out=out, workspace=ws)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        B.surgeon_prune_compact(x, 0.8, out=out, workspace=ws)
+    for i in (1, 2, 0, 1):                      # the replays of one graph carry the same call
+        x.copy_(xs[i])
+        graph.replay()
+        torch.cuda.synchronize()
+        assert out.read_header().status == B.SURGEON_OK
+        assert all(np.array_equal(u, v) for u, v in zip(out.to_numpy()[:3], ref[i]))
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    outs = [B.CompressedActivation(n, B.SURGEON_F32, 0.0, "cuda") for _ in range(3)]
+    wss = [torch.empty_like(ws) for _ in range(3)]
+    torch.cuda.synchronize()
+    for _ in range(4):
+        for i in range(3):
+            B.surgeon_prune_compact(xs[i], 0.8, out=outs[i], workspace=wss[i], stream=streams[i])
+    torch.cuda.synchronize()
+    for i in range(3):
+        assert all(np.array_equal(u, v) for u, v in zip(outs[i].to_numpy()[:3], ref[i]))
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("n", [1, 31, 1023, 1025, 4 * 8192 + 5])
+def test_rebuild(n, bf16):
+    x = W.draw("normal", n, seed=30)
+    x = x.to(torch.bfloat16) if bf16 else x
+    for ratio in (0.0, 0.5, 0.97):
+        comp, ref = assert_store_equals_oracle(x, ratio)
+        got = B.surgeon_decompress(comp).cpu()
+        got = got.view(torch.int16).numpy() if bf16 else got.numpy()
+        exp = oracle.decompress(ref["bitmap"], ref["values"], n)
+        assert np.array_equal(got.view(np.uint8), exp.view(np.uint8))
