@@ -13,13 +13,14 @@
 //      what a tap reads for consecutive output positions is then consecutive, whatever the stride;
 //   2. a thread copies one chunk of 8 positions of four operand rows per K-tile: five 4-byte loads, a
 //      funnel shift where the tap's column offset is odd, one 16-byte store.
-// One group rebuilds while the other copies; the bitmap words and offsets of a macro's first pieces are
-// fetched while the macro before it is copied.  Bound by the latency of step 1's two dependent loads
-// and by the gradient tiles' traffic from L2.  The kernels before it copied element by element
+// One group rebuilds while the other copies; the words and the values of a macro's first pieces are
+// fetched while the macro before it is copied.  Bound by the instructions of the two steps.  The kernels before it copied element by element
 // (7x7 stride 2 on 224x224, 3 -> 64 channels, batch 64: 465 us a call) or rebuilt the rows for every
 // K-tile (3x3 stride 2 on 56x56, 128 channels: 215 us).
 // Every wait is bounded and ends in SURGEON_ERR_TIMEOUT.
 #include <cuda.h>
+
+#include <cstddef>
 
 #include "surgeon_internal.cuh"
 #include "tc_common.cuh"
@@ -41,16 +42,75 @@ constexpr int kMaxStages = 8;
 constexpr int kATileBytes = kTileM * kTileK * 2;
 constexpr int kMaxPatchBytes = 44 * 1024;                 // per group
 constexpr int kPiece = 16;                                // elements of a row that one lane rebuilds
-constexpr int kAhead = 8;                                 // values in flight per lane
 
 __device__ __forceinline__ void group_sync(int g) {
   asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(kGroupThreads) : "memory");
 }
 
+// A piece whose values are on their way: the 16-byte vectors that hold its up to 16 packed values (a load per
+// value touches a cache line per lane and value, and the L1 takes one line per clock).
+template <int DT>
+struct PieceValues {
+  static constexpr int kVals = DT == 0 ? 4 : 8;           // values per vector
+  static constexpr int kVecs = kPiece / kVals + 1;        // vectors a piece can span
+  uint32_t w[4 * kVecs];
+  uint32_t a, bits, dst, col;                             // misalignment of the first value; bits; place
+  int m;                                                  // macro
+};
+template <int DT>
+__device__ __forceinline__ void load_values(const void* __restrict__ values, uint32_t rank, uint32_t count,
+                                            uint32_t n_keep, PieceValues<DT>& v) {
+  constexpr uint32_t V = PieceValues<DT>::kVals;
+  constexpr int NV = PieceValues<DT>::kVecs;
+  v.a = rank & (V - 1);
+  const uint32_t base = rank - v.a;
+  const uint32_t n_vec = count ? (v.a + count + V - 1) / V : 0u;
+  const unsigned char* src = static_cast<const unsigned char*>(values) + static_cast<size_t>(base) * (16 / V);
+  if (base + n_vec * V <= n_keep) {
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      uint4 q = make_uint4(0, 0, 0, 0);
+      if (static_cast<uint32_t>(j) < n_vec) q = __ldg(reinterpret_cast<const uint4*>(src) + j);
+      v.w[4 * j] = q.x; v.w[4 * j + 1] = q.y; v.w[4 * j + 2] = q.z; v.w[4 * j + 3] = q.w;
+    }
+  } else {                                                // a vector that ends past the last value
+#pragma unroll
+    for (int j = 0; j < 4 * NV; ++j) {
+      constexpr uint32_t kPerWord = V / 4;
+      uint32_t t = 0;
+#pragma unroll
+      for (uint32_t i = 0; i < kPerWord; ++i) {
+        const uint32_t e = base + j * kPerWord + i;
+        if (e < n_keep)
+          t |= DT == 0 ? __ldg(static_cast<const uint32_t*>(values) + e)
+                       : static_cast<uint32_t>(__ldg(static_cast<const unsigned short*>(values) + e)) << (16 * i);
+      }
+      v.w[j] = t;
+    }
+  }
+}
+// The values as bf16 pairs in order (h[0] holds the first two).
+template <int DT>
+__device__ __forceinline__ void line_up(PieceValues<DT>& v, uint32_t (&h)[8]) {
+  constexpr int N = 4 * PieceValues<DT>::kVecs;
+  const uint32_t words = DT == 0 ? v.a : v.a >> 1;        // whole words to drop: 0-3
+#pragma unroll
+  for (int j = 0; j < N - 2; ++j) v.w[j] = (words & 2u) ? v.w[j + 2] : v.w[j];
+#pragma unroll
+  for (int j = 0; j < N - 3; ++j) v.w[j] = (words & 1u) ? v.w[j + 1] : v.w[j];
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    h[j] = DT == 0 ? pack_bf16x2(__uint_as_float(v.w[2 * j]), __uint_as_float(v.w[2 * j + 1]))
+                   : __funnelshift_r(v.w[j], v.w[j + 1], (v.a & 1u) * 16u);
+}
+
 // What a lane fetches for its piece: the kept count before the 128-element block the piece starts in, the
-// words of the block before the piece's, its word and the one after it.
+// block's words and the one after the piece's; and where the piece goes.
 struct PieceRaw {
-  uint32_t off, b0, b1, b2, w0, w1, sh;
+  uint32_t off, next, start, len;
+  uint4 words;
+  uint32_t dst, col;       // patch element of the row's first column, the piece's first column
+  int m;                   // its macro
 };
 
 template <int DT>
@@ -163,6 +223,7 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
     unsigned char* patch = smem + p.stages * stage_bytes + g * p.patch_bytes;
     unsigned short* patch16 = reinterpret_cast<unsigned short*>(patch);
     const uint32_t patch_addr = smem_u32(patch);
+    const uint32_t n_keep = static_cast<uint32_t>(__ldg(p.n_keep_ptr));   // packed values in the store
     const int c_first = nn0 / p.RS;
     const int c_last = min(nn0 + kTileM - 1, p.n_gemm - 1) / p.RS;
     const int n_ch = c_last - c_first + 1;
@@ -189,49 +250,53 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
       }
     }
     // A macro's input rows and its pieces (channel, row, 16 columns).
-    struct Macro { int img, kt0, n_t, iy_lo, n_pieces, per_ch; };
-    const int per_row = (p.W + kPiece - 1) / kPiece;
+    // (32-bit indices, and divisions by multiplication: a piece costs a few hundred instructions in all, and
+    // they are what the kernel spends its time on)
+    struct Macro { int kt0, n_t, iy_lo; uint32_t n_pieces, per_ch, inv_ch, start; };
+    const uint32_t per_row = (p.W + kPiece - 1) / kPiece;
+    const uint32_t inv_row = p.inv_per_row;
     auto geometry = [&](int m) {
       Macro q;
-      q.img = m / p.macros_per_img;
-      q.kt0 = (m - q.img * p.macros_per_img) * p.macro;
+      const int img = m / p.macros_per_img;
+      q.kt0 = (m - img * p.macros_per_img) * p.macro;
       q.n_t = tiles_of(m);
       const int y_first = q.kt0 * kTileK / p.OWp;
       const int y_last = min((q.kt0 + q.n_t) * kTileK - 1, p.P - 1) / p.OWp;
       q.iy_lo = max(y_first * p.stride - p.pad, 0);
       const int iy_hi = min(y_last * p.stride + p.KH - 1 - p.pad, p.H - 1);
-      q.per_ch = (iy_hi - q.iy_lo + 1) * per_row;
+      q.per_ch = static_cast<uint32_t>(iy_hi - q.iy_lo + 1) * per_row;
+      q.inv_ch = q.per_ch > 1 ? 0xFFFFFFFFu / q.per_ch + 1u : 0u;       // exact below 2^16 pieces
       q.n_pieces = n_ch * q.per_ch;
+      q.start = (static_cast<uint32_t>(img) * p.C + c_first) * (p.H * p.W) + q.iy_lo * p.W;
       return q;
     };
-    auto place = [&](const Macro& q, int t, int* ci, int* row, int* col) {
-      *ci = t / q.per_ch;
-      const int rest = t - *ci * q.per_ch;
-      *row = rest / per_row;
-      *col = (rest - *row * per_row) * kPiece;
-    };
-    auto fetch = [&](const Macro& q, int t) {
-      PieceRaw r = {};
+    auto fetch = [&](const Macro& q, uint32_t t) {
+      PieceRaw r;
+      r.m = 0x7FFFFFFF; r.len = 0; r.off = 0; r.next = 0; r.start = 0; r.words = make_uint4(0, 0, 0, 0); r.dst = 0; r.col = 0;
       if (t < q.n_pieces) {
-        int ci, row, col;
-        place(q, t, &ci, &row, &col);
-        const long long start =
-            ((static_cast<long long>(q.img) * p.C + c_first + ci) * p.H + q.iy_lo + row) * p.W + col;
-        const long long blk = start >> kBlockShift, wi = start >> 5;
-        const int before = static_cast<int>(wi - blk * kBlockWords);
-        r.sh = static_cast<uint32_t>(start & 31);
+        const uint32_t ci = q.per_ch > 1 ? __umulhi(t, q.inv_ch) : t;
+        const uint32_t rest = t - ci * q.per_ch;
+        const uint32_t row = per_row > 1 ? __umulhi(rest, inv_row) : rest;
+        r.col = (rest - row * per_row) * kPiece;
+        r.dst = (ci * p.patch_rows + row) * row_len + 8;
+        r.start = q.start + ci * (p.H * p.W) + row * p.W + r.col;
+        r.len = min(static_cast<uint32_t>(kPiece), p.W - r.col);
+        const uint32_t blk = r.start >> kBlockShift;
         r.off = __ldg(offsets + blk);
-        r.b0 = before > 0 ? __ldg(bitmap + wi - before) : 0u;
-        r.b1 = before > 1 ? __ldg(bitmap + wi - before + 1) : 0u;
-        r.b2 = before > 2 ? __ldg(bitmap + wi - before + 2) : 0u;
-        r.w0 = __ldg(bitmap + wi);
-        r.w1 = (r.sh > 32u - kPiece && wi + 1 < p.n_words) ? __ldg(bitmap + wi + 1) : 0u;
+        if (blk != p.partial_blk) {
+          r.words = __ldg(reinterpret_cast<const uint4*>(bitmap) + blk);
+        } else {                                   // the last, partial block of the bitmap
+          const uint32_t w0 = blk * kBlockWords;
+          r.words.x = __ldg(bitmap + w0);
+          r.words.y = (w0 + 1 < p.n_words) ? __ldg(bitmap + w0 + 1) : 0u;
+          r.words.z = (w0 + 2 < p.n_words) ? __ldg(bitmap + w0 + 2) : 0u;
+          r.words.w = (w0 + 3 < p.n_words) ? __ldg(bitmap + w0 + 3) : 0u;
+        }
+        const uint32_t wi = r.start >> 5;          // (within the block the next word is at hand)
+        if ((wi & 3u) == 3u && (r.start & 31u) > 32u - kPiece && wi + 1 < p.n_words) r.next = __ldg(bitmap + wi + 1);
       }
       return r;
     };
-    // The ring place of the next tile.  A barrier's phase is told by one bit: a macro is shorter than the
-    // ring (see the plan), so that the tile of this place two rounds ago is known to be consumed when
-    // the warp comes to wait for the last one.
     int s = 0;
     uint32_t round = 0;
     auto skip_tiles = [&](int n) {                 // the other group's
@@ -247,12 +312,39 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
         atomicMax(status, static_cast<uint32_t>(SURGEON_ERR_TIMEOUT));
       }
     };
-    PieceRaw raw[2] = {};                          // the next two pieces
-    if (m_begin + g < m_end) {
-      const Macro q = geometry(m_begin + g);
-      raw[0] = fetch(q, gtid);
-      raw[1] = fetch(q, gtid + kGroupThreads);
-    }
+    // The thread's pieces are one stream over the group's macros: the words of a piece are fetched while the
+    // values of the one before it are on their way, and those while the one before that is placed.
+    // What is fetched ahead at a macro's end hides behind the copying of its operand tiles.
+    int fm = m_begin + g;                          // macro and index of the next piece to fetch
+    uint32_t ft = gtid;
+    Macro fq = geometry(fm < m_end ? fm : m_begin);
+    auto fetch_next = [&]() {
+      while (fm < m_end && ft >= fq.n_pieces) {
+        fm += kGroups;
+        ft = gtid;
+        if (fm < m_end) fq = geometry(fm);
+      }
+      PieceRaw r = fetch(fq, fm < m_end ? ft : 0xFFFFFFFFu);
+      if (fm < m_end) { r.m = fm; ft += kGroupThreads; }
+      return r;
+    };
+    auto issue = [&](const PieceRaw& r, PieceValues<DT>& v) {
+      const uint32_t wq = (r.start >> 5) & 3u, sh = r.start & 31u;
+      uint32_t rank = r.off;
+      rank += wq > 0 ? __popc(r.words.x) : 0u;
+      rank += wq > 1 ? __popc(r.words.y) : 0u;
+      rank += wq > 2 ? __popc(r.words.z) : 0u;
+      const uint32_t w0 = wq == 0 ? r.words.x : (wq == 1 ? r.words.y : (wq == 2 ? r.words.z : r.words.w));
+      const uint32_t w1 = wq == 3 ? r.next : (wq == 0 ? r.words.y : (wq == 1 ? r.words.z : r.words.w));
+      rank += __popc(w0 & ((1u << sh) - 1u));
+      v.bits = __funnelshift_r(w0, w1, sh) & ((1u << r.len) - 1u);
+      v.dst = r.dst; v.col = r.col; v.m = r.m;
+      load_values<DT>(values, rank, __popc(v.bits), n_keep, v);
+    };
+    PieceValues<DT> ready;
+    PieceRaw raw = fetch_next();
+    issue(raw, ready);
+    raw = fetch_next();
     for (int m = m_begin + g; m < m_end; m += kGroups) {
       const Macro q = geometry(m);
       const int kt0 = q.kt0, n_t = q.n_t, iy_lo = q.iy_lo;
@@ -260,40 +352,30 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
       for (int v = gtid; v < p.patch_bytes / 16; v += kGroupThreads)
         reinterpret_cast<uint4*>(patch)[v] = make_uint4(0, 0, 0, 0);
       group_sync(g);
-      for (int t = gtid; t < q.n_pieces; t += kGroupThreads) {
-        const PieceRaw r = raw[0];
-        raw[0] = raw[1];
-        raw[1] = fetch(q, t + 2 * kGroupThreads);
-        int ci, row, col;
-        place(q, t, &ci, &row, &col);
-        uint32_t rank = r.off + __popc(r.b0) + __popc(r.b1) + __popc(r.b2) + __popc(r.w0 & ((1u << r.sh) - 1u));
-        const int len = min(kPiece, p.W - col);
-        uint32_t bits = __funnelshift_r(r.w0, r.w1, r.sh) & ((1u << len) - 1u);
-        unsigned short* dst = patch16 + (ci * p.patch_rows + row) * row_len + 8;
-        for (int left = __popc(bits); left > 0; left -= kAhead) {
-          uint32_t v[kAhead];
+      while (ready.m == m) {
+        PieceValues<DT> now = ready;
+        issue(raw, ready);
+        raw = fetch_next();
+        uint32_t h[8], bits = now.bits;
+        const uint32_t count = __popc(bits), col = now.col;
+        unsigned short* dst = patch16 + now.dst;
+        line_up<DT>(now, h);
 #pragma unroll
-          for (int i = 0; i < kAhead; ++i) v[i] = ld_packed<DT>(values, rank + i, i < left);
-          rank += kAhead;
+        for (int i0 = 0; i0 < kPiece; i0 += 4) {
+          if (static_cast<uint32_t>(i0) < count) {
 #pragma unroll
-          for (int i = 0; i < kAhead; ++i) {
-            if (i < left) {
-              const uint32_t ix = col + __ffs(bits) - 1;
-              bits &= bits - 1;
-              const uint32_t qq = (ix * p.inv_stride) >> 16;       // ix / stride
-              if (qq + 8 < static_cast<uint32_t>(p.plane))         // (columns no tap reads)
-                dst[(ix - qq * p.stride) * p.plane + qq] =
-                    (DT == 0) ? to_bf16_bits(__uint_as_float(v[i])) : static_cast<unsigned short>(v[i]);
+            for (int i = i0; i < i0 + 4; ++i) {
+              if (static_cast<uint32_t>(i) < count) {
+                const uint32_t ix = col + __ffs(bits) - 1;         // (bits has a set bit left)
+                bits &= bits - 1;
+                const uint32_t qq = (ix * p.inv_stride) >> 16;     // ix / stride
+                dst[(ix - qq * p.stride) * p.plane + qq] = static_cast<unsigned short>(h[i >> 1] >> (16 * (i & 1)));
+              }
             }
           }
         }
       }
       group_sync(g);
-      if (m + kGroups < m_end) {                   // in flight while this macro's tiles are copied
-        const Macro nx = geometry(m + kGroups);
-        raw[0] = fetch(nx, gtid);
-        raw[1] = fetch(nx, gtid + kGroupThreads);
-      }
       // ---- the operand tiles ----
       for (int t = 0; t < n_t; ++t) {
         wait_stage();
@@ -387,10 +469,14 @@ bool compute_plan_strided(const surgeon_layer_desc& d, StridedParams* out) {
   p.n_gemm = d.c_in * p.RS;
   // 8 zeros to the left of a plane: tap columns reach at most 8 places over the edge; ix / stride by a multiplication
   if ((d.pad + d.stride - 1) / d.stride > 8 || (d.kw - 1) / d.stride > 5 || d.stride > 64 || d.w > 4096) return false;
+  const unsigned per_row = (d.w + kPiece - 1) / kPiece;
+  p.inv_per_row = per_row > 1 ? 0xFFFFFFFFu / per_row + 1u : 0u;
   p.inv_stride = (65536 + d.stride - 1) / d.stride;
   for (int ix = 0; ix < d.w; ++ix)
     if (static_cast<int>((static_cast<unsigned>(ix) * p.inv_stride) >> 16) != ix / d.stride) return false;
-  p.plane = p.OWp + 16;                            // elements; an odd number of words, against bank conflicts
+  // elements of a plane: 8 zeros, then the row or what its last chunk reads, whichever is longer; an odd number of
+  // words, against bank conflicts
+  p.plane = p.OWp + 16 > (d.w - 1) / d.stride + 9 ? p.OWp + 16 : ((d.w - 1) / d.stride + 9 + 1) / 2 * 2;
   if ((p.plane / 2) % 2 == 0) p.plane += 2;
   p.m_tiles = (p.n_gemm + kTileM - 1) / kTileM;
   const int n_ch = p.RS >= kTileM ? 2 : (p.C < (kTileM - 2) / p.RS + 2 ? p.C : (kTileM - 2) / p.RS + 2);
@@ -472,6 +558,9 @@ cudaError_t launch_strided(const surgeon_compressed& act, const StridedParams& p
                            void* grad_bf16, float* partial, uint32_t* status, cudaStream_t stream) {
   StridedParams p = plan;
   p.n_words = (act.n + 31) / 32;
+  p.partial_blk = (act.n % SURGEON_BLOCK) ? static_cast<unsigned>(act.n / SURGEON_BLOCK) : 0xFFFFFFFFu;
+  p.n_keep_ptr = reinterpret_cast<const long long*>(reinterpret_cast<const char*>(act.header) +
+                                                    offsetof(surgeon_header, n_keep));
   cudaError_t e = p.OW == p.OWp
                       ? launch_grad_to_bf16(grad_out, static_cast<long long>(p.B) * p.O * p.P, grad_bf16, status, stream)
                       : launch_grad_to_bf16_rows(grad_out, static_cast<long long>(p.B) * p.O * p.OH, p.OW, p.OWp,
