@@ -130,7 +130,8 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
   const int tid = threadIdx.x;
   const int warp = tid >> 5;
   const uint32_t lane = lane_id();
-  const int nn0 = blockIdx.x * kTileM;
+  const int nn0 = blockIdx.x * p.rows_per_tile;           // the im2col rows are spread evenly over the row tiles
+  const int nn_end = min(nn0 + p.rows_per_tile, p.n_gemm);
   const int o0 = blockIdx.y * n_cols;
   const int n_acc_here = min(p.n_acc, (p.O - o0 + p.acc_n - 1) / p.acc_n);
   const int split = blockIdx.z;
@@ -225,7 +226,7 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
     const uint32_t patch_addr = smem_u32(patch);
     const uint32_t n_keep = static_cast<uint32_t>(__ldg(p.n_keep_ptr));   // packed values in the store
     const int c_first = nn0 / p.RS;
-    const int c_last = min(nn0 + kTileM - 1, p.n_gemm - 1) / p.RS;
+    const int c_last = (nn_end - 1) / p.RS;
     const int n_ch = c_last - c_first + 1;
     const int row_len = p.stride * p.plane;        // elements of one input row in the patch
     // this thread's four operand rows and its chunk of 8 positions
@@ -240,7 +241,7 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
       dst_off[i] = tile_off(row, chunk);
       row_base[i] = 0;
       row_r[i] = -1000000;
-      if (nn < p.n_gemm) {
+      if (nn < nn_end) {
         const int c = nn / p.RS, rs = nn - c * p.RS;
         const int r = rs / p.KW, s = rs - r * p.KW;
         const int d = s - p.pad;
@@ -249,6 +250,12 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
         row_r[i] = r - p.pad;
       }
     }
+    // Rows past the tile's share stay zero in every stage.
+    const int n_mine = max(0, min(4, (p.rows_per_tile - (gtid >> 3) + 31) / 32));
+    for (int st = 0; st < p.stages; ++st)
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (i >= n_mine) *reinterpret_cast<uint4*>(smem + st * stage_bytes + dst_off[i]) = make_uint4(0, 0, 0, 0);
     // A macro's input rows and its pieces (channel, row, 16 columns).
     // (32-bit indices, and divisions by multiplication: a piece costs a few hundred instructions in all, and
     // they are what the kernel spends its time on)
@@ -386,6 +393,7 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
         const int nv = pos < p.P ? p.OW - x0 : 0;          // positions of the chunk that exist
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
+          if (i >= n_mine) break;
           const int iy = y * p.stride + row_r[i];
           uint4 out = make_uint4(0, 0, 0, 0);
           if (iy >= 0 && iy < p.H && nv > 0) {
@@ -431,7 +439,7 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
       for (int col = 16 * ((warp - 2) >> 2); col < cols_here; col += 16 * (kGroups * kGroupWarps / 4)) {
         uint32_t r[16];
         tmem_ld16(tmem_base + (static_cast<uint32_t>(lane_grp * 32) << 16) + col, r);
-        if (nn < p.n_gemm) {
+        if (nn < nn_end) {
 #pragma unroll
           for (int e = 0; e < 16; ++e) {
             const int o = o0 + col + e;
@@ -479,7 +487,9 @@ bool compute_plan_strided(const surgeon_layer_desc& d, StridedParams* out) {
   p.plane = p.OWp + 16 > (d.w - 1) / d.stride + 9 ? p.OWp + 16 : ((d.w - 1) / d.stride + 9 + 1) / 2 * 2;
   if ((p.plane / 2) % 2 == 0) p.plane += 2;
   p.m_tiles = (p.n_gemm + kTileM - 1) / kTileM;
-  const int n_ch = p.RS >= kTileM ? 2 : (p.C < (kTileM - 2) / p.RS + 2 ? p.C : (kTileM - 2) / p.RS + 2);
+  p.rows_per_tile = ((p.n_gemm + p.m_tiles - 1) / p.m_tiles + 7) / 8 * 8;
+  // channels a tile's rows can touch
+  const int n_ch = p.rows_per_tile < 2 ? 1 : (p.C < (p.rows_per_tile - 2) / p.RS + 2 ? p.C : (p.rows_per_tile - 2) / p.RS + 2);
   p.tiles_per_img = (p.P + kTileK - 1) / kTileK;
   // columns: one or two accumulators of at most 256 columns, the fewest padded columns first
   int best_waste = -1;
