@@ -469,15 +469,10 @@ __device__ __forceinline__ uint32_t count_above_mine(uint32_t b, uint32_t* s_war
   const int warp = threadIdx.x >> 5;
   if (lane_id() == 31) s_warp[warp] = excl + b;
   __syncthreads();
-  uint32_t above = excl, all = 0;
-#pragma unroll
-  for (int w = 0; w < kWarps; ++w) {
-    const uint32_t v = s_warp[w];
-    if (w < warp) above += v;
-    all += v;
-  }
-  *total = all;
-  return above;
+  const uint32_t mine = lane_id() < kWarps ? s_warp[lane_id()] : 0u;
+  const uint32_t before = warp_excl_scan(mine);
+  *total = __shfl_sync(kFull, before, 31);       // (lanes past the warps add nothing)
+  return excl + __shfl_sync(kFull, before, warp);
 }
 // The bin with #(bins above) < want <= #(bins >= it): its thread stores it, the count above it and its own.
 __device__ __forceinline__ void place_rank(uint32_t b, uint32_t above, uint32_t want, uint32_t* res) {
@@ -491,33 +486,71 @@ __device__ __forceinline__ uint32_t my_bin(const uint32_t* hist) {
   return threadIdx.x < kSelBins ? hist[kSelBins - 1 - threadIdx.x] : 0u;
 }
 
-// The first n_in keys of a slot, f(key): a warp together (slots in shared memory, a few chunks per
-// warp), or one lane alone with its loads in flight together (slots in global memory, a chunk per lane).
+// The first n_in keys of a slot in shared memory, f(key), a warp together.
 template <int DT, typename F>
 __device__ __forceinline__ void slot_keys_warp(const typename Elem<DT>::type* slot, uint32_t n_in, F f) {
   for (uint32_t i = lane_id(); i < n_in; i += 32) f(static_cast<uint32_t>(slot[i]));
 }
-// f(acc, key) for the listed keys of chunks 0 .. n_local - 1, then done(c, cnt[c], acc); a lane per chunk.
+// Of slots in global memory: f(c, acc, key) for the listed keys of chunks 0 .. n_local - 1, then done(c, cnt[c],
+// the chunk's acc) on one lane.  Half a warp per chunk, 8 bytes per lane (32 fp32 or 64 bf16 keys; few chunks
+// have more) and four chunks in flight: one trip to L2 for 128 chunks.  (A lane per chunk, 64 bytes at a time,
+// took 5-7 us a call.)  Of a larger tensor (`many`) a lane per chunk, which has four times as many chunks in
+// flight and asks for little more than the keys: 128 at a time made 4.3 GB 6 % slower.
 template <int DT, typename F, typename D>
-__device__ __forceinline__ void slot_keys_lane(const typename Elem<DT>::type* slots, const uint32_t* cnt, int n_local, F f, D done) {
-  constexpr uint32_t EPV = 16 / sizeof(typename Elem<DT>::type);
-  for (int c = threadIdx.x; c < n_local; c += kThreads) {
-    const uint32_t v = cnt[c], n_in = min(v >> 16, static_cast<uint32_t>(slot_entries(DT)));
-    uint32_t acc = 0;
-    const uint4* p = reinterpret_cast<const uint4*>(slots + static_cast<long long>(c) * slot_entries(DT));
-    for (uint32_t v0 = 0; v0 * EPV < n_in; v0 += 4) {
-      uint4 q[4];
+__device__ __forceinline__ void slot_keys_global(const typename Elem<DT>::type* slots, const uint32_t* cnt, int n_local, bool many, F f, D done) {
+  if (many) {
+    constexpr uint32_t EPV = 16 / sizeof(typename Elem<DT>::type);
+    for (int c = threadIdx.x; c < n_local; c += kThreads) {
+      const uint32_t v = cnt[c], n_in = min(v >> 16, static_cast<uint32_t>(slot_entries(DT)));
+      uint32_t acc = 0;
+      const uint4* p = reinterpret_cast<const uint4*>(slots + static_cast<long long>(c) * slot_entries(DT));
+      for (uint32_t v0 = 0; v0 * EPV < n_in; v0 += 4) {
+        uint4 q[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) q[u] = (v0 + u) * EPV < n_in ? p[v0 + u] : make_uint4(0, 0, 0, 0);
+        for (int u = 0; u < 4; ++u) q[u] = (v0 + u) * EPV < n_in ? p[v0 + u] : make_uint4(0, 0, 0, 0);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const uint32_t w[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
+        for (int u = 0; u < 4; ++u) {
+          const uint32_t w[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
 #pragma unroll
-        for (uint32_t e = 0; e < EPV; ++e)
-          if ((v0 + u) * EPV + e < n_in) f(acc, (DT == 0) ? w[e % 4] : (w[e >> 1] >> (16 * (e & 1))) & 0xFFFFu);
+          for (uint32_t e = 0; e < EPV; ++e)
+            if ((v0 + u) * EPV + e < n_in) f(c, acc, (DT == 0) ? w[e % 4] : (w[e >> 1] >> (16 * (e & 1))) & 0xFFFFu);
+        }
       }
+      done(c, v, acc);
     }
-    done(c, v, acc);
+    return;
+  }
+  constexpr uint32_t EPW = 8 / sizeof(typename Elem<DT>::type);     // keys of a lane
+  constexpr int kFlight = 4;
+  const uint32_t hl = threadIdx.x & 15u;
+  for (int c0 = (threadIdx.x >> 5) * 2; c0 < n_local; c0 += kFlight * (kThreads / 16)) {
+    const int cf = c0 + static_cast<int>((threadIdx.x >> 4) & 1u);
+    uint32_t v[kFlight];
+    uint2 q[kFlight];
+#pragma unroll
+    for (int u = 0; u < kFlight; ++u) {
+      const int c = cf + u * (kThreads / 16);
+      v[u] = c < n_local ? cnt[c] : 0u;
+      const uint2* p = reinterpret_cast<const uint2*>(slots + static_cast<long long>(c) * slot_entries(DT)) + hl;
+      q[u] = hl * EPW < (v[u] >> 16) ? *p : make_uint2(0, 0);
+    }
+#pragma unroll
+    for (int u = 0; u < kFlight; ++u) {
+      const int c = cf + u * (kThreads / 16);
+      const uint32_t n_in = min(v[u] >> 16, static_cast<uint32_t>(slot_entries(DT)));
+      uint32_t acc = 0;
+#pragma unroll
+      for (uint32_t e = 0; e < EPW; ++e) {
+        const uint32_t w = (DT == 0 ? e : e >> 1) ? q[u].y : q[u].x;
+        if (hl * EPW + e < n_in) f(c, acc, DT == 0 ? w : (w >> (16 * (e & 1))) & 0xFFFFu);
+      }
+#pragma unroll 1
+      for (uint32_t i = 16 * EPW + hl; i < n_in; i += 16)
+        f(c, acc, static_cast<uint32_t>(slots[static_cast<long long>(c) * slot_entries(DT) + i]));
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
+      if (hl == 0 && c < n_local) done(c, v[u], acc);
+    }
   }
 }
 
@@ -566,6 +599,8 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
   __shared__ uint32_t s_tot[4];                // keys above / inside the bracket, largest key inside, largest ~key inside
   __shared__ uint32_t s_over, s_fail, s_nkeys;
   __shared__ unsigned long long s_ans[2];
+  __shared__ uint32_t s_bin_key[kMaxKeys];      // the keys that this CTA reports at the last exchange,
+  __shared__ int s_bin_chunk[kMaxKeys];        // and their chunks
 
   const int tid = threadIdx.x;
   const int warp = tid >> 5;
@@ -701,8 +736,8 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     if (master) {
       if (tid < G) {
         ok = word_wait(a.arrive + phase * kSelMaxCtas + tid, a.token, &ignored);
-        a.arrive[phase * kSelMaxCtas + tid].x = 0ull;
         fence_gpu();
+        a.arrive[phase * kSelMaxCtas + tid].x = 0ull;
       }
       prepare_phase(a, phase + 1);
       ok = __syncthreads_and(ok);
@@ -741,15 +776,20 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
   // A resident tensor: 2048 vectors of 32 (fp32) or 16 (bf16) bytes, one per stratum, the same for
   // every CTA (each starts elsewhere in it, so that they do not all ask for the same lines at the
   // same time).  More would not pay: 148 CTAs that read 8192 places took 12 us.  The margin is 4
-  // standard deviations (a miss costs a round).  A larger tensor, for which a miss is another read
-  // of it and a narrow bracket pays: every CTA takes its own 512 or 1024 strata; CTA 0's part gives
-  // a window of bins, in which the CTAs' histograms are added up (all bins together: 150 thousand
-  // additions, 4 us); the first loads are under way meanwhile.
+  // standard deviations (a miss costs a round).
+  // A larger tensor, for which a miss is another read of it and a narrow bracket pays: every CTA
+  // samples the whole tensor at places of its own (stratum G i + p of the G i-th row, p scrambled from
+  // row to row so that no period of the data falls to one CTA) and reports where the threshold lies in
+  // its own 4 or 8 thousand elements.  The CTAs' answers are independent draws whose median is the
+  // threshold, however the elements are distributed, so the ones 2.5 sqrt(G) places (5 standard
+  // deviations) to either side of the middle bound it: 0.4 % of the elements to each side, as the sum of
+  // all histograms would give.  One exchange of one word per CTA, 4 us less than a window from CTA 0's part
+  // and added-up histograms took.
   uint32_t lo = 1, hi = kKeyMax;
   const uint32_t n_vec = static_cast<uint32_t>(a.n / EPV);
   constexpr int kPer = RES ? (DT == 0 ? 8 : 4) : 2;       // vectors per thread
   constexpr int kBinShift = Elem<DT>::kKeyBits - kSampleBinsLog2;
-  constexpr float kSigmas = RES ? 4.0f : 5.0f;
+  constexpr int kFineShift = kBinShift > kSelBinsLog2 ? kBinShift - kSelBinsLog2 : 0;     // (!RES)
   uint4 v[kPer];
   {
     constexpr uint32_t kStrata = kPer * kThreads / (DT == 0 ? 2 : 1);     // of this CTA
@@ -759,7 +799,12 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     for (int u = 0; u < kPer; ++u) {
       uint32_t loc = u * kThreads + tid, part = 0;
       if (DT == 0) { part = loc & 1u; loc >>= 1; }         // two lanes share a stratum: 32 bytes
-      loc = RES ? (loc + blockIdx.x * 37u) % kStrata : blockIdx.x * kStrata + loc;
+      if (RES) {
+        loc = (loc + blockIdx.x * 37u) % kStrata;
+      } else {
+        const uint32_t at_row = blockIdx.x + __umulhi(hash_u32(loc + 0x9E3779B9u), static_cast<uint32_t>(G));
+        loc = loc * G + (at_row >= static_cast<uint32_t>(G) ? at_row - G : at_row);
+      }
       const float at = (static_cast<float>(loc) + static_cast<float>(hash_u32(loc) >> 8) * (1.0f / 16777216.0f)) * stride;
       uint32_t pos = static_cast<uint32_t>(at);
       if (DT == 0) pos = (pos & ~1u) + part;
@@ -789,21 +834,23 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
       if (key) atomicAdd(&hist[bin >> 1], 1u << (16 * (bin & 1)));   // (not the zeros, half of post-ReLU data)
     }
   }
-  // rank of the threshold inside the sample, and a margin of some standard deviations of a binomial count
+  // rank of the threshold inside the sample, and (RES) a margin of some standard deviations of a binomial count
   const float q = static_cast<float>(a.k) / static_cast<float>(a.n);
-  auto ranks = [&](float S, float sigmas, uint32_t* r_hi, uint32_t* r_lo) {
-    const float delta = sigmas * sqrtf(S * q * (1.0f - q)) + 16.0f;
-    *r_hi = (q * S - delta >= 1.0f) ? static_cast<uint32_t>(q * S - delta) : 0u;           // 0: none
-    *r_lo = (q * S + delta <= S - 1.0f) ? static_cast<uint32_t>(q * S + delta) + 1u : 0u;  // 0: none
-  };
   constexpr float kOwn = static_cast<float>(kPer * kThreads * EPV);        // elements in this CTA's histogram
-  uint32_t r_hi, r_lo;
-  ranks(kOwn, RES ? kSigmas : 6.0f, &r_hi, &r_lo);
-  if (!RES && r_hi == 0) r_hi = 1;               // (a window: from the largest key seen)
-  if (tid < 2) s_res[tid] = tid == 0 && r_hi == 0 ? kSampleBins - 1u : 0u;
+  const float up = q * kOwn, down = kOwn - up;   // of them above and below the threshold
+  const bool no_hi = up < 16.0f, no_lo = down < 16.0f;     // (!RES) too few for a median that means something:
+  uint32_t r_hi, r_lo = 0;                       // that side stays open, and the rank moves to the other
+  if (RES) {
+    const float delta = 4.0f * sqrtf(kOwn * q * (1.0f - q)) + 16.0f;
+    r_hi = up - delta >= 1.0f ? static_cast<uint32_t>(up - delta) : 0u;                        // 0: none
+    r_lo = up + delta <= kOwn - 1.0f ? static_cast<uint32_t>(up + delta) + 1u : 0u;            // 0: none
+  } else {
+    r_hi = static_cast<uint32_t>(no_hi ? up + sqrtf(up) + 2.0f : no_lo ? up - sqrtf(down) - 2.0f : up + 0.5f);
+  }
+  if (tid < 2) s_res[tid] = RES && tid == 0 && r_hi == 0 ? kSampleBins - 1u : 0u;
   __syncthreads();
-  if (RES || master) {
-    // the bins of the two ranks in the CTA's own histogram
+  {
+    // the bins of the ranks in the CTA's own histogram
     // thread t owns the 32 bins below 2^14 - 32 t
     const uint4* mine = reinterpret_cast<const uint4*>(hist) + 4 * (kSampleBins / 32 - 1 - tid);
     uint32_t sum = 0;
@@ -817,103 +864,92 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     }
     uint32_t all;
     const uint32_t above = count_above_mine(sum, s_warp, &all);
-#pragma unroll
-    for (int which = 0; which < 2; ++which) {
+#pragma unroll 1
+    for (int which = 0; which < (RES ? 2 : 1); ++which) {
       // (a rank among the zeros lies below every counted bin: bin 0)
       const uint32_t want = which ? r_lo : r_hi;
       if (want && above < want && want <= above + sum) {
         uint32_t acc = above;
         int bin = 31;
+#pragma unroll 1
         for (; bin > 0; --bin) {
           const uint32_t c = (reinterpret_cast<const uint32_t*>(mine)[bin >> 1] >> (16 * (bin & 1))) & 0xFFFFu;
           if (acc + c >= want) break;
           acc += c;
         }
         s_res[which] = static_cast<uint32_t>(kSampleBins - 32 - 32 * tid + bin);
+        if (!RES) s_res[1] = want - acc;         // the rank among the bin's elements
       }
     }
     __syncthreads();
+  }
+  if (RES) {
     lo = max(s_res[1] << kBinShift, 1u);
     hi = (s_res[0] << kBinShift) | ((1u << kBinShift) - 1u);
-    if (!RES && tid == 0) {
-      fence_gpu();
-      word_store(a.answer, a.token, s_res[0]);   // phase 0 as above, and the window's top bin
-      s_ans[0] = s_res[0];
-    }
-  } else if (tid == 0) {
-    unsigned long long ans = 0;
-    if (!RES && !word_wait(a.answer, a.token, &ans)) s_fail = 1;
-    fence_gpu();
-    s_ans[0] = ans;
-  }
-  if (!RES) {
+  } else {
+    // the key's next bits, among the bin's elements (a bin holds about as many elements as the bracket will)
+    const uint32_t bin = s_res[0], want = s_res[1];
+    if (tid < kSelBins) hist[tid] = 0;
     __syncthreads();
-    if (s_fail) { drain(); quit(); return; }
-    // the window: kSelBins bins from its top down (8 octaves; what lies lower, lies lower)
-    const int top = static_cast<int>(s_ans[0]);
-    uint32_t over_top = 0;
-    for (int i = (top >> 1) + tid; i < kSampleBins / 2; i += kThreads) {
-      const uint32_t h = hist[i];
-      over_top += (2 * i > top ? h & 0xFFFFu : 0u) + (2 * i + 1 > top ? h >> 16 : 0u);
-    }
-    over_top = warp_sum(over_top);
-    if (lane == 0 && over_top) atomicAdd(&s_tot[0], over_top);
-    if (tid < kSelBins && tid <= top) {
-      const uint32_t h = (hist[(top - tid) >> 1] >> (16 * ((top - tid) & 1))) & 0xFFFFu;
-      if (h) atomicAdd(&a.hist[kSelBins - 1 - tid], h);
-    }
-    __syncthreads();
-    if (tid == 0) {
-      fence_gpu();
-      word_store(a.arrive + phase * kSelMaxCtas + blockIdx.x, a.token, s_tot[0]);
-    }
-    if (master) {
-      int ok = 1;
-      unsigned long long n_over = 0;
-      if (tid < G) {
-        ok = word_wait(a.arrive + phase * kSelMaxCtas + tid, a.token, &n_over);
-        a.arrive[phase * kSelMaxCtas + tid].x = 0ull;
-        fence_gpu();
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+      for (int e = 0; e < EPV; ++e) {
+        const uint32_t key = ((DT == 0) ? w[e % 4] : (w[e >> 1] >> (16 * (e & 1)))) & kMask;
+        if (key && key >> kBinShift == bin) atomicAdd(&hist[(key & ((1u << kBinShift) - 1u)) >> kFineShift], 1u);
       }
-      prepare_phase(a, phase + 1);
-      prepare_round(a, 1);
-      if (tid == 0) s_tot[1] = 0;
+    }
+    if (tid == 0) s_res[3] = 0;
+    __syncthreads();
+    uint32_t all;
+    const uint32_t b = my_bin(hist);
+    const uint32_t above = count_above_mine(b, s_warp, &all);
+    if (want) place_rank(b, above, want, s_res + 3);
+    __syncthreads();
+    if (tid == 0)                                // phase 0: where it lies
+      word_store(a.arrive + blockIdx.x, a.token, want ? (bin << (kBinShift - kFineShift)) | s_res[3] : 0u);
+    unsigned long long w = 0;
+    int ok = 1;
+    if (master) {
+      uint32_t* bins = hist;                     // (the sample is done with)
+      if (tid < G) {
+        ok = word_wait(a.arrive + tid, a.token, &w);
+        a.arrive[tid].x = 0ull;
+      }
+      // distinct, in the keys' order
+      if (tid < kSelMaxCtas) bins[tid] = tid < G ? (static_cast<uint32_t>(w) << 8) | (kSelMaxCtas - 1u - tid) : 0u;
       if (!__syncthreads_and(ok)) { drain(); quit(); return; }
-      const uint32_t w_over = __reduce_add_sync(kFull, static_cast<uint32_t>(n_over));
-      if (lane == 0 && w_over) atomicAdd(&s_tot[1], w_over);
-      const uint32_t b = tid < kSelBins ? __ldcg(a.hist + kSelBins - 1 - tid) : 0u;
-      uint32_t all;
-      ranks(kOwn * static_cast<float>(G), kSigmas, &r_hi, &r_lo);
-      const uint32_t above = count_above_mine(b, s_warp, &all) + s_tot[1];
-      if (r_hi) place_rank(b, above, r_hi, s_res);
-      if (r_lo) place_rank(b, above, r_lo, s_res + 3);
+      const int margin = static_cast<int>(2.5f * sqrtf(static_cast<float>(G))) + 1;
+      const int at_hi = G / 2 - margin, at_lo = G / 2 + margin;
+      if (tid < G) {
+        const uint32_t my = bins[tid];
+        int larger = 0;
+#pragma unroll 4
+        for (int i = 0; i < (G + 3) / 4; ++i) {
+          const uint4 o = reinterpret_cast<const uint4*>(bins)[i];
+          larger += (o.x > my ? 1 : 0) + (o.y > my ? 1 : 0) + (o.z > my ? 1 : 0) + (o.w > my ? 1 : 0);
+        }
+        if (larger == at_hi) s_res[0] = my >> 8;
+        if (larger == at_lo) s_res[1] = my >> 8;
+      }
       __syncthreads();
-      // (a rank above or below the window bounds its side of the bracket by the window's end, or not at all)
-      const int bottom = top - (kSelBins - 1);
-      const uint32_t below = s_tot[1] + all;     // ranks past this one lie below the window
-      hi = r_hi <= s_tot[1] ? kKeyMax
-           : r_hi > below   ? (static_cast<uint32_t>(max(bottom, 1)) << kBinShift) - 1u
-                            : (static_cast<uint32_t>(bottom + static_cast<int>(s_res[0])) << kBinShift) | ((1u << kBinShift) - 1u);
-      lo = r_lo == 0 || r_lo > below ? 1u
-           : r_lo <= s_tot[1]        ? static_cast<uint32_t>(top + 1) << kBinShift
-                                     : max(static_cast<uint32_t>(bottom + static_cast<int>(s_res[3])) << kBinShift, 1u);
+      hi = no_hi || at_hi < 0 ? kKeyMax : (s_res[0] << kFineShift) | ((1u << kFineShift) - 1u);
+      lo = no_lo || at_lo >= G ? 1u : max(s_res[1] << kFineShift, 1u);
       if (tid == 0) {
-        fence_gpu();
-        word_store(a.answer + phase * (kSelMaxCtas + 2), a.token, lo | (static_cast<unsigned long long>(hi) << 32));
-        a.answer[0].x = 0ull;
+        fence_gpu();                             // the histogram is zero, the claims, the header begun
+        word_store(a.answer, a.token, lo | (static_cast<unsigned long long>(hi) << 32));
       }
     } else {
       if (tid == 0) {
-        unsigned long long ans = 0;
-        if (!word_wait(a.answer + phase * (kSelMaxCtas + 2), a.token, &ans)) s_fail = 1;
-        s_ans[1] = ans;
+        ok = word_wait(a.answer, a.token, &w);
+        fence_gpu();
+        s_ans[0] = w;
       }
-      __syncthreads();
-      if (s_fail) { drain(); quit(); return; }
-      lo = static_cast<uint32_t>(s_ans[1]);
-      hi = static_cast<uint32_t>(s_ans[1] >> 32);
+      if (!__syncthreads_and(ok)) { drain(); quit(); return; }
+      lo = static_cast<uint32_t>(s_ans[0]);
+      hi = static_cast<uint32_t>(s_ans[0] >> 32);
     }
-    ++phase;
   }
 
   // ---- the threshold ----
@@ -922,7 +958,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
   uint32_t step = kRead, n_above = 0;            // n_above: keys above hi
   bool listed = false, loaded = true;            // (CTA 0) the last pass's lists are complete
   int shift = 0;
-  int round = RES ? 0 : 1;                       // (the shared sample used histogram 0)
+  int round = 0;
   uint32_t tau = 0, n_greater = 0;
   unsigned long long before = 0;
   for (;;) {
@@ -1052,7 +1088,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
       if (RES) {
         for (int c = warp; c < n_local; c += kWarps) slot_keys_warp<DT>(s_slots + c * kSlot, cnt[c] >> 16, add);
       } else {
-        slot_keys_lane<DT>(g_slots, cnt, n_local, [&](uint32_t&, uint32_t key) { add(key); }, [](int, uint32_t, uint32_t) {});
+        slot_keys_global<DT>(g_slots, cnt, n_local, n_local > kThreads / 2, [&](int, uint32_t&, uint32_t key) { add(key); }, [](int, uint32_t, uint32_t) {});
       }
     }
     if (RES && round == 0 && tid == 0) {         // CTA 0 has zeroed the histograms
@@ -1080,8 +1116,8 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
       int ok = 1;
       if (tid < G) {
         ok = word_wait(a.arrive + phase * kSelMaxCtas + tid, a.token, &v, a.stall != 0);
+        fence_gpu();                             // (before the clearing: a fence waits for the stores before it)
         a.arrive[phase * kSelMaxCtas + tid].x = 0ull;
-        fence_gpu();
       }
       prepare_phase(a, phase + 1);
       prepare_round(a, round + 1);
@@ -1096,11 +1132,11 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
       uint32_t n_in;
       const uint32_t above = count_above_mine(b, s_warp, &n_in);
       uint32_t sum = 0, key_max = 0, key_inv = 0, over = 0;
-#pragma unroll
-      for (int w = 0; w < kWarps; ++w) {
-        const uint4 u = s_red[w];
-        sum += u.x; key_max = max(key_max, u.y); key_inv = max(key_inv, u.z); over |= u.w;
-      }
+      const uint4 red = lane < kWarps ? s_red[lane] : make_uint4(0, 0, 0, 0);
+      sum = __reduce_add_sync(kFull, red.x);
+      key_max = __reduce_max_sync(kFull, red.y);
+      key_inv = __reduce_max_sync(kFull, red.z);
+      over = __any_sync(kFull, red.w != 0u) ? 1u : 0u;
       const bool was_read = step == kRead;
       if (was_read) { n_above = sum; listed = over == 0; }
       const long long r = static_cast<long long>(a.k) - n_above;     // rank among the keys of [0, hi]
@@ -1126,7 +1162,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
         fence_gpu();                             // the cleared words and bins of what comes next
         word_store(a.answer + phase * (kSelMaxCtas + 2), a.token, lo | (static_cast<unsigned long long>(hi) << 32));
         word_store(a.answer + phase * (kSelMaxCtas + 2) + 1, a.token, n_above | (static_cast<unsigned long long>(step) << 32));
-        if (RES && phase == 1) a.answer[0].x = 0ull;
+        if (phase == 1) a.answer[0].x = 0ull;
       }
     } else {
       if (tid < 2) {
@@ -1179,42 +1215,38 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
   if (s_fail) { quit(); return; }
   uint32_t n_gt = 0, n_eq = 0;
   if (step == kListed || step == kKeys) {
-    auto report = [&](uint32_t key, uint32_t& g, uint32_t& e) {
-      if (key > hi) ++g;
+    // acc: keys above hi, and (upper half) keys of [lo, hi]
+    auto report = [&](int c, uint32_t& acc, uint32_t key) {
+      if (key > hi) ++acc;
       else if (key >= lo) {
-        ++e;
+        acc += 0x10000u;
         if (step == kKeys) {
           const uint32_t at = atomicAdd(&s_nkeys, 1u);
-          if (at < static_cast<uint32_t>(kMaxKeys)) a.keys[blockIdx.x * kMaxKeys + at] = key;
+          if (at < static_cast<uint32_t>(kMaxKeys)) {
+            a.keys[blockIdx.x * kMaxKeys + at] = key;
+            s_bin_key[at] = key;
+            s_bin_chunk[at] = c;
+          }
         }
       }
+    };
+    auto done = [&](int c, uint32_t v, uint32_t acc) {       // (one lane)
+      acc += v & 0xFFFFu;
+      if (step == kListed) cnt[c] = acc;
+      else prefix[c] = acc & 0xFFFFu;            // (cnt stands: there may be another round)
+      n_gt += acc & 0xFFFFu;
+      n_eq += acc >> 16;
     };
     if (RES) {
       for (int c = warp; c < n_local; c += kWarps) {
         const uint32_t v = cnt[c];
-        uint32_t g = 0, e = 0;
-        slot_keys_warp<DT>(s_slots + c * kSlot, v >> 16, [&](uint32_t key) { report(key, g, e); });
-        if (lane == 0) g += v & 0xFFFFu;
-        n_gt += g;
-        n_eq += e;
-        if (step == kListed) {
-          const uint32_t both = __reduce_add_sync(kFull, g | (e << 16));
-          if (lane == 0) cnt[c] = both;
-        }
+        uint32_t acc = 0;
+        slot_keys_warp<DT>(s_slots + c * kSlot, v >> 16, [&](uint32_t key) { report(c, acc, key); });
+        acc = __reduce_add_sync(kFull, acc);
+        if (lane == 0) done(c, v, acc);
       }
     } else {
-      slot_keys_lane<DT>(g_slots, cnt, n_local,
-                         [&](uint32_t& acc, uint32_t key) {
-                           uint32_t g = 0, e = 0;
-                           report(key, g, e);
-                           acc += g | (e << 16);
-                         },
-                         [&](int c, uint32_t v, uint32_t acc) {
-                           acc += v & 0xFFFFu;
-                           if (step == kListed) cnt[c] = acc;
-                           n_gt += acc & 0xFFFFu;
-                           n_eq += acc >> 16;
-                         });
+      slot_keys_global<DT>(g_slots, cnt, n_local, n_local > kThreads / 2, report, done);
     }
   } else {
     for (int c = tid; c < n_local; c += kThreads) {
@@ -1249,32 +1281,32 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     int ok = 1;
     if (tid < G) {
       ok = word_wait(a.arrive + phase * kSelMaxCtas + tid, a.token, &v);
-      a.arrive[phase * kSelMaxCtas + tid].x = 0ull;
       fence_gpu();
+      a.arrive[phase * kSelMaxCtas + tid].x = 0ull;
     }
     prepare_phase(a, phase + 1);
     if (step == kKeys && tid < kSelBins) hist[tid] = hist[kSelBins + tid] = 0;
     if (!__syncthreads_and(ok)) { quit(); return; }
     if (step == kKeys) {
       const uint32_t n_k = tid < G ? static_cast<uint32_t>(v) : 0u;
-      uint32_t* nk = reinterpret_cast<uint32_t*>(aux + kAuxPrefix);     // [3][kSelMaxCtas]: keys, above, ties per CTA
+      uint32_t* nk = hist + 2 * kSelBins;        // [3][kSelMaxCtas]: keys, above, ties per CTA
       if (tid < kSelMaxCtas) { nk[tid] = n_k; nk[kSelMaxCtas + tid] = 0; nk[2 * kSelMaxCtas + tid] = 0; }
       const uint32_t w_most = __reduce_max_sync(kFull, n_k);
       if (lane == 0) s_warp[warp] = w_most;
       __syncthreads();
-      int most = 0;
-#pragma unroll
-      for (int w = 0; w < kWarps; ++w) most = max(most, static_cast<int>(s_warp[w]));
+      const int most = static_cast<int>(__reduce_max_sync(kFull, lane < kWarps ? s_warp[lane] : 0u));
       __syncthreads();
       constexpr int kPer = kKeysPerThread;
       again = most > kMaxKeys || most * G > kKeysAtOnce;
       if (!again) {
+        // (idx / most by multiplication: idx * most < 2^32)
+        const uint32_t inv = most > 1 ? 0xFFFFFFFFu / static_cast<uint32_t>(most) + 1u : 0u;
         uint32_t key[kPer];
         int who[kPer];
 #pragma unroll
         for (int u = 0; u < kPer; ++u) {
           const int idx = u * kThreads + tid;
-          who[u] = idx / most;
+          who[u] = most > 1 ? static_cast<int>(__umulhi(static_cast<uint32_t>(idx), inv)) : idx;
           const int i = idx - who[u] * most;
           const bool have = who[u] < G && i < static_cast<int>(nk[min(who[u], kSelMaxCtas - 1)]);
           key[u] = have ? __ldcg(a.keys + who[u] * kMaxKeys + i) : 0u;
@@ -1316,12 +1348,9 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     const unsigned long long incl = warp_incl_u64(v);
     if (lane == 31) s_warp64[warp] = incl;
     __syncthreads();
-    unsigned long long all = 0, base = 0;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
-      if (w < warp) base += s_warp64[w];
-      all += s_warp64[w];
-    }
+    const unsigned long long upto = warp_incl_u64(lane < kWarps ? s_warp64[lane] : 0ull);
+    const unsigned long long all = __shfl_sync(kFull, upto, 31);
+    const unsigned long long base = warp ? __shfl_sync(kFull, upto, warp - 1) : 0ull;
     const bool nz = a.drop_zeros && tau == 0u;   // store variant without kept zeros
     const long long quota = nz ? 0 : static_cast<long long>(a.k) - n_greater;
     const long long n_stored = nz ? static_cast<long long>(n_greater) : static_cast<long long>(a.k);
@@ -1376,20 +1405,15 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
   const long long n_stored = nz ? static_cast<long long>(n_greater) : static_cast<long long>(a.k);
 
   // ---- per-chunk counts and places ----
-  if (RES && step == kKeys) {
-    for (int c = warp; c < n_local; c += kWarps) {
-      const uint32_t v = cnt[c];
-      uint32_t both = 0;
-      slot_keys_warp<DT>(s_slots + c * kSlot, v >> 16, [&](uint32_t key) { if (key >= tau) both += key > tau ? 1u : 0x10000u; });
-      both = __reduce_add_sync(kFull, both);
-      if (lane == 0) cnt[c] = (v & 0xFFFFu) + both;
+  if (step == kKeys) {                           // what was above the bin, and the CTA's few keys inside it
+    const int n_bin = static_cast<int>(s_nkeys);
+    for (int c = tid; c < n_local; c += kThreads) {
+      uint32_t both = static_cast<uint32_t>(prefix[c]);
+#pragma unroll 1
+      for (int i = 0; i < n_bin; ++i)
+        if (s_bin_chunk[i] == c && s_bin_key[i] >= tau) both += s_bin_key[i] > tau ? 1u : 0x10000u;
+      cnt[c] = both;
     }
-    __syncthreads();
-  }
-  if (!RES && step == kKeys) {
-    slot_keys_lane<DT>(g_slots, cnt, n_local,
-                       [&](uint32_t& acc, uint32_t key) { if (key >= tau) acc += key > tau ? 1u : 0x10000u; },
-                       [&](int c, uint32_t v, uint32_t acc) { cnt[c] = (v & 0xFFFFu) + acc; });
     __syncthreads();
   }
   unsigned long long carry = before;
@@ -1406,12 +1430,9 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     const unsigned long long incl = warp_incl_u64(sum);
     if (lane == 31) s_warp64[warp] = incl;
     __syncthreads();
-    unsigned long long base = carry + incl - sum;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
-      if (w < warp) base += s_warp64[w];
-      carry += s_warp64[w];
-    }
+    const unsigned long long upto = warp_incl_u64(lane < kWarps ? s_warp64[lane] : 0ull);
+    unsigned long long base = carry + incl - sum + (warp ? __shfl_sync(kFull, upto, warp - 1) : 0ull);
+    carry += __shfl_sync(kFull, upto, 31);
 #pragma unroll
     for (int j = 0; j < kScan; ++j) {
       if (c + j < n_local) prefix[c + j] = base;

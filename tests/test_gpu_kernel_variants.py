@@ -124,6 +124,18 @@ def test_sample_that_misleads(bf16):
             assert_store_equals_oracle(x, ratio)
 
 
+@pytest.mark.parametrize("dist, n, bf16", [("normal", 9_000_001, False), ("relu_normal", 15_500_001, True),
+                                           ("ties16", 8_000_000, False), ("normal", 40_000_003, False)])
+def test_streamed_tensor_at_extreme_ratios(dist, n, bf16):
+    """Thresholds of which a CTA's own sample holds few elements, or none, above or below; and more chunks per
+    CTA than one trip to the lists takes."""
+    x = W.draw(dist, n, seed=31, device="cuda")
+    x = x.to(torch.bfloat16) if bf16 else x
+    ratios = (0.9,) if n > 1 << 24 else (1 - 3 / n, 0.9995, 0.996, 0.5, 0.004, 0.0005, 2 / n)
+    for ratio in ratios:
+        assert_store_equals_oracle(x.cpu(), ratio)
+
+
 @pytest.mark.parametrize("n", [5000, (1 << 23) + 77])
 def test_captured_call_replays_and_alternating_streams(n):
     xs = [W.draw("normal", n, seed=20 + i).cuda() for i in range(3)]
