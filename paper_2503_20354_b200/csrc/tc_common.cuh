@@ -137,6 +137,35 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// 16 accumulator columns of a warp's 32 TMEM lanes (r: this lane's) into 16 rows of a row-major fp32 array whose
+// columns are the lanes: element (e, lane) at dst[e * pitch + lane], for e < n_rows and lane < n_lanes.  `buf`: 2 KB
+// of the warp's own in shared memory.  Through it the warp stores 16 bytes per lane where the rows are
+// 16-byte aligned (`vec`): 16 stores of 4 bytes per lane took 1500 clocks a block, 8 us for the 512 columns of
+// a CTA, as long as a small layer's products.  `at`: index of dst in an array of `limit` elements.
+__device__ __forceinline__ void store_cols16(float* buf, const uint32_t (&r)[16], float* dst, long long pitch,
+                                             int n_rows, int n_lanes, bool vec, long long at, long long limit,
+                                             uint32_t* status) {
+  const int lane = static_cast<int>(lane_id());
+  if (vec) {
+    __syncwarp();                                // the previous block has been read out
+#pragma unroll
+    for (int e = 0; e < 16; ++e) buf[e * 32 + lane] = __uint_as_float(r[e]);
+    __syncwarp();
+    const int c = 4 * (lane & 7);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int e = 4 * i + (lane >> 3);
+      const float4 v = *reinterpret_cast<const float4*>(buf + e * 32 + c);
+      if (e < n_rows && c < n_lanes && SURGEON_IN_BOUNDS(at + e * pitch + c + 3, limit, status))
+        *reinterpret_cast<float4*>(dst + e * pitch + c) = v;
+    }
+  } else if (lane < n_lanes) {
+#pragma unroll
+    for (int e = 0; e < 16; ++e)
+      if (e < n_rows && SURGEON_IN_BOUNDS(at + e * pitch + lane, limit, status)) dst[e * pitch + lane] = __uint_as_float(r[e]);
+  }
+}
+
 // Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows of 128 bytes, groups
 // of 8 rows 1024 bytes apart (tile base 1024-byte aligned).
 __device__ __forceinline__ uint64_t make_desc(uint32_t saddr) {

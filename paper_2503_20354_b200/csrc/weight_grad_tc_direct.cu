@@ -725,35 +725,37 @@ dw_direct_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ v
   if (warp >= 2) {
     // a warp may read the 32 TMEM lanes of its quarter (warp % 4); the warps of a quarter take
     // the groups of 16 columns in turn
+    // (MODE != 0) the tap of the accumulator at hand and its first channel; a column's place in the accumulator
+    int tap = 0, o_acc = 0, rel = 16 * ((warp - 2) >> 2);
+    if (MODE != 0) {
+      const int u = TG >= 2 ? n_tile : u0;         // TG >= 2: accumulator a is kernel row a of this CTA's kernel column
+      tap = u / p.upt;
+      o_acc = (u - tap * p.upt) * p.acc_n;
+    }
     const bool done = mbar_wait(acc_bar, 0, 64);
     tc_fence_after();
     if (done && !fail) {
       const int lane_grp = warp & 3;
-      const int c = c0 + lane_grp * 32 + static_cast<int>(lane);
-      float* out = partial + static_cast<long long>(split) * p.O * p.C;
+      const long long first = static_cast<long long>(split) * p.O * p.C + c0 + lane_grp * 32;
+      float* buf = reinterpret_cast<float*>(smem) + (warp - 2) * 512;      // (the rings are done with)
+      const bool vec = (p.C & 3) == 0;             // (a row tile begins at a multiple of 16, and so a tile's end is one of 4)
       const int cols_here = n_acc_here * p.acc_n;
-      for (int col = 16 * ((warp - 2) >> 2); col < cols_here; col += 16 * (kProdWarps / 4)) {
+      for (int col = rel; col < cols_here; col += 16 * (kProdWarps / 4), rel += 16 * (kProdWarps / 4)) {
         uint32_t r[16];
         tmem_ld16(tmem_base + (static_cast<uint32_t>(lane_grp * 32) << 16) + col, r);
         int row0, n_ok;                   // first partial row of the 16 columns, how many exist
         if (MODE == 0) {
           row0 = o0 + col; n_ok = p.O - row0;
         } else {
-          const int a = col / p.acc_n;
-          const int u = u0 + a;
-          // TG >= 2: accumulator a is kernel row a of this CTA's kernel column
-          const int tap = TG >= 2 ? a * p.kw + n_tile / p.upt : u / p.upt;
-          const int o_lo = (TG >= 2 ? n_tile % p.upt : u - tap * p.upt) * p.acc_n + (col - a * p.acc_n);
-          row0 = tap * p.o_real + o_lo; n_ok = p.o_real - o_lo;
+          for (; rel >= p.acc_n; rel -= p.acc_n) {
+            if (TG >= 2) tap += p.kw;
+            else if ((o_acc += p.acc_n) == p.upt * p.acc_n) { o_acc = 0; ++tap; }
+          }
+          row0 = tap * p.o_real + o_acc + rel; n_ok = p.o_real - (o_acc + rel);
         }
-        if (lane_grp * 32 + static_cast<int>(lane) < rows_here) {
-#pragma unroll
-          for (int e = 0; e < 16; ++e)
-            if (e < n_ok && SURGEON_IN_BOUNDS(static_cast<long long>(split) * p.O * p.C +
-                                                  static_cast<long long>(row0 + e) * p.C + c,
-                                              static_cast<long long>(p.splits) * p.O * p.C, status))
-              out[static_cast<long long>(row0 + e) * p.C + c] = __uint_as_float(r[e]);
-        }
+        const long long at = first + static_cast<long long>(row0) * p.C;
+        store_cols16(buf, r, partial + at, p.C, n_ok, rows_here - lane_grp * 32, vec, at,
+                     static_cast<long long>(p.splits) * p.O * p.C, status);
       }
     } else if (!done && lane == 0) {
       atomicMax(status, static_cast<uint32_t>(SURGEON_ERR_TIMEOUT));
