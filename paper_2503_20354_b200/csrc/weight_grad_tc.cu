@@ -19,6 +19,7 @@
 // the scratch status word, frees its tensor memory and returns.
 #include <cuda.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "surgeon_internal.cuh"
@@ -774,7 +775,7 @@ static void launch_reduce_splits(const float* partial, long long mn, int splits,
 // run along c (contiguous in the partial, a kilobyte per warp), the writes along (c, tap)
 // (contiguous in dw), transposed through shared memory.  taps <= 49.  `sp` threads share an element's splits (see
 // reduce_splits_kernel) where a chunk has too few elements for the block.
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(512)
 reduce_splits_taps_kernel(const float* __restrict__ partial, int o_real, int c_in, int taps,
                           int chunk, int splits, int sp, float* __restrict__ dw, int accumulate,
                           const uint32_t* __restrict__ status, surgeon_header* __restrict__ hdr) {
@@ -792,7 +793,7 @@ reduce_splits_taps_kernel(const float* __restrict__ partial, int o_real, int c_i
     // multiple of 32 and n_c of 4, so both stay aligned); the split sums keep their order
     const int n_c4 = n_c >> 2;
     const int items = n_c4 * taps, per = (splits + sp - 1) / sp;
-    for (int idx = threadIdx.x; idx < items * sp; idx += 256) {
+    for (int idx = threadIdx.x; idx < items * sp; idx += blockDim.x) {
       const int y = sp == 1 ? 0 : idx / items, it = idx - y * items;
       const int tap = it / n_c4, cl = (it - tap * n_c4) * 4;
       const float* src = partial + (static_cast<long long>(tap) * o_real + o) * c_in + c0 + cl;
@@ -811,7 +812,7 @@ reduce_splits_taps_kernel(const float* __restrict__ partial, int o_real, int c_i
     }
     __syncthreads();
     const int n4 = (n_c * taps) >> 2;                  // n_c is a multiple of 4
-    for (int idx = threadIdx.x; idx < n4; idx += 256) {
+    for (int idx = threadIdx.x; idx < n4; idx += blockDim.x) {
       float4 v = *reinterpret_cast<const float4*>(tile + 4 * idx);
       for (int y = 1; y < sp; ++y) {
         const float4 u = *reinterpret_cast<const float4*>(tile + y * chunk * taps + 4 * idx);
@@ -825,7 +826,7 @@ reduce_splits_taps_kernel(const float* __restrict__ partial, int o_real, int c_i
     }
     return;
   }
-  for (int idx = threadIdx.x; idx < n_c * taps; idx += 256) {
+  for (int idx = threadIdx.x; idx < n_c * taps; idx += blockDim.x) {
     const int tap = idx / n_c, cl = idx - tap * n_c;     // consecutive threads, consecutive channels
     const float* src = partial + (static_cast<long long>(tap) * o_real + o) * c_in + c0 + cl;
     float s = src[0];
@@ -833,7 +834,7 @@ reduce_splits_taps_kernel(const float* __restrict__ partial, int o_real, int c_i
     tile[cl * taps + tap] = s;
   }
   __syncthreads();
-  for (int idx = threadIdx.x; idx < n_c * taps; idx += 256)
+  for (int idx = threadIdx.x; idx < n_c * taps; idx += blockDim.x)
     out[idx] = accumulate ? out[idx] + tile[idx] : tile[idx];
 }
 
@@ -992,9 +993,11 @@ cudaError_t launch_weight_grad_tc(const surgeon_compressed& act, const surgeon_l
       while (chunk > 32 && (static_cast<long long>(dp.o_real) * ((dp.C + chunk - 1) / chunk) < 4LL * sm_count() ||
                             chunk * dp.taps * 4 > 48 * 1024))
         chunk >>= 1;
-      int sp = 1;
-      while (dp.C % 4 == 0 && sp < 8 && chunk / 4 * dp.taps * sp < 256 && dp.splits >= 4 * sp) sp *= 2;
-      launch_kernel(reduce_splits_taps_kernel, dim3((dp.C + chunk - 1) / chunk, dp.o_real), dim3(256),
+      // as many threads per element as fit 512, while each has four parts left, and no second round of them
+      const int items = std::min(chunk, dp.C) / 4 * dp.taps;
+      const int sp = dp.C % 4 == 0 ? std::max(1, std::min({8, 512 / items, dp.splits / 4})) : 1;
+      const int threads = sp > 1 ? (items * sp + 31) / 32 * 32 : 256;
+      launch_kernel(reduce_splits_taps_kernel, dim3((dp.C + chunk - 1) / chunk, dp.o_real), dim3(threads),
                     static_cast<size_t>(chunk) * dp.taps * sp * sizeof(float), stream, true,
                     static_cast<const float*>(partial), dp.o_real, dp.C, dp.taps, chunk, dp.splits, sp, dw, accumulate,
                     static_cast<const uint32_t*>(status), act.header);

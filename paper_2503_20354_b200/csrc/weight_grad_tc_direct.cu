@@ -38,6 +38,7 @@
 // order by the caller.  Every wait is bounded and ends in SURGEON_ERR_TIMEOUT.
 #include <cuda.h>
 
+#include <algorithm>
 #include <cstddef>
 #include <cstdlib>
 
@@ -1100,19 +1101,43 @@ static bool compute_plan_direct(const surgeon_layer_desc& d, bool transposed_ok,
       p.b_bytes = p.tg == 1 ? p.n_acc * p.unit_bytes : p.unit_bytes;
     }
   }
-  p.n_cols = p.acc_n * p.n_acc;
-  p.n_tiles = p.tg >= 2 ? p.kw * p.upt
-              : (p.mode == 0) ? (p.O + p.n_cols - 1) / p.n_cols : (p.n_units + p.n_acc - 1) / p.n_acc;
   p.tiles_per_img = (p.T + (p.tg ? p.kpos : kTileK) - 1) / (p.tg ? p.kpos : kTileK);
   const long long total = static_cast<long long>(p.imgs) * p.tiles_per_img;
   if (total > 2147483647LL / 4) return false;
   p.total_ktiles = static_cast<int>(total);
   const int sms = sm_count();
+  auto n_tiles_of = [&](int acc_n, int n_acc) {
+    return p.tg >= 2 ? p.kw * p.upt
+           : (p.mode == 0) ? (p.O + acc_n * n_acc - 1) / (acc_n * n_acc) : (p.n_units + n_acc - 1) / n_acc;
+  };
+  // The K-tiles in splits of four or more: a CTA's time is that of its K-tiles and some five tiles' worth for its
+  // start, its partial tile and its share of the reduction.
+  const int max_splits = static_cast<int>(std::min<long long>((total + 3) / 4, 128));
+  if (!p.pair && p.tg < 2 && static_cast<long long>(p.m_tiles) * n_tiles_of(p.acc_n, p.n_acc) * max_splits < sms) {
+    // The widest column tiles leave SMs without work: narrower ones.  They rebuild the activation once more each, on
+    // SMs that would idle, and the partial tile (7 K-tiles' worth at 512 columns: it leaves at 25 to 30 bytes a
+    // clock) is written by more of them.
+    double best_cost = 1e30;
+    int best_n = p.acc_n, best_a = p.n_acc;
+    auto consider = [&](int acc_n, int n_acc) {
+      const long long tiles = static_cast<long long>(p.m_tiles) * n_tiles_of(acc_n, n_acc);
+      const int s = static_cast<int>(std::max<long long>(1, std::min<long long>(max_splits, sms / tiles)));
+      const double waves = static_cast<double>((tiles * s + sms - 1) / sms);
+      const double cost = waves * ((total + s - 1) / s + 5 + 7.0 * acc_n * n_acc / 512);
+      if (cost < best_cost - 1e-9) { best_cost = cost; best_n = acc_n; best_a = n_acc; }
+    };
+    consider(p.acc_n, p.n_acc);
+    if (p.mode == 0) for (int a = 256; a >= 64; a -= 64) { if (a < p.acc_n * p.n_acc) consider(a, 1); }
+    else for (int a = p.n_acc - 1; a >= 1; --a) consider(p.acc_n, a);
+    p.acc_n = best_n; p.n_acc = best_a;
+    if (p.tg) p.b_bytes = p.n_acc * p.unit_bytes;
+  }
+  p.n_cols = p.acc_n * p.n_acc;
+  p.n_tiles = n_tiles_of(p.acc_n, p.n_acc);
   const long long tiles_mn = static_cast<long long>(p.m_tiles) * p.n_tiles;
-  const int max_splits = (p.total_ktiles + 7) / 8 < 1 ? 1 : (p.total_ktiles + 7) / 8;
   int best = 1;
   double best_cost = 1e30;
-  for (int s = 1; s <= max_splits && s <= 128; ++s) {
+  for (int s = 1; s <= max_splits; ++s) {
     const long long ctas = tiles_mn * s;
     const long long waves = (ctas + sms - 1) / sms;
     const int kts = (p.total_ktiles + s - 1) / s;

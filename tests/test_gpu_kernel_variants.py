@@ -99,6 +99,16 @@ def test_reductions_of_small_weights(batch, c_in, c_out, k):
     torch.testing.assert_close(acc, 1 + torch.from_numpy(dw).cuda(), rtol=1e-5, atol=1e-6)
 
 
+@pytest.mark.parametrize("layer", [
+    W.linear("few_rows", 200, 320, 320), W.linear("ragged", 333, 136, 200), W.linear("wide", 260, 64, 1288),
+    W.conv("one_image", 1, 40, 14, 72, 1, 1, 0), W.conv("one_image_3x3", 1, 24, 13, 56), W.conv("taps_part", 2, 20, 8, 48),
+    W.conv("one_map", 1, 132, 16, 500, 1, 1, 0)], ids=lambda l: l.name)
+def test_small_reductions_on_narrow_column_tiles(layer):
+    """Fewer tiles than SMs: narrower column tiles, splits of four K-tiles, partial tiles of every width."""
+    dw, ref = _dw(layer, 0.5, B.PATH_TENSOR_CORE)
+    assert rel_frobenius(dw, ref) <= 5e-3
+
+
 # prune: whole chunks and one element around them, resident and streamed ranges (a CTA's range is resident up to 48
 # chunks of 4 KB), counts in global memory (beyond 512 chunks per CTA on 148 SMs)
 @pytest.mark.parametrize("bf16", [False, True])
