@@ -125,6 +125,7 @@ struct DirectParams {
   int tmem_cols, smem_bytes;
   long long n_words;        // words of the bitmap (filled by the launcher)
   const long long* n_keep_ptr;  // device address of the store's count of packed values (launcher)
+  unsigned few_keep;        // packed values up to which runs are rebuilt element by element (launcher)
   unsigned partial_blk;     // index of the bitmap's last block if it is partial, else 0xFFFFFFFF
 };
 bool plan_direct(const surgeon_layer_desc& d, DirectParams* out);

@@ -101,12 +101,15 @@ def test_reductions_of_small_weights(batch, c_in, c_out, k):
 
 @pytest.mark.parametrize("layer", [
     W.linear("few_rows", 200, 320, 320), W.linear("ragged", 333, 136, 200), W.linear("wide", 260, 64, 1288),
-    W.conv("one_image", 1, 40, 14, 72, 1, 1, 0), W.conv("one_image_3x3", 1, 24, 13, 56), W.conv("taps_part", 2, 20, 8, 48),
+    W.conv("one_image", 1, 40, 14, 72, 1, 1, 0), W.conv("one_image_3x3", 1, 24, 13, 56, 3), W.conv("taps_part", 2, 20, 8, 48, 3),
     W.conv("one_map", 1, 132, 16, 500, 1, 1, 0)], ids=lambda l: l.name)
-def test_small_reductions_on_narrow_column_tiles(layer):
-    """Fewer tiles than SMs: narrower column tiles, splits of four K-tiles, partial tiles of every width."""
-    dw, ref = _dw(layer, 0.5, B.PATH_TENSOR_CORE)
-    assert rel_frobenius(dw, ref) <= 5e-3
+@pytest.mark.parametrize("ratio", [0.5, 0.9])
+def test_small_reductions_on_narrow_column_tiles(layer, ratio):
+    """Fewer tiles than SMs: narrower column tiles, splits of four K-tiles, partial tiles of every width; and runs
+    with few kept elements."""
+    for dt in (W.BF16, W.F32):
+        dw, ref = _dw(replace(layer, dt=dt), ratio, B.PATH_TENSOR_CORE)
+        assert rel_frobenius(dw, ref) <= 5e-3
 
 
 # prune: whole chunks and one element around them, resident and streamed ranges (a CTA's range is resident up to 48
