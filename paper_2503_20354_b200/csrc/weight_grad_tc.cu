@@ -930,11 +930,6 @@ size_t im2col_grad_bytes(const TcParams& p, int pitch) {
 
 }  // namespace
 
-static size_t fast_partial_bytes(const FastParams& f) {
-  const size_t b = static_cast<size_t>(f.splits) * f.O * f.n_gemm * sizeof(float);
-  return (b + 255) & ~static_cast<size_t>(255);
-}
-
 static size_t direct_partial_bytes(const DirectParams& p) {
   const size_t b = static_cast<size_t>(p.splits) * p.O * p.C * sizeof(float);
   return (b + 255) & ~static_cast<size_t>(255);
@@ -947,9 +942,6 @@ size_t weight_grad_tc_workspace(const surgeon_layer_desc& d) {
   if (plan_direct(d, &dp)) return kStatusBytes + direct_partial_bytes(dp) + direct_grad_bf16_bytes(dp);
   StridedParams st;
   if (plan_strided(d, &st)) return kStatusBytes + strided_partial_bytes(st) + strided_grad_bf16_bytes(st);
-  FastParams f;
-  if (plan_conv_fast(d, &f))
-    return kStatusBytes + fast_partial_bytes(f) + conv_fast_grad_bf16_bytes(f);
   TcParams p;
   int pitch = 0;
   if (plan_im2col(d, 0, &p, &pitch))
@@ -1015,16 +1007,6 @@ cudaError_t launch_weight_grad_tc(const surgeon_compressed& act, const surgeon_l
     if (e != cudaSuccess) return e;
     launch_reduce_splits(partial, static_cast<long long>(strided.O) * strided.n_gemm, strided.splits, dw, accumulate,
                          status, act.header, stream);
-    note_launches(1);
-    return cudaGetLastError();
-  }
-  FastParams f;
-  if (plan_conv_fast(d, &f)) {
-    void* grad_bf16 = reinterpret_cast<char*>(partial) + fast_partial_bytes(f);
-    e = launch_conv_fast(act, f, grad_out, grad_bf16, partial, status, stream);
-    if (e != cudaSuccess) return e;
-    const long long fmn = static_cast<long long>(f.O) * f.n_gemm;
-    launch_reduce_splits(partial, fmn, f.splits, dw, accumulate, status, act.header, stream);
     note_launches(1);
     return cudaGetLastError();
   }

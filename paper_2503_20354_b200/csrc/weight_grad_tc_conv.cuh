@@ -1,4 +1,4 @@
-// Plan and launcher of the fast stride-1 convolution kernel (weight_grad_tc_conv.cu).
+// Plans and launchers of the tensor-core weight-gradient kernels, and the gradient pre-passes (weight_grad_tc_conv.cu).
 #pragma once
 
 #include <cuda.h>
@@ -36,30 +36,6 @@ inline bool memo_plan(const surgeon_layer_desc& d, int extra, P* out, F compute)
   if (e.ok) *out = e.p;
   return e.ok;
 }
-
-struct FastParams {
-  int mode;                 // 0 = 3x3 pad 1 through a shared-memory patch, 1 = 1x1 direct
-  int stride;               // 1 or 2
-  int B, C, H, W, O, OH, OW;
-  int P;                    // output positions per image (= OH*OW)
-  int n_gemm;               // C*KH*KW
-  int acc_n, n_acc;         // columns per accumulator, accumulators per CTA (1 or 2)
-  int n_tiles, m_tiles;
-  int tiles_per_img, total_ktiles, ktiles_per_split, splits;
-  int tmem_cols, stages, smem_bytes;
-};
-
-// False when the layer is not one the fast kernel handles.
-bool plan_conv_fast(const surgeon_layer_desc& d, FastParams* out);
-
-// Bytes of scratch for the bf16 copy of the output gradient.
-size_t conv_fast_grad_bf16_bytes(const FastParams& p);
-
-// Enqueues the bf16 conversion of grad_out into grad_bf16 and the kernel;
-// partial = [splits][O][n_gemm] fp32, status = one word (the pre-pass zeroes it).
-cudaError_t launch_conv_fast(const surgeon_compressed& act, const FastParams& p,
-                             const float* grad_out, void* grad_bf16, float* partial,
-                             uint32_t* status, cudaStream_t stream);
 
 // fp32 -> bf16 (round to nearest even) copy of n elements, as one streaming kernel.
 // As every gradient pre-pass, it also zeroes the call's status word.
