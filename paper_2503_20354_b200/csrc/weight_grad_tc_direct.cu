@@ -1124,8 +1124,8 @@ static bool compute_plan_direct(const surgeon_layer_desc& d, bool transposed_ok,
     // columns (a multiple of 16 with the fewest padded columns, then the widest); a CTA holds up
     // to three units (<= 512 TMEM columns).
     int best_waste = -1;
-    // (TG >= 2: the kh accumulators of a kernel column share the 512 columns)
-    for (int c = p.tg >= 2 ? 512 / p.kh / 16 * 16 : 256; c >= 16; c -= 16) {
+    // (TG >= 2: the kh accumulators of a kernel column share the 512 columns; an MMA has at most 256)
+    for (int c = p.tg >= 2 ? std::min(256, 512 / p.kh / 16 * 16) : 256; c >= 16; c -= 16) {
       const int upt = (p.o_real + c - 1) / c;
       const int waste = upt * c - p.o_real;
       if (best_waste < 0 || waste < best_waste) { best_waste = waste; p.acc_n = c; p.upt = upt; }
@@ -1175,6 +1175,7 @@ static bool compute_plan_direct(const surgeon_layer_desc& d, bool transposed_ok,
     p.acc_n = best_n; p.n_acc = best_a;
     if (p.tg) p.b_bytes = p.n_acc * p.unit_bytes;
   }
+  if (p.acc_n < 16 || p.acc_n > 256 || p.acc_n % 16 != 0) return false;      // not a shape that an MMA has
   p.n_cols = p.acc_n * p.n_acc;
   p.n_tiles = n_tiles_of(p.acc_n, p.n_acc);
   const long long tiles_mn = static_cast<long long>(p.m_tiles) * p.n_tiles;

@@ -38,6 +38,11 @@ TRANSPOSED = [
     W.conv("halo56", 1, 40, 56, 48, 3),
     W.conv("halo16_nopad", 2, 20, 16, 64, 3, 1, 0),
     W.Layer("halo16_2x3", 1, 2, 20, 9, 16, 48, 2, 3, 1, 1),
+    # one kernel row: its single accumulator is as wide as an MMA allows, not as the 512 columns would
+    W.Layer("halo8_1x3", 1, 3, 20, 9, 8, 264, 1, 3, 1, 0),
+    W.Layer("halo16_1x5", 1, 2, 40, 5, 16, 320, 1, 5, 1, 0),
+    W.Layer("halo32_1x3", 1, 1, 20, 3, 32, 512, 1, 3, 1, 0),
+    W.Layer("halo56_1x2", 1, 1, 24, 2, 56, 768, 1, 2, 1, 0),
     # a box per tap (other widths, other kernels)
     W.conv("tap7", 9, 40, 7, 136, 3),
     W.conv("tap14", 3, 24, 14, 264, 3),
