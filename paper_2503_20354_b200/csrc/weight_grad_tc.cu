@@ -985,8 +985,10 @@ cudaError_t launch_weight_grad_tc(const surgeon_compressed& act, const surgeon_l
       while (chunk > 32 && (static_cast<long long>(dp.o_real) * ((dp.C + chunk - 1) / chunk) < 4LL * sm_count() ||
                             chunk * dp.taps * 4 > 48 * 1024))
         chunk >>= 1;
-      // as many threads per element as fit 512, while each has four parts left, and no second round of them
-      const int items = std::min(chunk, dp.C) / 4 * dp.taps;
+      chunk = std::min(chunk, dp.C);
+      // as many threads per element as fit 512, while each has four parts left, and no second round of them: the
+      // tile is then 16 bytes a thread, 8 KB at most
+      const int items = chunk / 4 * dp.taps;
       const int sp = dp.C % 4 == 0 ? std::max(1, std::min({8, 512 / items, dp.splits / 4})) : 1;
       const int threads = sp > 1 ? (items * sp + 31) / 32 * 32 : 256;
       launch_kernel(reduce_splits_taps_kernel, dim3((dp.C + chunk - 1) / chunk, dp.o_real), dim3(threads),

@@ -105,6 +105,15 @@ def test_reductions_of_small_weights(batch, c_in, c_out, k):
 
 
 @pytest.mark.parametrize("layer", [
+    W.Layer("7x5", 1, 47, 4, 11, 35, 624, 7, 5, 1, 2), W.conv("5x5", 51, 4, 28, 605, 5)], ids=lambda l: l.name)
+def test_tap_reduction_of_few_channels_and_many_outputs(layer):
+    """A block of the tap reduction has fewer channels than it could take and several threads per element: its
+    shared memory is that of the channels that exist (a buffer for 256 would exceed 48 KB)."""
+    dw, ref = _dw(layer, 0.5, B.PATH_TENSOR_CORE)
+    assert rel_frobenius(dw, ref) <= 5e-3
+
+
+@pytest.mark.parametrize("layer", [
     W.linear("few_rows", 200, 320, 320), W.linear("ragged", 333, 136, 200), W.linear("wide", 260, 64, 1288),
     W.conv("one_image", 1, 40, 14, 72, 1, 1, 0), W.conv("one_image_3x3", 1, 24, 13, 56, 3), W.conv("taps_part", 2, 20, 8, 48, 3),
     W.conv("one_map", 1, 132, 16, 500, 1, 1, 0)], ids=lambda l: l.name)
