@@ -172,6 +172,10 @@ surgeon_status surgeon_prune_compact(const void* x, int64_t n, surgeon_dtype dt,
  * surgeon_prune_compact.  Unknown flag bits: INVALID_ARG.
  * ---------------------------------------------------------------------------------------- */
 #define SURGEON_STORE_DROP_ZEROS 1u
+/* Other calls run on other streams at the same time: this one takes a part of the GPU (at most a
+ * quarter of the SMs) and leaves the rest to them.  By default a call takes what makes it fastest by
+ * itself, and calls of several streams then run one after the other.  Results are the same. */
+#define SURGEON_SHARE_GPU 2u
 /* Diagnostic without a counterpart in the paper, for testing the error path of the bounded
  * device-side waits: the select's grid-wide barrier is given an arrival target it cannot reach
  * and a cap of 1024 polls, so it gives up after some tens of microseconds.  Every kernel of the

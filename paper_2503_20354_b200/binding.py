@@ -288,6 +288,7 @@ class CompressedActivation:
 
 
 SURGEON_STORE_DROP_ZEROS = 1
+SURGEON_SHARE_GPU = 2
 SURGEON_DEBUG_STALL_BARRIER = 0x80000000
 
 
@@ -297,7 +298,9 @@ def surgeon_prune_compact(x: torch.Tensor, ratio: float, out: Optional[Compresse
                           flags: int = 0) -> CompressedActivation:
     """Prune ``x`` (CUDA tensor, fp32 or bf16, contiguous) at ``ratio`` into a compressed store.
     ``flags=SURGEON_STORE_DROP_ZEROS``: kept zeros get no bit and no value (the header's n_keep
-    is then the stored count; ``out.sizes.n_keep`` stays the upper bound the buffers are sized for)."""
+    is then the stored count; ``out.sizes.n_keep`` stays the upper bound the buffers are sized for).
+    ``flags=SURGEON_SHARE_GPU``: other streams' calls run at the same time, so this one takes a part of
+    the GPU; a call that is sent to another stream than the current one says so by that."""
     if not x.is_cuda or not x.is_contiguous():
         raise ValueError("x must be a contiguous CUDA tensor")
     dt = dtype_code(x.dtype)
@@ -309,10 +312,12 @@ def surgeon_prune_compact(x: torch.Tensor, ratio: float, out: Optional[Compresse
         raise ValueError("output store does not fit this tensor / ratio")
     if workspace is None:
         workspace = _scratch(surgeon_compact_sizes(n, dt, ratio).workspace_bytes, x.device, stream)
+    at = _stream_ptr(stream)
+    if stream is not None and at != _stream_ptr(None):
+        flags |= SURGEON_SHARE_GPU
     st = lib().surgeon_prune_compact_flags(x.data_ptr(), n, dt, ratio, int(flags), C.byref(out.c),
                                            workspace.data_ptr(),
-                                           workspace.numel() * workspace.element_size(),
-                                           _stream_ptr(stream))
+                                           workspace.numel() * workspace.element_size(), at)
     if st != SURGEON_OK:
         _check(st, "surgeon_prune_compact")
     out._now_at(ratio)

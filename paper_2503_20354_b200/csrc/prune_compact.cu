@@ -30,6 +30,7 @@
 // either way.  Every count fits 32 bits because n <= SURGEON_MAX_N < 2^31.
 #include <cuda.h>
 
+#include <algorithm>
 #include <atomic>
 #include <chrono>
 #include <random>
@@ -69,6 +70,9 @@ constexpr int kAuxBytes = kAuxPrefix + kMaxLocalChunks * 8 > kSampleBytes ? kAux
 constexpr int kStageBytes = (kAuxCnt / kWarps) & ~15;
 constexpr size_t kPruneSmem = static_cast<size_t>(kRingBytes) + kAuxBytes + 1024;
 static_assert(kChunkBytes == kTileVecs * 16, "chunk size");
+// A streamed tensor's bracket comes from order statistics 2.5 sqrt(G) + 1 places to either side of the middle of G
+// CTAs' answers: with fewer than 31 CTAs there are none, and every key would be a candidate.
+constexpr int kLeastStreamedCtas = 31;
 constexpr int kMaxKeys = 64;                     // keys one CTA reports at the last exchange
 constexpr int kKeysPerThread = 8;                // and CTA 0 takes in
 constexpr int kKeysAtOnce = kKeysPerThread * kThreads;
@@ -1607,7 +1611,7 @@ unsigned long long next_token() {
 }
 
 template <int DT>
-cudaError_t run_prune_compact(const void* x, long long n, long long k, int drop_zeros, int stall,
+cudaError_t run_prune_compact(const void* x, long long n, long long k, int drop_zeros, int stall, int share,
                               const surgeon_compressed& out, void* workspace,
                               cudaStream_t stream) {
   using E = typename Elem<DT>::type;
@@ -1641,16 +1645,22 @@ cudaError_t run_prune_compact(const void* x, long long n, long long k, int drop_
   a.slots = ws + L.slots;
   CUtensorMap map;
   if (!make_row_map(x, a.n_rows_full > 0 ? a.n_rows_full : 1, &map)) return cudaErrorNotSupported;
-  // as many chunks per warp as a full grid would give its busiest warp, on as few CTAs as that takes: the
-  // others leave their SMs to other streams.  A caller that changes streams from call to call (the
-  // prunes of several layers in flight) gets the smallest grid that keeps the tensor on chip: the
-  // kernel takes whole SMs, so grids of 148 run one after the other.
-  static std::atomic<cudaStream_t> last_stream{nullptr};
-  const bool alone = last_stream.exchange(stream, std::memory_order_relaxed) == stream;
+  // A call by itself: as many chunks per warp as a full grid would give its busiest warp, on as few CTAs as that
+  // takes.  A CTA takes a whole SM, so calls on full grids run one after the other, each with its chain of exchanges
+  // exposed (20 us of the 40 that 19 MB take).  A call that says that others run beside it (SURGEON_SHARE_GPU) gets
+  // the smallest grid that keeps the tensor on chip, and of a tensor that no quarter of the SMs can hold a
+  // quarter: four such grids fit exactly (of grids that leave a rest a fifth starts in part and spins).
+  // Whole stacks on eight streams, full grid / SMs / 2, / 3, / 4: ViT 2.46 / 1.70 / 1.57 / 1.61 ms, WideResNet
+  // 1.53 / 1.14 / 1.08 / 1.00, ResNet-50 1.68 / 1.28 / 1.09 / 1.04, ResNeXt 1.93 / 1.46 / 1.36 / 1.31.
   const int sms = sm_count() < kSelMaxCtas ? sm_count() : kSelMaxCtas;
-  int per_cta = (a.n_chunks + sms * kWarps - 1) / (sms * kWarps) * kWarps;
-  if (!alone && per_cta < kResidentChunks) per_cta = kResidentChunks;
-  const int grid = (a.n_chunks + per_cta - 1) / per_cta;
+  int grid;
+  if (share) {
+    const int most = std::min(sms, std::max(sms / 4, kLeastStreamedCtas));
+    grid = std::min(most, (a.n_chunks + kResidentChunks - 1) / kResidentChunks);
+  } else {
+    const int per_cta = (a.n_chunks + sms * kWarps - 1) / (sms * kWarps) * kWarps;
+    grid = (a.n_chunks + per_cta - 1) / per_cta;
+  }
   a.spread = a.n_chunks > grid * kMaxLocalChunks ? 1 : 0;
   const bool resident = (a.n_chunks + grid - 1) / grid <= kResidentChunks;
   const void* kernel = resident ? reinterpret_cast<const void*>(prune_kernel<DT, true>)
@@ -1668,9 +1678,9 @@ cudaError_t run_prune_compact(const void* x, long long n, long long k, int drop_
 
 cudaError_t launch_prune_compact(const void* x, int64_t n, int dt, int64_t k,
                                  const surgeon_compressed& out, void* workspace,
-                                 cudaStream_t stream, int drop_zeros, int stall) {
-  return dt == 0 ? run_prune_compact<0>(x, n, k, drop_zeros, stall, out, workspace, stream)
-                 : run_prune_compact<1>(x, n, k, drop_zeros, stall, out, workspace, stream);
+                                 cudaStream_t stream, int drop_zeros, int stall, int share) {
+  return dt == 0 ? run_prune_compact<0>(x, n, k, drop_zeros, stall, share, out, workspace, stream)
+                 : run_prune_compact<1>(x, n, k, drop_zeros, stall, share, out, workspace, stream);
 }
 
 cudaError_t launch_decompress(const surgeon_compressed& act, void* x_out, cudaStream_t stream) {

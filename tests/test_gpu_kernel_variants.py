@@ -139,6 +139,23 @@ def test_prune_ranges(chunks, extra, bf16):
 
 
 @pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("chunks,extra", [(1, -1), (49, 0), (48 * 37, 0), (48 * 37, 1), (512 * 37 + 1, 3)])
+def test_prune_on_a_part_of_the_gpu(chunks, extra, bf16):
+    """SURGEON_SHARE_GPU, asked for or implied by a stream that is not the current one: at most a quarter of the
+    SMs, resident up to 48 chunks a CTA, counts in global memory beyond 512."""
+    n = chunks * (2048 if bf16 else 1024) + extra
+    x = W.draw("relu_normal", n, seed=4, device="cuda").cpu()
+    x = x.to(torch.bfloat16) if bf16 else x
+    side = torch.cuda.Stream()
+    for ratio in (0.3, 0.85):
+        assert_store_equals_oracle(x, ratio, comp=B.surgeon_prune_compact(x.cuda(), ratio, flags=B.SURGEON_SHARE_GPU))
+    xd = x.cuda()
+    out = B.CompressedActivation(n, B.dtype_code(x.dtype), 0.0, "cuda")
+    side.wait_stream(torch.cuda.current_stream())
+    assert_store_equals_oracle(x, 0.85, comp=B.surgeon_prune_compact(xd, 0.85, out=out, stream=side))
+
+
+@pytest.mark.parametrize("bf16", [False, True])
 def test_sample_that_misleads(bf16):
     """A short stretch holds all the large values: the strided sample sees few of them or none, so the bracket can
     miss and the select has to start over with what its counts prove."""
