@@ -111,8 +111,8 @@ __device__ __forceinline__ uint32_t hash_u32(uint32_t v) {
 // No counter has to start at zero, so the call needs no memset: the token differs from call to
 // call.  For a captured graph, whose replays carry the same token, CTA 0 clears every report that it
 // has read, clears a phase's answers before it answers the phase before it, and clears the first
-// answer (phase 0) after the reports of phase 1.  All CTAs are resident (cooperative launch); polls
-// are bounded.
+// answer (phase 0) after the reports of phase 1; a CTA that gives up takes its own words back.  All CTAs are
+// resident (cooperative launch); polls are bounded.
 __device__ __forceinline__ void word_store(ulonglong2* p, unsigned long long token, unsigned long long v) {
   asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}"
                ::"l"(p), "l"(token), "l"(v) : "memory");
@@ -759,7 +759,14 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     ++phase;
     return ok != 0;
   };
-  auto quit = [&]() { if (tid == 0) atomicMax(&a.hdr->status, static_cast<uint32_t>(SURGEON_ERR_TIMEOUT)); };
+  // The whole CTA leaves after a wait gave up.  It takes back what it has stored for the others: a replay of a
+  // captured call carries the same token and must not find it.
+  auto quit = [&]() {
+    if (tid == 0) atomicMax(&a.hdr->status, static_cast<uint32_t>(SURGEON_ERR_TIMEOUT));
+    if (tid < kSelPhases) a.arrive[tid * kSelMaxCtas + blockIdx.x].x = 0ull;
+    if (master)
+      for (int i = tid; i < kSelPhases * (kSelMaxCtas + 2); i += kThreads) a.answer[i].x = 0ull;
+  };
 
   // ---- set-up ----
   if (lane == 0) {                               // a warp's barriers are its own
@@ -1598,7 +1605,7 @@ bool make_row_map(const void* x, long long n_rows_full, CUtensorMap* map) {
                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// A value that no other call of this or another process carries (see grid_arrive).
+// A value that no other call of this or another process carries (see the grid-wide exchange).
 unsigned long long next_token() {
   static std::atomic<unsigned long long> counter{[] {
     std::random_device rd;

@@ -57,7 +57,6 @@ extern "C" surgeon_status surgeon_prune_compact_static(const void* x, int64_t n,
   if (n > SURGEON_STATIC_MAX_N) return SURGEON_ERR_UNSUPPORTED;  // built-in scratch is too small
   void* scratch = nullptr;
   if (static_scratch(&scratch) != cudaSuccess) return SURGEON_ERR_CUDA;
-  // Same checks and the same kernels as the ordinary call; they clear the part of the scratch
-  // that has to start at zero, so whatever an earlier call left behind does no harm.
+  // Same checks and the same kernel as the ordinary call, which needs nothing in the scratch to start at any value.
   return surgeon_prune_compact(x, n, dt, ratio, out, scratch, kStaticScratchBytes, cuda_stream);
 }

@@ -212,6 +212,21 @@ def test_captured_call_replays_and_alternating_streams(n):
         assert all(np.array_equal(u, v) for u, v in zip(outs[i].to_numpy()[:3], ref[i]))
 
 
+@pytest.mark.parametrize("n", [5000, 1 << 20, 10_000_000])
+def test_call_that_timed_out_leaves_no_words_behind(n):
+    """Replays of a captured call carry one token, so the words {token, 8 bytes} that the CTAs exchange (the first
+    12 x 256 + 12 x 258 pairs of the scratch) have to be gone after a call that gave up."""
+    x = W.draw("normal", n, seed=8, device="cuda")
+    out = B.CompressedActivation(n, B.SURGEON_F32, 0.0, "cuda")
+    ws = torch.zeros(out.sizes.workspace_bytes, dtype=torch.uint8, device="cuda")
+    B.surgeon_prune_compact(x, 0.5, out=out, workspace=ws, flags=B.SURGEON_DEBUG_STALL_BARRIER)
+    torch.cuda.synchronize()
+    assert out.read_header().status == B.SURGEON_ERR_TIMEOUT
+    tokens = ws[:16 * 12 * (256 + 258)].view(torch.int64).view(-1, 2)[:, 0]
+    assert int(tokens.count_nonzero()) == 0
+    assert_store_equals_oracle(x.cpu(), 0.5, comp=B.surgeon_prune_compact(x, 0.5, out=out, workspace=ws))
+
+
 @pytest.mark.parametrize("bf16", [False, True])
 @pytest.mark.parametrize("n", [1, 31, 1023, 1025, 4 * 8192 + 5])
 def test_rebuild(n, bf16):
