@@ -180,7 +180,8 @@ surgeon_status surgeon_prune_compact(const void* x, int64_t n, surgeon_dtype dt,
  * device-side waits: the select's grid-wide barrier is given an arrival target it cannot reach
  * and a cap of 1024 polls, so it gives up after some tens of microseconds.  Every kernel of the
  * call then returns without storing to bitmap, values or block_offsets, and
- * surgeon_header::status reads SURGEON_ERR_TIMEOUT; the other header fields are undefined.
+ * surgeon_header::status reads SURGEON_ERR_TIMEOUT and n_keep 0; the other header fields are
+ * undefined.
  * Nothing faults and nothing spins past the cap. */
 #define SURGEON_DEBUG_STALL_BARRIER 0x80000000u
 surgeon_status surgeon_prune_compact_flags(const void* x, int64_t n, surgeon_dtype dt, double ratio,

@@ -823,7 +823,10 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     }
   }
   if (master) {                                  // meanwhile CTA 0 prepares the exchange
-    if (tid == 0) a.hdr->status = SURGEON_OK;
+    if (tid == 0) {                              // (no value yet: what reads the store trusts the count)
+      a.hdr->status = SURGEON_OK;
+      a.hdr->n_keep = 0;
+    }
     prepare_phase(a, 1);
     prepare_round(a, 0);
     if (!RES && tid < kSelPhases * kClaimSets) a.claims[tid * kClaimStride] = 0u;
