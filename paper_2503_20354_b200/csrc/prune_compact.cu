@@ -660,6 +660,8 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     }
     return true;
   };
+  // True where arrived() writes to the chunk's place itself: its last rows, or the zeros of a chunk without a whole row.
+  auto completed = [&](int c) { return static_cast<long long>(c) * 32 + 32 > a.n_rows_full; };
   // The warp's chunks of one pass in the order of their loads: next() is the next one, or n_chunks.
   static_assert(kSlotsPerWarp == 3, "three loads in flight");
   int fly0 = a.n_chunks, fly1 = a.n_chunks, fly2 = a.n_chunks;    // chunks in flight, the oldest first
@@ -703,7 +705,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     for (int s = 0; fly0 < a.n_chunks; s = s == 2 ? 0 : s + 1) {
       unsigned char* region = my_ring + s * kChunkBytes;
       if (!arrived(fly0, s)) { give_up(s); break; }
-      const bool written = f(fly0, region);
+      const bool written = f(fly0, region) || completed(fly0);
       fly0 = fly1; fly1 = fly2;
       int c = next();
       if (c < a.n_chunks) {
@@ -1486,7 +1488,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
         for (int j = i - 1; j >= 0 && j > i - kSlotsPerWarp; --j) arrived(chunk_of(j), j % kSlotsPerWarp);
         break;
       }
-      const bool written = emit(chunk_of(i), my_ring + sl * kChunkBytes);
+      const bool written = emit(chunk_of(i), my_ring + sl * kChunkBytes) || completed(chunk_of(i));
       if (i >= kSlotsPerWarp) {
         if (written) tc::fence_proxy_async();
         __syncwarp();

@@ -139,6 +139,21 @@ def test_prune_ranges(chunks, extra, bf16):
 
 
 @pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("share", [0, B.SURGEON_SHARE_GPU])
+@pytest.mark.parametrize("chunks,extra", [(48 * 148 + 600, 5), (48 * 148 + 601, 700), (512 * 148 + 33, 30)])
+def test_partial_last_row_of_a_streamed_tensor(chunks, extra, share, bf16):
+    """The emitting pass runs backwards: the place of the tensor's last chunk, whose partial row is put there by
+    ordinary stores, is the first that another chunk's load fills.  Little or nothing of it is kept."""
+    n = chunks * (2048 if bf16 else 1024) + extra
+    x = W.draw("normal", n, seed=6, device="cuda").cpu()
+    x = x.to(torch.bfloat16) if bf16 else x
+    for tail, ratio in ((1.0, 0.95), (0.0, 0.7)):
+        x[-(extra + 1500):] *= tail
+        comp = B.surgeon_prune_compact(x.cuda(), ratio, flags=share)
+        assert_store_equals_oracle(x, ratio, comp=comp)
+
+
+@pytest.mark.parametrize("bf16", [False, True])
 @pytest.mark.parametrize("chunks,extra", [(1, -1), (49, 0), (48 * 37, 0), (48 * 37, 1), (512 * 37 + 1, 3)])
 def test_prune_on_a_part_of_the_gpu(chunks, extra, bf16):
     """SURGEON_SHARE_GPU, asked for or implied by a stream that is not the current one: at most a quarter of the
