@@ -293,6 +293,7 @@ class Stack:
         # with those of its neighbours.  Both loops fork from and join the caller's stream.
         self.n_streams = max(1, int(n_streams))
         self.streams = [torch.cuda.Stream(device=device) for _ in range(self.n_streams)] if self.n_streams > 1 else []
+        self.flags = B.SURGEON_SHARE_GPU if self.n_streams > 1 else 0
         self.ws = [torch.empty(max(ws1, ws2, 256), dtype=torch.uint8, device=device)
                    for _ in range(self.n_streams)]
         self.ratios = None
@@ -335,7 +336,7 @@ class Stack:
             if x_ready is not None:
                 (st or torch.cuda.current_stream(self.device)).wait_event(x_ready[i])
             B.surgeon_prune_compact(self.x[i], float(self.ratios[i]), out=self.store[i], workspace=self.ws[k],
-                                    stream=st)
+                                    stream=st, flags=self.flags)
         self._join()
         if ev: ev[1].record()
         self._fork()
@@ -345,7 +346,7 @@ class Stack:
             if g_ready is not None:
                 (st or torch.cuda.current_stream(self.device)).wait_event(g_ready[i])
             B.surgeon_weight_grad(self.store[i], self.desc[i], self.g[i], dw=self.dw[i], workspace=self.ws[k],
-                                  stream=st)
+                                  stream=st, flags=self.flags)
             if dw_done is not None:
                 dw_done[i].record(st or torch.cuda.current_stream(self.device))
         self._join()

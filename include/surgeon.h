@@ -261,6 +261,14 @@ surgeon_status surgeon_weight_grad(const surgeon_compressed* act, const surgeon_
                                    const float* grad_out, float* dw, int32_t accumulate,
                                    void* workspace, size_t workspace_bytes, void* cuda_stream);
 
+/* The same call with options.  SURGEON_SHARE_GPU: other calls run on other streams at the same time, so a
+ * small layer is cut into fewer parts than make it fastest by itself; its sums are then grouped
+ * otherwise (fixed as well, but not bit for bit those of a call without the flag).  The workspace query
+ * covers both.  flags = 0 is surgeon_weight_grad.  Unknown flag bits: INVALID_ARG. */
+surgeon_status surgeon_weight_grad_flags(const surgeon_compressed* act, const surgeon_layer_desc* d,
+                                         const float* grad_out, float* dw, int32_t accumulate, uint32_t flags,
+                                         void* workspace, size_t workspace_bytes, void* cuda_stream);
+
 /* ------------------------------------------------------------------------------------------
  * Algorithm 1: Reshape step ("Reshape") as a stand-alone utility: x_out[j] = kept ? value : +0 for
  * all j < act->n, in act->dt.  x_out: device pointer to n elements.  surgeon_weight_grad does

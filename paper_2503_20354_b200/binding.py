@@ -91,6 +91,9 @@ def lib():
         l.surgeon_weight_grad.restype = C.c_int
         l.surgeon_weight_grad.argtypes = [C.POINTER(Compressed), C.POINTER(LayerDesc), C.c_void_p,
                                           C.c_void_p, C.c_int32, C.c_void_p, C.c_size_t, C.c_void_p]
+        l.surgeon_weight_grad_flags.restype = C.c_int
+        l.surgeon_weight_grad_flags.argtypes = [C.POINTER(Compressed), C.POINTER(LayerDesc), C.c_void_p, C.c_void_p,
+                                                C.c_int32, C.c_uint32, C.c_void_p, C.c_size_t, C.c_void_p]
         l.surgeon_decompress.restype = C.c_int
         l.surgeon_decompress.argtypes = [C.POINTER(Compressed), C.c_void_p, C.c_void_p]
         l.surgeon_launch_count.restype = C.c_uint64
@@ -380,8 +383,10 @@ def surgeon_weight_grad_workspace(desc: LayerDesc) -> int:
 def surgeon_weight_grad(act: CompressedActivation, desc: LayerDesc, grad_out: torch.Tensor,
                         dw: Optional[torch.Tensor] = None, accumulate: bool = False,
                         workspace: Optional[torch.Tensor] = None,
-                        stream: Optional[torch.cuda.Stream] = None) -> torch.Tensor:
-    """dW of the layer from the compressed activation and fp32 ``grad_out``; returns ``dw``."""
+                        stream: Optional[torch.cuda.Stream] = None, flags: int = 0) -> torch.Tensor:
+    """dW of the layer from the compressed activation and fp32 ``grad_out``; returns ``dw``.
+    ``flags=SURGEON_SHARE_GPU``: other streams' calls run at the same time, so a small layer is cut into
+    fewer parts (its sums are grouped otherwise, which is why a ``stream`` argument does not imply it)."""
     if grad_out.dtype != torch.float32 or not grad_out.is_cuda or not grad_out.is_contiguous():
         raise ValueError("grad_out must be a contiguous fp32 CUDA tensor")
     if dw is None:
@@ -391,8 +396,8 @@ def surgeon_weight_grad(act: CompressedActivation, desc: LayerDesc, grad_out: to
         dw = torch.empty(shape, dtype=torch.float32, device=grad_out.device)
     if workspace is None:
         workspace = _scratch(surgeon_weight_grad_workspace(desc), grad_out.device, stream)
-    st = lib().surgeon_weight_grad(C.byref(act.c), C.byref(desc), grad_out.data_ptr(), dw.data_ptr(),
-                                   1 if accumulate else 0, workspace.data_ptr(),
-                                   workspace.numel() * workspace.element_size(), _stream_ptr(stream))
+    st = lib().surgeon_weight_grad_flags(C.byref(act.c), C.byref(desc), grad_out.data_ptr(), dw.data_ptr(),
+                                         1 if accumulate else 0, int(flags), workspace.data_ptr(),
+                                         workspace.numel() * workspace.element_size(), _stream_ptr(stream))
     _check(st, "surgeon_weight_grad")
     return dw

@@ -248,8 +248,15 @@ size_t surgeon_weight_grad_workspace(const surgeon_layer_desc* d) {
 surgeon_status surgeon_weight_grad(const surgeon_compressed* act, const surgeon_layer_desc* d,
                                    const float* grad_out, float* dw, int32_t accumulate,
                                    void* workspace, size_t workspace_bytes, void* cuda_stream) {
+  return surgeon_weight_grad_flags(act, d, grad_out, dw, accumulate, 0u, workspace, workspace_bytes, cuda_stream);
+}
+
+surgeon_status surgeon_weight_grad_flags(const surgeon_compressed* act, const surgeon_layer_desc* d,
+                                         const float* grad_out, float* dw, int32_t accumulate, uint32_t flags,
+                                         void* workspace, size_t workspace_bytes, void* cuda_stream) {
   surgeon_status why;
   if (!desc_ok(d, &why)) return why;
+  if (flags & ~static_cast<uint32_t>(SURGEON_SHARE_GPU)) return SURGEON_ERR_INVALID_ARG;
   if (!act || !grad_out || !dw || !act->bitmap || !act->block_offsets) return SURGEON_ERR_INVALID_ARG;
   if (act->dt != SURGEON_F32 && act->dt != SURGEON_BF16) return SURGEON_ERR_INVALID_ARG;
   if (act->n != static_cast<int64_t>(d->batch) * d->c_in * d->h * d->w) return SURGEON_ERR_INVALID_ARG;
@@ -263,7 +270,8 @@ surgeon_status surgeon_weight_grad(const surgeon_compressed* act, const surgeon_
   const cudaError_t e =
       d->groups > 1 ? launch_weight_grad_grouped(*act, *d, grad_out, dw, accumulate ? 1 : 0, workspace, s)
       : d->path == 1 ? launch_weight_grad_fp32(*act, *d, grad_out, dw, accumulate ? 1 : 0, workspace, s)
-                     : launch_weight_grad_tc(*act, *d, grad_out, dw, accumulate ? 1 : 0, workspace, s);
+                     : launch_weight_grad_tc(*act, *d, grad_out, dw, accumulate ? 1 : 0, flags & SURGEON_SHARE_GPU ? 1 : 0,
+                                             workspace, s);
   if (e == cudaErrorNotSupported) return SURGEON_ERR_UNSUPPORTED;
   if (e != cudaSuccess && getenv("SURGEON_VERBOSE"))
     fprintf(stderr, "surgeon_weight_grad: %s\n", cudaGetErrorString(e));

@@ -94,7 +94,7 @@ cudaError_t launch_weight_grad_grouped(const surgeon_compressed& act, const surg
 
 size_t weight_grad_tc_workspace(const surgeon_layer_desc& d);
 cudaError_t launch_weight_grad_tc(const surgeon_compressed& act, const surgeon_layer_desc& d,
-                                  const float* grad_out, float* dw, int accumulate,
+                                  const float* grad_out, float* dw, int accumulate, int share,
                                   void* workspace, cudaStream_t stream);
 
 // The driver's cuTensorMapEncodeTiled, looked up through the runtime (the library carries no

@@ -939,7 +939,11 @@ size_t weight_grad_tc_workspace(const surgeon_layer_desc& d) {
   SwapParams sp;
   if (plan_swap(d, &sp)) return kStatusBytes + swap_partial_bytes(sp) + direct_grad_bf16_bytes(sp.d);
   DirectParams dp;
-  if (plan_direct(d, &dp)) return kStatusBytes + direct_partial_bytes(dp) + direct_grad_bf16_bytes(dp);
+  if (plan_direct(d, false, &dp)) {              // (the splits of a call that shares the GPU may be others)
+    const size_t alone = direct_partial_bytes(dp) + direct_grad_bf16_bytes(dp);
+    if (!plan_direct(d, true, &dp)) return kStatusBytes + alone;
+    return kStatusBytes + std::max(alone, direct_partial_bytes(dp) + direct_grad_bf16_bytes(dp));
+  }
   StridedParams st;
   if (plan_strided(d, &st)) return kStatusBytes + strided_partial_bytes(st) + strided_grad_bf16_bytes(st);
   TcParams p;
@@ -952,7 +956,7 @@ size_t weight_grad_tc_workspace(const surgeon_layer_desc& d) {
 }
 
 cudaError_t launch_weight_grad_tc(const surgeon_compressed& act, const surgeon_layer_desc& d,
-                                  const float* grad_out, float* dw, int accumulate,
+                                  const float* grad_out, float* dw, int accumulate, int share,
                                   void* workspace, cudaStream_t stream) {
   // No geometry plan fits: say so before anything touches the workspace (its size query gave 0).
   if (weight_grad_tc_workspace(d) == 0 || workspace == nullptr) return cudaErrorNotSupported;
@@ -966,7 +970,7 @@ cudaError_t launch_weight_grad_tc(const surgeon_compressed& act, const surgeon_l
   DirectParams dp;
   SwapParams sp;
   const bool swapped = plan_swap(d, &sp);
-  if (swapped || plan_direct(d, &dp)) {
+  if (swapped || plan_direct(d, share != 0, &dp)) {
     if (swapped) {
       dp = sp.d;
       dp.splits = sp.splits;

@@ -104,7 +104,7 @@ struct DirectParams {
   unsigned few_keep;        // packed values up to which runs are rebuilt element by element (launcher)
   unsigned partial_blk;     // index of the bitmap's last block if it is partial, else 0xFFFFFFFF
 };
-bool plan_direct(const surgeon_layer_desc& d, DirectParams* out);
+bool plan_direct(const surgeon_layer_desc& d, bool share, DirectParams* out);   // share: other streams' calls run beside it
 bool plan_direct_copies(const surgeon_layer_desc& d, DirectParams* out);   // never a transposed gradient copy
 size_t direct_grad_bf16_bytes(const DirectParams& p);
 // partial = [splits][O][C] fp32 (O counts the stacked taps), status = one word (the pre-pass zeroes it).

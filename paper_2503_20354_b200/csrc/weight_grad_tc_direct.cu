@@ -1041,7 +1041,7 @@ static bool size_rings(DirectParams* p, int stage_bytes) {
   return true;
 }
 
-static bool compute_plan_direct(const surgeon_layer_desc& d, bool transposed_ok, DirectParams* out) {
+static bool compute_plan_direct(const surgeon_layer_desc& d, bool transposed_ok, bool share, DirectParams* out) {
   DirectParams p{};
   if (d.kind == 0) {
     p.mode = 0;
@@ -1154,9 +1154,13 @@ static bool compute_plan_direct(const surgeon_layer_desc& d, bool transposed_ok,
            : (p.mode == 0) ? (p.O + acc_n * n_acc - 1) / (acc_n * n_acc) : (p.n_units + n_acc - 1) / n_acc;
   };
   // The K-tiles in splits of four or more: a CTA's time is that of its K-tiles and some five tiles' worth for its
-  // start, its partial tile and its share of the reduction.
-  const int max_splits = static_cast<int>(std::min<long long>((total + 3) / 4, 128));
-  if (!p.pair && p.tg < 2 && static_cast<long long>(p.m_tiles) * n_tiles_of(p.acc_n, p.n_acc) * max_splits < sms) {
+  // start, its partial tile and its share of the reduction.  Next to other streams' calls (SURGEON_SHARE_GPU) the SMs
+  // that a layer leaves idle are not idle: splits of eight, and the widest column tiles (320 -> 320 channels of 4096
+  // rows take 24 SMs for 23.6 us instead of 144 for 19.5; a Segformer-shaped stack on eight streams 5.0 instead of
+  // 5.9 ms, on one stream 8.3 instead of 7.7).
+  const int least = share ? 8 : 4;
+  const int max_splits = static_cast<int>(std::min<long long>((total + least - 1) / least, 128));
+  if (!share && !p.pair && p.tg < 2 && static_cast<long long>(p.m_tiles) * n_tiles_of(p.acc_n, p.n_acc) * max_splits < sms) {
     // The widest column tiles leave SMs without work: narrower ones.  They rebuild the activation once more each, on
     // SMs that would idle, and the partial tile (7 K-tiles' worth at 512 columns: it leaves at 25 to 30 bytes a
     // clock) is written by more of them.
@@ -1197,15 +1201,15 @@ static bool compute_plan_direct(const surgeon_layer_desc& d, bool transposed_ok,
   return true;
 }
 
-bool plan_direct(const surgeon_layer_desc& d, DirectParams* out) {
+bool plan_direct(const surgeon_layer_desc& d, bool share, DirectParams* out) {
   struct Tag {};
-  return memo_plan<Tag>(d, use_pairs() ? 1 : 0, out, [&](DirectParams* p) {
+  return memo_plan<Tag>(d, (use_pairs() ? 1 : 0) + (share ? 2 : 0), out, [&](DirectParams* p) {
     // (a stage of boxes with halo rows can be too large for the rings)
-    return compute_plan_direct(d, !use_pairs(), p) || compute_plan_direct(d, false, p);
+    return compute_plan_direct(d, !use_pairs(), share, p) || compute_plan_direct(d, false, share, p);
   });
 }
 
-bool plan_direct_copies(const surgeon_layer_desc& d, DirectParams* out) { return compute_plan_direct(d, false, out); }
+bool plan_direct_copies(const surgeon_layer_desc& d, DirectParams* out) { return compute_plan_direct(d, false, false, out); }
 
 size_t direct_grad_bf16_bytes(const DirectParams& p) {
   const size_t b = p.tg ? static_cast<size_t>(p.imgs) * p.oh * p.ow * p.o_real * 2

@@ -126,6 +126,25 @@ def test_small_reductions_on_narrow_column_tiles(layer, ratio):
         assert rel_frobenius(dw, ref) <= 5e-3
 
 
+@pytest.mark.parametrize("layer", [
+    W.linear("few_rows", 200, 320, 320), W.linear("ragged", 1333, 136, 200), W.conv("one_map", 1, 132, 16, 500, 1, 1, 0),
+    W.conv("taps_part", 2, 20, 8, 48, 3), W.conv("s2", 2, 20, 14, 24, 3, 2)], ids=lambda l: l.name)
+def test_layers_cut_into_fewer_parts(layer):
+    """SURGEON_SHARE_GPU: other splits than the default's, in the scratch that the query asks for."""
+    a, g = W.activation(layer, 5), W.grad_out(layer, 5)
+    comp, ref = assert_store_equals_oracle(a, 0.5)
+    d = B.layer_desc(layer, B.PATH_TENSOR_CORE)
+    ws = torch.empty(B.surgeon_weight_grad_workspace(d), dtype=torch.uint8, device="cuda")
+    dense = oracle.decompress(ref["bitmap"], ref["values"], a.numel())
+    exp = oracle_dw(layer, dense.view(np.uint16) if layer.dt == W.BF16 else dense, g.numpy())
+    for flags in (B.SURGEON_SHARE_GPU, 0):
+        dw = B.surgeon_weight_grad(comp, d, g.cuda(), workspace=ws, flags=flags).cpu().numpy()
+        assert rel_frobenius(dw, exp) <= 5e-3
+    with pytest.raises(B.SurgeonError) as e:
+        B.surgeon_weight_grad(comp, d, g.cuda(), workspace=ws, flags=B.SURGEON_STORE_DROP_ZEROS)
+    assert e.value.status == B.SURGEON_ERR_INVALID_ARG
+
+
 # prune: whole chunks and one element around them, resident and streamed ranges (a CTA's range is resident up to 48
 # chunks of 4 KB), counts in global memory (beyond 512 chunks per CTA on 148 SMs)
 @pytest.mark.parametrize("bf16", [False, True])
