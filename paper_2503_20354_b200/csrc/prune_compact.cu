@@ -57,7 +57,7 @@ constexpr int kChunkBytes = 4096;
 constexpr int kRingBytes = kWarps * kSlotsPerWarp * kChunkBytes;
 constexpr int kResidentChunks = kWarps * kSlotsPerWarp;
 // The rest of the shared memory.  Slots: the listed keys, room for 1/16 of every chunk.
-constexpr int kMaxLocalChunks = 512;             // per-chunk counts in shared memory up to here
+constexpr int kMaxLocalChunks = 1024;            // per-chunk counts in shared memory up to here
 constexpr int kSlotBytes = 256;
 constexpr int kAuxSlots = 8192;                  // (histograms before it)
 constexpr int kAuxCnt = kAuxSlots + kResidentChunks * kSlotBytes;
@@ -83,7 +83,7 @@ struct PruneArgs {
   uint32_t k;
   int n_chunks;                  // chunks in all
   int drop_zeros, stall;
-  int spread;                    // the counts do not fit shared memory: the second pass is dealt out chunk by chunk
+  int spread;                    // the chunks are claimed, and the counts are in global memory
   unsigned long long token;      // unlike any other call's
   surgeon_header* hdr;
   uint32_t* bitmap;
@@ -94,7 +94,7 @@ struct PruneArgs {
   uint32_t* keys;                // [kSelMaxCtas][kMaxKeys]
   uint32_t* hist;                // [kSelHists][kSelBins]
   uint32_t* claims;              // [kSelPhases][kClaimSets], kClaimStride words apart: groups claimed in each pass
-  uint32_t* cnt;                 // per chunk (used when a CTA has more than kMaxLocalChunks)
+  uint32_t* cnt;                 // per chunk (spread)
   unsigned long long* prefix;    // likewise
   void* slots;                   // per chunk, listed keys of ranges that are not resident
 };
@@ -1663,7 +1663,7 @@ cudaError_t run_prune_compact(const void* x, long long n, long long k, int drop_
   // the smallest grid that keeps the tensor on chip, and of a tensor that no quarter of the SMs can hold a
   // quarter: four such grids fit exactly (of grids that leave a rest a fifth starts in part and spins).
   // Whole stacks on eight streams, full grid / SMs / 2, / 3, / 4: ViT 2.46 / 1.70 / 1.57 / 1.61 ms, WideResNet
-  // 1.53 / 1.14 / 1.08 / 1.00, ResNet-50 1.68 / 1.28 / 1.09 / 1.04, ResNeXt 1.93 / 1.46 / 1.36 / 1.31.
+  // 1.53 / 1.14 / 1.08 / 0.96, ResNet-50 1.68 / 1.28 / 1.09 / 1.02, ResNeXt 1.93 / 1.46 / 1.36 / 1.24.
   const int sms = sm_count() < kSelMaxCtas ? sm_count() : kSelMaxCtas;
   int grid;
   if (share) {
@@ -1673,7 +1673,9 @@ cudaError_t run_prune_compact(const void* x, long long n, long long k, int drop_
     const int per_cta = (a.n_chunks + sms * kWarps - 1) / (sms * kWarps) * kWarps;
     grid = (a.n_chunks + per_cta - 1) / per_cta;
   }
-  a.spread = a.n_chunks > grid * kMaxLocalChunks ? 1 : 0;
+  // claimed chunks (see the kernel): by itself from 512 chunks per CTA on, where equal shares end unevenly; on a part
+  // of the GPU only where the counts do not fit (on a quarter, 131 MB: 335 -> 310 us bf16, 260 -> 238 fp32)
+  a.spread = a.n_chunks > grid * (share ? kMaxLocalChunks : 512) ? 1 : 0;
   const bool resident = (a.n_chunks + grid - 1) / grid <= kResidentChunks;
   const void* kernel = resident ? reinterpret_cast<const void*>(prune_kernel<DT, true>)
                                 : reinterpret_cast<const void*>(prune_kernel<DT, false>);

@@ -173,10 +173,10 @@ def test_partial_last_row_of_a_streamed_tensor(chunks, extra, share, bf16):
 
 
 @pytest.mark.parametrize("bf16", [False, True])
-@pytest.mark.parametrize("chunks,extra", [(1, -1), (49, 0), (48 * 37, 0), (48 * 37, 1), (512 * 37 + 1, 3)])
+@pytest.mark.parametrize("chunks,extra", [(1, -1), (49, 0), (48 * 37, 0), (48 * 37, 1), (1024 * 37, 0), (1024 * 37 + 1, 3)])
 def test_prune_on_a_part_of_the_gpu(chunks, extra, bf16):
     """SURGEON_SHARE_GPU, asked for or implied by a stream that is not the current one: at most a quarter of the
-    SMs, resident up to 48 chunks a CTA, counts in global memory beyond 512."""
+    SMs, resident up to 48 chunks a CTA, counts in global memory beyond 1024."""
     n = chunks * (2048 if bf16 else 1024) + extra
     x = W.draw("relu_normal", n, seed=4, device="cuda").cpu()
     x = x.to(torch.bfloat16) if bf16 else x
