@@ -7,12 +7,17 @@
 // fp32 in a fixed order, and the chunk sums are added in double in a fixed order by a second
 // kernel, so the result is reproducible and stays within ~3e-6 relative error of exact arithmetic.
 //
-// Bound by the FMA pipes.  A CTA of 128 threads owns 64 x 128 outputs (8 x 8 per thread, packed
-// two to an instruction) and works in K-tiles of 32: every thread rebuilds the 32 positions of one
+// A CTA of 128 threads owns 64 x 128 outputs (8 x 8 per thread, packed two to an instruction) and
+// works in K-tiles of 32 positions of one or more images: every thread rebuilds the 32 positions of one
 // column - one rank computation per row of the map, then a bit test and a predicated load per
-// element - and four CTAs per SM hide the latency of that behind one another's products.
+// element, or a rank per element where rows are shorter than four - and four CTAs per SM hide the
+// latency of that behind one another's products.
 // Measured on 320 -> 320 channels, 3x3 on 16x16, batch 16 (7.5 GFLOP): 1084 us with a rank
-// computation per element and 4 x 4 outputs per thread, 264 us now (28.6 TFLOP/s).
+// computation per element and 4 x 4 outputs per thread, 264 us now: 28.6 TFLOP/s, 38 % of what the
+// FMA pipes could do, since rebuilding and products take turns.  Small maps (128 -> 128 channels on
+// 1x1, 200 000 images: 0.42 ms) and linear layers (4096 rows, 320 -> 320: 70 us) by elements.
+#include <type_traits>
+
 #include "surgeon_internal.cuh"
 
 namespace surgeon {
@@ -27,9 +32,12 @@ constexpr int kGPitch = TM + 4, kAPitch = TN + 4;
 
 struct Geom {
   int kind, B, C, H, W, O, KH, KW, stride, pad, OH, OW;
-  int P, tiles_per_img;  // positions per image (linear: rows), K-tiles per image
+  int P;                 // positions per image (linear: rows)
+  int by_element;        // conv: stretches of a row too short to be worth a rank computation each
   int k_tiles, per_chunk, chunks;
-  long long M, N;        // GEMM extents
+  int tiles_per_img;     // 0: K-tiles run over the images
+  int K;                 // what the GEMM sums over
+  long long M, N;        // its other extents
   long long n_words;
 };
 
@@ -40,8 +48,16 @@ Geom make_geom(const surgeon_layer_desc& d) {
   g.OH = (d.h + 2 * d.pad - d.kh) / d.stride + 1;
   g.OW = (d.w + 2 * d.pad - d.kw) / d.stride + 1;
   g.P = d.kind == 1 ? g.OH * g.OW : d.batch;
-  g.tiles_per_img = (g.P + TK - 1) / TK;
-  g.k_tiles = g.B * g.tiles_per_img;
+  g.by_element = g.OW < 4 || 63 / d.stride + 1 < 4;
+  // A K-tile stays inside an image, whose last one is partly used, unless that would leave more than a fifth of K
+  // unused (or K beyond what the grid takes): 49 positions 772 -> 730 us, one position 5.7 -> 0.42 ms; at 196
+  // positions (12 % unused) tiles over images cost 95 -> 100 us.
+  const long long padded = (static_cast<long long>(g.P) + TK - 1) / TK * TK;
+  const bool inside = 4 * padded <= 5LL * g.P && g.B * padded <= 65535LL * kMaxTiles * TK;
+  g.tiles_per_img = inside ? static_cast<int>(padded / TK) : 0;
+  const long long k_all = inside ? g.B * padded : static_cast<long long>(g.B) * g.P;
+  g.k_tiles = static_cast<int>((k_all + TK - 1) / TK);
+  g.K = static_cast<int>(k_all);
   g.M = d.c_out;
   g.N = static_cast<long long>(d.c_in) * d.kh * d.kw;
   g.n_words = (static_cast<long long>(d.batch) * d.c_in * d.h * d.w + 31) / 32;
@@ -50,9 +66,10 @@ Geom make_geom(const surgeon_layer_desc& d) {
   const long long tiles = ((g.M + TM - 1) / TM) * ((g.N + TN - 1) / TN);
   const long long slots = static_cast<long long>(kCtasPerSm) * sm_count();
   double best = 1e300;
-  g.per_chunk = 1;
+  g.per_chunk = kMaxTiles;
   for (int per = 1; per <= kMaxTiles; ++per) {
     const long long chunks = (g.k_tiles + per - 1) / per;
+    if (chunks > 65535) continue;                // (blockIdx.z)
     const long long waves = (tiles * chunks + slots - 1) / slots;
     const double cost = static_cast<double>(waves) * (per + 2.0);
     if (cost <= best) { best = cost; g.per_chunk = per; }
@@ -67,6 +84,40 @@ __device__ __forceinline__ float packed_value(const void* __restrict__ values, u
   if (DT == 0) return on ? __ldg(reinterpret_cast<const float*>(values) + idx) : 0.0f;
   const uint32_t h = on ? static_cast<uint32_t>(__ldg(reinterpret_cast<const unsigned short*>(values) + idx)) : 0u;
   return __uint_as_float(h << 16);
+}
+
+// The elements at flat indices j[i] (negative: zero).  First the words of all, then the values of all.
+template <int DT, int N>
+__device__ __forceinline__ void element_values(const uint32_t* __restrict__ bitmap, const void* __restrict__ values,
+                                               const uint32_t* __restrict__ offsets, uint32_t n_words,
+                                               const int (&j)[N], float (&v)[N]) {
+  static_assert(kBlockWords == 4, "a block's words are one vector");
+  uint4 q[N];
+  uint32_t idx[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const uint32_t blk = static_cast<uint32_t>(j[i]) >> kBlockShift, w0 = blk * kBlockWords;
+    q[i] = make_uint4(0, 0, 0, 0);
+    idx[i] = 0;
+    if (j[i] >= 0) {
+      idx[i] = __ldg(offsets + blk);
+      if (w0 + 4 <= n_words) {
+        q[i] = __ldg(reinterpret_cast<const uint4*>(bitmap) + blk);
+      } else {                                     // the last, partial block
+        q[i].x = __ldg(bitmap + w0);
+        q[i].y = w0 + 1 < n_words ? __ldg(bitmap + w0 + 1) : 0u;
+        q[i].z = w0 + 2 < n_words ? __ldg(bitmap + w0 + 2) : 0u;
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const uint32_t wq = (static_cast<uint32_t>(j[i]) >> 5) & 3u, bit = static_cast<uint32_t>(j[i]) & 31u;
+    const uint32_t w = wq == 0 ? q[i].x : (wq == 1 ? q[i].y : (wq == 2 ? q[i].z : q[i].w));
+    idx[i] += (wq > 0 ? __popc(q[i].x) : 0) + (wq > 1 ? __popc(q[i].y) : 0) + (wq > 2 ? __popc(q[i].z) : 0) +
+              __popc(w & ((1u << bit) - 1u));
+    v[i] = packed_value<DT>(values, idx[i], ((w >> bit) & 1u) != 0u);
+  }
 }
 
 // 64 bitmap bits from flat index j on, and the number of kept elements before j.
@@ -97,7 +148,9 @@ __device__ __forceinline__ unsigned long long twice(float v) {
   return r;
 }
 
-template <int DT, int KIND>
+// KIND: 0 linear, 1 convolution by stretches of a row, 2 convolution by elements (Geom::by_element).
+// SPAN: K-tiles run over the images (Geom::tiles_per_img is 0).
+template <int DT, int KIND, bool SPAN>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 dw_fp32_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ values,
                const uint32_t* __restrict__ offsets, const float* __restrict__ grad,
@@ -113,7 +166,7 @@ dw_fp32_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ val
   const long long col = n0 + tid;
   const bool col_ok = col < g.N;
   int c = 0, r = 0, s = 0;
-  if (KIND == 1 && col_ok) {
+  if (KIND != 0 && col_ok) {
     const int RS = g.KH * g.KW;
     c = static_cast<int>(col / RS);
     const int rs = static_cast<int>(col - static_cast<long long>(c) * RS);
@@ -127,14 +180,16 @@ dw_fp32_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ val
 #pragma unroll
     for (int b = 0; b < 4; ++b) acc[a][b] = 0ull;
   const int ty = tid >> 4, tx = tid & 15;
-  const bool vec4 = (g.P & 3) == 0;                // gradient rows readable with 16-byte loads
+  const bool vec4 = (g.P & 3) == 0;                // four positions from a multiple of 4 on: one image, 16 bytes
 
   for (int kt = kt_begin; kt < kt_end; ++kt) {
-    const int img = KIND == 1 ? kt / g.tiles_per_img : 0;
-    const int p0 = (kt - img * g.tiles_per_img) * TK;
-    const int n_pos = min(TK, g.P - p0);
+    // the tile's first position: its image and its place there
+    int img = KIND == 0 ? 0 : (SPAN ? kt * TK / g.P : kt / g.tiles_per_img);
+    const int p0 = SPAN ? kt * TK - img * g.P : (kt - img * g.tiles_per_img) * TK;
+    const int n_pos = min(TK, SPAN ? g.K - kt * TK : g.P - p0);
+    const int n_used = KIND == 1 ? TK : (n_pos + 7) & ~7;      // rows of the tiles that the products read
     // ---- the gradient tile, transposed ----
-    if (KIND == 1) {                               // [b][m][position]
+    if (KIND != 0) {                               // [b][m][position]
       const int mm = tid >> 1, half = tid & 1;
       const float* src = grad + (static_cast<long long>(img) * g.O + m0 + mm) * g.P + p0;
       const bool ok = m0 + mm < g.M;
@@ -142,7 +197,22 @@ dw_fp32_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ val
       for (int i = 0; i < 4; ++i) {                // (the two threads of a row alternate: no bank conflicts)
         const int k = 8 * i + 4 * half;
         float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (ok) {
+        if (SPAN && ok && k < n_pos) {
+          int p = (p0 + k) % g.P;
+          const float* at = src - p0 + static_cast<long long>((p0 + k) / g.P) * g.O * g.P + p;
+          if (vec4) {                              // (n_pos is a multiple of 4 as well)
+            v = __ldg(reinterpret_cast<const float4*>(at));
+          } else {
+            float* f = reinterpret_cast<float*>(&v);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              if (k + e < n_pos) f[e] = __ldg(at);
+              ++at;
+              if (++p == g.P) { p = 0; at += (g.O - 1LL) * g.P; }
+            }
+          }
+        }
+        if (!SPAN && ok) {
           if (vec4 && k + 4 <= n_pos) {
             v = __ldg(reinterpret_cast<const float4*>(src + k));
           } else {
@@ -165,9 +235,9 @@ dw_fp32_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ val
     // ---- this thread's column of the activation tile ----
     if (KIND == 1) {
       int y = p0 / g.OW, x = p0 - y * g.OW;
-      for (int k = 0; k < TK;) {
+      for (int k = 0; k < n_used;) {
         // a piece: positions of one output row, at most 64 input elements wide
-        int len = TK - k;
+        int len = n_used - k;
         uint32_t rank = 0;
         unsigned long long win = 0;
         if (k < n_pos) {
@@ -186,7 +256,7 @@ dw_fp32_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ val
             win <<= skip * g.stride;
           }
         }
-        const unsigned long long step_mask = (1ull << g.stride) - 1ull;
+        const unsigned long long step_mask = (1ull << g.stride) - 1ull;    // (stride at most 21: see by_element)
         for (int e0 = 0; e0 < len; e0 += 8) {
           float v[8];
 #pragma unroll
@@ -201,28 +271,44 @@ dw_fp32_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ val
         }
         k += len;
         x += len;
-        if (x >= g.OW) { x = 0; ++y; }
+        if (x >= g.OW) {
+          x = 0;
+          ++y;
+          if (SPAN && y == g.OH) { y = 0; ++img; }
+        }
       }
     } else {
-#pragma unroll 4
-      for (int k = 0; k < TK; ++k) {
-        float v = 0.0f;
-        if (k < n_pos && col_ok) {
-          const long long j = static_cast<long long>(p0 + k) * g.C + col;
-          const long long wi = j >> 5, blk = j >> kBlockShift;
-          const uint32_t w = __ldg(bitmap + wi), bit = static_cast<uint32_t>(j & 31);
-          if ((w >> bit) & 1u) {
-            uint32_t idx = __ldg(offsets + blk) + __popc(w & ((1u << bit) - 1u));
-            for (long long t = blk * kBlockWords; t < wi; ++t) idx += __popc(__ldg(bitmap + t));
-            v = packed_value<DT>(values, idx, true);
+      int y = 0, x = 0;
+      if (KIND == 2) { y = p0 / g.OW; x = p0 - y * g.OW; }
+      constexpr int kAtOnce = 8;
+#pragma unroll 1
+      for (int k = 0; k < n_used; k += kAtOnce) {
+        int j[kAtOnce];
+        float v[kAtOnce];
+#pragma unroll
+        for (int e = 0; e < kAtOnce; ++e) {
+          j[e] = -1;
+          if (KIND == 0) {
+            if (k + e < n_pos && col_ok) j[e] = (p0 + k + e) * g.C + static_cast<int>(col);
+          } else {
+            const int iy = y * g.stride + r - g.pad, ix = x * g.stride + s - g.pad;
+            if (k + e < n_pos && col_ok && iy >= 0 && iy < g.H && ix >= 0 && ix < g.W)
+              j[e] = ((img * g.C + c) * g.H + iy) * g.W + ix;
+            if (++x == g.OW) {
+              x = 0;
+              ++y;
+              if (SPAN && y == g.OH) { y = 0; ++img; }
+            }
           }
         }
-        As[k][tid] = v;
+        element_values<DT>(bitmap, values, offsets, static_cast<uint32_t>(g.n_words), j, v);
+#pragma unroll
+        for (int e = 0; e < kAtOnce; ++e) As[k + e][tid] = v[e];
       }
     }
     __syncthreads();
 #pragma unroll 8
-    for (int kk = 0; kk < TK; ++kk) {
+    for (int kk = 0; kk < n_used; ++kk) {          // (a multiple of 8)
       const ulonglong2 a0 = *reinterpret_cast<const ulonglong2*>(&As[kk][tx * 4]);
       const ulonglong2 a1 = *reinterpret_cast<const ulonglong2*>(&As[kk][TN / 2 + tx * 4]);
       const float4 g0 = *reinterpret_cast<const float4*>(&Gs[kk][ty * 8]);
@@ -285,8 +371,17 @@ cudaError_t launch_weight_grad_fp32(const surgeon_compressed& act, const surgeon
     auto launch = [&](auto kernel) {
       kernel<<<grid, kThreads, 0, stream>>>(act.bitmap, act.values, act.block_offsets, grad_out, partial, g);
     };
-    if (d.kind == 1) act.dt == 0 ? launch(dw_fp32_kernel<0, 1>) : launch(dw_fp32_kernel<1, 1>);
-    else act.dt == 0 ? launch(dw_fp32_kernel<0, 0>) : launch(dw_fp32_kernel<1, 0>);
+    auto launch_kind = [&](auto kind, auto span) {
+      act.dt == 0 ? launch(dw_fp32_kernel<0, decltype(kind)::value, decltype(span)::value>)
+                  : launch(dw_fp32_kernel<1, decltype(kind)::value, decltype(span)::value>);
+    };
+    using std::integral_constant;
+    const bool span = g.tiles_per_img == 0;
+    if (d.kind != 1) launch_kind(integral_constant<int, 0>{}, std::false_type{});
+    else if (g.by_element) span ? launch_kind(integral_constant<int, 2>{}, std::true_type{})
+                                : launch_kind(integral_constant<int, 2>{}, std::false_type{});
+    else span ? launch_kind(integral_constant<int, 1>{}, std::true_type{})
+              : launch_kind(integral_constant<int, 1>{}, std::false_type{});
     note_launches(1);
   }
   const long long mn = g.M * g.N;

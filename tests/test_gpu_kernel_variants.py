@@ -92,6 +92,20 @@ def test_fp32_tiles(layer):
     assert rel_frobenius(dw, ref) <= 1e-5
 
 
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("layer", [
+    W.conv("map1", 70, 40, 1, 65, 1, 1, 0), W.conv("map2", 37, 33, 2, 20, 1, 1, 0), W.conv("map2_2x2", 75, 20, 2, 24, 2, 1, 0),
+    W.conv("map3", 15, 20, 3, 66, 3), W.Layer("rows_of_3", 1, 5, 9, 8, 3, 130, 3, 3, 1, 1), W.conv("map7", 5, 20, 7, 24, 3),
+    W.Layer("rows_of_4", 1, 7, 9, 5, 4, 20, 3, 3, 1, 1), W.conv("map9", 3, 10, 9, 70, 3, 2), W.conv("one_output", 45, 12, 5, 24, 5, 1, 0),
+    W.conv("stride21", 2, 6, 90, 9, 3, 21), W.conv("stride22", 2, 6, 90, 9, 3, 22), W.conv("stride64", 3, 4, 130, 9, 2, 64, 1),
+    W.conv("stride70", 2, 3, 211, 8, 70, 70, 0), W.linear("ragged", 61, 77, 70, dt=W.F32), W.linear("rows8", 8, 200, 9, dt=W.F32)],
+    ids=lambda l: l.name)
+def test_fp32_tiles_over_images(layer, bf16):
+    """K-tiles that end inside an image, hold several, or are partly used; columns by rows of the map and by elements."""
+    dw, ref = _dw(replace(layer, dt=W.BF16 if bf16 else W.F32), 0.5, B.PATH_FP32)
+    assert rel_frobenius(dw, ref) <= 1e-5
+
+
 @pytest.mark.parametrize("batch,c_in,c_out,k", [(256, 16, 20, 1), (300, 64, 64, 1), (64, 7, 9, 1), (64, 20, 20, 3)])
 def test_reductions_of_small_weights(batch, c_in, c_out, k):
     layer = W.conv("r", batch, c_in, 8, c_out, k)
