@@ -647,6 +647,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     } else {
       for (int v = lane; v < kChunkBytes / 16; v += 32)
         *reinterpret_cast<uint4*>(region + v * 16) = make_uint4(0, 0, 0, 0);
+      tc::fence_proxy_async();                   // (these stores precede the next TMA fill of the place)
       __syncwarp();
     }
     if (row0 + 32 > a.n_rows_full && a.n > a.n_rows_full * EPR) {
@@ -656,12 +657,11 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
         *reinterpret_cast<E*>(region + r * 128 + (((byte >> 4) ^ (r & 7)) << 4) + (byte & 15)) =
             x[a.n_rows_full * EPR + e];
       }
+      tc::fence_proxy_async();
       __syncwarp();
     }
     return true;
   };
-  // True where arrived() writes to the chunk's place itself: its last rows, or the zeros of a chunk without a whole row.
-  auto completed = [&](int c) { return static_cast<long long>(c) * 32 + 32 > a.n_rows_full; };
   // The warp's chunks of one pass in the order of their loads: next() is the next one, or n_chunks.
   static_assert(kSlotsPerWarp == 3, "three loads in flight");
   int fly0 = a.n_chunks, fly1 = a.n_chunks, fly2 = a.n_chunks;    // chunks in flight, the oldest first
@@ -705,7 +705,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     for (int s = 0; fly0 < a.n_chunks; s = s == 2 ? 0 : s + 1) {
       unsigned char* region = my_ring + s * kChunkBytes;
       if (!arrived(fly0, s)) { give_up(s); break; }
-      const bool written = f(fly0, region) || completed(fly0);
+      const bool written = f(fly0, region);
       fly0 = fly1; fly1 = fly2;
       int c = next();
       if (c < a.n_chunks) {
@@ -1488,7 +1488,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
         for (int j = i - 1; j >= 0 && j > i - kSlotsPerWarp; --j) arrived(chunk_of(j), j % kSlotsPerWarp);
         break;
       }
-      const bool written = emit(chunk_of(i), my_ring + sl * kChunkBytes) || completed(chunk_of(i));
+      const bool written = emit(chunk_of(i), my_ring + sl * kChunkBytes);
       if (i >= kSlotsPerWarp) {
         if (written) tc::fence_proxy_async();
         __syncwarp();
