@@ -666,6 +666,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
   static_assert(kSlotsPerWarp == 3, "three loads in flight");
   int fly0 = a.n_chunks, fly1 = a.n_chunks, fly2 = a.n_chunks;    // chunks in flight, the oldest first
   int at_i = 0, claim = 0, pass = 0;             // (not spread) index of the next one; (spread) the claimed group; passes begun
+  uint32_t ahead = 0;                            // (lane 0) the group claimed one chunk ahead
   auto next = [&]() -> int {
     if (!spread) return at_i < n_mine ? chunk_of(at_i++) : a.n_chunks;
     if ((at_i & 3) == 0) {
@@ -673,11 +674,12 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
       const int n_sets = min(kClaimSets, G), set = static_cast<int>(blockIdx.x) * n_sets / G;
       const int set_begin = (set * G + n_sets - 1) / n_sets, set_end = ((set + 1) * G + n_sets - 1) / n_sets;
       uint32_t g = (blockIdx.x - set_begin) * kWarps + warp;
-      if (at_i > 0) {
-        if (lane == 0) g = (set_end - set_begin) * kWarps + atomicAdd(&a.claims[(pass * kClaimSets + set) * kClaimStride], 1u);
-        g = __shfl_sync(kFull, g, 0);
-      }
+      if (at_i > 0) g = (set_end - set_begin) * kWarps + __shfl_sync(kFull, ahead, 0);
       claim = static_cast<int>(min(4u * (g * n_sets + set), static_cast<uint32_t>(a.n_chunks)));
+    }
+    if ((at_i & 3) == 3 && lane == 0) {          // the round trip hides behind a chunk
+      const int set = static_cast<int>(blockIdx.x) * min(kClaimSets, G) / G;
+      ahead = atomicAdd(&a.claims[(pass * kClaimSets + set) * kClaimStride], 1u);
     }
     const int c = claim + (at_i++ & 3);
     return c < a.n_chunks ? c : a.n_chunks;
