@@ -935,7 +935,7 @@ static size_t direct_partial_bytes(const DirectParams& p) {
   return (b + 255) & ~static_cast<size_t>(255);
 }
 
-size_t weight_grad_tc_workspace(const surgeon_layer_desc& d) {
+static size_t plan_workspace(const surgeon_layer_desc& d) {
   SwapParams sp;
   if (plan_swap(d, &sp)) return kStatusBytes + swap_partial_bytes(sp) + direct_grad_bf16_bytes(sp.d);
   DirectParams dp;
@@ -953,6 +953,13 @@ size_t weight_grad_tc_workspace(const surgeon_layer_desc& d) {
            im2col_grad_bytes(p, pitch);
   if (!plan(d, 0, &p)) return 0;
   return kStatusBytes + static_cast<size_t>(p.splits) * p.O * p.n_gemm * sizeof(float);
+}
+
+// (asked for twice by every call: one look-up instead of one per kind of plan)
+size_t weight_grad_tc_workspace(const surgeon_layer_desc& d) {
+  struct Tag {};
+  size_t bytes = 0;
+  return memo_plan<Tag>(d, 0, &bytes, [&](size_t* b) { return (*b = plan_workspace(d)) != 0; }) ? bytes : 0;
 }
 
 cudaError_t launch_weight_grad_tc(const surgeon_compressed& act, const surgeon_layer_desc& d,

@@ -16,7 +16,7 @@ namespace surgeon {
 template <typename Tag, typename P, typename F>
 inline bool memo_plan(const surgeon_layer_desc& d, int extra, P* out, F compute) {
   struct Entry { surgeon_layer_desc d; int extra, dev; bool used, ok; P p; };
-  constexpr int kEntries = 64;
+  constexpr int kEntries = 128;                  // (a layer has up to two plans)
   thread_local Entry table[kEntries] = {};
   thread_local int next = 0;
   int dev = 0;
