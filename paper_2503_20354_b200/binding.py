@@ -316,7 +316,7 @@ def surgeon_prune_compact(x: torch.Tensor, ratio: float, out: Optional[Compresse
     if workspace is None:
         workspace = _scratch(surgeon_compact_sizes(n, dt, ratio).workspace_bytes, x.device, stream)
     at = _stream_ptr(stream)
-    if stream is not None and at != _stream_ptr(None):
+    if stream is not None and at != torch._C._cuda_getCurrentRawStream(stream.device_index):
         flags |= SURGEON_SHARE_GPU
     st = lib().surgeon_prune_compact_flags(x.data_ptr(), n, dt, ratio, int(flags), C.byref(out.c),
                                            workspace.data_ptr(),
