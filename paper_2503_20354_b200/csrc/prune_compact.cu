@@ -34,6 +34,7 @@
 #include <atomic>
 #include <chrono>
 #include <random>
+#include <type_traits>
 
 #include "surgeon_internal.cuh"
 #include "tc_common.cuh"
@@ -56,26 +57,36 @@ constexpr int kSlotsPerWarp = 3;                 // chunks in flight per warp: 1
 constexpr int kChunkBytes = 4096;
 constexpr int kRingBytes = kWarps * kSlotsPerWarp * kChunkBytes;
 constexpr int kResidentChunks = kWarps * kSlotsPerWarp;
-// The rest of the shared memory.  Slots: the listed keys, room for 1/16 of every chunk.
+// The rest of the shared memory: 32 KB, all of it the sample's bins first.
 constexpr int kMaxLocalChunks = 1024;            // per-chunk counts in shared memory up to here
-constexpr int kSlotBytes = 256;
-constexpr int kAuxSlots = 8192;                  // (histograms before it)
-constexpr int kAuxCnt = kAuxSlots + kResidentChunks * kSlotBytes;
-constexpr int kAuxPrefix = kAuxCnt + kMaxLocalChunks * 4;
 constexpr int kSampleBinsLog2 = 14;              // top 14 key bits: 64 bins per octave; 16-bit counters here
-constexpr int kSampleBytes = 2 << kSampleBinsLog2;
+constexpr int kAuxBytes = 2 << kSampleBinsLog2;
 static_assert((1 << kSampleBinsLog2) == kSampleBins, "bins of the sample");
-constexpr int kAuxBytes = kAuxPrefix + kMaxLocalChunks * 8 > kSampleBytes ? kAuxPrefix + kMaxLocalChunks * 8 : kSampleBytes;
-// emit: per-warp staging of the kept values of a sparse chunk, in the place of histogram and slots
-constexpr int kStageBytes = (kAuxCnt / kWarps) & ~15;
+constexpr int kAuxSlots = 8192;                  // (histograms before it)
+// A resident range: the listed keys of a chunk have a slot of their own, 12 % of its elements.
+constexpr int kResSlotBytes = 496;
+constexpr int kResCnt = kAuxSlots + kResidentChunks * kResSlotBytes;
+constexpr int kResPrefix = kResCnt + kResidentChunks * 4;
+static_assert(kResPrefix % 8 == 0 && kResPrefix + kResidentChunks * 8 <= kAuxBytes, "shared memory of a resident range");
+// Others: a staging slot per warp (room for 1/16 of a chunk), and one list of the keys of all chunks, each chunk's
+// in one piece.  What does not fit there goes to the chunk's slot in global memory.  The places take the list's room when
+// it is done with.
+constexpr int kSlotBytes = 256;
+constexpr int kListStart = kAuxSlots + kWarps * kSlotBytes;          // where a chunk's keys begin, 16 bits
+constexpr int kListAcc = kListStart + kMaxLocalChunks * 2;           // its count above the bin, 16 bits
+constexpr int kList = kListAcc + kMaxLocalChunks * 2;
+constexpr int kListBytes = 12288;
+// Counts and places of the chunks that there are lie at the end.
+static_assert(kList + kListBytes + kMaxLocalChunks * 4 <= kAuxBytes, "shared memory of a streamed range");
 constexpr size_t kPruneSmem = static_cast<size_t>(kRingBytes) + kAuxBytes + 1024;
 static_assert(kChunkBytes == kTileVecs * 16, "chunk size");
 // A streamed tensor's bracket comes from order statistics 2.5 sqrt(G) + 1 places to either side of the middle of G
 // CTAs' answers: with fewer than 31 CTAs there are none, and every key would be a candidate.
 constexpr int kLeastStreamedCtas = 31;
-constexpr int kMaxKeys = 64;                     // keys one CTA reports at the last exchange
-constexpr int kKeysPerThread = 8;                // and CTA 0 takes in
-constexpr int kKeysAtOnce = kKeysPerThread * kThreads;
+constexpr int kMaxKeys = 64;                     // keys one CTA reports at the last exchange, where the scratch has room
+constexpr uint32_t kKeysAtOnce = 960;            // and CTA 0 takes in, two threads per CTA
+static_assert(2 * kSelMaxCtas <= kThreads && kSelMaxCtas <= 256 &&
+              4 * (kSelBins + kKeysAtOnce + kSelMaxCtas) + kKeysAtOnce <= kAuxSlots, "room of the keys at CTA 0");
 
 struct PruneArgs {
   const void* x;
@@ -83,7 +94,6 @@ struct PruneArgs {
   uint32_t k;
   int n_chunks;                  // chunks in all
   int drop_zeros, stall;
-  int spread;                    // the chunks are claimed, and the counts are in global memory
   unsigned long long token;      // unlike any other call's
   surgeon_header* hdr;
   uint32_t* bitmap;
@@ -91,10 +101,10 @@ struct PruneArgs {
   uint32_t* offsets;
   ulonglong2* arrive;            // [kSelPhases][kSelMaxCtas]: {token, what the CTA reports}
   ulonglong2* answer;            // [kSelPhases][kSelMaxCtas + 2]: {token, what CTA 0 answers}
-  uint32_t* keys;                // [kSelMaxCtas][kMaxKeys]
+  unsigned long long* keys;      // [CTAs][key_room()]: {half a token, key}
   uint32_t* hist;                // [kSelHists][kSelBins]
   uint32_t* claims;              // [kSelPhases][kClaimSets], kClaimStride words apart: groups claimed in each pass
-  uint32_t* cnt;                 // per chunk (spread)
+  uint32_t* cnt;                 // per chunk (kClaimed)
   unsigned long long* prefix;    // likewise
   void* slots;                   // per chunk, listed keys of ranges that are not resident
 };
@@ -108,11 +118,16 @@ __device__ __forceinline__ uint32_t hash_u32(uint32_t v) {
 // A CTA reports by storing {token, 8 bytes} in its own word of the phase; CTA 0 polls these words,
 // one thread per CTA, and answers by storing {token, 8 bytes} in words that the others poll.  (Every
 // CTA polling the words of all others took 4-6 us on 148 SMs: the same L2 lines, 148 times over.)
-// No counter has to start at zero, so the call needs no memset: the token differs from call to
+// No word has to start at zero, so the call needs no memset: the token differs from call to
 // call.  For a captured graph, whose replays carry the same token, CTA 0 clears every report that it
-// has read, clears a phase's answers before it answers the phase before it, and clears the first
-// answer (phase 0) after the reports of phase 1; a CTA that gives up takes its own words back.  All CTAs are
-// resident (cooperative launch); polls are bounded.
+// has read, clears the answers of all phases before it gives the first one, and clears that one (phase 0)
+// after the reports of phase 1; a CTA takes its keys back when they have been read, and all its words when it gives up.
+// All CTAs are resident (cooperative launch); polls are bounded.
+//
+// No fence stands between a report and the answer: one waits for the stores before it, 0.3-0.5 us, and an exchange
+// used to have four of them in its chain.  Keys carry half the token each, so they are polled like the words; the
+// bins, which are added up by atomics, are complete when their sum is the sum of the counts in the words.  (148 CTAs:
+// words alone 1.3 us, with atomics behind fences 4.1; measured on exchanges alone.)
 __device__ __forceinline__ void word_store(ulonglong2* p, unsigned long long token, unsigned long long v) {
   asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}"
                ::"l"(p), "l"(token), "l"(v) : "memory");
@@ -123,6 +138,22 @@ __device__ __forceinline__ ulonglong2 word_load(const ulonglong2* p) {
                : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
   return v;
 }
+__device__ __forceinline__ void key_store(unsigned long long* p, unsigned long long token, uint32_t key) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"((token << 32) | key) : "memory");
+}
+// (not wanted: the token, and key 0)
+__device__ __forceinline__ unsigned long long key_load_if(const unsigned long long* p, bool wanted, unsigned long long token) {
+  unsigned long long v = token << 32;
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p ld.relaxed.gpu.global.u64 %0, [%1];\n\t}"
+               : "+l"(v) : "l"(p), "r"(static_cast<uint32_t>(wanted)) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint32_t count_load(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ int key_room(int ctas) { return min(kMaxKeys, kSelMaxCtas * kMaxKeys / 2 / ctas); }
 __device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 // One thread waits for a word of this call (what it announces apart from its own 8 bytes is visible
 // after a fence).  `stall` is the diagnostic of SURGEON_DEBUG_STALL_BARRIER: a value nobody ever
@@ -130,6 +161,7 @@ __device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" 
 __device__ __forceinline__ bool word_wait(const ulonglong2* p, unsigned long long token, unsigned long long* v,
                                           bool stall = false) {
   const uint32_t cap = stall ? 1024u : (1u << 22);
+#pragma unroll 1
   for (uint32_t spins = 0; spins <= cap; ++spins) {
     const ulonglong2 w = word_load(p);
     if (w.x == (stall ? ~token : token)) {
@@ -182,6 +214,43 @@ __device__ __forceinline__ uint32_t row_elem(const unsigned char* region, int e)
   const uint32_t lane = lane_id();
   const int byte = e * static_cast<int>(sizeof(E));
   return static_cast<uint32_t>(*reinterpret_cast<const E*>(region + lane * 128 + (((byte >> 4) ^ (lane & 7)) << 4) + (byte & 15)));
+}
+
+// put(which, value) for the elements of this lane's row whose bits are set; `which` = rank among them.  U elements of
+// each word per turn, so that their loads overlap: a turn is a chain of a bit search, a load and a store, 170 clocks.
+template <int DT, int WPL, int U, typename F>
+__device__ __forceinline__ void take_set(const unsigned char* region, const uint32_t (&word)[WPL], F put) {
+  using E = typename Elem<DT>::type;
+  const uint32_t lane = lane_id(), x = (lane & 7) << 4;
+  const unsigned char* row = region + lane * 128;
+  uint32_t m[WPL], at[WPL];
+#pragma unroll
+  for (int w = 0; w < WPL; ++w) {
+    m[w] = word[w];
+    at[w] = w ? __popc(word[0]) : 0u;
+  }
+#pragma unroll 1
+  while (m[0] | m[WPL - 1]) {
+    E val[WPL][U];
+    bool have[WPL][U];
+#pragma unroll
+    for (int w = 0; w < WPL; ++w) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        have[w][u] = m[w] != 0u;
+        const uint32_t e = 32 * w + (__clz(__brev(m[w])) & 31);      // (no bit left: some element of the row)
+        m[w] &= m[w] - 1u;
+        val[w][u] = *reinterpret_cast<const E*>(row + ((e * static_cast<uint32_t>(sizeof(E))) ^ x));
+      }
+    }
+#pragma unroll
+    for (int w = 0; w < WPL; ++w) {
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (have[w][u]) put(at[w] + u, val[w][u]);
+      at[w] += U;
+    }
+  }
 }
 
 // Masks of the elements with key >= t, bit e = element e, elements past nv cleared.  fp32 keys are
@@ -241,6 +310,22 @@ __device__ __noinline__ uint32_t one_key_of_chunk(const unsigned char* region, u
   return __reduce_add_sync(kFull, eq) == c_tot ? k0 : 0u;
 }
 
+// Keys of the chunk above t, and (upper half) equal to it.
+template <int DT>
+__device__ __noinline__ uint32_t count_chunk(const unsigned char* region, uint32_t t) {
+  constexpr int EPR = 128 / static_cast<int>(sizeof(typename Elem<DT>::type)), WPL = EPR / 32;
+  uint4 q[8];
+  load_row(region, q);
+  uint32_t m[WPL], ge = 0, gt = 0;               // (t >= 1: what lies past the tensor's end is below it)
+  mask_ge<DT, WPL>(q, EPR, t, m);
+#pragma unroll
+  for (int w = 0; w < WPL; ++w) ge += __popc(m[w]);
+  mask_ge<DT, WPL>(q, EPR, t + 1u, m);
+#pragma unroll
+  for (int w = 0; w < WPL; ++w) gt += __popc(m[w]);
+  return __reduce_add_sync(kFull, gt | ((ge - gt) << 16));
+}
+
 // Keep only the lowest `allowed` set bits of `m`.
 __device__ __forceinline__ uint32_t lowest_set_bits(uint32_t m, long long allowed) {
   if (allowed <= 0) return 0u;
@@ -262,12 +347,75 @@ __device__ __forceinline__ unsigned long long warp_incl_u64(unsigned long long v
   return v;
 }
 
+// The bits of a row in the one chunk inside which the tie quota ends: `above` and the first `allowed` ties of the chunk, which
+// are ranked by flat index (= lane, then bit).  Out of line, like all that one chunk of a tensor does: code that is not
+// in the instruction caches costs some 250 clocks per 128 bytes, and a call runs most of its code once.
+template <int DT>
+__device__ __noinline__ uint2 quota_words(const unsigned char* region, int nv, uint32_t tau, long long allowed, uint2 above) {
+  constexpr int WPL = 128 / static_cast<int>(sizeof(typename Elem<DT>::type)) / 32;
+  uint4 q[8];
+  load_row(region, q);
+  uint32_t word[2] = {above.x, above.y}, ge[WPL], ec = 0;
+  mask_ge<DT, WPL>(q, nv, tau, ge);
+#pragma unroll
+  for (int w = 0; w < WPL; ++w) { ge[w] &= ~word[w]; ec += __popc(ge[w]); }
+  allowed -= warp_excl_scan(ec);
+#pragma unroll
+  for (int w = 0; w < WPL; ++w) {
+    word[w] |= lowest_set_bits(ge[w], allowed);
+    allowed -= __popc(ge[w]);
+  }
+  return make_uint2(word[0], word[1]);
+}
+
+// The byte at address a of a packed sequence lives at a ^ ((a >> 5) & 0x7C): the 32-bit word
+// index is XORed with the index of its 128-byte row.  Without it, lanes that keep their whole
+// row (chunks before the end of a large tie quota, e.g. the zeros of post-ReLU data at a low
+// ratio) all start a multiple of 32 words apart and every store of the gather is a 32-way
+// bank conflict.
+__device__ __forceinline__ uint32_t packed_at(uint32_t addr) { return addr ^ ((addr >> 5) & 0x7Cu); }
+template <int DT>
+__device__ __forceinline__ uint32_t packed_elem(uint32_t rbase, uint32_t i) {        // element i of the sequence
+  const uint32_t addr = packed_at(rbase + i * static_cast<uint32_t>(sizeof(typename Elem<DT>::type)));
+  uint32_t u;
+  unsigned short h;
+  if (DT == 0) { asm volatile("ld.shared.u32 %0, [%1];" : "=r"(u) : "r"(addr) : "memory"); return u; }
+  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(h) : "r"(addr) : "memory");
+  return h;
+}
+// A full chunk with a misaligned destination: no room for the shift, the vectors are put together from elements.
+template <int DT>
+__device__ __noinline__ void copy_full_chunk(typename Elem<DT>::type* values, long long kept_before, uint32_t total, uint32_t rbase,
+                                             long long n_stored, uint32_t* status) {
+  using E = typename Elem<DT>::type;
+  constexpr int EPV = 16 / sizeof(E);
+  const uint32_t lane = lane_id(), mis = static_cast<uint32_t>(kept_before % EPV);
+  E* dst = values + kept_before;
+  const uint32_t head = min(mis ? EPV - mis : 0u, total);
+  const uint32_t n_vec = (total - head) / EPV;
+  if (lane < head && SURGEON_IN_BOUNDS(kept_before + lane, n_stored, status))
+    dst[lane] = static_cast<E>(packed_elem<DT>(rbase, lane));
+#pragma unroll 1
+  for (uint32_t v = lane; v < n_vec; v += 32) {
+    const uint32_t b = head + v * EPV;
+    uint32_t o[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      o[i] = DT == 0 ? packed_elem<DT>(rbase, b + i)
+                     : packed_elem<DT>(rbase, b + 2 * i) | (packed_elem<DT>(rbase, b + 2 * i + 1) << 16);
+    if (SURGEON_IN_BOUNDS(kept_before + head + v * EPV + EPV - 1, n_stored, status))
+      *reinterpret_cast<uint4*>(dst + head + v * EPV) = make_uint4(o[0], o[1], o[2], o[3]);
+  }
+  const uint32_t done = head + n_vec * EPV;
+  if (lane < total - done && SURGEON_IN_BOUNDS(kept_before + done + lane, n_stored, status))
+    dst[done + lane] = static_cast<E>(packed_elem<DT>(rbase, done + lane));
+}
+
 // ---- emit one chunk -------------------------------------------------------------------------------
 // before = (elements above the threshold before the chunk) << 32 | (ties before it); n_eq = its ties.
 // True when the chunk's place in the ring has been written to.
 template <int DT>
-__device__ __forceinline__ bool emit_chunk(const PruneArgs& a, unsigned char* region, unsigned char* stage,
-                                           int chunk, uint32_t tau, long long quota,
+__device__ __forceinline__ bool emit_chunk(const PruneArgs& a, unsigned char* region, int chunk, uint32_t tau, long long quota,
                                            unsigned long long before, uint32_t n_eq, long long n_stored) {
   using E = typename Elem<DT>::type;
   constexpr int EPR = 128 / sizeof(E);         // elements per row (= per lane): 32 / 64
@@ -290,16 +438,9 @@ __device__ __forceinline__ bool emit_chunk(const PruneArgs& a, unsigned char* re
   uint32_t word[WPL];
   mask_ge<DT, WPL>(q, nv, ties ? tau : tau + 1u, word);
   if (!ties && eq_b < quota) {
-    uint32_t ge[WPL], ec = 0;
-    mask_ge<DT, WPL>(q, nv, tau, ge);
-#pragma unroll
-    for (int w = 0; w < WPL; ++w) { ge[w] &= ~word[w]; ec += __popc(ge[w]); }
-    long long allowed = quota - eq_b - warp_excl_scan(ec);
-#pragma unroll
-    for (int w = 0; w < WPL; ++w) {
-      word[w] |= lowest_set_bits(ge[w], allowed);
-      allowed -= __popc(ge[w]);
-    }
+    const uint2 both = quota_words<DT>(region, nv, tau, quota - eq_b, make_uint2(word[0], word[WPL - 1]));
+    word[0] = both.x;
+    if (WPL == 2) word[WPL - 1] = both.y;
   }
   uint32_t cnt = 0;
 #pragma unroll
@@ -332,59 +473,16 @@ __device__ __forceinline__ bool emit_chunk(const PruneArgs& a, unsigned char* re
   // The sequence starts `mis` elements into its place, mis = the misalignment of its destination in
   // `values`: 16-byte vectors of the two then line up.
   const uint32_t mis = static_cast<uint32_t>(kept_before % EPV);
-  const uint32_t most = __reduce_max_sync(kFull, cnt);
-  // Sparse rows: a loop over the set bits, which fetches each kept element from the row; its cost is
-  // that of the fullest row (about 13 instructions per element), the unrolled gather's is 5 per element
-  // of the row, kept or not.
-  const bool sparse = most <= (DT == 0 ? 12u : 26u) &&
-                      (total + mis) * sizeof(E) <= static_cast<uint32_t>(kStageBytes);
-  if (sparse) {
-    uint32_t sa = smem_u32(stage) + (lane_pre + mis) * static_cast<uint32_t>(sizeof(E));
-#pragma unroll
-    for (int w = 0; w < WPL; ++w) {
-      uint32_t m = word[w];
-      while (m) {
-        const int e = 32 * w + __ffs(m) - 1;
-        m &= m - 1;
-        const uint32_t v = row_elem<DT>(region, e);
-        if (DT == 0) asm volatile("st.shared.u32 [%0], %1;" ::"r"(sa), "r"(v) : "memory");
-        else asm volatile("st.shared.u16 [%0], %1;" ::"r"(sa), "h"(static_cast<unsigned short>(v)) : "memory");
-        sa += static_cast<uint32_t>(sizeof(E));
-      }
-    }
-    __syncwarp();
-    const E* outp = reinterpret_cast<const E*>(stage);
-    E* gbase = values + (kept_before - mis);
-    const uint32_t end = mis + total, v_first = mis ? 1u : 0u, v_end = end / EPV;
-    if (mis) {
-      const uint32_t sl = mis + lane;
-      if (sl < static_cast<uint32_t>(EPV) && sl < end &&
-          SURGEON_IN_BOUNDS(kept_before - mis + sl, n_stored, &a.hdr->status))
-        gbase[sl] = outp[sl];
-    }
-    for (uint32_t g = v_first + lane; g < v_end; g += 32)
-      if (SURGEON_IN_BOUNDS(kept_before - mis + g * EPV + EPV - 1, n_stored, &a.hdr->status))
-        *reinterpret_cast<uint4*>(gbase + g * EPV) = *reinterpret_cast<const uint4*>(stage + g * 16);
-    const uint32_t t0 = (v_end > v_first ? v_end : v_first) * EPV;
-    if (t0 + lane < end && SURGEON_IN_BOUNDS(kept_before - mis + t0 + lane, n_stored, &a.hdr->status))
-      gbase[t0 + lane] = outp[t0 + lane];
-    __syncwarp();                                // the staging area is this warp's next chunk's
-    return false;
-  }
-  // Dense rows: gathered in place in the chunk's own part of the ring.
+  // Gathered in place in the chunk's own part of the ring, whatever share is kept.  (Sparse chunks by a loop over the set
+  // bits into a staging area took as long where 7-10 % are kept, and longer elsewhere: bf16, 77 MB, 30 % kept 72 against
+  // 65.5 us, 537 MB 353 against 314; 4.3 GB of fp32 1755 against 1710, by what the second path costs the first.)
   __syncwarp();                                  // every lane has its row in registers
-  // The byte at address a of the packed sequence lives at a ^ ((a >> 5) & 0x7C): the 32-bit word
-  // index is XORed with the index of its 128-byte row.  Without it, lanes that keep their whole
-  // row (chunks before the end of a large tie quota, e.g. the zeros of post-ReLU data at a low
-  // ratio) all start a multiple of 32 words apart and every store of the gather is a 32-way
-  // bank conflict.
   const uint32_t rbase = smem_u32(region);
-  auto swz = [](uint32_t addr) -> uint32_t { return addr ^ ((addr >> 5) & 0x7Cu); };
   const bool lined_up = total + mis <= static_cast<uint32_t>(32 * EPR);
   uint32_t pa = rbase + (lane_pre + (lined_up ? mis : 0u)) * static_cast<uint32_t>(sizeof(E));
   auto put = [&](uint32_t v) {
-    if (DT == 0) asm volatile("st.shared.u32 [%0], %1;" ::"r"(swz(pa)), "r"(v) : "memory");
-    else asm volatile("st.shared.u16 [%0], %1;" ::"r"(swz(pa)), "h"(static_cast<unsigned short>(v)) : "memory");
+    if (DT == 0) asm volatile("st.shared.u32 [%0], %1;" ::"r"(packed_at(pa)), "r"(v) : "memory");
+    else asm volatile("st.shared.u16 [%0], %1;" ::"r"(packed_at(pa)), "h"(static_cast<unsigned short>(v)) : "memory");
     pa += static_cast<uint32_t>(sizeof(E));
   };
 #pragma unroll
@@ -402,13 +500,6 @@ __device__ __forceinline__ bool emit_chunk(const PruneArgs& a, unsigned char* re
     }
   }
   __syncwarp();
-  auto elem_at = [&](uint32_t i) -> E {          // packed element i of the region
-    E v;
-    const uint32_t addr = swz(rbase + i * static_cast<uint32_t>(sizeof(E)));
-    if (DT == 0) { uint32_t u; asm volatile("ld.shared.u32 %0, [%1];" : "=r"(u) : "r"(addr) : "memory"); v = static_cast<E>(u); }
-    else { unsigned short u; asm volatile("ld.shared.u16 %0, [%1];" : "=h"(u) : "r"(addr) : "memory"); v = static_cast<E>(u); }
-    return v;
-  };
   if (lined_up) {
     // slots [mis, mis + total) of the region go to gbase[mis ...]; gbase is 16-byte aligned
     E* gbase = values + (kept_before - mis);
@@ -419,8 +510,9 @@ __device__ __forceinline__ bool emit_chunk(const PruneArgs& a, unsigned char* re
       const uint32_t sl = mis + lane;
       if (sl < static_cast<uint32_t>(EPV) && sl < end &&
           SURGEON_IN_BOUNDS(kept_before - mis + sl, n_stored, &a.hdr->status))
-        gbase[sl] = elem_at(sl);
+        gbase[sl] = static_cast<E>(packed_elem<DT>(rbase, sl));
     }
+#pragma unroll 2
     for (uint32_t g = v_first + lane; g < v_end; g += 32) {
       // the four words of a vector share their row: one 16-byte load, words permuted by the XOR
       const uint32_t la = rbase + g * 16u;
@@ -435,32 +527,9 @@ __device__ __forceinline__ bool emit_chunk(const PruneArgs& a, unsigned char* re
     }
     const uint32_t t0 = (v_end > v_first ? v_end : v_first) * EPV;
     if (t0 + lane < end && SURGEON_IN_BOUNDS(kept_before - mis + t0 + lane, n_stored, &a.hdr->status))
-      gbase[t0 + lane] = elem_at(t0 + lane);
+      gbase[t0 + lane] = static_cast<E>(packed_elem<DT>(rbase, t0 + lane));
   } else {
-    // a full chunk with a misaligned destination: no room for the shift, element-wise vectors
-    E* dst = values + kept_before;
-    uint32_t head = mis ? EPV - mis : 0;
-    if (head > total) head = total;
-    const uint32_t n_vec = (total - head) / EPV;
-    if (lane < head && SURGEON_IN_BOUNDS(kept_before + lane, n_stored, &a.hdr->status))
-      dst[lane] = elem_at(lane);
-    for (uint32_t v = lane; v < n_vec; v += 32) {
-      const uint32_t b = head + v * EPV;
-      uint4 o;
-      if (DT == 0) {
-        o = make_uint4(elem_at(b), elem_at(b + 1), elem_at(b + 2), elem_at(b + 3));
-      } else {
-        o = make_uint4(elem_at(b) | (static_cast<uint32_t>(elem_at(b + 1)) << 16),
-                       elem_at(b + 2) | (static_cast<uint32_t>(elem_at(b + 3)) << 16),
-                       elem_at(b + 4) | (static_cast<uint32_t>(elem_at(b + 5)) << 16),
-                       elem_at(b + 6) | (static_cast<uint32_t>(elem_at(b + 7)) << 16));
-      }
-      if (SURGEON_IN_BOUNDS(kept_before + head + v * EPV + EPV - 1, n_stored, &a.hdr->status))
-        *reinterpret_cast<uint4*>(dst + head + v * EPV) = o;
-    }
-    const uint32_t done = head + n_vec * EPV;
-    if (lane < total - done && SURGEON_IN_BOUNDS(kept_before + done + lane, n_stored, &a.hdr->status))
-      dst[done + lane] = elem_at(done + lane);
+    copy_full_chunk<DT>(values, kept_before, total, rbase, n_stored, &a.hdr->status);
   }
   return true;
 }
@@ -493,68 +562,32 @@ __device__ __forceinline__ uint32_t my_bin(const uint32_t* hist) {
 // The first n_in keys of a slot in shared memory, f(key), a warp together.
 template <int DT, typename F>
 __device__ __forceinline__ void slot_keys_warp(const typename Elem<DT>::type* slot, uint32_t n_in, F f) {
+#pragma unroll 1
   for (uint32_t i = lane_id(); i < n_in; i += 32) f(static_cast<uint32_t>(slot[i]));
 }
-// Of slots in global memory: f(c, acc, key) for the listed keys of chunks 0 .. n_local - 1, then done(c, cnt[c],
-// the chunk's acc) on one lane.  Half a warp per chunk, 8 bytes per lane (32 fp32 or 64 bf16 keys; few chunks
-// have more) and four chunks in flight: one trip to L2 for 128 chunks.  (A lane per chunk, 64 bytes at a time,
-// took 5-7 us a call.)  Of a larger tensor (`many`) a lane per chunk, which has four times as many chunks in
-// flight and asks for little more than the keys: 128 at a time made 4.3 GB 6 % slower.
+// Of slots in global memory (a large tensor's, whose chunks are claimed): f(c, acc, key) for the listed keys of chunks
+// 0 .. n_local - 1, then done(c, cnt[c], the chunk's acc).  A lane per chunk, 64 bytes at a time: many chunks in
+// flight, and little more asked for than the keys (half a warp per chunk made 4.3 GB 6 % slower).
 template <int DT, typename F, typename D>
-__device__ __forceinline__ void slot_keys_global(const typename Elem<DT>::type* slots, const uint32_t* cnt, int n_local, bool many, F f, D done) {
-  if (many) {
-    constexpr uint32_t EPV = 16 / sizeof(typename Elem<DT>::type);
-    for (int c = threadIdx.x; c < n_local; c += kThreads) {
-      const uint32_t v = cnt[c], n_in = min(v >> 16, static_cast<uint32_t>(slot_entries(DT)));
-      uint32_t acc = 0;
-      const uint4* p = reinterpret_cast<const uint4*>(slots + static_cast<long long>(c) * slot_entries(DT));
-      for (uint32_t v0 = 0; v0 * EPV < n_in; v0 += 4) {
-        uint4 q[4];
+__device__ __forceinline__ void slot_keys_global(const typename Elem<DT>::type* slots, const uint32_t* cnt, int n_local, F f, D done) {
+  constexpr uint32_t EPV = 16 / sizeof(typename Elem<DT>::type);
+  for (int c = threadIdx.x; c < n_local; c += kThreads) {
+    const uint32_t v = cnt[c], n_in = min(v >> 16, static_cast<uint32_t>(slot_entries(DT)));
+    uint32_t acc = 0;
+    const uint4* p = reinterpret_cast<const uint4*>(slots + static_cast<long long>(c) * slot_entries(DT));
+    for (uint32_t v0 = 0; v0 * EPV < n_in; v0 += 4) {
+      uint4 q[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) q[u] = (v0 + u) * EPV < n_in ? p[v0 + u] : make_uint4(0, 0, 0, 0);
+      for (int u = 0; u < 4; ++u) q[u] = (v0 + u) * EPV < n_in ? p[v0 + u] : make_uint4(0, 0, 0, 0);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const uint32_t w[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
+      for (int u = 0; u < 4; ++u) {
+        const uint32_t w[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
 #pragma unroll
-          for (uint32_t e = 0; e < EPV; ++e)
-            if ((v0 + u) * EPV + e < n_in) f(c, acc, (DT == 0) ? w[e % 4] : (w[e >> 1] >> (16 * (e & 1))) & 0xFFFFu);
-        }
+        for (uint32_t e = 0; e < EPV; ++e)
+          if ((v0 + u) * EPV + e < n_in) f(c, acc, (DT == 0) ? w[e % 4] : (w[e >> 1] >> (16 * (e & 1))) & 0xFFFFu);
       }
-      done(c, v, acc);
     }
-    return;
-  }
-  constexpr uint32_t EPW = 8 / sizeof(typename Elem<DT>::type);     // keys of a lane
-  constexpr int kFlight = 4;
-  const uint32_t hl = threadIdx.x & 15u;
-  for (int c0 = (threadIdx.x >> 5) * 2; c0 < n_local; c0 += kFlight * (kThreads / 16)) {
-    const int cf = c0 + static_cast<int>((threadIdx.x >> 4) & 1u);
-    uint32_t v[kFlight];
-    uint2 q[kFlight];
-#pragma unroll
-    for (int u = 0; u < kFlight; ++u) {
-      const int c = cf + u * (kThreads / 16);
-      v[u] = c < n_local ? cnt[c] : 0u;
-      const uint2* p = reinterpret_cast<const uint2*>(slots + static_cast<long long>(c) * slot_entries(DT)) + hl;
-      q[u] = hl * EPW < (v[u] >> 16) ? *p : make_uint2(0, 0);
-    }
-#pragma unroll
-    for (int u = 0; u < kFlight; ++u) {
-      const int c = cf + u * (kThreads / 16);
-      const uint32_t n_in = min(v[u] >> 16, static_cast<uint32_t>(slot_entries(DT)));
-      uint32_t acc = 0;
-#pragma unroll
-      for (uint32_t e = 0; e < EPW; ++e) {
-        const uint32_t w = (DT == 0 ? e : e >> 1) ? q[u].y : q[u].x;
-        if (hl * EPW + e < n_in) f(c, acc, DT == 0 ? w : (w >> (16 * (e & 1))) & 0xFFFFu);
-      }
-#pragma unroll 1
-      for (uint32_t i = 16 * EPW + hl; i < n_in; i += 16)
-        f(c, acc, static_cast<uint32_t>(slots[static_cast<long long>(c) * slot_entries(DT) + i]));
-#pragma unroll
-      for (int o = 8; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
-      if (hl == 0 && c < n_local) done(c, v[u], acc);
-    }
+    done(c, v, acc);
   }
 }
 
@@ -570,27 +603,40 @@ enum Step : uint32_t {
   kRecount = 6,    // the threshold is lo; the lists overflowed: count once more
 };
 
-// CTA 0: the answers of a phase and the histogram of a round, before the exchange that leads to them.
-__device__ __forceinline__ void prepare_phase(const PruneArgs& a, int phase) {
-  if (phase < kSelPhases)
-    for (int i = threadIdx.x; i < kSelMaxCtas + 2; i += kThreads) a.answer[phase * (kSelMaxCtas + 2) + i].x = 0ull;
+// CTA 0: no phase of [p0, p1) has an answer, and the bins and counts of the rounds [r0, r1) are zero.
+__device__ __forceinline__ uint32_t* above_count(const PruneArgs& a, int round) {     // (between the counters of claims)
+  return a.claims + round * kClaimSets * kClaimStride + 1;
 }
-__device__ __forceinline__ void prepare_round(const PruneArgs& a, int round) {
-  if (round < kSelHists && threadIdx.x < kSelBins) a.hist[round * kSelBins + threadIdx.x] = 0u;
+__device__ __forceinline__ void prepare_exchanges(const PruneArgs& a, int p0, int p1, int r0, int r1) {
+  constexpr int kRow = kSelMaxCtas + 2;
+  static_assert(kRow <= kThreads && kSelBins <= kThreads && kSelHists <= kSelPhases, "one thread per answer and bin");
+  for (int p = p0; p < p1; ++p)
+    if (threadIdx.x < gridDim.x + 2u) a.answer[p * kRow + threadIdx.x].x = 0ull;
+  for (int r = r0; r < r1; ++r) {
+    if (threadIdx.x < kSelBins) a.hist[r * kSelBins + threadIdx.x] = 0u;
+    if (threadIdx.x == 0) *above_count(a, r) = 0u;
+  }
 }
 
-// RES: the CTA's whole range stays in the ring (at most kResidentChunks chunks per CTA).
-template <int DT, bool RES>
+// MODE kResident: the CTA's whole range stays in the ring (at most kResidentChunks chunks per CTA).
+//      kStreamed: it goes through the ring twice; counts and lists are in shared memory.
+//      kClaimed: of a gigabyte tensor the warps claim their chunks four at a time, in either pass: equal
+//      shares took some SMs 620 us and others 760, and all wait for the last.  Four sets of CTAs claim
+//      from counters of their own (one counter for all passes on a claim every 3 ns, too slow).  Only
+//      what is counted and placed per CTA stays a contiguous range then; counts and lists are in global memory.
+enum Mode { kResident = 0, kStreamed = 1, kClaimed = 2 };
+template <int DT, int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
 prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ PruneArgs a) {
   using E = typename Elem<DT>::type;
+  constexpr bool RES = MODE == kResident, spread = MODE == kClaimed;
   constexpr uint32_t kMask = Elem<DT>::kKeyMask;
   constexpr uint32_t kKeyMax = kMask;
   constexpr int EPR = 128 / sizeof(E);
   constexpr int WPL = EPR / 32;
   constexpr int EPV = 16 / sizeof(E);
-  constexpr int kSlot = slot_entries(DT);
-  static_assert(kSlot * sizeof(E) == kSlotBytes, "slot size");
+  constexpr int kSlot = RES ? kResSlotBytes / static_cast<int>(sizeof(E)) : slot_entries(DT);
+  static_assert(RES || kSlot * sizeof(E) == kSlotBytes, "slot size");
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* ring = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -601,7 +647,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
   __shared__ unsigned long long s_warp64[kWarps];
   __shared__ uint32_t s_res[8];
   __shared__ uint32_t s_tot[4];                // keys above / inside the bracket, largest key inside, largest ~key inside
-  __shared__ uint32_t s_over, s_fail, s_nkeys;
+  __shared__ uint32_t s_over, s_fail, s_nkeys, s_list_n, s_list_lo;
   __shared__ unsigned long long s_ans[2];
   __shared__ uint32_t s_bin_key[kMaxKeys];      // the keys that this CTA reports at the last exchange,
   __shared__ int s_bin_chunk[kMaxKeys];        // and their chunks
@@ -614,15 +660,17 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
   const int c_begin = static_cast<int>(static_cast<long long>(a.n_chunks) * blockIdx.x / G);
   const int c_end = static_cast<int>(static_cast<long long>(a.n_chunks) * (blockIdx.x + 1) / G);
   const int n_local = c_end - c_begin;
-  // Of a gigabyte tensor (a.spread) the warps claim their chunks four at a time, in either pass: equal
-  // shares took some SMs 620 us and others 760, and all wait for the last.  Four sets of CTAs claim
-  // from counters of their own (one counter for all passes on a claim every 3 ns, too slow).  Only
-  // what is counted and placed per CTA stays a contiguous range then.
-  const bool spread = !RES && a.spread != 0;
   const int n_mine = warp < n_local ? (n_local - 1 - warp) / kWarps + 1 : 0;   // (not spread) chunks c_begin + warp + 16 i
-  uint32_t* cnt = spread ? a.cnt + c_begin : reinterpret_cast<uint32_t*>(aux + kAuxCnt);
+  const int n_even = (n_local + 1) & ~1;         // (the places are 8 bytes each)
+  uint32_t* cnt = spread ? a.cnt + c_begin : reinterpret_cast<uint32_t*>(aux + (RES ? kResCnt : kAuxBytes - 4 * n_even));
   unsigned long long* prefix =
-      spread ? a.prefix + c_begin : reinterpret_cast<unsigned long long*>(aux + kAuxPrefix);
+      spread ? a.prefix + c_begin : reinterpret_cast<unsigned long long*>(aux + (RES ? kResPrefix : kAuxBytes - 12 * n_even));
+  // (streamed, not claimed) the list: fp32 keys, or bf16 keys less the bracket's lower end in a byte
+  using L = typename std::conditional<DT == 0, uint32_t, unsigned char>::type;
+  L* list = reinterpret_cast<L*>(aux + kList);
+  unsigned short* list_start = reinterpret_cast<unsigned short*>(aux + kListStart);
+  unsigned short* list_acc = reinterpret_cast<unsigned short*>(aux + kListAcc);
+  constexpr uint32_t kNotListed = 0xFFFFu;       // the chunk's keys are in its slot in global memory
   E* s_slots = reinterpret_cast<E*>(aux + kAuxSlots);     // RES: the chunks' slots, else a staging slot per warp
   E* g_slots = reinterpret_cast<E*>(a.slots) + static_cast<long long>(c_begin) * kSlot;
   const E* __restrict__ x = reinterpret_cast<const E*>(a.x);
@@ -631,27 +679,41 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
   unsigned char* my_ring = ring + warp * (kSlotsPerWarp * kChunkBytes);
   const uint32_t my_bars = smem_u32(bars + warp * kSlotsPerWarp);
   uint32_t parity = 0;                           // bit s: phase of place s's next wait
+  uint32_t under_way = 0;                        // bit s: a load of place s has been started and not waited for
   auto chunk_of = [&](int i) { return c_begin + warp + kWarps * i; };
   auto issue = [&](int c, int s) {               // start the load of chunk c into place s (one lane)
-    if (lane == 0 && static_cast<long long>(c) * 32 < a.n_rows_full) {
+    if (static_cast<long long>(c) * 32 >= a.n_rows_full) return;
+    under_way |= 1u << s;
+    if (lane == 0) {
       tc::mbar_arrive_expect_tx(my_bars + 8 * s, kChunkBytes);
       tc::tma_load_2d(smem_u32(my_ring + s * kChunkBytes), &xmap, 0, c * 32, my_bars + 8 * s);
     }
   };
+  auto landed = [&](int s) -> bool {             // wait for the load of place s
+    const uint32_t bar = my_bars + 8 * s, phase_bit = (parity >> s) & 1u;
+    parity ^= 1u << s;
+    under_way &= ~(1u << s);
+#pragma unroll 1
+    for (uint32_t i = 0; i < tc::kWaitCap; ++i)
+      if (tc::mbar_try_wait(bar, phase_bit)) return true;
+    return false;
+  };
   auto arrived = [&](int c, int s) -> bool {     // wait for it; the tensor's last, partial row is added
     unsigned char* region = my_ring + s * kChunkBytes;
     const long long row0 = static_cast<long long>(c) * 32;
+    if (row0 + 32 <= a.n_rows_full) return landed(s);
     if (row0 < a.n_rows_full) {
-      if (!tc::mbar_wait(my_bars + 8 * s, (parity >> s) & 1u)) return false;
-      parity ^= 1u << s;
+      if (!landed(s)) return false;
     } else {
+#pragma unroll 1
       for (int v = lane; v < kChunkBytes / 16; v += 32)
         *reinterpret_cast<uint4*>(region + v * 16) = make_uint4(0, 0, 0, 0);
       tc::fence_proxy_async();                   // (these stores precede the next TMA fill of the place)
       __syncwarp();
     }
-    if (row0 + 32 > a.n_rows_full && a.n > a.n_rows_full * EPR) {
+    if (a.n > a.n_rows_full * EPR) {
       const int r = static_cast<int>(a.n_rows_full - row0);       // the map fills the rows past it with zeros
+#pragma unroll 1
       for (int e = lane; e < static_cast<int>(a.n - a.n_rows_full * EPR); e += 32) {
         const int byte = e * static_cast<int>(sizeof(E));
         *reinterpret_cast<E*>(region + r * 128 + (((byte >> 4) ^ (r & 7)) << 4) + (byte & 15)) =
@@ -684,29 +746,24 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     const int c = claim + (at_i++ & 3);
     return c < a.n_chunks ? c : a.n_chunks;
   };
-  auto begin_pass = [&](bool reverse) {          // the first three loads; reverse: from the tensor's end
-    at_i = 0;
-    auto one = [&](int s) -> int {
-      int c = next();
-      if (c < a.n_chunks) {
-        if (reverse) c = a.n_chunks - 1 - c;
-        issue(c, s);
-      }
-      return c;
-    };
-    fly0 = one(0); fly1 = one(1); fly2 = one(2);
+  auto start = [&](bool reverse, int s) -> int { // the load of the next chunk; reverse: from the tensor's end
+    int c = next();
+    if (c < a.n_chunks) {
+      if (reverse) c = a.n_chunks - 1 - c;
+      issue(c, s);
+    }
+    return c;
   };
-  // A wait gave up: the loads behind it are waited for (with a limit) as well.
-  auto give_up = [&](int s) {
-    s_fail = 1;
-    if (fly1 < a.n_chunks) arrived(fly1, (s + 1) % 3);
-    if (fly2 < a.n_chunks) arrived(fly2, (s + 2) % 3);
+  auto begin_pass = [&](bool reverse) {          // the first three loads
+    at_i = 0;
+    fly0 = start(reverse, 0); fly1 = start(reverse, 1); fly2 = start(reverse, 2);
   };
   // One pass over the warp's chunks: f(chunk, region) is true where it wrote to the region.
   auto run_pass = [&](bool reverse, auto f) {
+#pragma unroll 1
     for (int s = 0; fly0 < a.n_chunks; s = s == 2 ? 0 : s + 1) {
       unsigned char* region = my_ring + s * kChunkBytes;
-      if (!arrived(fly0, s)) { give_up(s); break; }
+      if (!arrived(fly0, s)) { s_fail = 1; break; }
       const bool written = f(fly0, region);
       fly0 = fly1; fly1 = fly2;
       int c = next();
@@ -722,15 +779,31 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
   };
   // (RES) the chunks are where the first loads put them.
   auto run_resident = [&](bool loading, auto f) {
+#pragma unroll 1
     for (int i = 0; i < n_mine; ++i) {
-      if (loading && !arrived(chunk_of(i), i)) { s_fail = 1; for (++i; i < n_mine; ++i) arrived(chunk_of(i), i); break; }
+      if (loading && !arrived(chunk_of(i), i)) { s_fail = 1; break; }
       f(chunk_of(i), my_ring + i * kChunkBytes);
     }
   };
-  auto drain = [&]() {                           // before leaving with the first loads under way
-    if (fly0 < a.n_chunks) arrived(fly0, 0);
-    if (fly1 < a.n_chunks) arrived(fly1, 1);
-    if (fly2 < a.n_chunks) arrived(fly2, 2);
+  // (streamed, not claimed) f(c, acc, key) for the listed keys of every chunk, then done(c, cnt[c], the chunk's acc) on
+  // one lane: eight lanes per chunk.
+  auto listed_keys = [&](auto f, auto done) {
+#pragma unroll 1
+    for (int c0 = warp * 4; c0 < n_local; c0 += kWarps * 4) {
+      const int c = c0 + static_cast<int>(lane >> 3);
+      const uint32_t v = c < n_local ? cnt[c] : 0u, n_in = min(v >> 16, static_cast<uint32_t>(kSlot));
+      const uint32_t start = n_in ? list_start[c] : 0u;
+      uint32_t acc = 0;
+#pragma unroll 1
+      for (uint32_t i = lane & 7u; i < n_in; i += 8) {
+        const uint32_t key = start == kNotListed ? static_cast<uint32_t>(g_slots[static_cast<long long>(c) * kSlot + i])
+                                                 : list[start + i] + (DT == 0 ? 0u : s_list_lo);
+        f(c, acc, key);
+      }
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
+      if ((lane & 7u) == 0 && c < n_local) done(c, v, acc);
+    }
   };
   int phase = 1;                                 // of the next exchange
   auto meet = [&]() -> bool {                    // an exchange without a message: what was written before is visible after
@@ -747,7 +820,6 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
         fence_gpu();
         a.arrive[phase * kSelMaxCtas + tid].x = 0ull;
       }
-      prepare_phase(a, phase + 1);
       ok = __syncthreads_and(ok);
       if (ok && tid == 0) {
         fence_gpu();
@@ -763,57 +835,38 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     ++phase;
     return ok != 0;
   };
-  // The whole CTA leaves after a wait gave up.  It takes back what it has stored for the others: a replay of a
-  // captured call carries the same token and must not find it.
-  auto quit = [&]() {
-    if (tid == 0) atomicMax(&a.hdr->status, static_cast<uint32_t>(SURGEON_ERR_TIMEOUT));
-    if (tid < kSelPhases) a.arrive[tid * kSelMaxCtas + blockIdx.x].x = 0ull;
-    if (master)
-      for (int i = tid; i < kSelPhases * (kSelMaxCtas + 2); i += kThreads) a.answer[i].x = 0ull;
-  };
-
-  // ---- set-up ----
-  if (lane == 0) {                               // a warp's barriers are its own
-    for (int s = 0; s < kSlotsPerWarp; ++s) tc::mbar_init(my_bars + 8 * s, 1);
-    tc::fence_barrier_init();
-  }
-  __syncwarp();
-  begin_pass(false);
-  if (tid == 0) {
-    s_fail = 0;
-    s_over = 0;
-  }
-  if (tid < 4) s_tot[tid] = 0;
-  for (int i = tid; i < kSampleBytes / 16; i += kThreads) reinterpret_cast<uint4*>(aux)[i] = make_uint4(0, 0, 0, 0);
-  __syncthreads();
-
+  enum Leave { kDone = 0, kTimedOut = 1, kUnsound = 2 };
+  const int left_as = [&]() -> int {
   // ---- the sample ----
-  // A resident tensor: 2048 vectors of 32 (fp32) or 16 (bf16) bytes, one per stratum, the same for
+  // A resident tensor: 1024 vectors of four elements, one per stratum, the same for
   // every CTA (each starts elsewhere in it, so that they do not all ask for the same lines at the
-  // same time).  More would not pay: 148 CTAs that read 8192 places took 12 us.  The margin is 4
-  // standard deviations (a miss costs a round).
+  // same time).  The margin is 3.5 standard deviations (a miss costs another pass over shared memory): at most 6 % of
+  // the elements lie inside, for which the slots have twice the room.  Four times as many elements, with half the
+  // bracket, cost 3 us more (up to 8 us of shared-memory atomics where many keys are equal) and saved 0.5.
   // A larger tensor, for which a miss is another read of it and a narrow bracket pays: every CTA
   // samples the whole tensor at places of its own (stratum G i + p of the G i-th row, p scrambled from
   // row to row so that no period of the data falls to one CTA) and reports where the threshold lies in
-  // its own 4 or 8 thousand elements.  The CTAs' answers are independent draws whose median is the
+  // its own 4 thousand elements.  The CTAs' answers are independent draws whose median is the
   // threshold, however the elements are distributed, so the ones 2.5 sqrt(G) places (5 standard
   // deviations) to either side of the middle bound it: 0.4 % of the elements to each side, as the sum of
   // all histograms would give.  One exchange of one word per CTA, 4 us less than a window from CTA 0's part
   // and added-up histograms took.
   uint32_t lo = 1, hi = kKeyMax;
-  const uint32_t n_vec = static_cast<uint32_t>(a.n / EPV);
-  constexpr int kPer = RES ? (DT == 0 ? 8 : 4) : 2;       // vectors per thread
+  constexpr int kPer = RES || DT == 0 ? 2 : 1;   // vectors per thread
+  constexpr int kVecElems = RES ? 4 : EPV;       // elements of one
+  constexpr int kVecWords = kVecElems * static_cast<int>(sizeof(E)) / 4;
   constexpr int kBinShift = Elem<DT>::kKeyBits - kSampleBinsLog2;
   constexpr int kFineShift = kBinShift > kSelBinsLog2 ? kBinShift - kSelBinsLog2 : 0;     // (!RES)
   uint4 v[kPer];
   {
-    constexpr uint32_t kStrata = kPer * kThreads / (DT == 0 ? 2 : 1);     // of this CTA
+    constexpr uint32_t kStrata = kPer * kThreads / (!RES && DT == 0 ? 2 : 1);     // of this CTA
     const uint32_t strata = RES ? kStrata : kStrata * G;
+    const uint32_t n_vec = static_cast<uint32_t>(a.n / kVecElems);
     const float stride = static_cast<float>(n_vec) / static_cast<float>(strata);
 #pragma unroll
     for (int u = 0; u < kPer; ++u) {
       uint32_t loc = u * kThreads + tid, part = 0;
-      if (DT == 0) { part = loc & 1u; loc >>= 1; }         // two lanes share a stratum: 32 bytes
+      if (!RES && DT == 0) { part = loc & 1u; loc >>= 1; }         // two lanes share a stratum: 32 bytes
       if (RES) {
         loc = (loc + blockIdx.x * 37u) % kStrata;
       } else {
@@ -822,50 +875,77 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
       }
       const float at = (static_cast<float>(loc) + static_cast<float>(hash_u32(loc) >> 8) * (1.0f / 16777216.0f)) * stride;
       uint32_t pos = static_cast<uint32_t>(at);
-      if (DT == 0) pos = (pos & ~1u) + part;
-      v[u] = n_vec ? __ldg(reinterpret_cast<const uint4*>(a.x) + min(pos, n_vec - 1)) : make_uint4(0, 0, 0, 0);
+      if (!RES && DT == 0) pos = (pos & ~1u) + part;
+      v[u] = make_uint4(0, 0, 0, 0);
+      if (n_vec) {
+        pos = min(pos, n_vec - 1);
+        if (kVecWords == 4) {
+          v[u] = __ldg(reinterpret_cast<const uint4*>(a.x) + pos);
+        } else {
+          const uint2 half = __ldg(reinterpret_cast<const uint2*>(a.x) + pos);
+          v[u].x = half.x;
+          v[u].y = half.y;
+        }
+      }
     }
   }
-  if (master) {                                  // meanwhile CTA 0 prepares the exchange
+
+  // ---- set-up ----
+  if (lane == 0) {                               // a warp's barriers are its own
+    for (int s = 0; s < kSlotsPerWarp; ++s) tc::mbar_init(my_bars + 8 * s, 1);
+    tc::fence_barrier_init();
+  }
+  __syncwarp();
+  fly0 = start(false, 0);                        // (the others when the sample is there: it would queue behind them)
+  if (tid == 0) {
+    s_fail = 0;
+    s_over = 0;
+  }
+  if (tid < 4) s_tot[tid] = 0;
+  for (int i = tid; i < kAuxBytes / 16; i += kThreads) reinterpret_cast<uint4*>(aux)[i] = make_uint4(0, 0, 0, 0);
+  __syncthreads();
+
+  if (master) {                                  // meanwhile CTA 0 prepares the exchanges
     if (tid == 0) {                              // (no value yet: what reads the store trusts the count)
       a.hdr->status = SURGEON_OK;
       a.hdr->n_keep = 0;
     }
-    prepare_phase(a, 1);
-    prepare_round(a, 0);
+    // what the usual call needs, the rest where a round is added
+    prepare_exchanges(a, 1, spread ? kSelPhases : 3, 0, spread ? kSelHists : 1);
     if (!RES && tid < kSelPhases * kClaimSets) a.claims[tid * kClaimStride] = 0u;
-    if (RES) {
-      __syncthreads();
-      if (tid == 0) {
-        fence_gpu();
-        word_store(a.answer, a.token, 0ull);     // phase 0: the histogram is zero, the header begun
-      }
-    }
+    __syncthreads();
   }
 #pragma unroll
   for (int u = 0; u < kPer; ++u) {
     const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
 #pragma unroll
-    for (int e = 0; e < EPV; ++e) {
+    for (int e = 0; e < kVecElems; ++e) {
       const uint32_t key = ((DT == 0) ? w[e % 4] : (w[e >> 1] >> (16 * (e & 1)))) & kMask;
       const uint32_t bin = key >> kBinShift;
       if (key) atomicAdd(&hist[bin >> 1], 1u << (16 * (bin & 1)));   // (not the zeros, half of post-ReLU data)
     }
   }
+  fly1 = start(false, 1);
+  fly2 = start(false, 2);
+  if (master && tid == 0) {                      // (by now its stores have arrived)
+    fence_gpu();
+    if (RES) word_store(a.answer, a.token, 0ull);      // phase 0: prepared
+  }
   // rank of the threshold inside the sample, and (RES) a margin of some standard deviations of a binomial count
   const float q = static_cast<float>(a.k) / static_cast<float>(a.n);
-  constexpr float kOwn = static_cast<float>(kPer * kThreads * EPV);        // elements in this CTA's histogram
+  constexpr float kOwn = static_cast<float>(kPer * kThreads * kVecElems);   // elements in this CTA's histogram
   const float up = q * kOwn, down = kOwn - up;   // of them above and below the threshold
   const bool no_hi = up < 16.0f, no_lo = down < 16.0f;     // (!RES) too few for a median that means something:
   uint32_t r_hi, r_lo = 0;                       // that side stays open, and the rank moves to the other
   if (RES) {
-    const float delta = 4.0f * sqrtf(kOwn * q * (1.0f - q)) + 16.0f;
+    const float delta = 3.5f * sqrtf(kOwn * q * (1.0f - q)) + 8.0f;
     r_hi = up - delta >= 1.0f ? static_cast<uint32_t>(up - delta) : 0u;                        // 0: none
     r_lo = up + delta <= kOwn - 1.0f ? static_cast<uint32_t>(up + delta) + 1u : 0u;            // 0: none
   } else {
     r_hi = static_cast<uint32_t>(no_hi ? up + sqrtf(up) + 2.0f : no_lo ? up - sqrtf(down) - 2.0f : up + 0.5f);
   }
   if (tid < 2) s_res[tid] = RES && tid == 0 && r_hi == 0 ? kSampleBins - 1u : 0u;
+  if (tid < 2) s_res[4 + 2 * tid] = kThreads;    // (no thread has the rank)
   __syncthreads();
   {
     // the bins of the ranks in the CTA's own histogram
@@ -882,20 +962,22 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     }
     uint32_t all;
     const uint32_t above = count_above_mine(sum, s_warp, &all);
-#pragma unroll 1
+#pragma unroll
     for (int which = 0; which < (RES ? 2 : 1); ++which) {
       // (a rank among the zeros lies below every counted bin: bin 0)
       const uint32_t want = which ? r_lo : r_hi;
       if (want && above < want && want <= above + sum) {
-        uint32_t acc = above;
-        int bin = 31;
-#pragma unroll 1
-        for (; bin > 0; --bin) {
-          const uint32_t c = (reinterpret_cast<const uint32_t*>(mine)[bin >> 1] >> (16 * (bin & 1))) & 0xFFFFu;
-          if (acc + c >= want) break;
-          acc += c;
-        }
-        s_res[which] = static_cast<uint32_t>(kSampleBins - 32 - 32 * tid + bin);
+        s_res[4 + 2 * which] = tid;
+        s_res[5 + 2 * which] = above;
+      }
+    }
+    __syncthreads();
+    if (warp < (RES ? 2 : 1) && s_res[4 + 2 * warp] < kThreads) {     // a warp for each rank, a lane per bin
+      const uint32_t owner = s_res[4 + 2 * warp], want = warp ? r_lo : r_hi, bin = kSampleBins - 1u - 32u * owner - lane;
+      const uint32_t c = (hist[bin >> 1] >> (16 * (bin & 1))) & 0xFFFFu;
+      const uint32_t acc = s_res[5 + 2 * warp] + warp_excl_scan(c);
+      if (acc < want && want <= acc + c) {
+        s_res[warp] = bin;
         if (!RES) s_res[1] = want - acc;         // the rank among the bin's elements
       }
     }
@@ -913,7 +995,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     for (int u = 0; u < kPer; ++u) {
       const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
 #pragma unroll
-      for (int e = 0; e < EPV; ++e) {
+      for (int e = 0; e < kVecElems; ++e) {
         const uint32_t key = ((DT == 0) ? w[e % 4] : (w[e >> 1] >> (16 * (e & 1)))) & kMask;
         if (key && key >> kBinShift == bin) atomicAdd(&hist[(key & ((1u << kBinShift) - 1u)) >> kFineShift], 1u);
       }
@@ -937,7 +1019,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
       }
       // distinct, in the keys' order
       if (tid < kSelMaxCtas) bins[tid] = tid < G ? (static_cast<uint32_t>(w) << 8) | (kSelMaxCtas - 1u - tid) : 0u;
-      if (!__syncthreads_and(ok)) { drain(); quit(); return; }
+      if (!__syncthreads_and(ok)) return kTimedOut;
       const int margin = static_cast<int>(2.5f * sqrtf(static_cast<float>(G))) + 1;
       const int at_hi = G / 2 - margin, at_lo = G / 2 + margin;
       if (tid < G) {
@@ -954,8 +1036,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
       __syncthreads();
       hi = no_hi || at_hi < 0 ? kKeyMax : (s_res[0] << kFineShift) | ((1u << kFineShift) - 1u);
       lo = no_lo || at_lo >= G ? 1u : max(s_res[1] << kFineShift, 1u);
-      if (tid == 0) {
-        fence_gpu();                             // the histogram is zero, the claims, the header begun
+      if (tid == 0) {                            // (prepared behind a fence, above)
         word_store(a.answer, a.token, lo | (static_cast<unsigned long long>(hi) << 32));
       }
     } else {
@@ -964,7 +1045,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
         fence_gpu();
         s_ans[0] = w;
       }
-      if (!__syncthreads_and(ok)) { drain(); quit(); return; }
+      if (!__syncthreads_and(ok)) return kTimedOut;
       lo = static_cast<uint32_t>(s_ans[0]);
       hi = static_cast<uint32_t>(s_ans[0] >> 32);
     }
@@ -985,11 +1066,16 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     shift = max(0, 32 - __clz(range) - kSelBinsLog2);
     __syncthreads();
     if (tid < kSelBins) hist[tid] = 0;
-    if (step == kRead) {
-      if (tid < 4) s_tot[tid] = 0;
-      if (tid == 0) s_over = 0;
+    if (tid < 4 && (step == kRead || tid == 1)) s_tot[tid] = 0;
+    if (tid == 0 && step == kRead) {
+      s_over = 0;
+      s_list_n = 0;
+      s_list_lo = lo;
     }
     __syncthreads();
+    ulonglong2 prepared = make_ulonglong2(0, 0);   // (RES) CTA 0's first word, asked for ahead of its use
+    if (RES && round == 0 && tid == 0) prepared = word_load(a.answer);
+    uint32_t w_in = 0;                           // keys inside the bracket
     if (step == kRead) {
       if (!RES && !loaded) {                     // the pass starts over
         tc::fence_proxy_async();
@@ -1048,12 +1134,14 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
         const uint32_t a_tot = both & 0xFFFFu, c_tot = both >> 16;
         if (lane == 0) cnt[cl] = both;
         w_above += a_tot;
+        w_in += c_tot;
         if (c_tot > static_cast<uint32_t>(kSlot)) {
           // Massive ties.  If the chunk's keys inside the bracket all are one key, it is counted in
           // one go; if that holds everywhere with the same key, it is the threshold and the counts
           // are final without a list.
           const uint32_t k1 = one_key_of_chunk<DT>(region, cw[0], cw[WPL - 1], c_tot);
           if (lane == 0) s_over = 1;
+          if (MODE == kStreamed && lane == 0) list_start[cl] = kNotListed;
           if (k1) {
             if (lane == 0) atomicAdd(&hist[(k1 - lo) >> shift], c_tot);
             kmax = max(kmax, k1);
@@ -1071,18 +1159,25 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
         } else if (c_tot) {
           // the lanes put their keys into the slot, then share the rest of the work evenly
           E* sl = s_slots + (RES ? cl : warp) * kSlot;
-          uint32_t pos = warp_excl_scan(cc);
-#pragma unroll
-          for (int w = 0; w < WPL; ++w)
-            for (uint32_t m = cw[w]; m; m &= m - 1)
-              sl[pos++] = static_cast<E>(row_elem<DT>(region, 32 * w + __ffs(m) - 1) & kMask);
+          E* to = sl + warp_excl_scan(cc);
+          take_set<DT, WPL, 2>(region, cw, [&](uint32_t i, E v) { to[i] = v & static_cast<E>(kMask); });
           __syncwarp();
+          uint32_t at = kNotListed;
+          if (MODE == kStreamed && (DT == 0 || range < 256u)) {
+            if (lane == 0) at = atomicAdd(&s_list_n, c_tot);
+            at = __shfl_sync(kFull, at, 0);
+            if (at + c_tot > kListBytes / sizeof(L)) at = kNotListed;
+          }
+          if (MODE == kStreamed && lane == 0) list_start[cl] = static_cast<unsigned short>(at);
           for (uint32_t t = lane; t < c_tot; t += 32) {
             const uint32_t key = sl[t];
             atomicAdd(&hist[(key - lo) >> shift], 1u);
             kmax = max(kmax, key);
             kinv = max(kinv, ~key);
-            if (!RES) g_slots[static_cast<long long>(cl) * kSlot + t] = static_cast<E>(key);
+            if (!RES) {
+              if (at != kNotListed) list[at + t] = static_cast<L>(DT == 0 ? key : key - lo);
+              else g_slots[static_cast<long long>(cl) * kSlot + t] = static_cast<E>(key);
+            }
           }
           __syncwarp();
         }
@@ -1095,68 +1190,83 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
       kinv = __reduce_max_sync(kFull, kinv);
       if (lane == 0) {
         if (w_above) atomicAdd(&s_tot[0], w_above);
+        if (w_in) atomicAdd(&s_tot[1], w_in);
         if (kmax) atomicMax(&s_tot[2], kmax);
         if (kinv) atomicMax(&s_tot[3], kinv);
       }
     } else {
       auto add = [&](uint32_t key) {
         const uint32_t rel = key - lo;           // (below lo: wraps far above the range)
-        if (rel <= range) atomicAdd(&hist[rel >> shift], 1u);
+        if (rel <= range) {
+          atomicAdd(&hist[rel >> shift], 1u);
+          ++w_in;
+        }
       };
       if (RES) {
         for (int c = warp; c < n_local; c += kWarps) slot_keys_warp<DT>(s_slots + c * kSlot, cnt[c] >> 16, add);
+      } else if (spread) {
+        slot_keys_global<DT>(g_slots, cnt, n_local, [&](int, uint32_t&, uint32_t key) { add(key); }, [](int, uint32_t, uint32_t) {});
       } else {
-        slot_keys_global<DT>(g_slots, cnt, n_local, n_local > kThreads / 2, [&](int, uint32_t&, uint32_t key) { add(key); }, [](int, uint32_t, uint32_t) {});
+        listed_keys([&](int, uint32_t&, uint32_t key) { add(key); }, [](int, uint32_t, uint32_t) {});
       }
+      w_in = warp_sum(w_in);
+      if (lane == 0 && w_in) atomicAdd(&s_tot[1], w_in);
     }
     if (RES && round == 0 && tid == 0) {         // CTA 0 has zeroed the histograms
       unsigned long long ignored;
-      if (!word_wait(a.answer, a.token, &ignored)) s_fail = 1;
+      if (prepared.x != a.token && !word_wait(a.answer, a.token, &ignored)) s_fail = 1;
       fence_gpu();
     }
     __syncthreads();
-    if (s_fail) { quit(); return; }
+    if (s_fail) return kTimedOut;
     uint32_t* gh = a.hist + round * kSelBins;
     if (tid < kSelBins) {
       const uint32_t h = hist[tid];
       if (h) atomicAdd(&gh[tid], h);
     }
-    __syncthreads();
     if (tid == 0) {
-      // reported: keys above, whether a list overflowed, and the one key inside (0: none, ~0: several)
-      fence_gpu();
+      // reported: how many keys this CTA has put into the bins and the count above them, whether a list overflowed, and
+      // the one key inside (0: none, ~0: several)
+      const uint32_t n_up = step == kRead ? s_tot[0] : 0u;
+      if (n_up) atomicAdd(above_count(a, round), n_up);
       const uint32_t one = s_tot[2] == 0u ? 0u : (s_tot[2] == ~s_tot[3] ? s_tot[2] : 0xFFFFFFFFu);
+      if (spread) fence_gpu();                   // (the counts and lists, which other CTAs will read)
       word_store(a.arrive + phase * kSelMaxCtas + blockIdx.x, a.token,
-                 (static_cast<unsigned long long>(one) << 32) | s_tot[0] | (s_over << 31));
+                 (static_cast<unsigned long long>(one) << 32) | (n_up + s_tot[1]) | (s_over << 31));
     }
     if (master) {
       unsigned long long v = 0;
       int ok = 1;
       if (tid < G) {
         ok = word_wait(a.arrive + phase * kSelMaxCtas + tid, a.token, &v, a.stall != 0);
-        fence_gpu();                             // (before the clearing: a fence waits for the stores before it)
+        if (spread) fence_gpu();
         a.arrive[phase * kSelMaxCtas + tid].x = 0ull;
       }
-      prepare_phase(a, phase + 1);
-      prepare_round(a, round + 1);
-      if (!__syncthreads_and(ok)) { quit(); return; }
-      const uint32_t b = tid < kSelBins ? __ldcg(gh + kSelBins - 1 - tid) : 0u;
+      if (!__syncthreads_and(ok)) return kTimedOut;
       const uint32_t one = static_cast<uint32_t>(v >> 32);
       const uint32_t w_max = __reduce_max_sync(kFull, one), w_inv = __reduce_max_sync(kFull, one ? ~one : 0u);
       const uint32_t w_over = __any_sync(kFull, (static_cast<uint32_t>(v) >> 31) != 0u) ? 1u : 0u;
       const uint32_t w_sum = __reduce_add_sync(kFull, static_cast<uint32_t>(v) & 0x7FFFFFFFu);
       __shared__ uint4 s_red[kWarps];
+      __shared__ uint32_t s_up;
       if (lane == 0) s_red[warp] = make_uint4(w_sum, w_max, w_inv, w_over);
-      uint32_t n_in;
-      const uint32_t above = count_above_mine(b, s_warp, &n_in);
-      uint32_t sum = 0, key_max = 0, key_inv = 0, over = 0;
+      uint32_t b, n_in, above, n_up, all = 0;
+      for (uint32_t spins = 0;; ++spins) {       // until everything that was reported has arrived in the bins
+        b = tid < kSelBins ? count_load(gh + kSelBins - 1 - tid) : 0u;
+        if (tid == 0) s_up = count_load(above_count(a, round));
+        above = count_above_mine(b, s_warp, &n_in);
+        n_up = s_up;
+        if (spins == 0) all = __reduce_add_sync(kFull, lane < kWarps ? s_red[lane].x : 0u);
+        if (n_in + n_up == all || spins > (1u << 18)) break;
+        __syncthreads();
+      }
+      if (n_in + n_up != all) return kTimedOut;
       const uint4 red = lane < kWarps ? s_red[lane] : make_uint4(0, 0, 0, 0);
-      sum = __reduce_add_sync(kFull, red.x);
-      key_max = __reduce_max_sync(kFull, red.y);
-      key_inv = __reduce_max_sync(kFull, red.z);
-      over = __any_sync(kFull, red.w != 0u) ? 1u : 0u;
+      const uint32_t key_max = __reduce_max_sync(kFull, red.y);
+      const uint32_t key_inv = __reduce_max_sync(kFull, red.z);
+      const bool over = __any_sync(kFull, red.w != 0u);
       const bool was_read = step == kRead;
-      if (was_read) { n_above = sum; listed = over == 0; }
+      if (was_read) { n_above = n_up; listed = !over; }
       const long long r = static_cast<long long>(a.k) - n_above;     // rank among the keys of [0, hi]
       if (r < 1) {                               // the bracket lies too low: the threshold is above it
         lo = hi + 1u; hi = kKeyMax; step = kRead;
@@ -1173,11 +1283,15 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
         hi = min(hi, lo + ((1u << shift) - 1u));
         if (shift == 0) step = listed ? kListed : kRecount;
         else if (!listed) step = kRead;
-        else step = s_res[2] <= static_cast<uint32_t>(kKeysAtOnce / 2) && shift <= 2 * kSelBinsLog2 ? kKeys : kRefine;
+        else step = s_res[2] <= kKeysAtOnce && shift <= 2 * kSelBinsLog2 ? kKeys : kRefine;
       }
-      __syncthreads();
+      if (step <= kRefine && !spread && round == 0) {        // an unusual call: prepare the rest
+        prepare_exchanges(a, 3, kSelPhases, 1, kSelHists);
+        __syncthreads();
+        if (tid == 0) fence_gpu();
+      }
       if (tid == 0) {
-        fence_gpu();                             // the cleared words and bins of what comes next
+        if (spread) fence_gpu();
         word_store(a.answer + phase * (kSelMaxCtas + 2), a.token, lo | (static_cast<unsigned long long>(hi) << 32));
         word_store(a.answer + phase * (kSelMaxCtas + 2) + 1, a.token, n_above | (static_cast<unsigned long long>(step) << 32));
         if (phase == 1) a.answer[0].x = 0ull;
@@ -1186,11 +1300,11 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
       if (tid < 2) {
         unsigned long long v = 0;
         if (!word_wait(a.answer + phase * (kSelMaxCtas + 2) + tid, a.token, &v, a.stall != 0)) s_fail = 1;
-        if (!RES) fence_gpu();                   // (spread: the counts and lists of the other CTAs)
+        if (spread) fence_gpu();                 // the counts and lists of the other CTAs
         s_ans[tid] = v;
       }
       __syncthreads();
-      if (s_fail) { quit(); return; }
+      if (s_fail) return kTimedOut;
       lo = static_cast<uint32_t>(s_ans[0]);
       hi = static_cast<uint32_t>(s_ans[0] >> 32);
       n_above = static_cast<uint32_t>(s_ans[1]);
@@ -1199,7 +1313,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     ++phase;
     if (round + 1 >= kSelHists && step <= kRefine) {   // cannot happen: a miss, three levels and a pass for ties are the most
       if (tid == 0) atomicMax(&a.hdr->status, static_cast<uint32_t>(SURGEON_ERR_INTERNAL));
-      return;
+      return kUnsound;
     }
   }
 
@@ -1207,14 +1321,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
   if (step == kRecount) {                        // the lists overflowed: count once more from the chunks
     __syncthreads();
     auto recount = [&](int c, unsigned char* region) -> bool {
-      uint4 q[8];
-      load_row(region, q);
-      uint32_t ge[WPL], gt[WPL], g = 0, e = 0;   // (lo >= 1: what lies past the tensor's end is below it)
-      mask_ge<DT, WPL>(q, EPR, lo, ge);
-      mask_ge<DT, WPL>(q, EPR, lo + 1u, gt);
-#pragma unroll
-      for (int w = 0; w < WPL; ++w) { g += __popc(gt[w]); e += __popc(ge[w] & ~gt[w]); }
-      const uint32_t both = __reduce_add_sync(kFull, g | (e << 16));
+      const uint32_t both = count_chunk<DT>(region, lo);
       if (lane == 0) cnt[c - c_begin] = both;
       return false;
     };
@@ -1226,11 +1333,11 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
       begin_pass(false);
       run_pass(false, recount);
     }
-    if (spread && !meet()) { quit(); return; }
+    if (spread && !meet()) return kTimedOut;
   }
   if (tid == 0) s_nkeys = 0;
   __syncthreads();
-  if (s_fail) { quit(); return; }
+  if (s_fail) return kTimedOut;
   uint32_t n_gt = 0, n_eq = 0;
   if (step == kListed || step == kKeys) {
     // acc: keys above hi, and (upper half) keys of [lo, hi]
@@ -1240,8 +1347,8 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
         acc += 0x10000u;
         if (step == kKeys) {
           const uint32_t at = atomicAdd(&s_nkeys, 1u);
-          if (at < static_cast<uint32_t>(kMaxKeys)) {
-            a.keys[blockIdx.x * kMaxKeys + at] = key;
+          if (at < static_cast<uint32_t>(key_room(G))) {
+            key_store(a.keys + blockIdx.x * key_room(G) + at, a.token, key);
             s_bin_key[at] = key;
             s_bin_chunk[at] = c;
           }
@@ -1251,6 +1358,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     auto done = [&](int c, uint32_t v, uint32_t acc) {       // (one lane)
       acc += v & 0xFFFFu;
       if (step == kListed) cnt[c] = acc;
+      else if (MODE == kStreamed) list_acc[c] = static_cast<unsigned short>(acc);
       else prefix[c] = acc & 0xFFFFu;            // (cnt stands: there may be another round)
       n_gt += acc & 0xFFFFu;
       n_eq += acc >> 16;
@@ -1263,8 +1371,10 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
         acc = __reduce_add_sync(kFull, acc);
         if (lane == 0) done(c, v, acc);
       }
+    } else if (spread) {
+      slot_keys_global<DT>(g_slots, cnt, n_local, report, done);
     } else {
-      slot_keys_global<DT>(g_slots, cnt, n_local, n_local > kThreads / 2, report, done);
+      listed_keys(report, done);
     }
   } else {
     for (int c = tid; c < n_local; c += kThreads) {
@@ -1287,7 +1397,6 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
   if (tid == 0) {
     unsigned long long t = 0;
     for (int w = 0; w < kWarps; ++w) t += s_warp64[w];
-    fence_gpu();
     word_store(a.arrive + phase * kSelMaxCtas + blockIdx.x, a.token, t);
   }
 
@@ -1295,74 +1404,107 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
   tau = lo; n_greater = n_above;
   bool again = false;                            // a CTA has more keys than it can report: narrow the bin first
   if (master) {
+    // two threads per CTA, which share its keys
+    const int who = tid >> 1;
     unsigned long long v = 0;
     int ok = 1;
-    if (tid < G) {
-      ok = word_wait(a.arrive + phase * kSelMaxCtas + tid, a.token, &v);
-      fence_gpu();
-      a.arrive[phase * kSelMaxCtas + tid].x = 0ull;
+    if (who < G) {
+      ok = word_wait(a.arrive + phase * kSelMaxCtas + who, a.token, &v);
+      if (!(tid & 1)) a.arrive[phase * kSelMaxCtas + who].x = 0ull;
     }
-    prepare_phase(a, phase + 1);
-    if (step == kKeys && tid < kSelBins) hist[tid] = hist[kSelBins + tid] = 0;
-    if (!__syncthreads_and(ok)) { quit(); return; }
     if (step == kKeys) {
-      const uint32_t n_k = tid < G ? static_cast<uint32_t>(v) : 0u;
-      uint32_t* nk = hist + 2 * kSelBins;        // [3][kSelMaxCtas]: keys, above, ties per CTA
-      if (tid < kSelMaxCtas) { nk[tid] = n_k; nk[kSelMaxCtas + tid] = 0; nk[2 * kSelMaxCtas + tid] = 0; }
-      const uint32_t w_most = __reduce_max_sync(kFull, n_k);
-      if (lane == 0) s_warp[warp] = w_most;
+      const uint32_t n_k = static_cast<uint32_t>(v);
+      const bool fits = n_k <= static_cast<uint32_t>(key_room(G));
+      const unsigned long long* mine = a.keys + who * key_room(G) + (tid & 1);
+      // the keys, with their CTA, in shared memory; their histogram by the upper bits of key - lo
+      uint32_t* got = hist + kSelBins;           // [kKeysAtOnce]
+      uint32_t* nk = got + kKeysAtOnce;          // [kSelMaxCtas] keys of a CTA above the threshold, and (upper half) ties
+      unsigned char* owner = reinterpret_cast<unsigned char*>(nk + kSelMaxCtas);
+      const int coarse = shift > kSelBinsLog2 ? shift - kSelBinsLog2 : 0;
+      if (tid < kSelBins) hist[tid] = 0;
+      if (tid < kSelMaxCtas) nk[tid] = 0;
+      if (tid == 0) s_res[6] = s_res[7] = 0;
       __syncthreads();
-      const int most = static_cast<int>(__reduce_max_sync(kFull, lane < kWarps ? s_warp[lane] : 0u));
-      __syncthreads();
-      constexpr int kPer = kKeysPerThread;
-      again = most > kMaxKeys || most * G > kKeysAtOnce;
-      if (!again) {
-        // (idx / most by multiplication: idx * most < 2^32)
-        const uint32_t inv = most > 1 ? 0xFFFFFFFFu / static_cast<uint32_t>(most) + 1u : 0u;
-        uint32_t key[kPer];
-        int who[kPer];
+      const int turns = __reduce_max_sync(kFull, fits ? static_cast<int>((n_k + 7u) / 8u) : 0);
+#pragma unroll 1
+      for (int turn = 0; turn < turns; ++turn) { // four keys of each thread at a time
+        unsigned long long w[4];
+        bool late;
+        uint32_t spins = 0;
+        do {
+          late = false;
 #pragma unroll
-        for (int u = 0; u < kPer; ++u) {
-          const int idx = u * kThreads + tid;
-          who[u] = most > 1 ? static_cast<int>(__umulhi(static_cast<uint32_t>(idx), inv)) : idx;
-          const int i = idx - who[u] * most;
-          const bool have = who[u] < G && i < static_cast<int>(nk[min(who[u], kSelMaxCtas - 1)]);
-          key[u] = have ? __ldcg(a.keys + who[u] * kMaxKeys + i) : 0u;
+          for (int u = 0; u < 4; ++u)
+            w[u] = key_load_if(mine + 8 * turn + 2 * u, fits && 8u * turn + 2u * u + (tid & 1u) < n_k, a.token);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) late |= static_cast<uint32_t>(w[u] >> 32) != static_cast<uint32_t>(a.token);
+        } while (late && ++spins < (1u << 20));
+        if (late) ok = 0;
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const uint32_t key = static_cast<uint32_t>(w[u]), have = __ballot_sync(kFull, key != 0u);
+          uint32_t at = 0;
+          if (lane == 0 && have) at = atomicAdd(&s_res[6], __popc(have));
+          at = __shfl_sync(kFull, at, 0) + __popc(have & lanemask_lt());
+          if (key && at < kKeysAtOnce) {
+            got[at] = key;
+            owner[at] = static_cast<unsigned char>(who);
+            atomicAdd(&hist[(key - lo) >> coarse], 1u);
+          }
         }
-        // the rank among them: by the upper bits of key - lo, then by the rest
-        const int coarse = shift > kSelBinsLog2 ? shift - kSelBinsLog2 : 0;
-#pragma unroll
-        for (int u = 0; u < kPer; ++u)
-          if (key[u]) atomicAdd(&hist[(key[u] - lo) >> coarse], 1u);
-        __syncthreads();
+      }
+      again = __syncthreads_or(!fits) != 0;
+      if (!__syncthreads_and(ok)) return kTimedOut;
+      if (!again) {
+        const uint32_t n_got = min(s_res[6], kKeysAtOnce);
         uint32_t all;
         uint32_t b = my_bin(hist);
         place_rank(b, count_above_mine(b, s_warp, &all), a.k - n_above, s_res);
         __syncthreads();
-        tau = lo + (s_res[0] << coarse);
+        const uint32_t in_bin = s_res[2], bin = lo + (s_res[0] << coarse);
+        tau = bin;
         n_greater = n_above + s_res[1];
-        if (coarse) {
-#pragma unroll
-          for (int u = 0; u < kPer; ++u)
-            if (key[u] >= tau && ((key[u] - tau) >> coarse) == 0u) atomicAdd(&hist[kSelBins + key[u] - tau], 1u);
+        if (coarse) {                            // its keys, which a warp can hold (few lie in a bin of 512)
+          __shared__ uint32_t s_few[32];
+          if (in_bin > 32u) hist[tid] = 0;       // (massive ties: their low bits are counted)
           __syncthreads();
-          b = my_bin(hist + kSelBins);
-          place_rank(b, count_above_mine(b, s_warp, &all), a.k - n_greater, s_res + 3);
+#pragma unroll 1
+          for (uint32_t i = tid; i < n_got; i += kThreads) {
+            const uint32_t rel = got[i] - bin;   // (below the bin: wraps)
+            if (rel >> coarse == 0u) {
+              if (in_bin <= 32u) s_few[atomicAdd(&s_res[7], 1u)] = got[i];
+              else atomicAdd(&hist[rel], 1u);
+            }
+          }
           __syncthreads();
-          tau += s_res[3];
-          n_greater += s_res[4];
+          if (in_bin <= 32u) {                   // every warp ranks them
+            const uint32_t k0 = lane < in_bin ? s_few[lane] : 0u;
+            uint32_t larger = 0;
+#pragma unroll 1
+            for (uint32_t i = 0; i < in_bin; ++i) larger += __shfl_sync(kFull, k0, i) > k0 ? 1u : 0u;
+            // the threshold: the smallest key with fewer than the wanted rank above it
+            tau = __reduce_min_sync(kFull, lane < in_bin && larger < a.k - n_greater ? k0 : 0xFFFFFFFFu);
+            n_greater += __popc(__ballot_sync(kFull, lane < in_bin && k0 > tau));
+          } else {
+            b = my_bin(hist);
+            place_rank(b, count_above_mine(b, s_warp, &all), a.k - n_greater, s_res + 3);
+            __syncthreads();
+            tau += s_res[3];
+            n_greater += s_res[4];
+          }
         }
-#pragma unroll
-        for (int u = 0; u < kPer; ++u) {
-          if (key[u] > tau) atomicAdd(&nk[kSelMaxCtas + who[u]], 1u);
-          else if (key[u] == tau) atomicAdd(&nk[2 * kSelMaxCtas + who[u]], 1u);
-        }
+#pragma unroll 1
+        for (uint32_t i = tid; i < n_got; i += kThreads)
+          if (got[i] >= tau) atomicAdd(&nk[owner[i]], got[i] > tau ? 1u : 0x10000u);
         __syncthreads();
-        if (tid < G)
-          v = ((v >> 32 << 32) + (static_cast<unsigned long long>(nk[kSelMaxCtas + tid]) << 32)) | nk[2 * kSelMaxCtas + tid];
+        if (who < G) v = (((v >> 32) + (nk[who] & 0xFFFFu)) << 32) | (nk[who] >> 16);
       }
+    } else if (!__syncthreads_and(ok)) {
+      return kTimedOut;
     }
     // exclusive scan over the CTAs
+    if (tid & 1) v = 0;
     const unsigned long long incl = warp_incl_u64(v);
     if (lane == 31) s_warp64[warp] = incl;
     __syncthreads();
@@ -1378,11 +1520,13 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     const bool sound = static_cast<long long>(all >> 32) == n_greater && quota >= 0 &&
                        n_greater + (eq_all < quota ? eq_all : quota) == n_stored;
     const uint32_t verdict = again ? 1u : (sound ? 0u : 2u);
-    if (step == kKeys) {                         // (the cleared words of a further round)
+    if (again && !spread && phase == 2) {        // an unusual call: prepare what its next rounds need
+      prepare_exchanges(a, 3, kSelPhases, 1, kSelHists);
+      __syncthreads();
       if (tid == 0) fence_gpu();
       __syncthreads();
     }
-    if (tid < G) word_store(a.answer + phase * (kSelMaxCtas + 2) + 2 + tid, a.token, base + incl - v);
+    if (who < G && !(tid & 1)) word_store(a.answer + phase * (kSelMaxCtas + 2) + 2 + who, a.token, base + incl - v);
     if (tid == 0) {
       word_store(a.answer + phase * (kSelMaxCtas + 2), a.token, tau | (static_cast<unsigned long long>(n_greater) << 32));
       word_store(a.answer + phase * (kSelMaxCtas + 2) + 1, a.token, verdict);
@@ -1397,7 +1541,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
       }
     }
     before = 0;                                  // CTA 0's chunks are the first
-    if (verdict == 2u) return;
+    if (verdict == 2u) return kUnsound;
   } else {
     __shared__ unsigned long long s_last[3];
     if (tid < 3) {
@@ -1407,14 +1551,16 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
       s_last[tid] = v;
     }
     __syncthreads();
-    if (s_fail) { quit(); return; }
-    if (s_last[1] == 2ull) return;
+    if (s_fail) return kTimedOut;
+    if (s_last[1] == 2ull) return kUnsound;
     again = s_last[1] == 1ull;
     tau = static_cast<uint32_t>(s_last[0]);
     n_greater = static_cast<uint32_t>(s_last[0] >> 32);
     before = s_last[2];
   }
   ++phase;
+  if (step == kKeys && tid < min(static_cast<int>(s_nkeys), key_room(G)))     // they have been read
+    a.keys[blockIdx.x * key_room(G) + tid] = 0ull;
   if (!again) break;
   step = kRefine;
   }
@@ -1426,7 +1572,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
   if (step == kKeys) {                           // what was above the bin, and the CTA's few keys inside it
     const int n_bin = static_cast<int>(s_nkeys);
     for (int c = tid; c < n_local; c += kThreads) {
-      uint32_t both = static_cast<uint32_t>(prefix[c]);
+      uint32_t both = MODE == kStreamed ? list_acc[c] : static_cast<uint32_t>(prefix[c]);
 #pragma unroll 1
       for (int i = 0; i < n_bin; ++i)
         if (s_bin_chunk[i] == c && s_bin_key[i] >= tau) both += s_bin_key[i] > tau ? 1u : 0x10000u;
@@ -1434,8 +1580,28 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     }
     __syncthreads();
   }
+  if (RES) {                                     // every warp for itself: at most 48 chunks
+    uint32_t up[2], tie[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int c = 32 * j + static_cast<int>(lane);
+      const uint32_t v = c < n_local ? cnt[c] : 0u;
+      up[j] = v & 0xFFFFu;
+      tie[j] = v >> 16;
+    }
+    unsigned long long base = before;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int c = 32 * j + static_cast<int>(lane);
+      const uint32_t u0 = warp_excl_scan(up[j]), t0 = warp_excl_scan(tie[j]);
+      if (c < n_local && c % kWarps == warp) prefix[c] = base + ((static_cast<unsigned long long>(u0) << 32) | t0);
+      base += (static_cast<unsigned long long>(__shfl_sync(kFull, u0 + up[j], 31)) << 32) | __shfl_sync(kFull, t0 + tie[j], 31);
+    }
+    __syncwarp();
+  } else {
   unsigned long long carry = before;
   constexpr int kScan = 4;                       // consecutive chunks per thread
+#pragma unroll 1
   for (int c0 = 0; c0 < n_local; c0 += kScan * kThreads) {
     const int c = c0 + kScan * tid;
     unsigned long long val[kScan], sum = 0;
@@ -1459,44 +1625,69 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     __syncthreads();
   }
 
+  }
   // ---- emit ----
-  unsigned char* stage = aux + warp * kStageBytes;
-  auto emit = [&](int c, unsigned char* region) -> bool {
-    const unsigned long long at = prefix[c - c_begin];
-    return emit_chunk<DT>(a, region, stage, c, tau, quota, at, cnt[c - c_begin] >> 16, n_stored);
-  };
   if (RES) {
-    run_resident(false, emit);
-  } else if (spread) {
-    if (!meet()) { quit(); return; }             // every CTA's places are known to all
+    run_resident(false, [&](int c, unsigned char* region) -> bool {
+      return emit_chunk<DT>(a, region, c, tau, quota, prefix[c - c_begin], cnt[c - c_begin] >> 16, n_stored);
+    });
+    return kDone;
+  }
+  // From the end, where the ring (not claimed: its places still hold the last three) and the L2 cache have it.
+  unsigned long long at_next = 0;                // (claimed) place and ties of the next chunk, fetched one chunk ahead
+  uint32_t n_next = 0;
+  if (spread) {
+    if (!meet()) return kTimedOut;               // every CTA's places are known to all
     tc::fence_proxy_async();
     __syncwarp();
-    begin_pass(true);                            // from the end, where the L2 cache holds some of it
-    unsigned long long at_next = fly0 < a.n_chunks ? prefix[fly0 - c_begin] : 0ull;    // fetched one chunk ahead
-    uint32_t n_next = fly0 < a.n_chunks ? cnt[fly0 - c_begin] : 0u;
-    run_pass(true, [&](int c, unsigned char* region) -> bool {
-      const unsigned long long at = at_next;
-      const uint32_t n_at = n_next >> 16;
-      if (fly1 < a.n_chunks) { at_next = prefix[fly1 - c_begin]; n_next = cnt[fly1 - c_begin]; }
-      return emit_chunk<DT>(a, region, stage, c, tau, quota, at, n_at, n_stored);
-    });
-    if (s_fail && lane == 0) atomicMax(&a.hdr->status, static_cast<uint32_t>(SURGEON_ERR_TIMEOUT));
-  } else {
-    // the chunks still in the ring first, then backwards through the rest
-    for (int i = n_mine - 1; i >= 0; --i) {
-      const int sl = i % kSlotsPerWarp;
-      if (i + kSlotsPerWarp < n_mine && !arrived(chunk_of(i), sl)) {
-        atomicMax(&a.hdr->status, static_cast<uint32_t>(SURGEON_ERR_TIMEOUT));
-        for (int j = i - 1; j >= 0 && j > i - kSlotsPerWarp; --j) arrived(chunk_of(j), j % kSlotsPerWarp);
-        break;
-      }
-      const bool written = emit(chunk_of(i), my_ring + sl * kChunkBytes);
-      if (i >= kSlotsPerWarp) {
-        if (written) tc::fence_proxy_async();
-        __syncwarp();
-        issue(chunk_of(i - kSlotsPerWarp), sl);
-      }
+    begin_pass(true);
+    if (fly0 < a.n_chunks) { at_next = prefix[fly0 - c_begin]; n_next = cnt[fly0 - c_begin]; }
+  }
+  int i = n_mine - 1;                            // (not claimed) the next one
+  int s = spread || i < 0 ? 0 : i % kSlotsPerWarp;
+#pragma unroll 1
+  while (spread ? fly0 < a.n_chunks : i >= 0) {
+    const int c = spread ? fly0 : chunk_of(i);
+    if ((spread || i + kSlotsPerWarp < n_mine) && !arrived(c, s)) {
+      atomicMax(&a.hdr->status, static_cast<uint32_t>(SURGEON_ERR_TIMEOUT));
+      break;
     }
+    unsigned long long at = at_next;
+    uint32_t n_at = n_next;
+    if (!spread) { at = prefix[c - c_begin]; n_at = cnt[c - c_begin]; }
+    else if (fly1 < a.n_chunks) { at_next = prefix[fly1 - c_begin]; n_next = cnt[fly1 - c_begin]; }
+    const bool written = emit_chunk<DT>(a, my_ring + s * kChunkBytes, c, tau, quota, at, n_at >> 16, n_stored);
+    int c_load;                                  // what the place takes next
+    if (spread) {
+      fly0 = fly1; fly1 = fly2;
+      c_load = next();
+      fly2 = c_load;
+      if (c_load < a.n_chunks) fly2 = c_load = a.n_chunks - 1 - c_load;
+    } else {
+      c_load = i >= kSlotsPerWarp ? chunk_of(i - kSlotsPerWarp) : a.n_chunks;
+      --i;
+    }
+    if (c_load < a.n_chunks) {
+      if (written) tc::fence_proxy_async();      // this warp's writes to the place precede the next TMA fill
+      __syncwarp();                              // every lane has read the place
+      issue(c_load, s);
+    }
+    s = spread ? (s == 2 ? 0 : s + 1) : (s == 0 ? 2 : s - 1);
+  }
+  return kDone;
+  }();
+
+  // A wait gave up somewhere: the loads under way are waited for (with a limit) as well, and the CTA takes back what it
+  // has stored for the others: a replay of a captured call carries the same token and must not find it.
+#pragma unroll 1
+  for (int s = 0; s < kSlotsPerWarp; ++s)
+    if ((under_way >> s) & 1u) landed(s);
+  if (left_as == kTimedOut) {
+    if (tid == 0) atomicMax(&a.hdr->status, static_cast<uint32_t>(SURGEON_ERR_TIMEOUT));
+    if (tid < kSelPhases) a.arrive[tid * kSelMaxCtas + blockIdx.x].x = 0ull;
+    if (tid < key_room(G)) a.keys[blockIdx.x * key_room(G) + tid] = 0ull;
+    if (master)
+      for (int i = tid; i < kSelPhases * (kSelMaxCtas + 2); i += kThreads) a.answer[i].x = 0ull;
   }
 }
 
@@ -1620,8 +1811,10 @@ unsigned long long next_token() {
         std::chrono::steady_clock::now().time_since_epoch().count());
     return ((static_cast<unsigned long long>(rd()) << 32) | rd()) ^ (t << 20);
   }()};
-  unsigned long long v = counter.fetch_add(1, std::memory_order_relaxed);
-  return v ? v : counter.fetch_add(1, std::memory_order_relaxed);
+  unsigned long long v;
+  do v = counter.fetch_add(1, std::memory_order_relaxed);
+  while (static_cast<uint32_t>(v) == 0u);        // (a cleared key must not carry its lower half)
+  return v;
 }
 
 template <int DT>
@@ -1651,7 +1844,7 @@ cudaError_t run_prune_compact(const void* x, long long n, long long k, int drop_
   a.hdr = out.header; a.bitmap = out.bitmap; a.values = out.values; a.offsets = out.block_offsets;
   a.arrive = reinterpret_cast<ulonglong2*>(ws + L.arrive);
   a.answer = reinterpret_cast<ulonglong2*>(ws + L.answer);
-  a.keys = reinterpret_cast<uint32_t*>(ws + L.keys);
+  a.keys = reinterpret_cast<unsigned long long*>(ws + L.keys);
   a.hist = reinterpret_cast<uint32_t*>(ws + L.hist);
   a.claims = reinterpret_cast<uint32_t*>(ws + L.claims);
   a.cnt = reinterpret_cast<uint32_t*>(ws + L.cnt);
@@ -1677,10 +1870,11 @@ cudaError_t run_prune_compact(const void* x, long long n, long long k, int drop_
   }
   // claimed chunks (see the kernel): by itself from 512 chunks per CTA on, where equal shares end unevenly; on a part
   // of the GPU only where the counts do not fit (on a quarter, 131 MB: 335 -> 310 us bf16, 260 -> 238 fp32)
-  a.spread = a.n_chunks > grid * (share ? kMaxLocalChunks : 512) ? 1 : 0;
+  const bool claimed = a.n_chunks > grid * (share ? kMaxLocalChunks : 512);
   const bool resident = (a.n_chunks + grid - 1) / grid <= kResidentChunks;
-  const void* kernel = resident ? reinterpret_cast<const void*>(prune_kernel<DT, true>)
-                                : reinterpret_cast<const void*>(prune_kernel<DT, false>);
+  const void* kernel = resident  ? reinterpret_cast<const void*>(prune_kernel<DT, kResident>)
+                       : claimed ? reinterpret_cast<const void*>(prune_kernel<DT, kClaimed>)
+                                 : reinterpret_cast<const void*>(prune_kernel<DT, kStreamed>);
   cudaError_t e = allow_dynamic_smem(kernel, static_cast<int>(kPruneSmem));
   if (e != cudaSuccess) return e;
   void* args[] = {&map, &a};

@@ -228,6 +228,46 @@ def test_streamed_tensor_at_extreme_ratios(dist, n, bf16):
         assert_store_equals_oracle(x.cpu(), ratio)
 
 
+def _awkward(kind, n):
+    """Values that lead the select off its usual way: brackets of many keys (bf16: more than the list's bytes can
+    tell apart), all keys near the threshold in one place (lists and the keys of one CTA overflow), many more
+    of them in a bin than CTA 0 takes at once, or a bin of few distinct keys with many copies each."""
+    g = torch.Generator().manual_seed(n)
+    if kind == "log_uniform":
+        return torch.exp2(240.0 * torch.rand(n, generator=g) - 120.0)
+    if kind == "sorted":
+        return torch.linspace(-1.0, 1.0, n)
+    x = torch.randn(n, generator=g)
+    if kind == "clustered":                      # a tenth of the tensor, in one place, has two in three of its keys in 1e-3 of the range
+        x[n // 2:n // 2 + n // 10] = 1.0 + 1e-3 * torch.rand(n // 10, generator=g)
+    if kind == "few_keys":                       # neighbouring fp32 numbers around the threshold, ten thousand copies each
+        at = torch.randint(0, n, (n // 4,), generator=g)
+        x[at] = (torch.tensor(1.0).view(torch.int32) + torch.randint(0, max(2, n // 40000), (n // 4,), generator=g)).int().view(torch.float32)
+    return x
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("n", [40000, 3_000_001, 18_000_003])        # one CTA or two, resident, streamed
+@pytest.mark.parametrize("kind", ["log_uniform", "sorted", "clustered", "few_keys"])
+def test_select_off_its_usual_way(kind, n, bf16):
+    x = _awkward(kind, n)
+    x = x.to(torch.bfloat16) if bf16 else x
+    ratio = 1.0 - float((x.abs() > 1.0005).double().mean()) if kind == "clustered" else 0.7
+    comp, _ = assert_store_equals_oracle(x, ratio)
+    ref = [v.copy() for v in comp.to_numpy()[:3]]
+    xc, ws = x.cuda(), torch.empty(comp.sizes.workspace_bytes, dtype=torch.uint8, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        B.surgeon_prune_compact(xc, ratio, out=comp, workspace=ws)
+    for _ in range(2):                           # replays carry the same token: nothing of the first is taken for the second
+        for part in (comp.bitmap, comp.values, comp.block_offsets):
+            part.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert comp.read_header().status == B.SURGEON_OK
+        assert all(np.array_equal(u.view(np.uint8), v.view(np.uint8)) for u, v in zip(comp.to_numpy()[:3], ref))
+
+
 @pytest.mark.parametrize("n", [5000, (1 << 23) + 77])
 def test_captured_call_replays_and_alternating_streams(n):
     xs = [W.draw("normal", n, seed=20 + i).cuda() for i in range(3)]
