@@ -4,7 +4,8 @@
 // scheduling.  The first cuts dw into at most kGiBlocks contiguous slices, one per CTA: a thread
 // adds the squares of every 256th element of its slice in double (a product of two fp32 values is
 // exact in double), the CTA adds its threads' sums in a fixed tree and writes one partial.  The
-// second adds the partials in index order, divides by N and takes the root.
+// second adds the partials in index order, divides by N and takes the root.  Both are dependent launches:
+// the kernels are 2 us each, and so were the gaps before them (an importance pass over eight layers: 485 -> 451 us).
 #include "surgeon_internal.cuh"
 
 namespace surgeon {
@@ -31,6 +32,8 @@ __device__ __forceinline__ double block_sum_fixed(double v, double* s_warp) {
 __global__ void __launch_bounds__(kGiThreads)
 gi_partial_kernel(const float* __restrict__ dw, long long n, long long per_block,
                   double* __restrict__ partial) {
+  pdl_wait();                                    // (the dw; and the partials of a call before this one have been read)
+  pdl_trigger();
   __shared__ double s_warp[kGiThreads / 32];
   const long long begin = static_cast<long long>(blockIdx.x) * per_block;
   const long long end = begin + per_block < n ? begin + per_block : n;
@@ -46,6 +49,8 @@ gi_partial_kernel(const float* __restrict__ dw, long long n, long long per_block
 __global__ void __launch_bounds__(kGiThreads)
 gi_final_kernel(const double* __restrict__ partial, int n_partials, long long n,
                 double* __restrict__ gi_out) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ double s_warp[kGiThreads / 32];
   // thread t adds the partials t, t + 256, ... in that order
   double acc = 0.0;
@@ -66,10 +71,10 @@ cudaError_t launch_gradient_importance(const float* dw, long long n, double* gi_
     if (per_block < 4096) per_block = 4096;
     per_block = (per_block + kGiThreads - 1) / kGiThreads * kGiThreads;
     blocks = static_cast<int>((n + per_block - 1) / per_block);
-    gi_partial_kernel<<<blocks, kGiThreads, 0, stream>>>(dw, n, per_block, partial);
+    launch_kernel(gi_partial_kernel, dim3(blocks), dim3(kGiThreads), 0, stream, true, dw, n, per_block, partial);
     note_launches(1);
   }
-  gi_final_kernel<<<1, kGiThreads, 0, stream>>>(partial, blocks, n, gi_out);
+  launch_kernel(gi_final_kernel, dim3(1), dim3(kGiThreads), 0, stream, true, partial, blocks, n, gi_out);
   note_launches(1);
   return cudaGetLastError();
 }
