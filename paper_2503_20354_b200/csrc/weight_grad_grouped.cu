@@ -265,11 +265,15 @@ __device__ __forceinline__ int fast_div(int n, uint32_t rcp) {
 // hides that latency is the other CTAs' work.  That leaves a CTA 85 registers per thread (tiles of
 // at most 4 channel pairs: 36 accumulators) and about 74 KB of shared memory.
 constexpr int kG3CtasPerSm = 2;
+// One channel per group: 9 sums per thread need no 128 registers, and a tile of half the size leaves room for twice as
+// many CTAs, which hide one another's load phases.
+constexpr int kG3CtasPerSmDepthwise = 4;
 constexpr int kG3Smem = 110 * 1024;
+constexpr int kG3SmemDepthwise = 54 * 1024;
 constexpr int kG3MaxTile = 8;
 
 template <int TO, int TC, int ST>
-__global__ void __launch_bounds__(kThreads, kG3CtasPerSm)
+__global__ void __launch_bounds__(kThreads, TO * TC == 1 ? kG3CtasPerSmDepthwise : kG3CtasPerSm)
 dw_grouped3_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ values,
                    const uint32_t* __restrict__ offsets, const float* __restrict__ grad,
                    double* __restrict__ partial, Grouped3Params p) {
@@ -502,10 +506,17 @@ dw_grouped3_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__
   __syncthreads();
   const int ncol = p.Cg * 9;
   double* out = partial + static_cast<long long>(chunk * p.n_bands + band) * p.O * ncol;
-  for (int i = tid; i < p.units * ACC; i += kThreads) {
+  // One channel per group: 9 sums of 256 parts would be a chain of 5 us for a thread each; 16 lanes share one.
+  constexpr int per = TO * TC == 1 ? 16 : 1;          // lanes of a sum
+  for (int i0 = tid; i0 < (per == 1 ? p.units * ACC : (p.units * ACC * per + 31) / 32 * 32); i0 += kThreads) {      // (whole warps)
+    const int i = i0 / per, part = i0 % per;
     const int u = i / ACC, a = i - u * ACC;
     double s = 0.0;
-    for (int sp = 0; sp < p.S; ++sp) s += static_cast<double>(red[(u * p.S + sp) * ACC + a]);
+    if (per == 1 || i < p.units * ACC)
+      for (int sp = part; sp < p.S; sp += per) s += static_cast<double>(red[(u * p.S + sp) * ACC + a]);
+#pragma unroll
+    for (int o = per / 2; o > 0; o /= 2) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+    if (i >= p.units * ACC || part) continue;
     const int uo = u / p.n_cb, uc = u - uo * p.n_cb;
     const int o = a / (TC * 9), rem = a - o * (TC * 9);
     const int c = rem / 9, rs = rem - c * 9;
@@ -588,6 +599,7 @@ bool plan_grouped3(const surgeon_layer_desc& d, Grouped3Params* out, Grouped3Til
   int to = p.Og % 4 == 0 ? 4 : (p.Og % 2 == 0 ? 2 : 1);
   int tc = p.Cg % 4 == 0 ? 4 : (p.Cg % 2 == 0 ? 2 : 1);
   while (to * tc > kG3MaxTile) { if (tc >= to) tc >>= 1; else to >>= 1; }
+  const long long room = to * tc == 1 ? kG3SmemDepthwise : kG3Smem;
   p.n_cb = p.Cg / tc;
   p.units = (p.Og / to) * p.n_cb;
   if (p.units > kThreads) return false;
@@ -600,16 +612,16 @@ bool plan_grouped3(const surgeon_layer_desc& d, Grouped3Params* out, Grouped3Til
     const long long in_rows = static_cast<long long>(band - 1) * d.stride + 3;
     const long long a = static_cast<long long>(p.Cg) * in_rows * p.Wp;
     const long long g = static_cast<long long>(p.Og) * band * p.OW;
-    if ((a + g) * 4 <= kG3Smem) { p.in_rows = static_cast<int>(in_rows); p.a_floats = static_cast<int>(a); p.g_floats = static_cast<int>(g); break; }
+    if ((a + g) * 4 <= room) { p.in_rows = static_cast<int>(in_rows); p.a_floats = static_cast<int>(a); p.g_floats = static_cast<int>(g); break; }
   }
-  if (red_bytes > kG3Smem) return false;
+  if (red_bytes > room) return false;
   p.band = band;
   p.n_bands = (p.OH + band - 1) / band;
-  p.nb = static_cast<int>(kG3Smem / (static_cast<long long>(p.a_floats + p.g_floats) * 4));
+  p.nb = static_cast<int>(room / (static_cast<long long>(p.a_floats + p.g_floats) * 4));
   if (p.nb > 8) p.nb = 8;
   // image chunks: one resident wave of CTAs, and no thread adds more than kTermsPerThread terms in fp32
   const long long per_chunk0 = static_cast<long long>(p.G) * p.n_bands;
-  long long chunks = (static_cast<long long>(kG3CtasPerSm) * sm_count()) / per_chunk0;
+  long long chunks = (static_cast<long long>(to * tc == 1 ? kG3CtasPerSmDepthwise : kG3CtasPerSm) * sm_count()) / per_chunk0;
   const long long strips = static_cast<long long>(band) * (p.OW / 8);
   const long long max_imgs = (static_cast<long long>(kTermsPerThread) / 8) * p.S / strips;   // strips per thread = imgs * strips / S
   if (max_imgs < 1) return false;

@@ -63,6 +63,28 @@ def test_stride_one_taps(layer, bf16):
     assert rel_frobenius(dw, ref) <= 5e-3
 
 
+DEPTHWISE = [
+    # one band and several, one strip a thread and none, one image and more than a tile holds
+    W.conv("dw8", 3, 3, 8, 3, 3, groups=3),
+    W.conv("dw64", 1, 5, 64, 5, 3, groups=5),
+    W.conv("dw56_b9", 9, 4, 56, 4, 3, groups=4),
+    W.conv("dw128_bands", 1, 2, 128, 2, 3, groups=2),
+    W.conv("dw112_s2", 2, 3, 112, 3, 3, 2, groups=3),
+]
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("layer", DEPTHWISE, ids=lambda l: l.name)
+def test_depthwise_sums_shared_by_lanes(layer, bf16):
+    layer = replace(layer, dt=W.BF16 if bf16 else W.F32)
+    a, g = W.activation(layer, 6), W.grad_out(layer, 6)
+    comp, ref = assert_store_equals_oracle(a, 0.5)
+    dw = B.surgeon_weight_grad(comp, B.layer_desc(layer, B.PATH_TENSOR_CORE), g.cuda()).cpu().numpy()
+    dense = oracle.decompress(ref["bitmap"], ref["values"], a.numel()).reshape(layer.act_shape)
+    exp = oracle.dw_conv2d_grouped(dense.view(np.uint16) if bf16 else dense, g.numpy(), 3, 3, layer.stride, 1, layer.groups)
+    assert rel_frobenius(dw, exp) <= 1e-5      # fp32 sums of at most 4096 terms (3e-6), doubles after
+
+
 STRIDED = [
     W.conv("s2_w17", 3, 20, 17, 40, 3, 2),
     W.conv("s2_w112_many_macros", 1, 3, 112, 16, 7, 2, 3),
