@@ -1023,13 +1023,16 @@ using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, voi
 }  // namespace
 
 // Shared memory: the staging area of the packed values (fp32 activations only), the gradient
-// ring (as many tiles as fit beside four activation tiles, up to 4), then as many activation tiles
-// as fit (up to 8).
+// ring (as many tiles as fit beside four activation tiles, up to 4; slabs beside three, up to 6), then as many
+// activation tiles as fit (up to 8).
 static bool size_rings(DirectParams* p, int stage_bytes) {
   const int budget = 224 * 1024 - 1024 - stage_bytes;
   const int b_bytes = p->tg ? p->b_bytes : p->n_cols * (p->pair ? 64 : 128);
-  const int least = p->tg >= 3 ? 4 : 2, most = p->tg >= 3 ? kMaxBStages : 4;    // (a K-tile holds three slabs)
-  int b_stages = (budget - 4 * kATileBytes) / b_bytes;
+  // Slabs: a K-tile holds three, so two more are wanted under way (with one, the MMA thread waited 420-690 of 1700-2000
+  // clocks a K-tile for them; 160 channels on 32x32, 7 % kept, 173 -> 160 us, 320 on 16x16 148 -> 140), and three
+  // activation tiles beside them do; more than three under way take activation tiles for nothing.
+  const int least = p->tg >= 3 ? 4 : 2, most = p->tg >= 3 ? 6 : 4;
+  int b_stages = (budget - (p->tg >= 3 ? 3 : 4) * kATileBytes) / b_bytes;
   if (b_stages > most) b_stages = most;
   if (b_stages < least) b_stages = least;
   if (b_stages * b_bytes + 2 * kATileBytes > budget) return false;
