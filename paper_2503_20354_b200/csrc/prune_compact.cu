@@ -9,7 +9,7 @@
 // three grid-wide exchanges, at which CTA 0 collects, decides and answers:
 //
 //   sample    a scattered sample gives a bracket [lo, hi] of keys that contains the threshold with
-//             overwhelming probability (1-4 % of the elements)
+//             overwhelming probability (1-6 % of the elements)
 //   classify  first pass over the CTA's chunks: keys above the bracket are counted per chunk, the
 //             keys inside are listed and counted in a histogram of 512 bins over the bracket
 //   exchange  the summed histogram gives the threshold's bin: one key for bf16, whose brackets are
@@ -351,7 +351,7 @@ __device__ __forceinline__ unsigned long long warp_incl_u64(unsigned long long v
 // are ranked by flat index (= lane, then bit).  Out of line, like all that one chunk of a tensor does: code that is not
 // in the instruction caches costs some 250 clocks per 128 bytes, and a call runs most of its code once.
 template <int DT>
-__device__ __noinline__ uint2 quota_words(const unsigned char* region, int nv, uint32_t tau, long long allowed, uint2 above) {
+__device__ __forceinline__ uint2 quota_words_inline(const unsigned char* region, int nv, uint32_t tau, long long allowed, uint2 above) {
   constexpr int WPL = 128 / static_cast<int>(sizeof(typename Elem<DT>::type)) / 32;
   uint4 q[8];
   load_row(region, q);
@@ -366,6 +366,10 @@ __device__ __noinline__ uint2 quota_words(const unsigned char* region, int nv, u
     allowed -= __popc(ge[w]);
   }
   return make_uint2(word[0], word[1]);
+}
+template <int DT>
+__device__ __noinline__ uint2 quota_words(const unsigned char* region, int nv, uint32_t tau, long long allowed, uint2 above) {
+  return quota_words_inline<DT>(region, nv, tau, allowed, above);
 }
 
 // The byte at address a of a packed sequence lives at a ^ ((a >> 5) & 0x7C): the 32-bit word
@@ -385,7 +389,7 @@ __device__ __forceinline__ uint32_t packed_elem(uint32_t rbase, uint32_t i) {   
 }
 // A full chunk with a misaligned destination: no room for the shift, the vectors are put together from elements.
 template <int DT>
-__device__ __noinline__ void copy_full_chunk(typename Elem<DT>::type* values, long long kept_before, uint32_t total, uint32_t rbase,
+__device__ __forceinline__ void copy_full_chunk_inline(typename Elem<DT>::type* values, long long kept_before, uint32_t total, uint32_t rbase,
                                              long long n_stored, uint32_t* status) {
   using E = typename Elem<DT>::type;
   constexpr int EPV = 16 / sizeof(E);
@@ -410,11 +414,18 @@ __device__ __noinline__ void copy_full_chunk(typename Elem<DT>::type* values, lo
   if (lane < total - done && SURGEON_IN_BOUNDS(kept_before + done + lane, n_stored, status))
     dst[done + lane] = static_cast<E>(packed_elem<DT>(rbase, done + lane));
 }
+template <int DT>
+__device__ __noinline__ void copy_full_chunk(typename Elem<DT>::type* values, long long kept_before, uint32_t total, uint32_t rbase,
+                                             long long n_stored, uint32_t* status) {
+  copy_full_chunk_inline<DT>(values, kept_before, total, rbase, n_stored, status);
+}
 
 // ---- emit one chunk -------------------------------------------------------------------------------
 // before = (elements above the threshold before the chunk) << 32 | (ties before it); n_eq = its ties.
 // True when the chunk's place in the ring has been written to.
-template <int DT, bool kPlain>
+// kClaimedTensor: of a gigabyte tensor, whose kernel runs its loop some thousand times: what is rare is in line there (calls in the loop
+// cost 4.3 GB of fp32 1745 -> 1810 us).
+template <int DT, bool kPlain, bool kClaimedTensor>
 __device__ __forceinline__ bool emit_chunk(const PruneArgs& a, unsigned char* region, int chunk, uint32_t tau, long long quota,
                                            unsigned long long before, uint32_t n_eq, long long n_stored) {
   using E = typename Elem<DT>::type;
@@ -438,7 +449,9 @@ __device__ __forceinline__ bool emit_chunk(const PruneArgs& a, unsigned char* re
   uint32_t word[WPL];
   mask_ge<DT, WPL>(q, nv, ties ? tau : tau + 1u, word);
   if (!ties && eq_b < quota) {
-    const uint2 both = quota_words<DT>(region, nv, tau, quota - eq_b, make_uint2(word[0], word[WPL - 1]));
+    const uint2 above = make_uint2(word[0], word[WPL - 1]);
+    const uint2 both = kClaimedTensor ? quota_words_inline<DT>(region, nv, tau, quota - eq_b, above)
+                                      : quota_words<DT>(region, nv, tau, quota - eq_b, above);
     word[0] = both.x;
     if (WPL == 2) word[WPL - 1] = both.y;
   }
@@ -516,7 +529,7 @@ __device__ __forceinline__ bool emit_chunk(const PruneArgs& a, unsigned char* re
       gbase[mis + lane] = packed[mis + lane];
     if (tail + lane < end && SURGEON_IN_BOUNDS(kept_before - mis + tail + lane, n_stored, &a.hdr->status))
       gbase[tail + lane] = packed[tail + lane];
-#pragma unroll 2
+#pragma unroll 4
     for (uint32_t g = v_first + lane; g < v_end; g += 32)
       if (SURGEON_IN_BOUNDS(kept_before - mis + g * EPV + EPV - 1, n_stored, &a.hdr->status))
         *reinterpret_cast<uint4*>(gbase + g * EPV) = *reinterpret_cast<const uint4*>(region + g * 16);
@@ -536,7 +549,7 @@ __device__ __forceinline__ bool emit_chunk(const PruneArgs& a, unsigned char* re
           SURGEON_IN_BOUNDS(kept_before - mis + sl, n_stored, &a.hdr->status))
         gbase[sl] = static_cast<E>(packed_elem<DT>(rbase, sl));
     }
-#pragma unroll 2
+#pragma unroll 4
     for (uint32_t g = v_first + lane; g < v_end; g += 32) {
       // the four words of a vector share their row: one 16-byte load, words permuted by the XOR
       const uint32_t la = rbase + g * 16u;
@@ -553,7 +566,8 @@ __device__ __forceinline__ bool emit_chunk(const PruneArgs& a, unsigned char* re
     if (t0 + lane < end && SURGEON_IN_BOUNDS(kept_before - mis + t0 + lane, n_stored, &a.hdr->status))
       gbase[t0 + lane] = static_cast<E>(packed_elem<DT>(rbase, t0 + lane));
   } else {
-    copy_full_chunk<DT>(values, kept_before, total, rbase, n_stored, &a.hdr->status);
+    if (kClaimedTensor) copy_full_chunk_inline<DT>(values, kept_before, total, rbase, n_stored, &a.hdr->status);
+    else copy_full_chunk<DT>(values, kept_before, total, rbase, n_stored, &a.hdr->status);
   }
   return true;
 }
@@ -1653,7 +1667,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
   // ---- emit ----
   if (RES) {
     run_resident(false, [&](int c, unsigned char* region) -> bool {
-      return emit_chunk<DT, (DT == 1 || MODE != kClaimed)>(a, region, c, tau, quota, prefix[c - c_begin], cnt[c - c_begin] >> 16, n_stored);
+      return emit_chunk<DT, (DT == 1 || MODE != kClaimed), MODE == kClaimed>(a, region, c, tau, quota, prefix[c - c_begin], cnt[c - c_begin] >> 16, n_stored);
     });
     return kDone;
   }
@@ -1680,7 +1694,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     uint32_t n_at = n_next;
     if (!spread) { at = prefix[c - c_begin]; n_at = cnt[c - c_begin]; }
     else if (fly1 < a.n_chunks) { at_next = prefix[fly1 - c_begin]; n_next = cnt[fly1 - c_begin]; }
-    const bool written = emit_chunk<DT, (DT == 1 || MODE != kClaimed)>(a, my_ring + s * kChunkBytes, c, tau, quota, at, n_at >> 16, n_stored);
+    const bool written = emit_chunk<DT, (DT == 1 || MODE != kClaimed), MODE == kClaimed>(a, my_ring + s * kChunkBytes, c, tau, quota, at, n_at >> 16, n_stored);
     int c_load;                                  // what the place takes next
     if (spread) {
       fly0 = fly1; fly1 = fly2;
