@@ -101,7 +101,7 @@ struct PruneArgs {
   uint32_t* offsets;
   ulonglong2* arrive;            // [kSelPhases][kSelMaxCtas]: {token, what the CTA reports}
   ulonglong2* answer;            // [kSelPhases][kSelMaxCtas + 2]: {token, what CTA 0 answers}
-  unsigned long long* keys;      // [CTAs][key_room()]: {half a token, key}
+  unsigned long long* keys;      // [CTAs][key_room()]: {tag, key}
   uint32_t* hist;                // [kSelHists][kSelBins]
   uint32_t* claims;              // [kSelPhases][kClaimSets], kClaimStride words apart: groups claimed in each pass
   uint32_t* cnt;                 // per chunk (kClaimed)
@@ -121,13 +121,17 @@ __device__ __forceinline__ uint32_t hash_u32(uint32_t v) {
 // No word has to start at zero, so the call needs no memset: the token differs from call to
 // call.  For a captured graph, whose replays carry the same token, CTA 0 clears every report that it
 // has read, clears the answers of all phases before it gives the first one, and clears that one (phase 0)
-// after the reports of phase 1; a CTA takes its keys back when they have been read, and all its words when it gives up.
+// after the reports of phase 1; a CTA takes its words back when it gives up.
 // All CTAs are resident (cooperative launch); polls are bounded.
 //
 // No fence stands between a report and the answer: one waits for the stores before it, 0.3-0.5 us, and an exchange
-// used to have four of them in its chain.  Keys carry half the token each, so they are polled like the words; the
+// used to have four of them in its chain.  Keys carry a tag each, so they are polled like the words; the
 // bins, which are added up by atomics, are complete when their sum is the sum of the counts in the words.  (148 CTAs:
 // words alone 1.3 us, with atomics behind fences 4.1; measured on exchanges alone.)
+//
+// A tag is 32 bits, which something that the scratch happens to hold, or that an earlier replay left there, could match.
+// So every CTA clears its key words before the fence that precedes its first report, and CTA 0 has a fence behind
+// these reports where it asks for keys, off the chain (it has answered by then): it sees cleared words or this call's.
 __device__ __forceinline__ void word_store(ulonglong2* p, unsigned long long token, unsigned long long v) {
   asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}"
                ::"l"(p), "l"(token), "l"(v) : "memory");
@@ -138,12 +142,14 @@ __device__ __forceinline__ ulonglong2 word_load(const ulonglong2* p) {
                : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
   return v;
 }
-__device__ __forceinline__ void key_store(unsigned long long* p, unsigned long long token, uint32_t key) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"((token << 32) | key) : "memory");
+// (never that of a cleared word)
+__device__ __forceinline__ uint32_t key_tag(unsigned long long token) { return static_cast<uint32_t>(token) | 1u; }
+__device__ __forceinline__ void key_store(unsigned long long* p, uint32_t tag, uint32_t key) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"((static_cast<unsigned long long>(tag) << 32) | key) : "memory");
 }
-// (not wanted: the token, and key 0)
-__device__ __forceinline__ unsigned long long key_load_if(const unsigned long long* p, bool wanted, unsigned long long token) {
-  unsigned long long v = token << 32;
+// (not wanted: the tag and `otherwise`)
+__device__ __forceinline__ unsigned long long key_load_if(const unsigned long long* p, bool wanted, uint32_t tag, uint32_t otherwise) {
+  unsigned long long v = (static_cast<unsigned long long>(tag) << 32) | otherwise;
   asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p ld.relaxed.gpu.global.u64 %0, [%1];\n\t}"
                : "+l"(v) : "l"(p), "r"(static_cast<uint32_t>(wanted)) : "memory");
   return v;
@@ -940,6 +946,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     s_over = 0;
   }
   if (tid < 4) s_tot[tid] = 0;
+  if (tid < key_room(G)) a.keys[blockIdx.x * key_room(G) + tid] = 0ull;      // (see the grid-wide exchange)
   for (int i = tid; i < kAuxBytes / 16; i += kThreads) reinterpret_cast<uint4*>(aux)[i] = make_uint4(0, 0, 0, 0);
   __syncthreads();
 
@@ -1334,6 +1341,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
         word_store(a.answer + phase * (kSelMaxCtas + 2) + 1, a.token, n_above | (static_cast<unsigned long long>(step) << 32));
         if (phase == 1) a.answer[0].x = 0ull;
       }
+      if (!spread && step == kKeys && tid < G) fence_gpu();  // the key words of all CTAs have been cleared
     } else {
       if (tid < 2) {
         unsigned long long v = 0;
@@ -1386,7 +1394,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
         if (step == kKeys) {
           const uint32_t at = atomicAdd(&s_nkeys, 1u);
           if (at < static_cast<uint32_t>(key_room(G))) {
-            key_store(a.keys + blockIdx.x * key_room(G) + at, a.token, key);
+            key_store(a.keys + blockIdx.x * key_room(G) + at, key_tag(a.token), key);
             s_bin_key[at] = key;
             s_bin_chunk[at] = c;
           }
@@ -1469,23 +1477,26 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
         unsigned long long w[4];
         bool late;
         uint32_t spins = 0;
+        const uint32_t first = 8u * turn + (tid & 1u), left = fits && n_k > first ? n_k - first : 0u;      // word u: 2 u < left
         do {
           late = false;
 #pragma unroll
-          for (int u = 0; u < 4; ++u)
-            w[u] = key_load_if(mine + 8 * turn + 2 * u, fits && 8u * turn + 2u * u + (tid & 1u) < n_k, a.token);
+          for (int u = 0; u < 4; ++u) w[u] = key_load_if(mine + 8 * turn + 2 * u, 2u * u < left, key_tag(a.token), lo);
 #pragma unroll
-          for (int u = 0; u < 4; ++u) late |= static_cast<uint32_t>(w[u] >> 32) != static_cast<uint32_t>(a.token);
+          for (int u = 0; u < 4; ++u)            // (a number outside the bin is no index below)
+            late |= static_cast<uint32_t>(w[u] >> 32) != key_tag(a.token) || static_cast<uint32_t>(w[u]) - lo > hi - lo;
         } while (late && ++spins < (1u << 20));
         if (late) ok = 0;
         __syncwarp();
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          const uint32_t key = static_cast<uint32_t>(w[u]), have = __ballot_sync(kFull, key != 0u);
+          const uint32_t key = static_cast<uint32_t>(w[u]);
+          const bool got_one = !late && 2u * u < left;
+          const uint32_t have = __ballot_sync(kFull, got_one);
           uint32_t at = 0;
           if (lane == 0 && have) at = atomicAdd(&s_res[6], __popc(have));
           at = __shfl_sync(kFull, at, 0) + __popc(have & lanemask_lt());
-          if (key && at < kKeysAtOnce) {
+          if (got_one && at < kKeysAtOnce) {
             got[at] = key;
             owner[at] = static_cast<unsigned char>(who);
             atomicAdd(&hist[(key - lo) >> coarse], 1u);
@@ -1597,7 +1608,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     before = s_last[2];
   }
   ++phase;
-  if (step == kKeys && tid < min(static_cast<int>(s_nkeys), key_room(G)))     // they have been read
+  if (step == kKeys && tid < min(static_cast<int>(s_nkeys), key_room(G)))     // they have been read, and there may be others
     a.keys[blockIdx.x * key_room(G) + tid] = 0ull;
   if (!again) break;
   step = kRefine;
@@ -1723,7 +1734,6 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
   if (left_as == kTimedOut) {
     if (tid == 0) atomicMax(&a.hdr->status, static_cast<uint32_t>(SURGEON_ERR_TIMEOUT));
     if (tid < kSelPhases) a.arrive[tid * kSelMaxCtas + blockIdx.x].x = 0ull;
-    if (tid < key_room(G)) a.keys[blockIdx.x * key_room(G) + tid] = 0ull;
     if (master)
       for (int i = tid; i < kSelPhases * (kSelMaxCtas + 2); i += kThreads) a.answer[i].x = 0ull;
   }
@@ -1875,10 +1885,7 @@ unsigned long long next_token() {
         std::chrono::steady_clock::now().time_since_epoch().count());
     return ((static_cast<unsigned long long>(rd()) << 32) | rd()) ^ (t << 20);
   }()};
-  unsigned long long v;
-  do v = counter.fetch_add(1, std::memory_order_relaxed);
-  while (static_cast<uint32_t>(v) == 0u);        // (a cleared key must not carry its lower half)
-  return v;
+  return counter.fetch_add(1, std::memory_order_relaxed);
 }
 
 template <int DT>

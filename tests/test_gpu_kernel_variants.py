@@ -338,6 +338,43 @@ def test_call_that_timed_out_leaves_no_words_behind(n):
     assert_store_equals_oracle(x.cpu(), 0.5, comp=B.surgeon_prune_compact(x, 0.5, out=out, workspace=ws))
 
 
+KEY_WORDS = slice(16 * 12 * (256 + 258), 16 * 12 * (256 + 258) + 256 * 64 * 4)      # of the scratch: the keys that CTAs report
+
+
+@pytest.mark.parametrize("n, flags", [(40000, 0), (3_000_001, 0), (18_000_003, 0), (1024 * (1024 * 37 + 1), B.SURGEON_SHARE_GPU)])
+def test_scratch_that_holds_what_looks_like_keys(n, flags):
+    """The scratch may hold anything, words with the very tag of the call among them (a replay carries the token of the
+    one before): keys inside and outside the bin, in every place that a CTA reports keys in."""
+    xs = [W.draw("normal", n, seed=40 + i, device="cuda") for i in range(2)]
+    refs = []
+    for x in xs:
+        comp = B.surgeon_prune_compact(x, 0.7, flags=flags)
+        assert_store_equals_oracle(x.cpu(), 0.7, comp=comp)
+        refs.append([v.copy() for v in comp.to_numpy()[:3]] + [comp.read_header().threshold_key])
+    x, out = xs[0].clone(), B.CompressedActivation(n, B.SURGEON_F32, 0.7, "cuda")
+    ws = torch.zeros(out.sizes.workspace_bytes, dtype=torch.uint8, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        B.surgeon_prune_compact(x, 0.7, out=out, workspace=ws, flags=flags)
+    rng = np.random.default_rng(n)
+    for turn in range(6):
+        ref = refs[turn % 2]
+        x.copy_(xs[turn % 2])
+        if turn:
+            low = token & 0xFFFFFFFF
+            tags = np.array([low, low | 1] + [(low << 4 | p) & 0xFFFFFFFF for p in range(12)], dtype=np.uint64)
+            near = (ref[3] + rng.integers(-300, 300, 8192)).astype(np.uint64)
+            far = rng.integers(0, 1 << 32, 8192, dtype=np.uint64)
+            words = tags[rng.integers(0, len(tags), 8192)] << np.uint64(32) | np.where(rng.random(8192) < 0.5, near, far)
+            ws[KEY_WORDS].copy_(torch.from_numpy(words.view(np.uint8)))
+        graph.replay()
+        torch.cuda.synchronize()
+        assert out.read_header().status == B.SURGEON_OK
+        assert all(np.array_equal(u.view(np.uint8), v.view(np.uint8)) for u, v in zip(out.to_numpy()[:3], ref))
+        answers = ws[16 * 12 * 256:KEY_WORDS.start].view(torch.int64).view(-1, 2)[:, 0].cpu()
+        token = int(answers[answers != 0][0])
+
+
 @pytest.mark.parametrize("bf16", [False, True])
 @pytest.mark.parametrize("n", [1, 31, 1023, 1025, 4 * 8192 + 5])
 def test_rebuild(n, bf16):
