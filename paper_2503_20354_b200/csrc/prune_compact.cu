@@ -132,6 +132,8 @@ __device__ __forceinline__ uint32_t hash_u32(uint32_t v) {
 // A tag is 32 bits, which something that the scratch happens to hold, or that an earlier replay left there, could match.
 // So every CTA clears its key words before the fence that precedes its first report, and CTA 0 has a fence behind
 // these reports where it asks for keys, off the chain (it has answered by then): it sees cleared words or this call's.
+// Where a CTA has more keys than it can report, the bin is narrowed and keys are reported once more, in the same words: the
+// tag names the phase.
 __device__ __forceinline__ void word_store(ulonglong2* p, unsigned long long token, unsigned long long v) {
   asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}"
                ::"l"(p), "l"(token), "l"(v) : "memory");
@@ -143,7 +145,10 @@ __device__ __forceinline__ ulonglong2 word_load(const ulonglong2* p) {
   return v;
 }
 // (never that of a cleared word)
-__device__ __forceinline__ uint32_t key_tag(unsigned long long token) { return static_cast<uint32_t>(token) | 1u; }
+__device__ __forceinline__ uint32_t key_tag(unsigned long long token, int phase) {
+  return (static_cast<uint32_t>(token) << 4) | static_cast<uint32_t>(phase);
+}
+static_assert(kSelPhases <= 16, "phase in four bits");
 __device__ __forceinline__ void key_store(unsigned long long* p, uint32_t tag, uint32_t key) {
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"((static_cast<unsigned long long>(tag) << 32) | key) : "memory");
 }
@@ -1107,6 +1112,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
   unsigned long long before = 0;
   for (;;) {
   for (; step <= kRefine; ++round) {
+    if (round > 0 && tid == 1) fence_gpu();      // (it has read the answer) the bins and answers that CTA 0 has cleared for this round
     const uint32_t range = hi - lo;
     shift = max(0, 32 - __clz(range) - kSelBinsLog2);
     __syncthreads();
@@ -1394,7 +1400,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
         if (step == kKeys) {
           const uint32_t at = atomicAdd(&s_nkeys, 1u);
           if (at < static_cast<uint32_t>(key_room(G))) {
-            key_store(a.keys + blockIdx.x * key_room(G) + at, key_tag(a.token), key);
+            key_store(a.keys + blockIdx.x * key_room(G) + at, key_tag(a.token, phase), key);
             s_bin_key[at] = key;
             s_bin_chunk[at] = c;
           }
@@ -1481,10 +1487,10 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
         do {
           late = false;
 #pragma unroll
-          for (int u = 0; u < 4; ++u) w[u] = key_load_if(mine + 8 * turn + 2 * u, 2u * u < left, key_tag(a.token), lo);
+          for (int u = 0; u < 4; ++u) w[u] = key_load_if(mine + 8 * turn + 2 * u, 2u * u < left, key_tag(a.token, phase), lo);
 #pragma unroll
           for (int u = 0; u < 4; ++u)            // (a number outside the bin is no index below)
-            late |= static_cast<uint32_t>(w[u] >> 32) != key_tag(a.token) || static_cast<uint32_t>(w[u]) - lo > hi - lo;
+            late |= static_cast<uint32_t>(w[u] >> 32) != key_tag(a.token, phase) || static_cast<uint32_t>(w[u]) - lo > hi - lo;
         } while (late && ++spins < (1u << 20));
         if (late) ok = 0;
         __syncwarp();
@@ -1608,8 +1614,9 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     before = s_last[2];
   }
   ++phase;
-  if (step == kKeys && tid < min(static_cast<int>(s_nkeys), key_room(G)))     // they have been read, and there may be others
-    a.keys[blockIdx.x * key_room(G) + tid] = 0ull;
+  // They have been read.  (Not needed: they carry this phase's tag.  Without a place where the paths of all steps meet, small
+  // calls that report no keys took 2-4 us longer.)
+  if (step == kKeys && tid < min(static_cast<int>(s_nkeys), key_room(G))) a.keys[blockIdx.x * key_room(G) + tid] = 0ull;
   if (!again) break;
   step = kRefine;
   }

@@ -338,6 +338,36 @@ def test_call_that_timed_out_leaves_no_words_behind(n):
     assert_store_equals_oracle(x.cpu(), 0.5, comp=B.surgeon_prune_compact(x, 0.5, out=out, workspace=ws))
 
 
+@pytest.mark.parametrize("n, flags", [(2_000_001, 0), (18_000_003, 0), (1024 * (1024 * 37 + 1), B.SURGEON_SHARE_GPU)])
+def test_keys_reported_more_than_once(n, flags):
+    """Two hundred copies of the threshold in one CTA: more keys than it can report, so the bin is narrowed and keys go
+    into the same words again.  Each replay of one captured call has other values, and ordinary ones in between."""
+    k = B.surgeon_compact_sizes(n, B.SURGEON_F32, 0.7).n_keep
+    xs, refs = [], []
+    for i in range(3):
+        x = W.draw("normal", n, seed=60 + i, device="cuda") * (1.0 + 0.3 * i)
+        if i != 1:
+            at = n // 2 + 37 * torch.arange(200, device="cuda")
+            x[at] = x.abs().kthvalue(n - k + 1).values * torch.tensor([1.0, -1.0], device="cuda").repeat(100)
+        comp = B.surgeon_prune_compact(x, 0.7, flags=flags)
+        assert_store_equals_oracle(x.cpu(), 0.7, comp=comp)
+        xs.append(x)
+        refs.append([v.copy() for v in comp.to_numpy()[:3]])
+    x, out = xs[0].clone(), B.CompressedActivation(n, B.SURGEON_F32, 0.7, "cuda")
+    ws = torch.zeros(out.sizes.workspace_bytes, dtype=torch.uint8, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        B.surgeon_prune_compact(x, 0.7, out=out, workspace=ws, flags=flags)
+    for i in (0, 2, 1, 2, 0, 0):
+        x.copy_(xs[i])
+        graph.replay()
+        torch.cuda.synchronize()
+        assert out.read_header().status == B.SURGEON_OK
+        assert all(np.array_equal(u.view(np.uint8), v.view(np.uint8)) for u, v in zip(out.to_numpy()[:3], refs[i]))
+        answered = ws[16 * 12 * 256:16 * 12 * (256 + 258)].view(torch.int64).view(12, 258, 2)[:, 0, 0].count_nonzero()
+        assert flags or int(answered) >= 4       # two rounds and two last exchanges
+
+
 KEY_WORDS = slice(16 * 12 * (256 + 258), 16 * 12 * (256 + 258) + 256 * 64 * 4)      # of the scratch: the keys that CTAs report
 
 
