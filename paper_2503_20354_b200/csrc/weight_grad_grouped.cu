@@ -15,6 +15,7 @@
 // planes beside them, and every thread accumulates up to 8 output channels of a few (c', r, s)
 // columns.  Partial sums per (band, image chunk) are added in a fixed order by a second kernel:
 // results are bitwise reproducible.
+#include <algorithm>
 #include <type_traits>
 
 #include "surgeon_internal.cuh"
@@ -261,19 +262,23 @@ __device__ __forceinline__ void cp_async_wait_all() {
 __device__ __forceinline__ int fast_div(int n, uint32_t rcp) {
   return rcp ? static_cast<int>(__umulhi(static_cast<uint32_t>(n), rcp)) : n;
 }
-// Three CTAs share an SM: rebuilding a tile is two dependent global loads per element, so what
-// hides that latency is the other CTAs' work.  That leaves a CTA 85 registers per thread (tiles of
-// at most 4 channel pairs: 36 accumulators) and about 74 KB of shared memory.
+// Two CTAs share an SM: rebuilding a tile is two dependent global loads per element, so what
+// hides that latency is the other CTA's work.  That leaves a CTA 128 registers per thread (tiles of
+// at most 8 channel pairs: 72 accumulators) and 110 KB of shared memory.
 constexpr int kG3CtasPerSm = 2;
-// One channel per group: 9 sums per thread need no 128 registers, and a tile of half the size leaves room for twice as
-// many CTAs, which hide one another's load phases.
-constexpr int kG3CtasPerSmDepthwise = 4;
 constexpr int kG3Smem = 110 * 1024;
-constexpr int kG3SmemDepthwise = 54 * 1024;
 constexpr int kG3MaxTile = 8;
+// One channel per group in and out (depthwise): 9 sums per thread need no 128 registers, and a tile of half the size
+// leaves room for twice as many CTAs, which hide one another's load phases.  1280 channels on 64x64, batch 1, half
+// kept: 51 -> 31 us a call.  Not where it has fewer than four rows, two of which are halo (16 channels 1536 wide, three
+// rows: 211 us, on tiles of 110 KB 184; 3072 wide, one row: 513 and 276), nor under stride 2 where the whole map
+// fits the larger tile only (256 channels on 128x128: 24.8 and 18.7; under stride 1 96x96 takes 26.8 and 33).
+constexpr int kG3CtasPerSmDepthwise = 4;
+constexpr int kG3SmemDepthwise = 54 * 1024;
+constexpr int kG3LeastRowsDepthwise = 4;
 
-template <int TO, int TC, int ST>
-__global__ void __launch_bounds__(kThreads, TO * TC == 1 ? kG3CtasPerSmDepthwise : kG3CtasPerSm)
+template <int TO, int TC, int ST, bool kDepthwise>
+__global__ void __launch_bounds__(kThreads, kDepthwise ? kG3CtasPerSmDepthwise : kG3CtasPerSm)
 dw_grouped3_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ values,
                    const uint32_t* __restrict__ offsets, const float* __restrict__ grad,
                    double* __restrict__ partial, Grouped3Params p) {
@@ -506,8 +511,8 @@ dw_grouped3_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__
   __syncthreads();
   const int ncol = p.Cg * 9;
   double* out = partial + static_cast<long long>(chunk * p.n_bands + band) * p.O * ncol;
-  // One channel per group: 9 sums of 256 parts would be a chain of 5 us for a thread each; 16 lanes share one.
-  constexpr int per = TO * TC == 1 ? 16 : 1;          // lanes of a sum
+  // Depthwise: 9 sums of 256 parts would be a chain of 5 us for a thread each; 16 lanes share one.
+  constexpr int per = kDepthwise ? 16 : 1;            // lanes of a sum
   for (int i0 = tid; i0 < (per == 1 ? p.units * ACC : (p.units * ACC * per + 31) / 32 * 32); i0 += kThreads) {      // (whole warps)
     const int i = i0 / per, part = i0 % per;
     const int u = i / ACC, a = i - u * ACC;
@@ -585,7 +590,7 @@ bool plan_grouped(const surgeon_layer_desc& d, GroupedParams* out) {
 // The register-tiled kernel's launch: 3x3, padding 1, stride 1 or 2, even maps under stride 2, output
 // rows a multiple of 8 wide.  TO / TC = the largest of 4, 2, 1 that divide the group's output /
 // input channels with TO * TC <= 4.
-struct Grouped3Tile { int to, tc; };
+struct Grouped3Tile { int to, tc; bool depthwise; };
 bool plan_grouped3(const surgeon_layer_desc& d, Grouped3Params* out, Grouped3Tile* tile) {
   if (d.kind != 1 || d.groups <= 1 || d.c_in % d.groups || d.c_out % d.groups) return false;
   if (d.kh != 3 || d.kw != 3 || d.pad != 1 || (d.stride != 1 && d.stride != 2)) return false;
@@ -599,29 +604,35 @@ bool plan_grouped3(const surgeon_layer_desc& d, Grouped3Params* out, Grouped3Til
   int to = p.Og % 4 == 0 ? 4 : (p.Og % 2 == 0 ? 2 : 1);
   int tc = p.Cg % 4 == 0 ? 4 : (p.Cg % 2 == 0 ? 2 : 1);
   while (to * tc > kG3MaxTile) { if (tc >= to) tc >>= 1; else to >>= 1; }
-  const long long room = to * tc == 1 ? kG3SmemDepthwise : kG3Smem;
   p.n_cb = p.Cg / tc;
   p.units = (p.Og / to) * p.n_cb;
   if (p.units > kThreads) return false;
   p.S = kThreads / p.units;
   p.Wp = p.W + 4;                                   // column 0 = input column -1; 16-byte aligned rows
   const long long red_bytes = static_cast<long long>(kThreads) * to * tc * 9 * 4;
-  int band = p.OH;
-  for (;; --band) {
-    if (band < 1) return false;
-    const long long in_rows = static_cast<long long>(band - 1) * d.stride + 3;
-    const long long a = static_cast<long long>(p.Cg) * in_rows * p.Wp;
-    const long long g = static_cast<long long>(p.Og) * band * p.OW;
-    if ((a + g) * 4 <= room) { p.in_rows = static_cast<int>(in_rows); p.a_floats = static_cast<int>(a); p.g_floats = static_cast<int>(g); break; }
-  }
-  if (red_bytes > room) return false;
+  // the tallest band whose two tiles fit: Cg ((rows - 1) stride + 3) Wp + Og rows OW floats; below 1: none
+  auto tallest = [&](long long bytes) {
+    const long long rest = bytes / 4 - static_cast<long long>(p.Cg) * (3 - d.stride) * p.Wp;
+    const long long rows = rest / (static_cast<long long>(p.Cg) * d.stride * p.Wp + static_cast<long long>(p.Og) * p.OW);
+    return static_cast<int>(std::min<long long>(p.OH, std::max<long long>(rows, 0)));
+  };
+  const bool depthwise = p.Cg == 1 && p.Og == 1;
+  const int rows_small = depthwise ? tallest(kG3SmemDepthwise) : 0, rows_large = tallest(kG3Smem);
+  const bool small = depthwise && (rows_small == p.OH || (rows_small >= kG3LeastRowsDepthwise &&
+                                                          !(d.stride == 2 && rows_large == p.OH)));
+  const int band = small ? rows_small : rows_large;
+  const long long room = small ? kG3SmemDepthwise : kG3Smem;
+  if (band < 1 || red_bytes > room) return false;
+  p.in_rows = (band - 1) * d.stride + 3;
+  p.a_floats = p.Cg * p.in_rows * p.Wp;
+  p.g_floats = p.Og * band * p.OW;
   p.band = band;
   p.n_bands = (p.OH + band - 1) / band;
   p.nb = static_cast<int>(room / (static_cast<long long>(p.a_floats + p.g_floats) * 4));
   if (p.nb > 8) p.nb = 8;
   // image chunks: one resident wave of CTAs, and no thread adds more than kTermsPerThread terms in fp32
   const long long per_chunk0 = static_cast<long long>(p.G) * p.n_bands;
-  long long chunks = (static_cast<long long>(to * tc == 1 ? kG3CtasPerSmDepthwise : kG3CtasPerSm) * sm_count()) / per_chunk0;
+  long long chunks = (static_cast<long long>(small ? kG3CtasPerSmDepthwise : kG3CtasPerSm) * sm_count()) / per_chunk0;
   const long long strips = static_cast<long long>(band) * (p.OW / 8);
   const long long max_imgs = (static_cast<long long>(kTermsPerThread) / 8) * p.S / strips;   // strips per thread = imgs * strips / S
   if (max_imgs < 1) return false;
@@ -636,7 +647,7 @@ bool plan_grouped3(const surgeon_layer_desc& d, Grouped3Params* out, Grouped3Til
   p.rcp_spr = div_magic(p.OW / 8);
   p.rcp_w = div_magic(p.W);
   *out = p;
-  tile->to = to; tile->tc = tc;
+  tile->to = to; tile->tc = tc; tile->depthwise = depthwise;
   return true;
 }
 size_t grouped3_smem(const Grouped3Params& p, const Grouped3Tile& t) {
@@ -685,13 +696,15 @@ cudaError_t launch_weight_grad_grouped(const surgeon_compressed& act, const surg
     };
     auto by_stride = [&](auto to, auto tc) {
       constexpr int TO = decltype(to)::value, TC = decltype(tc)::value;
-      if (d.stride == 1) launch(dw_grouped3_kernel<TO, TC, 1>);
-      else launch(dw_grouped3_kernel<TO, TC, 2>);
+      if (d.stride == 1) launch(dw_grouped3_kernel<TO, TC, 1, false>);
+      else launch(dw_grouped3_kernel<TO, TC, 2, false>);
     };
     using I1 = std::integral_constant<int, 1>;
     using I2 = std::integral_constant<int, 2>;
     using I4 = std::integral_constant<int, 4>;
-    if (t3.to == 4 && t3.tc == 2) by_stride(I4{}, I2{});
+    if (t3.depthwise && d.stride == 1) launch(dw_grouped3_kernel<1, 1, 1, true>);
+    else if (t3.depthwise) launch(dw_grouped3_kernel<1, 1, 2, true>);
+    else if (t3.to == 4 && t3.tc == 2) by_stride(I4{}, I2{});
     else if (t3.to == 2 && t3.tc == 4) by_stride(I2{}, I4{});
     else if (t3.to == 4) by_stride(I4{}, I1{});
     else if (t3.to == 2 && t3.tc == 2) by_stride(I2{}, I2{});

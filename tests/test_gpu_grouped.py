@@ -36,6 +36,16 @@ SHAPES = [
     W.conv("depthwise_w16", 9, 12, 16, 12, 3, groups=12),
     W.conv("t22_s2_w16", 3, 32, 32, 32, 3, 2, groups=4),            # 8 -> 8 per group, stride 2
     replace(W.conv("t22_tall_bands", 1, 8, 64, 8, 3, groups=2), h=240),   # several bands of output rows
+    # odd channels in and out (1 x 1 tiles, not depthwise), up to as many as a CTA has threads for
+    W.conv("t11_3to3", 3, 9, 16, 9, 3, groups=3),
+    W.conv("t11_15to15", 2, 30, 16, 30, 3, groups=2),
+    W.conv("t11_127to1", 1, 254, 40, 2, 3, groups=2),
+    W.conv("t11_1to51", 1, 2, 32, 102, 3, 2, groups=2),
+    # depthwise rows of which fewer than four, or none, fit the smaller tile; a map that fits the larger one only
+    replace(W.conv("depthwise_w1536", 1, 2, 1536, 2, 3, groups=2), h=7),
+    replace(W.conv("depthwise_w4096", 1, 2, 4096, 2, 3, groups=2), h=3),
+    replace(W.conv("depthwise_w4096_s2", 1, 2, 4096, 2, 3, 2, groups=2), h=6),
+    W.conv("depthwise_w144_s2", 2, 3, 144, 3, 3, 2, groups=3),
 ]
 
 

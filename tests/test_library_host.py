@@ -117,3 +117,11 @@ def test_argument_checks_need_no_device():
     assert B.surgeon_weight_grad_workspace(bad) == 0
     assert l.surgeon_weight_grad(ctypes.byref(comp), ctypes.byref(bad), 16, 16, 0, 0, 0, 0) == B.SURGEON_ERR_INVALID_ARG
     assert B.status_string(B.SURGEON_ERR_TIMEOUT).startswith("device-side")
+
+
+def test_grouped_layers_that_have_a_plan():
+    """Groups of many odd channel counts, and depthwise layers on wide maps: what a tile of 110 KB holds is not refused."""
+    for layer in (W.conv("wide_groups", 4, 254, 40, 2, 3, groups=2), W.conv("out51", 1, 4, 256, 204, 3, groups=4),
+                  W.conv("c15", 1, 30, 240, 30, 3, groups=2), W.conv("dw4096", 1, 2, 4096, 2, 3, groups=2),
+                  W.conv("dw6144_s2", 1, 2, 6144, 2, 3, 2, groups=2)):
+        assert B.surgeon_weight_grad_workspace(B.layer_desc(layer, B.PATH_TENSOR_CORE)) > 0, layer.name
