@@ -1023,16 +1023,19 @@ using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, voi
 }  // namespace
 
 // Shared memory: the staging area of the packed values (fp32 activations only), the gradient
-// ring (as many tiles as fit beside four activation tiles, up to 4; slabs beside three, up to 6), then as many
-// activation tiles as fit (up to 8).
+// ring (as many tiles as fit beside four activation tiles, up to 4; slabs up to 8, beside three activation tiles and up
+// to 6 for fp32 activations), then as many activation tiles as fit (up to 8).
 static bool size_rings(DirectParams* p, int stage_bytes) {
   const int budget = 224 * 1024 - 1024 - stage_bytes;
   const int b_bytes = p->tg ? p->b_bytes : p->n_cols * (p->pair ? 64 : 128);
-  // Slabs: a K-tile holds three, so two more are wanted under way (with one, the MMA thread waited 420-690 of 1700-2000
-  // clocks a K-tile for them; 160 channels on 32x32, 7 % kept, 173 -> 160 us, 320 on 16x16 148 -> 140), and three
-  // activation tiles beside them do; more than three under way take activation tiles for nothing.
-  const int least = p->tg >= 3 ? 4 : 2, most = p->tg >= 3 ? 6 : 4;
-  int b_stages = (budget - (p->tg >= 3 ? 3 : 4) * kATileBytes) / b_bytes;
+  // Slabs: a K-tile holds three, so two more are wanted under way.  Beside the staging area of fp32 activations a fourth
+  // activation tile leaves room for one (the MMA thread waited 420-690 of 1700-2000 clocks a K-tile for them; 160 channels
+  // on 32x32, 7 % kept, 173 -> 160 us, 320 on 16x16 148 -> 140); more than three under way take activation tiles for
+  // nothing.  bf16 activations have no staging area, and the fourth tile is worth more to them (256 channels on 64x64,
+  // batch 16, 70 % kept: 171 us, with three 174; 30 % kept 139 and 142).
+  const bool slabs = p->tg >= 3, few_tiles = slabs && stage_bytes > 0;
+  const int least = slabs ? 4 : 2, most = few_tiles ? 6 : (slabs ? kMaxBStages : 4);
+  int b_stages = (budget - (few_tiles ? 3 : 4) * kATileBytes) / b_bytes;
   if (b_stages > most) b_stages = most;
   if (b_stages < least) b_stages = least;
   if (b_stages * b_bytes + 2 * kATileBytes > budget) return false;
