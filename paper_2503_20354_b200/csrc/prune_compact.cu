@@ -614,13 +614,15 @@ __device__ __forceinline__ void slot_keys_warp(const typename Elem<DT>::type* sl
 #pragma unroll 1
   for (uint32_t i = lane_id(); i < n_in; i += 32) f(static_cast<uint32_t>(slot[i]));
 }
-// Of slots in global memory (a large tensor's, whose chunks are claimed): f(c, acc, key) for the listed keys of chunks
+// Of slots in global memory: f(c, acc, key) for the listed keys of the wanted ones of chunks
 // 0 .. n_local - 1, then done(c, cnt[c], the chunk's acc).  A lane per chunk, 64 bytes at a time: many chunks in
 // flight, and little more asked for than the keys (half a warp per chunk made 4.3 GB 6 % slower).
-template <int DT, typename F, typename D>
-__device__ __forceinline__ void slot_keys_global(const typename Elem<DT>::type* slots, const uint32_t* cnt, int n_local, F f, D done) {
+template <int DT, typename W, typename F, typename D>
+__device__ __forceinline__ void slot_keys_global(const typename Elem<DT>::type* slots, const uint32_t* cnt, int n_local, W wanted, F f, D done) {
   constexpr uint32_t EPV = 16 / sizeof(typename Elem<DT>::type);
+#pragma unroll 1
   for (int c = threadIdx.x; c < n_local; c += kThreads) {
+    if (!wanted(c)) continue;
     const uint32_t v = cnt[c], n_in = min(v >> 16, static_cast<uint32_t>(slot_entries(DT)));
     uint32_t acc = 0;
     const uint4* p = reinterpret_cast<const uint4*>(slots + static_cast<long long>(c) * slot_entries(DT));
@@ -835,13 +837,17 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     }
   };
   // (streamed, not claimed) f(c, acc, key) for the listed keys of every chunk, then done(c, cnt[c], the chunk's acc) on
-  // one lane: eight lanes per chunk.
+  // one lane: eight lanes per chunk; a lane per chunk whose keys are in global memory, where that is so of two thirds or
+  // more of the keys (a chain of loads for each eight keys; fp32 on a quarter of the SMs, 134 MB, 40 % kept 250 us and 233, 70 % kept
+  // 266 and 252.  Where few chunks are in global memory a second loop loses: 268 MB on all SMs 139 and 142).
   auto listed_keys = [&](auto f, auto done) {
+    const bool many = s_list_n > 3u * kListBytes / sizeof(L);
 #pragma unroll 1
     for (int c0 = warp * 4; c0 < n_local; c0 += kWarps * 4) {
       const int c = c0 + static_cast<int>(lane >> 3);
-      const uint32_t v = c < n_local ? cnt[c] : 0u, n_in = min(v >> 16, static_cast<uint32_t>(kSlot));
-      const uint32_t start = n_in ? list_start[c] : 0u;
+      const uint32_t v = c < n_local ? cnt[c] : 0u, start = (v >> 16) ? list_start[c] : 0u;
+      const bool later = many && start == kNotListed;
+      const uint32_t n_in = later ? 0u : min(v >> 16, static_cast<uint32_t>(kSlot));
       uint32_t acc = 0;
 #pragma unroll 1
       for (uint32_t i = lane & 7u; i < n_in; i += 8) {
@@ -851,7 +857,11 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
       }
 #pragma unroll
       for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
-      if ((lane & 7u) == 0 && c < n_local) done(c, v, acc);
+      if ((lane & 7u) == 0 && c < n_local && !later) done(c, v, acc);
+    }
+    if (many) {
+      __syncthreads();                           // (done writes cnt, by which the chunks are told apart)
+      slot_keys_global<DT>(g_slots, cnt, n_local, [&](int c) { return (cnt[c] >> 16) && list_start[c] == kNotListed; }, f, done);
     }
   };
   int phase = 1;                                 // of the next exchange
@@ -1256,7 +1266,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
       if (RES) {
         for (int c = warp; c < n_local; c += kWarps) slot_keys_warp<DT>(s_slots + c * kSlot, cnt[c] >> 16, add);
       } else if (spread) {
-        slot_keys_global<DT>(g_slots, cnt, n_local, [&](int, uint32_t&, uint32_t key) { add(key); }, [](int, uint32_t, uint32_t) {});
+        slot_keys_global<DT>(g_slots, cnt, n_local, [](int) { return true; }, [&](int, uint32_t&, uint32_t key) { add(key); }, [](int, uint32_t, uint32_t) {});
       } else {
         listed_keys([&](int, uint32_t&, uint32_t key) { add(key); }, [](int, uint32_t, uint32_t) {});
       }
@@ -1424,7 +1434,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
         if (lane == 0) done(c, v, acc);
       }
     } else if (spread) {
-      slot_keys_global<DT>(g_slots, cnt, n_local, report, done);
+      slot_keys_global<DT>(g_slots, cnt, n_local, [](int) { return true; }, report, done);
     } else {
       listed_keys(report, done);
     }

@@ -226,6 +226,25 @@ def test_prune_on_a_part_of_the_gpu(chunks, extra, bf16):
 
 
 @pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("chunks", [300 * 37, 385 * 37, 900 * 37 + 1])
+def test_calls_in_a_row_on_a_part_of_the_gpu(chunks, bf16):
+    """Lists of which a part, or most, is in global memory, read by eight lanes per chunk or by one, and
+    chunks that have no tie; thirty calls with nothing to wait for in between."""
+    n = chunks * (2048 if bf16 else 1024)
+    for dist, ratio in (("normal", 0.95), ("relu_normal", 0.6)):
+        x = W.draw(dist, n, seed=12, device="cuda")
+        x = x.to(torch.bfloat16) if bf16 else x
+        out = B.CompressedActivation(n, B.dtype_code(x.dtype), ratio, "cuda")
+        ws = torch.zeros(out.sizes.workspace_bytes, dtype=torch.uint8, device="cuda")
+        headers = []
+        for _ in range(30):
+            B.surgeon_prune_compact(x, ratio, out=out, workspace=ws, flags=B.SURGEON_SHARE_GPU)
+            headers.append(out.header.clone())
+        assert_store_equals_oracle(x.cpu(), ratio, comp=out)
+        assert all(torch.equal(h, headers[-1]) for h in headers)
+
+
+@pytest.mark.parametrize("bf16", [False, True])
 def test_sample_that_misleads(bf16):
     """A short stretch holds all the large values: the strided sample sees few of them or none, so the bracket can
     miss and the select has to start over with what its counts prove."""
