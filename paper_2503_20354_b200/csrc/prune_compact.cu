@@ -1122,7 +1122,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
   unsigned long long before = 0;
   for (;;) {
   for (; step <= kRefine; ++round) {
-    if (round > 0 && tid == 1) fence_gpu();      // (it has read the answer) the bins and answers that CTA 0 has cleared for this round
+    if (round > 0 && G > 1 && tid == 1) fence_gpu();       // (it has read the answer) the bins and answers that CTA 0 has cleared for this round
     const uint32_t range = hi - lo;
     shift = max(0, 32 - __clz(range) - kSelBinsLog2);
     __syncthreads();
@@ -1357,7 +1357,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
         word_store(a.answer + phase * (kSelMaxCtas + 2) + 1, a.token, n_above | (static_cast<unsigned long long>(step) << 32));
         if (phase == 1) a.answer[0].x = 0ull;
       }
-      if (!spread && step == kKeys && tid < G) fence_gpu();  // the key words of all CTAs have been cleared
+      if (!spread && step == kKeys && G > 1 && tid < G) fence_gpu();       // the key words of all CTAs have been cleared
     } else {
       if (tid < 2) {
         unsigned long long v = 0;

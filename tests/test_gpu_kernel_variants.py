@@ -269,11 +269,11 @@ def test_streamed_tensor_at_extreme_ratios(dist, n, bf16):
         assert_store_equals_oracle(x.cpu(), ratio)
 
 
-def _awkward(kind, n):
+def _awkward(kind, n, seed=0):
     """Values that lead the select off its usual way: brackets of many keys (bf16: more than the list's bytes can
     tell apart), all keys near the threshold in one place (lists and the keys of one CTA overflow), many more
     of them in a bin than CTA 0 takes at once, or a bin of few distinct keys with many copies each."""
-    g = torch.Generator().manual_seed(n)
+    g = torch.Generator().manual_seed(n + seed)
     if kind == "log_uniform":
         return torch.exp2(240.0 * torch.rand(n, generator=g) - 120.0)
     if kind == "sorted":
@@ -287,26 +287,36 @@ def _awkward(kind, n):
     return x
 
 
+# two or three CTAs, resident, streamed; claimed (on a part of the GPU, where that begins at the fewest chunks)
 @pytest.mark.parametrize("bf16", [False, True])
-@pytest.mark.parametrize("n", [40000, 3_000_001, 18_000_003])        # one CTA or two, resident, streamed
+@pytest.mark.parametrize("n", [40000, 3_000_001, 18_000_003, "claimed"])
 @pytest.mark.parametrize("kind", ["log_uniform", "sorted", "clustered", "few_keys"])
 def test_select_off_its_usual_way(kind, n, bf16):
-    x = _awkward(kind, n)
-    x = x.to(torch.bfloat16) if bf16 else x
-    ratio = 1.0 - float((x.abs() > 1.0005).double().mean()) if kind == "clustered" else 0.7
-    comp, _ = assert_store_equals_oracle(x, ratio)
-    ref = [v.copy() for v in comp.to_numpy()[:3]]
-    xc, ws = x.cuda(), torch.empty(comp.sizes.workspace_bytes, dtype=torch.uint8, device="cuda")
+    flags = B.SURGEON_SHARE_GPU if n == "claimed" else 0
+    n = (1024 * 37 + 1) * (2048 if bf16 else 1024) + 5 if flags else n
+    xs = [_awkward(kind, n), 1.25 * _awkward(kind, n, 1).flip(0), torch.randn(n, generator=torch.Generator().manual_seed(n))]
+    ratio = 1.0 - float((xs[0].abs() > 1.0005).double().mean()) if kind == "clustered" else 0.7
+    refs = []
+    for i, x in enumerate(xs):
+        xs[i] = x = (x.to(torch.bfloat16) if bf16 else x).cuda()
+        comp = B.surgeon_prune_compact(x, ratio)       # (claimed: the same tensor streamed on the whole GPU is the reference)
+        if not flags:
+            assert_store_equals_oracle(x.cpu(), ratio, comp=comp)
+        refs.append([v.clone() for v in (comp.bitmap, comp.values, comp.block_offsets, comp.header)])
+    x, out = xs[0].clone(), B.CompressedActivation(n, B.dtype_code(xs[0].dtype), ratio, "cuda")
+    ws = torch.zeros(out.sizes.workspace_bytes, dtype=torch.uint8, device="cuda")
     graph = torch.cuda.CUDAGraph()
     with torch.cuda.graph(graph):
-        B.surgeon_prune_compact(xc, ratio, out=comp, workspace=ws)
-    for _ in range(2):                           # replays carry the same token: nothing of the first is taken for the second
-        for part in (comp.bitmap, comp.values, comp.block_offsets):
+        B.surgeon_prune_compact(x, ratio, out=out, workspace=ws, flags=flags)
+    for i in (0, 1, 2, 1, 0, 0):                 # replays carry the same token, and find the scratch as another tensor's left it
+        x.copy_(xs[i])
+        for part in (out.bitmap, out.values, out.block_offsets):
             part.zero_()
         graph.replay()
         torch.cuda.synchronize()
-        assert comp.read_header().status == B.SURGEON_OK
-        assert all(np.array_equal(u.view(np.uint8), v.view(np.uint8)) for u, v in zip(comp.to_numpy()[:3], ref))
+        assert out.read_header().status == B.SURGEON_OK
+        for got, ref in zip((out.bitmap, out.values, out.block_offsets, out.header), refs[i]):
+            assert torch.equal(got.view(torch.uint8), ref.view(torch.uint8))
 
 
 @pytest.mark.parametrize("n", [5000, (1 << 23) + 77])
