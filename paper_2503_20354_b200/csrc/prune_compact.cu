@@ -362,7 +362,7 @@ __device__ __forceinline__ unsigned long long warp_incl_u64(unsigned long long v
 // are ranked by flat index (= lane, then bit).  Out of line, like all that one chunk of a tensor does: code that is not
 // in the instruction caches costs some 250 clocks per 128 bytes, and a call runs most of its code once.
 template <int DT>
-__device__ __forceinline__ uint2 quota_words_inline(const unsigned char* region, int nv, uint32_t tau, long long allowed, uint2 above) {
+__device__ __noinline__ uint2 quota_words(const unsigned char* region, int nv, uint32_t tau, long long allowed, uint2 above) {
   constexpr int WPL = 128 / static_cast<int>(sizeof(typename Elem<DT>::type)) / 32;
   uint4 q[8];
   load_row(region, q);
@@ -377,10 +377,6 @@ __device__ __forceinline__ uint2 quota_words_inline(const unsigned char* region,
     allowed -= __popc(ge[w]);
   }
   return make_uint2(word[0], word[1]);
-}
-template <int DT>
-__device__ __noinline__ uint2 quota_words(const unsigned char* region, int nv, uint32_t tau, long long allowed, uint2 above) {
-  return quota_words_inline<DT>(region, nv, tau, allowed, above);
 }
 
 // The byte at address a of a packed sequence lives at a ^ ((a >> 5) & 0x7C): the 32-bit word
@@ -400,7 +396,7 @@ __device__ __forceinline__ uint32_t packed_elem(uint32_t rbase, uint32_t i) {   
 }
 // A full chunk with a misaligned destination: no room for the shift, the vectors are put together from elements.
 template <int DT>
-__device__ __forceinline__ void copy_full_chunk_inline(typename Elem<DT>::type* values, long long kept_before, uint32_t total, uint32_t rbase,
+__device__ __noinline__ void copy_full_chunk(typename Elem<DT>::type* values, long long kept_before, uint32_t total, uint32_t rbase,
                                              long long n_stored, uint32_t* status) {
   using E = typename Elem<DT>::type;
   constexpr int EPV = 16 / sizeof(E);
@@ -425,18 +421,11 @@ __device__ __forceinline__ void copy_full_chunk_inline(typename Elem<DT>::type* 
   if (lane < total - done && SURGEON_IN_BOUNDS(kept_before + done + lane, n_stored, status))
     dst[done + lane] = static_cast<E>(packed_elem<DT>(rbase, done + lane));
 }
-template <int DT>
-__device__ __noinline__ void copy_full_chunk(typename Elem<DT>::type* values, long long kept_before, uint32_t total, uint32_t rbase,
-                                             long long n_stored, uint32_t* status) {
-  copy_full_chunk_inline<DT>(values, kept_before, total, rbase, n_stored, status);
-}
 
 // ---- emit one chunk -------------------------------------------------------------------------------
 // before = (elements above the threshold before the chunk) << 32 | (ties before it); n_eq = its ties.
 // True when the chunk's place in the ring has been written to.
-// kClaimedTensor: of a gigabyte tensor, whose kernel runs its loop some thousand times: what is rare is in line there (calls in the loop
-// cost 4.3 GB of fp32 1745 -> 1810 us).
-template <int DT, bool kPlain, bool kClaimedTensor>
+template <int DT>
 __device__ __forceinline__ bool emit_chunk(const PruneArgs& a, unsigned char* region, int chunk, uint32_t tau, long long quota,
                                            unsigned long long before, uint32_t n_eq, long long n_stored) {
   using E = typename Elem<DT>::type;
@@ -461,8 +450,7 @@ __device__ __forceinline__ bool emit_chunk(const PruneArgs& a, unsigned char* re
   mask_ge<DT, WPL>(q, nv, ties ? tau : tau + 1u, word);
   if (!ties && eq_b < quota) {
     const uint2 above = make_uint2(word[0], word[WPL - 1]);
-    const uint2 both = kClaimedTensor ? quota_words_inline<DT>(region, nv, tau, quota - eq_b, above)
-                                      : quota_words<DT>(region, nv, tau, quota - eq_b, above);
+    const uint2 both = quota_words<DT>(region, nv, tau, quota - eq_b, above);
     word[0] = both.x;
     if (WPL == 2) word[WPL - 1] = both.y;
   }
@@ -499,7 +487,7 @@ __device__ __forceinline__ bool emit_chunk(const PruneArgs& a, unsigned char* re
   const uint32_t mis = static_cast<uint32_t>(kept_before % EPV);
   // Gathered in place in the chunk's own part of the ring, whatever share is kept.  (Sparse chunks by a loop over the set
   // bits into a staging area took as long where 7-10 % are kept, and longer elsewhere: bf16, 77 MB, 30 % kept 72 against
-  // 65.5 us, 537 MB 353 against 314; 4.3 GB of fp32 1755 against 1710, by what the second path costs the first.)
+  // 65.5 us, 537 MB 353 against 314.)
   __syncwarp();                                  // every lane has its row in registers
   const uint32_t rbase = smem_u32(region);
   const bool lined_up = total + mis <= static_cast<uint32_t>(32 * EPR);
@@ -527,8 +515,9 @@ __device__ __forceinline__ bool emit_chunk(const PruneArgs& a, unsigned char* re
   };
   // Rows kept by five eighths at most start far enough from multiples of 32 words without the XOR, which is a third
   // of the gather's instructions: bf16, 2 GB, a tenth kept 980 -> 920 us, 537 MB 292 -> 274, 77 MB 65.5 -> 63.5; fp32,
-  // 131 MB 84.0 -> 81.9, but 4.3 GB 1795 -> 1805, which keep the one path (kPlain).
-  if (kPlain && lined_up && __reduce_max_sync(kFull, cnt) <= 5u * EPR / 8u) {
+  // 131 MB 84.0 -> 81.9, 4.3 GB, a tenth kept 1562 -> 1514 (half kept: 1857 and 1856, runs of one side differ by 20).
+  constexpr uint32_t kMost = 5u * EPR / 8u;
+  if (lined_up && total <= 32u * kMost && __reduce_max_sync(kFull, cnt) <= kMost) {
     gather([](uint32_t addr) { return addr; });
     __syncwarp();
     E* gbase = values + (kept_before - mis);
@@ -577,8 +566,7 @@ __device__ __forceinline__ bool emit_chunk(const PruneArgs& a, unsigned char* re
     if (t0 + lane < end && SURGEON_IN_BOUNDS(kept_before - mis + t0 + lane, n_stored, &a.hdr->status))
       gbase[t0 + lane] = static_cast<E>(packed_elem<DT>(rbase, t0 + lane));
   } else {
-    if (kClaimedTensor) copy_full_chunk_inline<DT>(values, kept_before, total, rbase, n_stored, &a.hdr->status);
-    else copy_full_chunk<DT>(values, kept_before, total, rbase, n_stored, &a.hdr->status);
+    copy_full_chunk<DT>(values, kept_before, total, rbase, n_stored, &a.hdr->status);
   }
   return true;
 }
@@ -1698,7 +1686,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
   // ---- emit ----
   if (RES) {
     run_resident(false, [&](int c, unsigned char* region) -> bool {
-      return emit_chunk<DT, (DT == 1 || MODE != kClaimed), MODE == kClaimed>(a, region, c, tau, quota, prefix[c - c_begin], cnt[c - c_begin] >> 16, n_stored);
+      return emit_chunk<DT>(a, region, c, tau, quota, prefix[c - c_begin], cnt[c - c_begin] >> 16, n_stored);
     });
     return kDone;
   }
@@ -1725,7 +1713,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     uint32_t n_at = n_next;
     if (!spread) { at = prefix[c - c_begin]; n_at = cnt[c - c_begin]; }
     else if (fly1 < a.n_chunks) { at_next = prefix[fly1 - c_begin]; n_next = cnt[fly1 - c_begin]; }
-    const bool written = emit_chunk<DT, (DT == 1 || MODE != kClaimed), MODE == kClaimed>(a, my_ring + s * kChunkBytes, c, tau, quota, at, n_at >> 16, n_stored);
+    const bool written = emit_chunk<DT>(a, my_ring + s * kChunkBytes, c, tau, quota, at, n_at >> 16, n_stored);
     int c_load;                                  // what the place takes next
     if (spread) {
       fly0 = fly1; fly1 = fly2;
