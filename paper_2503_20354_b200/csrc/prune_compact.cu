@@ -1948,7 +1948,8 @@ cudaError_t run_prune_compact(const void* x, long long n, long long k, int drop_
     grid = (a.n_chunks + per_cta - 1) / per_cta;
   }
   // claimed chunks (see the kernel): by itself from 512 chunks per CTA on, where equal shares end unevenly; on a part
-  // of the GPU only where the counts do not fit (on a quarter, 131 MB: 335 -> 310 us bf16, 260 -> 238 fp32)
+  // of the GPU only where the counts do not fit (on a quarter, 134 MB fp32, claimed and streamed: 40 % kept 249 and 233 us,
+  // 5 % kept 216 and 199, 70 % kept 250 and 252)
   const bool claimed = a.n_chunks > grid * (share ? kMaxLocalChunks : 512);
   const bool resident = (a.n_chunks + grid - 1) / grid <= kResidentChunks;
   const void* kernel = resident  ? reinterpret_cast<const void*>(prune_kernel<DT, kResident>)

@@ -272,7 +272,7 @@ constexpr int kG3MaxTile = 8;
 // leaves room for twice as many CTAs, which hide one another's load phases.  1280 channels on 64x64, batch 1, half
 // kept: 51 -> 31 us a call.  Not where it has fewer than four rows, two of which are halo (16 channels 1536 wide, three
 // rows: 211 us, on tiles of 110 KB 184; 3072 wide, one row: 513 and 276), nor under stride 2 where the whole map
-// fits the larger tile only (256 channels on 128x128: 24.8 and 18.7; under stride 1 96x96 takes 26.8 and 33).
+// fits the larger tile only (256 channels on 128x128: 24.8 and 20.7; under stride 1 96x96 takes 26.8 and 33).
 constexpr int kG3CtasPerSmDepthwise = 4;
 constexpr int kG3SmemDepthwise = 54 * 1024;
 constexpr int kG3LeastRowsDepthwise = 4;
