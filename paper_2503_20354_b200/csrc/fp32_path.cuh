@@ -1,0 +1,30 @@
+// The fp32 path of surgeon_weight_grad on the tensor cores (weight_grad_fp32_split.cu), as the path's launcher
+// (weight_grad_fp32.cu) uses it.
+#pragma once
+
+#include "surgeon_internal.cuh"
+
+namespace surgeon {
+
+struct SplitGeom {
+  int C, H, W, O, KW, RS, stride, pad, OH, OW;
+  int P, K, N;              // positions per image (linear: 1), what the GEMM sums over, its columns (c, r, s)
+  int step_y, step_x;       // 64 positions, in rows and columns of the output
+  int most_len;             // positions of one output row that 32 input elements hold
+  int linear, vec;          // vec: the gradient can be read 16 bytes at a time
+  int grad_blocks;          // blocks of the pre-pass that writes the gradient's planes
+  uint32_t n_words;         // words of the bitmap
+  uint32_t mul_p, shift_p, mul_w, shift_w;       // division by P and OW
+  int tile_n, nt, mt;       // output channels per CTA, tiles of them, tiles of 128 columns
+  int warp_cols, tmem_cols;
+  int k_tiles, per_chunk, chunks, ctas;
+};
+// False: the layer is not one for it.
+bool plan_split(const surgeon_layer_desc& d, SplitGeom* out);
+size_t split_planes_bytes(const SplitGeom& g);
+// partial: [chunks][O][N].  most: the largest magnitudes of the gradient (a word per block of the pre-pass) and then of the
+// activation (a word per CTA), as bf16 patterns; 0xFFFF from a CTA that gave up.
+cudaError_t launch_split(const surgeon_compressed& act, const SplitGeom& g, const float* grad_out, void* planes,
+                         float* partial, uint32_t* most, cudaStream_t stream);
+
+}  // namespace surgeon

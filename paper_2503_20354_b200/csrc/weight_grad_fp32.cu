@@ -1,4 +1,5 @@
-// fp32 CUDA-core path of surgeon_weight_grad (Algorithm 1: Reshape and gradient steps, Eq. 2).
+// fp32 path of surgeon_weight_grad (Algorithm 1: Reshape and gradient steps, Eq. 2): its launcher, and the kernel on CUDA
+// cores, for the layers that the tensor cores (weight_grad_fp32_split.cu) do not take and the operands that they cannot hold.
 //
 // Implicit GEMM  dW[m, nn] = sum_k G[k, m] * Acol[k, nn]  with m = output channel,
 // nn = (c, r, s) and k = (b, y, x) (or the row t of a linear layer).  The im2col operand is
@@ -16,9 +17,10 @@
 // computation per element and 4 x 4 outputs per thread, 264 us now: 28.6 TFLOP/s, 38 % of what the
 // FMA pipes could do, since rebuilding and products take turns.  Small maps (128 -> 128 channels on
 // 1x1, 200 000 images: 0.42 ms) and linear layers (4096 rows, 320 -> 320: 70 us) by elements.
+#include <algorithm>
 #include <type_traits>
 
-#include "surgeon_internal.cuh"
+#include "fp32_path.cuh"
 
 namespace surgeon {
 
@@ -40,6 +42,23 @@ struct Geom {
   long long M, N;        // its other extents
   long long n_words;
 };
+
+// What the tensor cores (weight_grad_fp32_split.cu) left behind, where they ran first.
+struct SplitResult {
+  const uint32_t* most;     // largest magnitudes: n_grad words of the gradient, n_act of the activation
+  int* n_parts;             // to be set: partial sums per output
+  int n_grad, n_act, chunks;
+};
+
+// Whether the three bf16 parts held all of every operand, given the bit patterns of the largest magnitudes.  Infinities and
+// NaN have no parts.  A third part lies 2^-24 below its number and is lost below 2^-133, products below 2^-126: ranges
+// that end well above both, and below 2^127.
+__device__ __forceinline__ bool split_holds(uint32_t a, uint32_t b) {
+  if (a >= 0x7F80u || b >= 0x7F80u) return false;
+  if (a == 0 || b == 0) return true;
+  const uint32_t ea = a >> 7, eb = b >> 7;       // exponents, 127 more than they are
+  return ea >= 127 - 80 && eb >= 127 - 80 && ea + eb >= 2 * 127 - 80 && ea + eb <= 2 * 127 + 100;
+}
 
 Geom make_geom(const surgeon_layer_desc& d) {
   Geom g;
@@ -154,7 +173,28 @@ template <int DT, int KIND, bool SPAN>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 dw_fp32_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ values,
                const uint32_t* __restrict__ offsets, const float* __restrict__ grad,
-               float* __restrict__ partial, Geom g) {
+               float* __restrict__ partial, Geom g, SplitResult split) {
+  if (split.most) {                              // the tensor cores' result stands unless their planes could not hold an operand
+    pdl_wait();
+    __shared__ uint32_t s_most[2];
+    if (threadIdx.x < 2) s_most[threadIdx.x] = 0;
+    __syncthreads();
+    uint32_t m[2] = {0, 0};
+    for (int i = threadIdx.x; i < split.n_grad + split.n_act; i += kThreads) {
+      uint32_t& x = m[i < split.n_grad ? 0 : 1];
+      x = max(x, split.most[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      m[i] = __reduce_max_sync(0xFFFFFFFFu, m[i]);
+      if (lane_id() == 0) atomicMax(&s_most[i], m[i]);
+    }
+    __syncthreads();
+    const bool stands = split_holds(s_most[0], s_most[1]);
+    if (threadIdx.x == 0 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) *split.n_parts = stands ? split.chunks : g.chunks;
+    pdl_trigger();
+    if (stands) return;
+  }
   __shared__ __align__(16) float Gs[TK][kGPitch];
   __shared__ __align__(16) float As[TK][kAPitch];
   const int tid = threadIdx.x;
@@ -341,22 +381,58 @@ dw_fp32_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ val
   }
 }
 
+// The partial sums, in double, in a fixed order.  n_parts: how many there are (null: `chunks`).  V outputs a thread, or
+// (V = 1, blocks of 32 x 8) one by eight threads, which take every eighth partial sum.
+template <int V, bool EIGHT>
 __global__ void __launch_bounds__(256)
-reduce_chunks_kernel(const float* __restrict__ partial, long long mn, int chunks,
+reduce_chunks_kernel(const float* __restrict__ partial, long long mn, int chunks, const int* n_parts,
                      float* __restrict__ dw, int accumulate) {
-  const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i >= mn) return;
-  double s = 0.0;
+  static_assert(V == 1 || !EIGHT, "one output");
+  pdl_wait();
+  if (n_parts) chunks = *n_parts;
+  const long long i = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) * V;
+  using Vec = typename std::conditional<V == 4, float4, float>::type;
+  double s[V];
+#pragma unroll
+  for (int e = 0; e < V; ++e) s[e] = 0.0;
+  if (i < mn) {
 #pragma unroll 8
-  for (int z = 0; z < chunks; ++z) s += static_cast<double>(__ldg(partial + z * mn + i));
-  dw[i] = accumulate ? static_cast<float>(static_cast<double>(dw[i]) + s) : static_cast<float>(s);
+    for (int z = EIGHT ? threadIdx.y : 0; z < chunks; z += EIGHT ? 8 : 1) {
+      const Vec v = __ldg(reinterpret_cast<const Vec*>(partial + z * mn + i));
+#pragma unroll
+      for (int e = 0; e < V; ++e) s[e] += static_cast<double>(reinterpret_cast<const float*>(&v)[e]);
+    }
+  }
+  if (EIGHT) {
+    __shared__ double part[8][32];
+    part[threadIdx.y][threadIdx.x] = s[0];
+    __syncthreads();
+    if (threadIdx.y != 0) return;
+#pragma unroll
+    for (int y = 1; y < 8; ++y) s[0] += part[y][threadIdx.x];
+  }
+  if (i >= mn) return;
+  float out[V];
+#pragma unroll
+  for (int e = 0; e < V; ++e)
+    out[e] = accumulate ? static_cast<float>(static_cast<double>(dw[i + e]) + s[e]) : static_cast<float>(s[e]);
+  *reinterpret_cast<Vec*>(dw + i) = *reinterpret_cast<const Vec*>(out);
 }
 
 }  // namespace
 
+// Scratch of a layer for the tensor cores: the count of partial sums per output and the largest magnitudes, the gradient's
+// planes, then the partial sums.
+static size_t split_head_bytes(const SplitGeom& s) {
+  return (16 + (static_cast<size_t>(s.grad_blocks) + s.ctas) * 4 + 255) & ~static_cast<size_t>(255);
+}
+
 size_t weight_grad_fp32_workspace(const surgeon_layer_desc& d) {
   const Geom g = make_geom(d);
-  return static_cast<size_t>(g.chunks < 1 ? 1 : g.chunks) * g.M * g.N * sizeof(float);
+  SplitGeom s;
+  const bool split = plan_split(d, &s);
+  const int chunks = std::max(std::max(g.chunks, 1), split ? s.chunks : 0);
+  return (split ? split_head_bytes(s) + split_planes_bytes(s) : 0) + static_cast<size_t>(chunks) * g.M * g.N * sizeof(float);
 }
 
 cudaError_t launch_weight_grad_fp32(const surgeon_compressed& act, const surgeon_layer_desc& d,
@@ -364,12 +440,24 @@ cudaError_t launch_weight_grad_fp32(const surgeon_compressed& act, const surgeon
                                     void* workspace, cudaStream_t stream) {
   const Geom g = make_geom(d);
   float* partial = static_cast<float*>(workspace);
+  SplitGeom s;
+  SplitResult result = {};
+  if (g.chunks > 0 && plan_split(d, &s)) {
+    int* n_parts = static_cast<int*>(workspace);
+    uint32_t* most = static_cast<uint32_t*>(workspace) + 4;
+    char* planes = static_cast<char*>(workspace) + split_head_bytes(s);
+    partial = reinterpret_cast<float*>(planes + split_planes_bytes(s));
+    result = {most, n_parts, s.grad_blocks, s.ctas, s.chunks};
+    const cudaError_t e = launch_split(act, s, grad_out, planes, partial, most, stream);
+    if (e != cudaSuccess) return e;
+  }
   if (g.chunks > 65535 || (g.M + TM - 1) / TM > 65535) return cudaErrorNotSupported;
   if (g.chunks > 0) {
     dim3 grid(static_cast<unsigned>((g.N + TN - 1) / TN), static_cast<unsigned>((g.M + TM - 1) / TM),
               static_cast<unsigned>(g.chunks));
     auto launch = [&](auto kernel) {
-      kernel<<<grid, kThreads, 0, stream>>>(act.bitmap, act.values, act.block_offsets, grad_out, partial, g);
+      launch_kernel(kernel, grid, dim3(kThreads), 0, stream, result.most != nullptr, act.bitmap,
+                    static_cast<const void*>(act.values), act.block_offsets, grad_out, partial, g, result);
     };
     auto launch_kind = [&](auto kind, auto span) {
       act.dt == 0 ? launch(dw_fp32_kernel<0, decltype(kind)::value, decltype(span)::value>)
@@ -385,8 +473,15 @@ cudaError_t launch_weight_grad_fp32(const surgeon_compressed& act, const surgeon
     note_launches(1);
   }
   const long long mn = g.M * g.N;
-  reduce_chunks_kernel<<<static_cast<unsigned>((mn + 255) / 256), 256, 0, stream>>>(
-      partial, mn, g.chunks, dw, accumulate);
+  const int parts = result.most ? result.chunks : g.chunks;
+  auto reduce = [&](auto kernel, int per_block, dim3 block) {
+    launch_kernel(kernel, dim3(static_cast<unsigned>((mn + per_block - 1) / per_block)), block, 0, stream,
+                  result.most != nullptr, partial, mn, g.chunks, result.n_parts, dw, accumulate);
+  };
+  // Few outputs of many partial sums: eight threads each (432 of 96: 14 us by one thread each).
+  if (parts >= 16 && mn < 65536) reduce(reduce_chunks_kernel<1, true>, 32, dim3(32, 8));
+  else if (mn % 4 == 0 && mn >= 262144) reduce(reduce_chunks_kernel<4, false>, 1024, dim3(256));
+  else reduce(reduce_chunks_kernel<1, false>, 256, dim3(256));
   note_launches(1);
   return cudaGetLastError();
 }

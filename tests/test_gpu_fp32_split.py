@@ -1,0 +1,85 @@
+"""The fp32 path on the tensor cores, against the fp64 oracle: edges of its tiles, and operands that the three bf16
+parts of a number cannot hold.
+
+Tolerance 1e-6 (relative Frobenius error).  A K-tile's sum of the large products is cut off four times, by a unit in the
+last place (2^-23) at most each: 4.8e-7.  At most 32 of them are added in fp32, errors of 2^-24 and random sign:
+3.4e-7.  What is left out of a product, and what is cut off the small ones, is below 1e-7."""
+import numpy as np
+import pytest
+import torch
+from dataclasses import replace
+
+import oracle
+from paper_2503_20354_b200 import binding as B
+from paper_2503_20354_b200 import workloads as W
+from gpu_util import oracle_dw, rel_frobenius
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [
+    # K-tiles of 64 positions over the images: one short of a tile, one more; maps whose rows are split
+    W.conv("k63", 1, 24, 7, 40, 1, 1, 0), W.conv("k65_chunks", 13, 130, 5, 17, 1, 1, 0),
+    W.conv("w14_c136_o161", 5, 136, 14, 161, 1, 1, 0), W.conv("w7_o159", 3, 15, 7, 159, 3),
+    W.conv("w4", 9, 9, 4, 33, 3), W.conv("w33_5x5", 1, 5, 33, 16, 5, 1, 2), W.conv("w16_o320", 2, 43, 16, 320, 3),
+    W.Layer("h3w50_2x3", 1, 2, 7, 3, 50, 20, 2, 3, 1, 1),
+    # strides: pieces of 16, 11, 7 and 4 positions
+    W.conv("s2", 6, 40, 30, 96, 3, 2), W.conv("s3", 8, 24, 40, 64, 5, 3, 1), W.conv("s5", 8, 16, 64, 96, 7, 5, 3),
+    W.conv("s8", 12, 64, 64, 32, 8, 8, 0),
+    # linear: columns and channels around the tiles, channels that are no multiple of 4 or 16
+    W.linear("t64", 64, 128, 64, dist="normal"), W.linear("t65", 65, 129, 65, dist="normal"),
+    W.linear("t1000", 1000, 31, 127, dist="normal"), W.linear("t2049", 2049, 17, 130, dist="normal"),
+    W.linear("t1", 1, 300, 10, dist="normal"),
+]
+
+
+@pytest.mark.parametrize("ratio", [0.0, 0.8])
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("layer", SHAPES, ids=lambda l: l.name)
+def test_tile_edges(layer, bf16, ratio):
+    layer = replace(layer, dt=W.BF16 if bf16 else W.F32)
+    a, g = W.activation(layer, 5), W.grad_out(layer, 5)
+    store = B.surgeon_prune_compact(a.cuda(), ratio)
+    dw = B.surgeon_weight_grad(store, B.layer_desc(layer, B.PATH_FP32), g.cuda())
+    bits = W.as_numpy_bits(a).reshape(-1)
+    r = oracle.prune_compact(bits, ratio)
+    ref = oracle_dw(layer, oracle.decompress(r["bitmap"], r["values"], bits.size), g.numpy())
+    assert rel_frobenius(dw.cpu().numpy(), ref) <= 1e-6
+    # added to what is there
+    twice = B.surgeon_weight_grad(store, B.layer_desc(layer, B.PATH_FP32), g.cuda(), dw=dw.clone(), accumulate=True)
+    assert rel_frobenius(twice.cpu().numpy(), 2 * ref) <= 1e-6
+
+
+LINEAR = W.linear("tokens", 700, 160, 96, dist="normal", dt=W.F32)
+
+
+@pytest.mark.parametrize("scale_a,scale_g", [(1e-32, 1.0), (1.0, 1e-36), (1e-18, 1e-17), (1e18, 1e17), (3e37, 1e-30)])
+def test_magnitudes_at_the_ends_of_the_range(scale_a, scale_g):
+    a, g = W.activation(LINEAR, 7) * scale_a, W.grad_out(LINEAR, 7) * scale_g
+    store = B.surgeon_prune_compact(a.cuda(), 0.0)
+    dw = B.surgeon_weight_grad(store, B.layer_desc(LINEAR, B.PATH_FP32), g.cuda()).cpu().numpy().astype(np.float64)
+    ref = g.numpy().astype(np.float64).T @ a.numpy().astype(np.float64).reshape(700, -1)
+    # (fp32 ends at 2^-149: half of it for each of the 700 terms where the products lie there)
+    assert np.linalg.norm(dw - ref) <= 1e-5 * np.linalg.norm(ref) + 2.0 ** -150 * 700 * np.sqrt(ref.size)
+
+
+@pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
+@pytest.mark.parametrize("where", ["activation", "gradient"])
+def test_infinities_and_nan(where, value):
+    a, g = W.activation(LINEAR, 8), W.grad_out(LINEAR, 8)
+    (a.view(700, -1) if where == "activation" else g)[123, 45] = value
+    store = B.surgeon_prune_compact(a.cuda(), 0.0)
+    dw = B.surgeon_weight_grad(store, B.layer_desc(LINEAR, B.PATH_FP32), g.cuda()).cpu().numpy()
+    with np.errstate(invalid="ignore"):
+        ref = g.numpy().astype(np.float64).T @ a.numpy().astype(np.float64).reshape(700, -1)
+    assert np.array_equal(np.isnan(dw), np.isnan(ref))
+    assert np.array_equal(np.where(np.isinf(dw), dw, 0), np.where(np.isinf(ref), ref, 0))
+    ok = np.isfinite(ref)
+    assert ok.any() and rel_frobenius(dw[ok], ref[ok]) <= 1e-5
+
+
+def test_an_exact_product_stays_exact():
+    """One row of the gradient is one value: dW is that row of the activation, to the last bit."""
+    a, g = W.activation(LINEAR, 9), torch.zeros(700, 96)
+    g[77, 5] = 1.0
+    dw = B.surgeon_weight_grad(B.surgeon_prune_compact(a.cuda(), 0.0), B.layer_desc(LINEAR, B.PATH_FP32), g.cuda()).cpu()
+    assert torch.equal(dw.view(96, -1)[5], a.view(700, -1)[77]) and not dw.view(96, -1)[6].any()
