@@ -14,7 +14,7 @@ struct SplitGeom {
   int linear, vec;          // vec: the gradient can be read 16 bytes at a time
   int grad_blocks;          // blocks of the pre-pass that writes the gradient's planes
   uint32_t n_words;         // words of the bitmap
-  uint32_t mul_p, shift_p, mul_w, shift_w;       // division by P and OW
+  FastDiv by_p, by_ow;      // division by P and OW
   int tile_n, nt, mt;       // output channels per CTA, tiles of them, tiles of 128 columns
   int warp_cols, tmem_cols;
   int k_tiles, per_chunk, chunks, ctas;

@@ -152,6 +152,18 @@ inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block
 #define SURGEON_IN_BOUNDS(idx, limit, status_word) true
 #endif
 
+// Division of numbers below 2^31 by one that the host knows: two instructions instead of some 35.
+struct FastDiv {
+  uint32_t mul, shift;
+};
+inline FastDiv make_div(uint32_t d) {            // d >= 1
+  FastDiv f{0, 0};
+  while ((1ull << f.shift) < d) ++f.shift;
+  f.mul = static_cast<uint32_t>(((1ull << 32) * ((1ull << f.shift) - d)) / d + 1);
+  return f;
+}
+__device__ __forceinline__ uint32_t divide(uint32_t n, FastDiv f) { return (__umulhi(n, f.mul) + n) >> f.shift; }
+
 __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31; }
 __device__ __forceinline__ uint32_t lanemask_lt() {
   uint32_t m;

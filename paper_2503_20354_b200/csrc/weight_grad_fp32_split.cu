@@ -52,11 +52,6 @@ constexpr int kMaxTileN = 160;                   // 40 sums a thread; two accumu
 constexpr int kPlaneA = kTileM * kTileK * 2;     // 16 KB
 constexpr int kMaxTiles = 2048 / kTileK;         // K-tiles of one chunk at most
 
-// Unsigned division by a constant of the layer, for numbers below 2^31.
-__device__ __forceinline__ uint32_t divide(uint32_t n, uint32_t mul, uint32_t shift) {
-  return (__umulhi(n, mul) + n) >> shift;
-}
-
 // x0, x1 -> their three parts, two to a word.
 __device__ __forceinline__ void split2(float x0, float x1, uint32_t& p1, uint32_t& p2, uint32_t& p3) {
   p1 = pack_bf16x2(x0, x1);
@@ -112,7 +107,7 @@ grad_split_kernel(const float* __restrict__ grad, unsigned char* __restrict__ ou
        i += static_cast<long long>(gridDim.x) * blockDim.x) {
     const int row = static_cast<int>(i / per_row), col = static_cast<int>(i - static_cast<long long>(row) * per_row) * 8;
     // a row's columns are in pieces of P, one per image (linear: in one piece)
-    const uint32_t img = g.linear ? 0u : divide(col, g.mul_p, g.shift_p), p = col - img * g.P;
+    const uint32_t img = g.linear ? 0u : divide(col, g.by_p), p = col - img * g.P;
     const float* at = grad + (g.linear ? static_cast<size_t>(row) * g.O + col : (static_cast<size_t>(img) * g.O + row) * g.P + p);
     const size_t skip = g.linear ? 0 : static_cast<size_t>(g.O - 1) * g.P;        // from an image's end to the next one
     const int len = row < n_rows ? n_cols : 0;
@@ -274,9 +269,9 @@ dw_split_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ va
     int img = 0, y = 0, x = 0, kp = 0;           // (convolution) the lane's first position of the tile that is asked for
     if (KIND != 0) {
       kp = kt_begin * kTileK + 16 * part;
-      img = divide(kp, g.mul_p, g.shift_p);
+      img = divide(kp, g.by_p);
       const int p = kp - img * g.P;
-      y = divide(p, g.mul_w, g.shift_w);
+      y = divide(p, g.by_ow);
       x = p - y * g.OW;
     }
     auto fetch = [&]() {
@@ -459,13 +454,6 @@ dw_split_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ va
   if (tid == 0) most[(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = fail ? 0xFFFFu : s_most;
 }
 
-void find_divisor(uint32_t d, uint32_t* mul, uint32_t* shift) {
-  uint32_t l = 0;
-  while ((1ull << l) < d) ++l;
-  *shift = l;
-  *mul = static_cast<uint32_t>(((1ull << 32) * ((1ull << l) - d)) / d + 1);
-}
-
 bool compute_plan_split(const surgeon_layer_desc& d, SplitGeom* out) {
   SplitGeom g{};
   const long long rows = d.batch;
@@ -487,8 +475,8 @@ bool compute_plan_split(const surgeon_layer_desc& d, SplitGeom* out) {
   g.linear = d.kind == 1 ? 0 : 1;
   g.vec = (g.linear ? d.c_out % 4 == 0 : P % 4 == 0) ? 1 : 0;
   g.n_words = static_cast<uint32_t>((rows * d.c_in * d.h * d.w + 31) / 32);
-  find_divisor(g.P, &g.mul_p, &g.shift_p);
-  find_divisor(d.kind == 1 ? g.OW : 1, &g.mul_w, &g.shift_w);
+  g.by_p = make_div(g.P);
+  g.by_ow = make_div(d.kind == 1 ? g.OW : 1);
   // Columns: as few tiles as 160 allows, of equal width (linear: slabs of 64).
   if (d.kind == 1) {
     g.nt = (g.O + kMaxTileN - 1) / kMaxTileN;

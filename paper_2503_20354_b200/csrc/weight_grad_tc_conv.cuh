@@ -59,10 +59,10 @@ struct StridedParams {
   int patch_rows, plane;    // input rows of a patch, elements of a phase plane of one row
   int patch_bytes, stages, tmem_cols, smem_bytes;
   unsigned inv_stride;      // ix / stride = ix * inv_stride >> 16
-  unsigned inv_per_row;     // division by the pieces per row (high word of a product)
+  FastDiv by_row, by_ch;    // division by the pieces per row, and per channel of the patch,
+  FastDiv by_owp, by_macros;         // by OWp, and by the macros of an image
   unsigned partial_blk;     // index of the bitmap's last block if it is partial, else 0xFFFFFFFF (launcher)
   long long n_words;        // words of the bitmap (filled by the launcher)
-  const long long* n_keep_ptr;  // device address of the store's count of packed values (launcher)
 };
 bool plan_strided(const surgeon_layer_desc& d, StridedParams* out);
 size_t strided_partial_bytes(const StridedParams& p);

@@ -10,17 +10,21 @@
 //   1. the input rows that the macro's positions touch are rebuilt from the store in a shared-memory
 //      patch, one lane per 16 elements of a row, once for all taps.  A row is kept as `stride` phase
 //      planes (column ix goes to plane ix mod stride, place ix div stride), with zeros around:
-//      what a tap reads for consecutive output positions is then consecutive, whatever the stride;
+//      what a tap reads for consecutive output positions is then consecutive, whatever the stride.  For strides 1 and 2
+//      a lane's elements are whole 16-byte vectors of the planes, put together in registers;
 //   2. a thread copies one chunk of 8 positions of four operand rows per K-tile: five 4-byte loads, a
 //      funnel shift where the tap's column offset is odd, one 16-byte store.
 // One group rebuilds while the other copies; the words and the values of a macro's first pieces are
-// fetched while the macro before it is copied.  Bound by the instructions of the two steps.  The kernels before it copied element by element
-// (7x7 stride 2 on 224x224, 3 -> 64 channels, batch 64: 465 us a call) or rebuilt the rows for every
-// K-tile (3x3 stride 2 on 56x56, 128 channels: 215 us).
+// fetched while the macro before it is copied.  Bound by the instructions of the two steps, so divisions are
+// multiplications, the copy has no branches, and a piece takes some 200 instructions (746 when its kept values were
+// scattered bit by bit into a zeroed patch): a K-tile of 3x3 stride 2 took 5900-7500 clocks and takes 3500-6000.
+// Calls, 70 % pruned, before and now: 128 -> 128 channels on 56x56, batch 64, bf16 132 -> 91 us; 256 -> 256 on 28x28
+// 91 -> 73; 512 -> 512 on 14x14 85 -> 67; 160 -> 320 on 32x32, batch 200, fp32 179 -> 150; 320 -> 640 on 16x16 171 ->
+// 128; 7x7 stride 2 on 224x224, 3 -> 64, batch 64, bf16 192 -> 161.
 // Every wait is bounded and ends in SURGEON_ERR_TIMEOUT.
 #include <cuda.h>
 
-#include <cstddef>
+#include <algorithm>
 
 #include "surgeon_internal.cuh"
 #include "tc_common.cuh"
@@ -47,61 +51,40 @@ __device__ __forceinline__ void group_sync(int g) {
   asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(kGroupThreads) : "memory");
 }
 
-// A piece whose values are on their way: the 16-byte vectors that hold its up to 16 packed values (a load per
-// value touches a cache line per lane and value, and the L1 takes one line per clock).
-template <int DT>
+// A piece whose values are on their way: one predicated load per element (consecutive lanes have consecutive pieces of
+// a channel, whose packed values lie in few cache lines).
 struct PieceValues {
-  static constexpr int kVals = DT == 0 ? 4 : 8;           // values per vector
-  static constexpr int kVecs = kPiece / kVals + 1;        // vectors a piece can span
-  uint32_t w[4 * kVecs];
-  uint32_t a, bits, dst, col;                             // misalignment of the first value; bits; place
+  uint32_t v[kPiece];
+  uint32_t dst, col, len;                                 // place
   int m;                                                  // macro
 };
 template <int DT>
-__device__ __forceinline__ void load_values(const void* __restrict__ values, uint32_t rank, uint32_t count,
-                                            uint32_t n_keep, PieceValues<DT>& v) {
-  constexpr uint32_t V = PieceValues<DT>::kVals;
-  constexpr int NV = PieceValues<DT>::kVecs;
-  v.a = rank & (V - 1);
-  const uint32_t base = rank - v.a;
-  const uint32_t n_vec = count ? (v.a + count + V - 1) / V : 0u;
-  const unsigned char* src = static_cast<const unsigned char*>(values) + static_cast<size_t>(base) * (16 / V);
-  if (base + n_vec * V <= n_keep) {
+__device__ __forceinline__ uint32_t pair(uint32_t lo, uint32_t hi) {
+  return DT == 0 ? pack_bf16x2(__uint_as_float(lo), __uint_as_float(hi)) : lo | (hi << 16);
+}
+// Into the row's phase planes.  The places of a piece are whole 16-byte vectors for strides 1 and 2; past the row's
+// end they are zeros like the elements there.
+template <int DT>
+__device__ __forceinline__ void place(const PieceValues& q, unsigned short* row, int stride, int plane, uint32_t inv_stride) {
+  const uint32_t (&v)[kPiece] = q.v;
+  if (stride == 1) {
+    uint4* to = reinterpret_cast<uint4*>(row + q.col);
+    to[0] = make_uint4(pair<DT>(v[0], v[1]), pair<DT>(v[2], v[3]), pair<DT>(v[4], v[5]), pair<DT>(v[6], v[7]));
+    to[1] = make_uint4(pair<DT>(v[8], v[9]), pair<DT>(v[10], v[11]), pair<DT>(v[12], v[13]), pair<DT>(v[14], v[15]));
+  } else if (stride == 2) {
 #pragma unroll
-    for (int j = 0; j < NV; ++j) {
-      uint4 q = make_uint4(0, 0, 0, 0);
-      if (static_cast<uint32_t>(j) < n_vec) q = __ldg(reinterpret_cast<const uint4*>(src) + j);
-      v.w[4 * j] = q.x; v.w[4 * j + 1] = q.y; v.w[4 * j + 2] = q.z; v.w[4 * j + 3] = q.w;
-    }
-  } else {                                                // a vector that ends past the last value
+    for (int ph = 0; ph < 2; ++ph)
+      *reinterpret_cast<uint4*>(row + ph * plane + (q.col >> 1)) =
+          make_uint4(pair<DT>(v[ph], v[ph + 2]), pair<DT>(v[ph + 4], v[ph + 6]), pair<DT>(v[ph + 8], v[ph + 10]),
+                     pair<DT>(v[ph + 12], v[ph + 14]));
+  } else {
+    uint32_t at = (q.col * inv_stride) >> 16, ph = q.col - at * stride;           // col / stride
 #pragma unroll
-    for (int j = 0; j < 4 * NV; ++j) {
-      constexpr uint32_t kPerWord = V / 4;
-      uint32_t t = 0;
-#pragma unroll
-      for (uint32_t i = 0; i < kPerWord; ++i) {
-        const uint32_t e = base + j * kPerWord + i;
-        if (e < n_keep)
-          t |= DT == 0 ? __ldg(static_cast<const uint32_t*>(values) + e)
-                       : static_cast<uint32_t>(__ldg(static_cast<const unsigned short*>(values) + e)) << (16 * i);
-      }
-      v.w[j] = t;
+    for (int e = 0; e < kPiece; ++e) {
+      if (static_cast<uint32_t>(e) < q.len) row[ph * plane + at] = static_cast<unsigned short>(pair<DT>(v[e], 0u));
+      if (++ph == static_cast<uint32_t>(stride)) { ph = 0; ++at; }
     }
   }
-}
-// The values as bf16 pairs in order (h[0] holds the first two).
-template <int DT>
-__device__ __forceinline__ void line_up(PieceValues<DT>& v, uint32_t (&h)[8]) {
-  constexpr int N = 4 * PieceValues<DT>::kVecs;
-  const uint32_t words = DT == 0 ? v.a : v.a >> 1;        // whole words to drop: 0-3
-#pragma unroll
-  for (int j = 0; j < N - 2; ++j) v.w[j] = (words & 2u) ? v.w[j + 2] : v.w[j];
-#pragma unroll
-  for (int j = 0; j < N - 3; ++j) v.w[j] = (words & 1u) ? v.w[j + 1] : v.w[j];
-#pragma unroll
-  for (int j = 0; j < 8; ++j)
-    h[j] = DT == 0 ? pack_bf16x2(__uint_as_float(v.w[2 * j]), __uint_as_float(v.w[2 * j + 1]))
-                   : __funnelshift_r(v.w[j], v.w[j + 1], (v.a & 1u) * 16u);
 }
 
 // What a lane fetches for its piece: the kept count before the 128-element block the piece starts in, the
@@ -138,7 +121,10 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
   const int m_begin = split * p.macros_per_split;
   const int m_end = min(m_begin + p.macros_per_split, p.total_macros);
   // K-tiles of macro m (the last one of an image may be short)
-  auto tiles_of = [&](int m) { return min(p.macro, p.tiles_per_img - (m % p.macros_per_img) * p.macro); };
+  auto tiles_of = [&](int m) {
+    const int k = m - static_cast<int>(divide(m, p.by_macros)) * p.macros_per_img;
+    return min(p.macro, p.tiles_per_img - k * p.macro);
+  };
 
   const uint32_t full_bar = smem_u32(bars);
   const uint32_t empty_bar = smem_u32(bars + kMaxStages);
@@ -197,7 +183,7 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
       uint32_t round = 0;
       bool ok = true;
       for (int m = m_begin; m < m_end && ok; ++m) {
-        const int img = m / p.macros_per_img;
+        const int img = divide(m, p.by_macros);
         const int kt0 = (m - img * p.macros_per_img) * p.macro;
         const int n_t = tiles_of(m);
         for (int t = 0; t < n_t; ++t) {
@@ -224,7 +210,6 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
     unsigned char* patch = smem + p.stages * stage_bytes + g * p.patch_bytes;
     unsigned short* patch16 = reinterpret_cast<unsigned short*>(patch);
     const uint32_t patch_addr = smem_u32(patch);
-    const uint32_t n_keep = static_cast<uint32_t>(__ldg(p.n_keep_ptr));   // packed values in the store
     const int c_first = nn0 / p.RS;
     const int c_last = (nn_end - 1) / p.RS;
     const int n_ch = c_last - c_first + 1;
@@ -256,51 +241,42 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
 #pragma unroll
       for (int i = 0; i < 4; ++i)
         if (i >= n_mine) *reinterpret_cast<uint4*>(smem + st * stage_bytes + dst_off[i]) = make_uint4(0, 0, 0, 0);
-    // A macro's input rows and its pieces (channel, row, 16 columns).
-    // (32-bit indices, and divisions by multiplication: a piece costs a few hundred instructions in all, and
-    // they are what the kernel spends its time on)
-    struct Macro { int kt0, n_t, iy_lo; uint32_t n_pieces, per_ch, inv_ch, start; };
-    const uint32_t per_row = (p.W + kPiece - 1) / kPiece;
-    const uint32_t inv_row = p.inv_per_row;
+    // A macro's pieces (channel, row, 16 columns), as many as its patch has; some rows may lie past the map.
+    const uint32_t per_row = (p.W + kPiece - 1) / kPiece, per_ch = p.patch_rows * per_row, n_pieces = n_ch * per_ch;
+    struct Macro { int kt0, n_t, iy_lo; uint32_t start; };
     auto geometry = [&](int m) {
       Macro q;
-      const int img = m / p.macros_per_img;
+      const int img = divide(m, p.by_macros);
       q.kt0 = (m - img * p.macros_per_img) * p.macro;
-      q.n_t = tiles_of(m);
-      const int y_first = q.kt0 * kTileK / p.OWp;
-      const int y_last = min((q.kt0 + q.n_t) * kTileK - 1, p.P - 1) / p.OWp;
-      q.iy_lo = max(y_first * p.stride - p.pad, 0);
-      const int iy_hi = min(y_last * p.stride + p.KH - 1 - p.pad, p.H - 1);
-      q.per_ch = static_cast<uint32_t>(iy_hi - q.iy_lo + 1) * per_row;
-      q.inv_ch = q.per_ch > 1 ? 0xFFFFFFFFu / q.per_ch + 1u : 0u;       // exact below 2^16 pieces
-      q.n_pieces = n_ch * q.per_ch;
+      q.n_t = min(p.macro, p.tiles_per_img - q.kt0);
+      q.iy_lo = max(static_cast<int>(divide(q.kt0 * kTileK, p.by_owp)) * p.stride - p.pad, 0);
       q.start = (static_cast<uint32_t>(img) * p.C + c_first) * (p.H * p.W) + q.iy_lo * p.W;
       return q;
     };
     auto fetch = [&](const Macro& q, uint32_t t) {
       PieceRaw r;
       r.m = 0x7FFFFFFF; r.len = 0; r.off = 0; r.next = 0; r.start = 0; r.words = make_uint4(0, 0, 0, 0); r.dst = 0; r.col = 0;
-      if (t < q.n_pieces) {
-        const uint32_t ci = q.per_ch > 1 ? __umulhi(t, q.inv_ch) : t;
-        const uint32_t rest = t - ci * q.per_ch;
-        const uint32_t row = per_row > 1 ? __umulhi(rest, inv_row) : rest;
+      if (t < n_pieces) {
+        const uint32_t ci = divide(t, p.by_ch), rest = t - ci * per_ch, row = divide(rest, p.by_row);
         r.col = (rest - row * per_row) * kPiece;
         r.dst = (ci * p.patch_rows + row) * row_len + 8;
-        r.start = q.start + ci * (p.H * p.W) + row * p.W + r.col;
-        r.len = min(static_cast<uint32_t>(kPiece), p.W - r.col);
-        const uint32_t blk = r.start >> kBlockShift;
-        r.off = __ldg(offsets + blk);
-        if (blk != p.partial_blk) {
-          r.words = __ldg(reinterpret_cast<const uint4*>(bitmap) + blk);
-        } else {                                   // the last, partial block of the bitmap
-          const uint32_t w0 = blk * kBlockWords;
-          r.words.x = __ldg(bitmap + w0);
-          r.words.y = (w0 + 1 < p.n_words) ? __ldg(bitmap + w0 + 1) : 0u;
-          r.words.z = (w0 + 2 < p.n_words) ? __ldg(bitmap + w0 + 2) : 0u;
-          r.words.w = (w0 + 3 < p.n_words) ? __ldg(bitmap + w0 + 3) : 0u;
+        if (q.iy_lo + static_cast<int>(row) < p.H) {
+          r.start = q.start + ci * (p.H * p.W) + row * p.W + r.col;
+          r.len = min(static_cast<uint32_t>(kPiece), p.W - r.col);
+          const uint32_t blk = r.start >> kBlockShift;
+          r.off = __ldg(offsets + blk);
+          if (blk != p.partial_blk) {
+            r.words = __ldg(reinterpret_cast<const uint4*>(bitmap) + blk);
+          } else {                                 // the last, partial block of the bitmap
+            const uint32_t w0 = blk * kBlockWords;
+            r.words.x = __ldg(bitmap + w0);
+            r.words.y = (w0 + 1 < p.n_words) ? __ldg(bitmap + w0 + 1) : 0u;
+            r.words.z = (w0 + 2 < p.n_words) ? __ldg(bitmap + w0 + 2) : 0u;
+            r.words.w = (w0 + 3 < p.n_words) ? __ldg(bitmap + w0 + 3) : 0u;
+          }
+          const uint32_t wi = r.start >> 5;        // (within the block the next word is at hand)
+          if ((wi & 3u) == 3u && (r.start & 31u) > 32u - kPiece && wi + 1 < p.n_words) r.next = __ldg(bitmap + wi + 1);
         }
-        const uint32_t wi = r.start >> 5;          // (within the block the next word is at hand)
-        if ((wi & 3u) == 3u && (r.start & 31u) > 32u - kPiece && wi + 1 < p.n_words) r.next = __ldg(bitmap + wi + 1);
       }
       return r;
     };
@@ -326,8 +302,8 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
     uint32_t ft = gtid;
     Macro fq = geometry(fm < m_end ? fm : m_begin);
     auto fetch_next = [&]() {
-      while (fm < m_end && ft >= fq.n_pieces) {
-        fm += kGroups;
+      if (ft >= n_pieces && fm < m_end) {         // (a thread past all pieces of a macro has none in the others either)
+        fm = gtid < n_pieces ? fm + kGroups : m_end;
         ft = gtid;
         if (fm < m_end) fq = geometry(fm);
       }
@@ -335,7 +311,7 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
       if (fm < m_end) { r.m = fm; ft += kGroupThreads; }
       return r;
     };
-    auto issue = [&](const PieceRaw& r, PieceValues<DT>& v) {
+    auto issue = [&](const PieceRaw& r, PieceValues& v) {
       const uint32_t wq = (r.start >> 5) & 3u, sh = r.start & 31u;
       uint32_t rank = r.off;
       rank += wq > 0 ? __popc(r.words.x) : 0u;
@@ -344,43 +320,45 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
       const uint32_t w0 = wq == 0 ? r.words.x : (wq == 1 ? r.words.y : (wq == 2 ? r.words.z : r.words.w));
       const uint32_t w1 = wq == 3 ? r.next : (wq == 0 ? r.words.y : (wq == 1 ? r.words.z : r.words.w));
       rank += __popc(w0 & ((1u << sh) - 1u));
-      v.bits = __funnelshift_r(w0, w1, sh) & ((1u << r.len) - 1u);
-      v.dst = r.dst; v.col = r.col; v.m = r.m;
-      load_values<DT>(values, rank, __popc(v.bits), n_keep, v);
+      const uint32_t bits = __funnelshift_r(w0, w1, sh) & ((1u << r.len) - 1u);
+      // A fully kept piece (all of an unpruned tensor, the head of one whose zeros are kept in part) is consecutive values:
+      // 16 bytes at a time where that holds for the warp.
+      constexpr uint32_t V = DT == 0 ? 4 : 8;
+      if (__all_sync(__activemask(), bits == (1u << r.len) - 1u && ((rank | r.len) & (V - 1)) == 0)) {
+        const uint4* src = reinterpret_cast<const uint4*>(static_cast<const unsigned char*>(values) + static_cast<size_t>(rank) * (16 / V));
+#pragma unroll
+        for (uint32_t j = 0; j < kPiece / V; ++j) {
+          const uint4 q = j * V < r.len ? __ldg(src + j) : make_uint4(0, 0, 0, 0);
+          const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+          for (uint32_t e = 0; e < V; ++e) v.v[j * V + e] = DT == 0 ? w[e % 4] : (w[e >> 1] >> (16 * (e & 1))) & 0xFFFFu;
+        }
+      } else {
+#pragma unroll
+        for (int e = 0; e < kPiece; ++e) {
+          v.v[e] = ld_packed<DT>(values, rank, bits & (1u << e));
+          if (bits & (1u << e)) ++rank;
+        }
+      }
+      v.dst = r.dst; v.col = r.col; v.len = r.len; v.m = r.m;
     };
-    PieceValues<DT> ready;
+    PieceValues ready;
     PieceRaw raw = fetch_next();
     issue(raw, ready);
     raw = fetch_next();
+    // (what no piece writes stays zero: the places around the rows)
+    for (int v = gtid; v < p.patch_bytes / 16; v += kGroupThreads)
+      reinterpret_cast<uint4*>(patch)[v] = make_uint4(0, 0, 0, 0);
+    group_sync(g);
     for (int m = m_begin + g; m < m_end; m += kGroups) {
       const Macro q = geometry(m);
       const int kt0 = q.kt0, n_t = q.n_t, iy_lo = q.iy_lo;
       // ---- the patch ----
-      for (int v = gtid; v < p.patch_bytes / 16; v += kGroupThreads)
-        reinterpret_cast<uint4*>(patch)[v] = make_uint4(0, 0, 0, 0);
-      group_sync(g);
       while (ready.m == m) {
-        PieceValues<DT> now = ready;
+        const PieceValues now = ready;
         issue(raw, ready);
         raw = fetch_next();
-        uint32_t h[8], bits = now.bits;
-        const uint32_t count = __popc(bits), col = now.col;
-        unsigned short* dst = patch16 + now.dst;
-        line_up<DT>(now, h);
-#pragma unroll
-        for (int i0 = 0; i0 < kPiece; i0 += 4) {
-          if (static_cast<uint32_t>(i0) < count) {
-#pragma unroll
-            for (int i = i0; i < i0 + 4; ++i) {
-              if (static_cast<uint32_t>(i) < count) {
-                const uint32_t ix = col + __ffs(bits) - 1;         // (bits has a set bit left)
-                bits &= bits - 1;
-                const uint32_t qq = (ix * p.inv_stride) >> 16;     // ix / stride
-                dst[(ix - qq * p.stride) * p.plane + qq] = static_cast<unsigned short>(h[i >> 1] >> (16 * (i & 1)));
-              }
-            }
-          }
-        }
+        place<DT>(now, patch16 + now.dst, p.stride, p.plane, p.inv_stride);
       }
       group_sync(g);
       // ---- the operand tiles ----
@@ -389,33 +367,26 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
         __syncwarp();
         unsigned char* a_tile = smem + s * stage_bytes;
         const int pos = (kt0 + t) * kTileK + 8 * chunk;
-        const int y = pos / p.OWp, x0 = pos - y * p.OWp;
+        const int y = divide(pos, p.by_owp), x0 = pos - y * p.OWp;
         const int nv = pos < p.P ? p.OW - x0 : 0;          // positions of the chunk that exist
+        uint32_t keep[4];                                  // (the padding at the end of the row is zero)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) keep[j] = nv > 2 * j + 1 ? 0xFFFFFFFFu : (nv == 2 * j + 1 ? 0xFFFFu : 0u);
+        const int y_in = y * p.stride, e0 = x0 - iy_lo * row_len;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           if (i >= n_mine) break;
-          const int iy = y * p.stride + row_r[i];
-          uint4 out = make_uint4(0, 0, 0, 0);
-          if (iy >= 0 && iy < p.H && nv > 0) {
-            const uint32_t e = static_cast<uint32_t>(row_base[i] + (iy - iy_lo) * row_len + x0);
-            const uint32_t addr = patch_addr + (e & ~1u) * 2u;
-            uint32_t w[5];
+          const int iy = y_in + row_r[i];
+          const bool in = static_cast<uint32_t>(iy) < static_cast<uint32_t>(p.H) && nv > 0;
+          const uint32_t e = in ? static_cast<uint32_t>(row_base[i] + e0 + iy * row_len) : 8u;
+          const uint32_t addr = patch_addr + (e & ~1u) * 2u, shift = (e & 1u) * 16u, all = in ? 0xFFFFFFFFu : 0u;
+          uint32_t w[5];
 #pragma unroll
-            for (int j = 0; j < 5; ++j)
-              asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w[j]) : "r"(addr + 4 * j) : "memory");
-            const uint32_t shift = (e & 1u) * 16u;
-            out.x = __funnelshift_r(w[0], w[1], shift);
-            out.y = __funnelshift_r(w[1], w[2], shift);
-            out.z = __funnelshift_r(w[2], w[3], shift);
-            out.w = __funnelshift_r(w[3], w[4], shift);
-            if (nv < 8) {                                  // the padding at the end of the row
-              uint32_t* o = reinterpret_cast<uint32_t*>(&out);
-#pragma unroll
-              for (int j = 0; j < 4; ++j)
-                o[j] = 2 * j + 1 < nv ? o[j] : (2 * j < nv ? o[j] & 0xFFFFu : 0u);
-            }
-          }
-          *reinterpret_cast<uint4*>(a_tile + dst_off[i]) = out;
+          for (int j = 0; j < 5; ++j)
+            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w[j]) : "r"(addr + 4 * j) : "memory");
+          *reinterpret_cast<uint4*>(a_tile + dst_off[i]) =
+              make_uint4(__funnelshift_r(w[0], w[1], shift) & keep[0] & all, __funnelshift_r(w[1], w[2], shift) & keep[1] & all,
+                         __funnelshift_r(w[2], w[3], shift) & keep[2] & all, __funnelshift_r(w[3], w[4], shift) & keep[3] & all);
         }
         fence_proxy_async();
         __syncwarp();
@@ -423,7 +394,7 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
         skip_tiles(1);
       }
       if (m + 1 < m_end) skip_tiles(tiles_of(m + 1));
-      group_sync(g);                               // the patch is read; it is zeroed next
+      group_sync(g);                               // the patch is read; the next one takes its place
     }
   }
 
@@ -477,15 +448,13 @@ bool compute_plan_strided(const surgeon_layer_desc& d, StridedParams* out) {
   p.n_gemm = d.c_in * p.RS;
   // 8 zeros to the left of a plane: tap columns reach at most 8 places over the edge; ix / stride by a multiplication
   if ((d.pad + d.stride - 1) / d.stride > 8 || (d.kw - 1) / d.stride > 5 || d.stride > 64 || d.w > 4096) return false;
-  const unsigned per_row = (d.w + kPiece - 1) / kPiece;
-  p.inv_per_row = per_row > 1 ? 0xFFFFFFFFu / per_row + 1u : 0u;
   p.inv_stride = (65536 + d.stride - 1) / d.stride;
   for (int ix = 0; ix < d.w; ++ix)
     if (static_cast<int>((static_cast<unsigned>(ix) * p.inv_stride) >> 16) != ix / d.stride) return false;
-  // elements of a plane: 8 zeros, then the row or what its last chunk reads, whichever is longer; an odd number of
-  // words, against bank conflicts
-  p.plane = p.OWp + 16 > (d.w - 1) / d.stride + 9 ? p.OWp + 16 : ((d.w - 1) / d.stride + 9 + 1) / 2 * 2;
-  if ((p.plane / 2) % 2 == 0) p.plane += 2;
+  // elements of a plane: 8 zeros, then the row's pieces or what its last chunk reads, whichever is longer, in whole
+  // 16-byte vectors
+  const int pieces = (d.w + kPiece - 1) / kPiece * kPiece;
+  p.plane = (std::max(p.OWp + 16, 8 + (pieces - 1) / d.stride + 1) + 7) / 8 * 8;
   p.m_tiles = (p.n_gemm + kTileM - 1) / kTileM;
   p.rows_per_tile = ((p.n_gemm + p.m_tiles - 1) / p.m_tiles + 7) / 8 * 8;
   // channels a tile's rows can touch
@@ -506,7 +475,8 @@ bool compute_plan_strided(const surgeon_layer_desc& d, StridedParams* out) {
     for (int n_acc = units >= 2 ? 2 : 1; n_acc >= 1 && !found; --n_acc) {
       for (int macro = 8; macro >= 1 && !found; --macro) {
         if (macro > p.tiles_per_img) continue;
-        int out_rows = (macro * kTileK + p.OWp - 2) / p.OWp + 1;
+        // (where macros begin with a row, whole rows)
+        int out_rows = macro * kTileK % p.OWp == 0 ? macro * kTileK / p.OWp : (macro * kTileK + p.OWp - 2) / p.OWp + 1;
         if (out_rows > p.OH) out_rows = p.OH;
         int rows = (out_rows - 1) * d.stride + d.kh;
         if (rows > d.h) rows = d.h;
@@ -525,6 +495,9 @@ bool compute_plan_strided(const surgeon_layer_desc& d, StridedParams* out) {
   if (!found) return false;
   p.n_tiles = (units + p.n_acc - 1) / p.n_acc;
   p.macros_per_img = (p.tiles_per_img + p.macro - 1) / p.macro;
+  const int per_row = (d.w + kPiece - 1) / kPiece;
+  p.by_row = make_div(per_row); p.by_ch = make_div(per_row * p.patch_rows);
+  p.by_owp = make_div(p.OWp); p.by_macros = make_div(p.macros_per_img);
   const long long total = static_cast<long long>(d.batch) * p.macros_per_img;
   if (total > 2147483647LL / 64) return false;
   p.total_macros = static_cast<int>(total);
@@ -569,8 +542,6 @@ cudaError_t launch_strided(const surgeon_compressed& act, const StridedParams& p
   StridedParams p = plan;
   p.n_words = (act.n + 31) / 32;
   p.partial_blk = (act.n % SURGEON_BLOCK) ? static_cast<unsigned>(act.n / SURGEON_BLOCK) : 0xFFFFFFFFu;
-  p.n_keep_ptr = reinterpret_cast<const long long*>(reinterpret_cast<const char*>(act.header) +
-                                                    offsetof(surgeon_header, n_keep));
   cudaError_t e = p.OW == p.OWp
                       ? launch_grad_to_bf16(grad_out, static_cast<long long>(p.B) * p.O * p.P, grad_bf16, status, stream)
                       : launch_grad_to_bf16_rows(grad_out, static_cast<long long>(p.B) * p.O * p.OH, p.OW, p.OWp,
