@@ -74,7 +74,7 @@ cudaError_t launch_strided(const surgeon_compressed& act, const StridedParams& p
 // ---- layers whose im2col operand is the activation itself (weight_grad_tc_direct.cu) ----------
 struct DirectParams {
   int mode;                 // 0 = linear [T, C] (MN-major operands), 1 = conv 1x1 stride 1 (K-major),
-                            // 2 = conv 1x1 stride 2 (K-major, sampled input)
+                            // 2 = conv 1x1 stride 2 (K-major, sampled input), 3 = the same on a transposed gradient copy
   int ow, in_w, in_hw;      // mode 2: output row length, input row length, input plane size
   int taps;                 // 1, or kh*kw for a k x k stride-1 conv (mode 1 over shifted gradients)
   int kh, kw, pad, in_h, oh;  // taps > 1: kernel and map sizes (with ow, in_w)
@@ -82,6 +82,8 @@ struct DirectParams {
   int row_shift;            // taps > 1: only the kw column shifts are stored; rows shift by TMA offset
   int tg;                   // k x k on one transposed gradient copy: 1-5 (see weight_grad_tc_direct.cu), else 0
   int map_rows, kpos;       // tg: whole map rows per K-tile, and their positions
+  int slot_w;               // mode 3: K positions per output row: 8, 16, 32 or 64
+  unsigned many_keep;       // mode 3: packed values above which a warp's lanes share each run (launcher)
   int k_rows;               // tg: k-rows of a 64-channel slab in shared memory
   int unit_bytes, b_bytes;  // tg: bytes of a unit's slabs, and of a stage
   unsigned box_bytes;       // tg: bytes one box brings

@@ -28,6 +28,13 @@
 //           ring; a tap's shift is a choice of slab and start address per MMA.  Every slab is loaded once.
 // 160 channels on 32x32, batch 200: 247 -> 189 us a call; 640 channels on 8x8: 167 -> 145.
 //
+// 1x1 layers of stride 2 on maps at most 128 wide take that copy as well (MODE 3): a K-tile is 64 / slot_w output rows, each at
+// a multiple of slot_w = 8, 16, 32 or 64 positions (the boxes are slot_w wide and bring zeros past a row's end), so that a
+// lane's run is one, two or four pieces of input rows at places that are known when the kernel is compiled.  A run that
+// began anywhere in a row was walked segment by segment and kept value by kept value (MODE 2, for the others), 13000 clocks a
+// K-tile: 1024 -> 2048 channels on 14x14, batch 64, bf16, 70 % pruned 108 -> 54 us; 512 -> 1024 on 28x28 97 -> 67; 256 ->
+// 512 on 56x56 97 -> 83, unpruned 165 -> 97.
+//
 // The activation operand is rebuilt from the compressed store by 16 producer warps, 8 per K-tile,
 // two tiles in flight: a lane owns a run of 32 consecutive elements (64 bytes of the swizzled
 // tile), finds the rank of its first kept element from the block offset and the block's bitmap
@@ -41,6 +48,7 @@
 #include <algorithm>
 #include <cstddef>
 #include <cstdlib>
+#include <type_traits>
 
 #include "surgeon_internal.cuh"
 #include "tc_common.cuh"
@@ -513,6 +521,163 @@ dw_direct_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ v
         if (lane == 0) { if (PAIR) mbar_arrive_rank0(full_a + 8 * sa); else mbar_arrive(full_a + 8 * sa); }
         next_stage();
       }
+    } else if (MODE == 3) {
+      // 1x1 stride 2: a K-tile is 64 / slot_w output rows, each at a multiple of slot_w positions: the lane's run is a part
+      // of one row (slot_w 32 and 64), two rows or four.  A row's positions are every other element of every other input
+      // row: the places of its kept ones count the elements between them.
+      const bool many = n_keep > p.many_keep;
+      auto rebuild = [&](auto segments) {
+        constexpr int SEGS = decltype(segments)::value, NE = 32 / SEGS;
+        struct Raw {
+          uint32_t base, j, n;                         // kept count before the block; first element; elements that exist
+          uint4 q;                                     // the block's words
+          uint2 after;                                 // and the two behind it
+        };
+        auto fetch = [&](int kt, Raw (&raw)[SEGS]) {
+          const int img = kt / p.tiles_per_img, kin = kt - img * p.tiles_per_img;
+          const int x0 = SEGS == 1 ? (32 * part) & (p.slot_w - 1) : 0;
+          const int ix = 2 * x0, n_row = max(0, min(NE, (p.in_w - ix + 1) >> 1));
+          const int y0 = kin * p.map_rows + 32 * part / p.slot_w;
+#pragma unroll
+          for (int i = 0; i < SEGS; ++i) {
+            Raw& r = raw[i];
+            const int iy = 2 * (y0 + i);
+            r.n = row < rows_here && iy < p.in_h ? n_row : 0;
+            r.base = 0; r.q = make_uint4(0, 0, 0, 0); r.after = make_uint2(0, 0);
+            r.j = ((static_cast<uint32_t>(img) * p.C + (c0 + row)) * p.in_h + iy) * p.in_w + ix;
+            if (r.n > 0) {
+              const uint32_t blk = r.j >> kBlockShift, w0 = blk * kBlockWords, n_words = static_cast<uint32_t>(p.n_words);
+              r.base = __ldg(offsets + blk);
+              if (blk != p.partial_blk) {
+                r.q = __ldg(reinterpret_cast<const uint4*>(bitmap) + blk);
+                if ((r.j & 64u) && w0 + 4 < n_words) {
+                  if (w0 + 5 < n_words) r.after = __ldg(reinterpret_cast<const uint2*>(bitmap + w0 + 4));
+                  else r.after.x = __ldg(bitmap + w0 + 4);
+                }
+              } else {                                 // the last, partial block of the bitmap
+                r.q.x = __ldg(bitmap + w0);
+                r.q.y = (w0 + 1 < n_words) ? __ldg(bitmap + w0 + 1) : 0u;
+                r.q.z = (w0 + 2 < n_words) ? __ldg(bitmap + w0 + 2) : 0u;
+                r.q.w = (w0 + 3 < n_words) ? __ldg(bitmap + w0 + 3) : 0u;
+              }
+            }
+          }
+        };
+        constexpr bool kAhead = SEGS <= 2;             // (four rows' words would take 36 registers)
+        Raw cur[SEGS];
+        if (kAhead && wg < n_kt) fetch(kt_begin + wg, cur);
+        for (int it = wg; it < n_kt; it += kGroups) {
+          Raw nxt[SEGS];
+          if (!kAhead) fetch(kt_begin + it, cur);
+          else if (it + kGroups < n_kt) fetch(kt_begin + it + kGroups, nxt);
+          // place of the first element's value, and the bits of the row's elements and of those between them
+          uint32_t rank[SEGS], win[SEGS][2];
+#pragma unroll
+          for (int i = 0; i < SEGS; ++i) {
+            const Raw& r = cur[i];
+            const uint32_t wq = (r.j >> 5) & 3u, sh = r.j & 31u;
+            rank[i] = r.base + (wq > 0 ? __popc(r.q.x) : 0u) + (wq > 1 ? __popc(r.q.y) : 0u) + (wq > 2 ? __popc(r.q.z) : 0u);
+            const uint32_t w0 = wq == 0 ? r.q.x : (wq == 1 ? r.q.y : (wq == 2 ? r.q.z : r.q.w));
+            const uint32_t w1 = wq == 0 ? r.q.y : (wq == 1 ? r.q.z : (wq == 2 ? r.q.w : r.after.x));
+            const uint32_t w2 = wq == 0 ? r.q.z : (wq == 1 ? r.q.w : (wq == 2 ? r.after.x : r.after.y));
+            rank[i] += __popc(w0 & ((1u << sh) - 1u));
+            win[i][0] = __funnelshift_r(w0, w1, sh);
+            win[i][1] = SEGS == 1 ? __funnelshift_r(w1, w2, sh) : 0u;
+            const uint32_t bits = 2 * r.n;
+            if (bits < 32) { win[i][0] &= (1u << bits) - 1u; win[i][1] = 0; }
+            else if (bits < 64) win[i][1] &= (1u << (bits - 32)) - 1u;
+          }
+          unsigned char* dst_row = smem + sa * kATileBytes + rowbase;
+          if (many) {
+            // A lane per element, run by run, so that a load's values lie side by side.  (A lane's own loads touch a
+            // cache line each, more lines than the L1 beside 200 KB of tiles holds until their last use.)
+            // The lanes of segment i ask for their numbers in the register that lane 32 / SEGS * i + ... holds: a run's
+            // segments are spread over the lanes first.
+            if (!wait_stage()) break;
+            constexpr int RUNS = 32 / SEGS;                            // runs per round
+            const int seg = static_cast<int>(lane) / NE, e2 = 2 * (static_cast<int>(lane) % NE);
+#pragma unroll
+            for (int round_no = 0; round_no < SEGS; ++round_no) {
+              // lane RUNS * i + k: segment i of run RUNS * round_no + k
+              uint32_t at = 0, wa = 0, wb = 0;
+#pragma unroll
+              for (int i = 0; i < SEGS; ++i) {
+                const int from = RUNS * round_no + static_cast<int>(lane) % RUNS;
+                const uint32_t x = SEGS == 1 ? rank[i] : __shfl_sync(0xFFFFFFFFu, rank[i], from);
+                const uint32_t y0 = SEGS == 1 ? win[i][0] : __shfl_sync(0xFFFFFFFFu, win[i][0], from);
+                if (static_cast<int>(lane) / RUNS == i) { at = x; wa = y0; }
+              }
+              if (SEGS == 1) wb = win[0][1];
+#pragma unroll 1
+              for (int l0 = 0; l0 < RUNS; l0 += 8) {
+                uint32_t v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                  const int from = RUNS * seg + l0 + u;
+                  const uint32_t w0 = __shfl_sync(0xFFFFFFFFu, wa, from);
+                  uint32_t idx = __shfl_sync(0xFFFFFFFFu, at, from), on;
+                  if (SEGS == 1) {
+                    const unsigned long long w = w0 | (static_cast<unsigned long long>(__shfl_sync(0xFFFFFFFFu, wb, from)) << 32);
+                    idx += __popcll(w & ((1ull << e2) - 1ull));
+                    on = static_cast<uint32_t>(w >> e2) & 1u;
+                  } else {
+                    idx += __popc(w0 & ((1u << e2) - 1u));
+                    on = (w0 >> e2) & 1u;
+                  }
+                  v[u] = ld_packed<DT>(values, idx, on);
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                  const int run = RUNS * round_no + l0 + u, rr = 16 * w8 + (run >> 1);     // whose: its tile row, and which half of it
+                  unsigned char* to = smem + sa * kATileBytes + rr * 128 +
+                                      ((((run & 1) * 4 + (static_cast<int>(lane) >> 3)) ^ (rr & 7)) << 4) + (lane & 7) * 2;
+                  *reinterpret_cast<unsigned short*>(to) =
+                      DT == 0 ? to_bf16_bits(__uint_as_float(v[u])) : static_cast<unsigned short>(v[u]);
+                }
+              }
+            }
+          } else {
+            uint32_t v[32];
+#pragma unroll
+            for (int i = 0; i < SEGS; ++i) {
+              uint32_t idx = rank[i];
+#pragma unroll
+              for (int e = 0; e < NE; ++e) {
+                const uint32_t w = win[i][e >> 4], bit = 1u << (2 * (e & 15));
+                v[i * NE + e] = ld_packed<DT>(values, idx, w & bit);
+                if (w & bit) ++idx;
+                if (w & (bit << 1)) ++idx;
+              }
+            }
+            uint4 chunk[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              uint32_t o[4];
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const uint32_t lo = v[8 * q + 2 * e], hi = v[8 * q + 2 * e + 1];
+                o[e] = DT == 0 ? pack_bf16x2(__uint_as_float(lo), __uint_as_float(hi)) : lo | (hi << 16);
+              }
+              chunk[q] = make_uint4(o[0], o[1], o[2], o[3]);
+            }
+            if (!wait_stage()) break;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              *reinterpret_cast<uint4*>(dst_row + (((y + q) ^ xr) << 4)) = chunk[q];
+          }
+          fence_proxy_async();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(full_a + 8 * sa);
+          next_stage();
+          if (kAhead) {
+#pragma unroll
+            for (int i = 0; i < SEGS; ++i) cur[i] = nxt[i];
+          }
+        }
+      };
+      if (p.slot_w >= 32) rebuild(std::integral_constant<int, 1>{});
+      else if (p.slot_w == 16) rebuild(std::integral_constant<int, 2>{});
+      else rebuild(std::integral_constant<int, 4>{});
     } else {
       // Flat index of the lane's run in the group's first tile, advanced by two tiles per round
       // without multiplications: linear j = t * C + c; conv j = (img * C + c) * T + position.
@@ -1056,6 +1221,17 @@ static bool compute_plan_direct(const surgeon_layer_desc& d, bool transposed_ok,
   } else if (d.kind == 1 && d.kh == 1 && d.kw == 1 && d.stride == 1 && d.pad == 0) {
     p.mode = 1;
     p.T = d.h * d.w; p.imgs = d.batch;
+  } else if (d.kind == 1 && d.kh == 1 && d.kw == 1 && d.stride == 2 && d.pad == 0 && transposed_ok && d.w <= 128 &&
+             d.c_out % 8 == 0 && d.c_out >= 48) {
+    p.mode = 3;                                    // rows of output positions at multiples of slot_w, the gradient transposed
+    p.tg = 1;
+    p.taps = p.kh = p.kw = 1;
+    p.in_h = d.h; p.in_w = d.w;
+    p.oh = (d.h + 1) / 2; p.ow = (d.w + 1) / 2;
+    p.slot_w = 8;
+    while (p.slot_w < p.ow) p.slot_w *= 2;
+    p.map_rows = kTileK / p.slot_w;
+    p.T = p.oh * p.slot_w; p.imgs = d.batch;
   } else if (d.kind == 1 && d.kh == 1 && d.kw == 1 && d.stride == 2 && d.pad == 0) {
     p.mode = 2;                                    // output positions; the input is sampled
     p.ow = (d.w - 1) / 2 + 1;
@@ -1142,10 +1318,10 @@ static bool compute_plan_direct(const surgeon_layer_desc& d, bool transposed_ok,
     while (p.n_acc < 3 && p.n_acc < p.n_units && (p.n_acc + 1) * p.acc_n <= col_cap) ++p.n_acc;
     if (p.tg) {
       if (p.tg >= 2) p.n_acc = p.kh;
-      p.kpos = p.map_rows * p.in_w;
+      p.kpos = p.map_rows * (p.mode == 3 ? p.slot_w : p.in_w);
       const int box_rows = p.tg == 2 ? p.map_rows + p.kh - 1 : p.map_rows;
       p.k_rows = p.tg == 2 ? box_rows * p.in_w + (kTileK - p.kpos) : kTileK;
-      p.box_bytes = static_cast<unsigned>(box_rows * p.in_w) * 128u;
+      p.box_bytes = static_cast<unsigned>(box_rows * (p.mode == 3 ? p.slot_w : p.in_w)) * 128u;
       p.unit_bytes = (p.acc_n + 63) / 64 * p.k_rows * 128;
       p.b_bytes = p.tg == 1 ? p.n_acc * p.unit_bytes : p.unit_bytes;
     }
@@ -1296,7 +1472,7 @@ cudaError_t encode_direct_grad_map(const DirectParams& p, void* grad_bf16, int b
     const cuuint64_t o = static_cast<cuuint64_t>(p.o_real), w = static_cast<cuuint64_t>(p.ow), h = static_cast<cuuint64_t>(p.oh);
     const cuuint64_t dims[4] = {o, w, h, static_cast<cuuint64_t>(p.imgs)};
     const cuuint64_t strides[3] = {o * 2, o * w * 2, o * w * h * 2};
-    const cuuint32_t box[4] = {64, static_cast<cuuint32_t>(p.in_w),
+    const cuuint32_t box[4] = {64, static_cast<cuuint32_t>(p.mode == 3 ? p.slot_w : p.in_w),
                                static_cast<cuuint32_t>(p.tg == 2 ? p.map_rows + p.kh - 1 : p.map_rows), 1};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     r = encode(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, grad_bf16, dims, strides, box, estr,
@@ -1329,7 +1505,7 @@ cudaError_t launch_direct(const surgeon_compressed& act, const DirectParams& pla
                           const float* grad_out, void* grad_bf16, float* partial,
                           uint32_t* status, cudaStream_t stream) {
   DirectParams p = plan;
-  if (!size_rings(&p, act.dt == 0 ? kStageBytes : 0)) return cudaErrorInvalidValue;
+  if (!size_rings(&p, act.dt == 0 && p.mode != 3 ? kStageBytes : 0)) return cudaErrorInvalidValue;
   p.n_words = (act.n + 31) / 32;
   p.few_keep = static_cast<unsigned>(act.n / 8);
   p.n_keep_ptr = reinterpret_cast<const long long*>(reinterpret_cast<const char*>(act.header) +
@@ -1362,6 +1538,15 @@ cudaError_t launch_direct(const surgeon_compressed& act, const DirectParams& pla
     return cudaLaunchKernelEx(&cfg, kernel, act.bitmap, act.values, act.block_offsets, map, partial,
                               status, p);
   };
+  if (p.mode == 3) {
+    // From where on a warp's lanes share each run (70 % / 50 % / 0 % pruned; each lane its own run, and shared: 256 -> 512
+    // channels on 56x56, batch 64, fp32 101, 142, 103 and 93, 97, 101 us; 512 -> 1024 on 28x28 79, 112, 126 and 95, 103,
+    // 126; bf16 67, 89, 108 and 91, 93, 116, 60 % kept 155 and 101; 1024 -> 2048 on 14x14 54, 67, 77 and 83, 73, 77).
+    p.many_keep = static_cast<unsigned>(act.n * (p.slot_w >= 32 ? 35 : (act.dt == 0 ? 40 : 48)) / 100);
+    e = act.dt ? launch(dw_direct_kernel<1, 3, 0, 1>) : launch(dw_direct_kernel<0, 3, 0, 1>);
+    note_launches(1);
+    return e;
+  }
   if (p.tg) {
     switch (p.tg * 2 + (act.dt ? 1 : 0)) {
       case 2: e = launch(dw_direct_kernel<0, 1, 0, 1>); break;
