@@ -40,6 +40,7 @@ constexpr int kSampleBins = 16384;     // bins of the sample
 constexpr int kSelPhases = 12;         // grid-wide exchanges of a call (3 in the common case)
 constexpr int kSelMaxCtas = 256;
 constexpr int kClaimSets = 4, kClaimStride = 32;
+__host__ __device__ constexpr int table_bins(int dt) { return dt == 0 ? 1 : 256; }       // whose counts every CTA shows to the others
 // Candidate slots: per chunk, room for 1/16 of its elements (fp32: 32-bit keys, bf16: 16-bit).
 __host__ __device__ constexpr int slot_entries(int dt) { return dt == 0 ? 64 : 128; }
 constexpr int slot_entry_bytes(int dt) { return dt == 0 ? 4 : 2; }
@@ -47,10 +48,10 @@ constexpr int slot_entry_bytes(int dt) { return dt == 0 ? 4 : 2; }
 // Byte offsets of the parts of the scratch buffer; nothing in it has to start at any value.
 // arrive / answer / keys: what the CTAs exchange; hist: the select's histograms, one per round; claims:
 // counters of claimed chunks; cnt
-// and prefix: per-chunk counts and places of CTAs with too many chunks for shared memory; slots:
-// the keys inside the bracket, per chunk.
+// and prefix: per-chunk counts and places of CTAs with too many chunks for shared memory; table: per CTA (16 chunks or more
+// of a tensor) the counts of its bins; slots: the keys inside the bracket, per chunk.
 struct PruneLayout {
-  size_t arrive, answer, keys, hist, claims, cnt, prefix, slots, total;
+  size_t arrive, answer, keys, hist, claims, cnt, prefix, table, slots, total;
   int64_t tiles;
 };
 constexpr PruneLayout prune_layout(int64_t n, int dt) {
@@ -66,6 +67,8 @@ constexpr PruneLayout prune_layout(int64_t n, int dt) {
   L.prefix = off; off += t * 8;
   L.cnt = off; off += t * 4;
   off = (off + 255) & ~static_cast<size_t>(255);
+  L.table = off;
+  off += (t / 16 + 1 < kSelMaxCtas ? t / 16 + 1 : static_cast<size_t>(kSelMaxCtas)) * table_bins(dt) * 16;
   L.slots = off;
   off += t * static_cast<size_t>(slot_entries(dt)) * slot_entry_bytes(dt);
   L.total = (off + 255) & ~static_cast<size_t>(255);
