@@ -56,7 +56,7 @@ struct StridedParams {
   int tiles_per_img;        // K-tiles of 64 positions
   int macro;                // K-tiles per rebuilt patch
   int macros_per_img, total_macros, macros_per_split;
-  int patch_rows, plane;    // input rows of a patch, elements of a phase plane of one row
+  int patch_rows, plane, row_len;    // input rows of a patch, elements of a phase plane of one row, of a row with its padding
   int patch_bytes, stages, tmem_cols, smem_bytes;
   unsigned inv_stride;      // ix / stride = ix * inv_stride >> 16
   FastDiv by_row, by_ch;    // division by the pieces per row, and per channel of the patch,

@@ -12,15 +12,18 @@
 //      planes (column ix goes to plane ix mod stride, place ix div stride), with zeros around:
 //      what a tap reads for consecutive output positions is then consecutive, whatever the stride.  For strides 1 and 2
 //      a lane's elements are whole 16-byte vectors of the planes, put together in registers;
-//   2. a thread copies one chunk of 8 positions of four operand rows per K-tile: five 4-byte loads, a
-//      funnel shift where the tap's column offset is odd, one 16-byte store.
+//   2. a thread copies one chunk of 8 positions of four operand rows per K-tile: the 16 bytes that the chunk begins in and,
+//      for a tap off a whole vector's start, the next 16, put in place by selects and a funnel shift.  Rows of the patch have
+//      a pitch that spreads the eight lanes of such a load over the banks (five 4-byte loads, 16 bytes from lane to lane and
+//      rows on the same banks, took 1440-2640 clocks a K-tile for what now takes 1040-1180).
 // One group rebuilds while the other copies; the words and the values of a macro's first pieces are
-// fetched while the macro before it is copied.  Bound by the instructions of the two steps, so divisions are
-// multiplications, the copy has no branches, and a piece takes some 200 instructions (746 when its kept values were
-// scattered bit by bit into a zeroed patch): a K-tile of 3x3 stride 2 took 5900-7500 clocks and takes 3500-6000.
-// Calls, 70 % pruned, before and now: 128 -> 128 channels on 56x56, batch 64, bf16 132 -> 91 us; 256 -> 256 on 28x28
-// 91 -> 73; 512 -> 512 on 14x14 85 -> 67; 160 -> 320 on 32x32, batch 200, fp32 179 -> 150; 320 -> 640 on 16x16 171 ->
-// 128; 7x7 stride 2 on 224x224, 3 -> 64, batch 64, bf16 192 -> 161.
+// fetched while the macro before it is copied.  Bound by the instructions of the two steps, 430 for a warp's 32 pieces and
+// 200 for its part of a K-tile: with 16 warps an SM issues at 0.56 of its rate and each warp every 8 clocks, for no one
+// reason above a quarter; tensor pipe 17 %, DRAM 4 %.  So divisions are multiplications, the copy has no branches, a kept
+// value costs one test for its load and its count, and a piece is put together in registers, not scattered bit by bit.
+// Calls, 70 % pruned, when bits were scattered, with 4-byte copies, and now: 128 -> 128 channels on 56x56, batch 64, bf16
+// 132, 94, 89 us; 256 -> 256 on 28x28 91, 73, 60; 512 -> 512 on 14x14 85, 68, 60; 160 -> 320 on 32x32, batch 200, fp32 179,
+// 148, 116; 320 -> 640 on 16x16 171, 126, 109; 7x7 stride 2 on 224x224, 3 -> 64, batch 64, bf16 192, 161, 160.
 // Every wait is bounded and ends in SURGEON_ERR_TIMEOUT.
 #include <cuda.h>
 
@@ -44,11 +47,42 @@ constexpr int kGroupThreads = kGroupWarps * 32;
 constexpr int kThreads = 64 + kGroups * kGroupThreads;    // warp 0: MMA, warp 1: TMA, then the groups
 constexpr int kMaxStages = 8;
 constexpr int kATileBytes = kTileM * kTileK * 2;
-constexpr int kMaxPatchBytes = 44 * 1024;                 // per group
+constexpr int kMaxPatchBytes = 46 * 1024;                 // per group
 constexpr int kPiece = 16;                                // elements of a row that one lane rebuilds
 
 __device__ __forceinline__ void group_sync(int g) {
   asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(kGroupThreads) : "memory");
+}
+
+// 16 bytes of shared memory: read, read where wanted (else zeros), written
+__device__ __forceinline__ uint4 ld_shared_vec(uint32_t addr) {
+  uint4 r;
+  asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "r"(addr));
+  return r;
+}
+__device__ __forceinline__ uint4 ld_shared_vec_if(uint32_t addr, bool wanted) {
+  uint4 r;
+  asm volatile("{.reg .pred q; setp.ne.u32 q, %5, 0; mov.u32 %0, 0; mov.u32 %1, 0; mov.u32 %2, 0; mov.u32 %3, 0;"
+               "@q ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];}"
+               : "=&r"(r.x), "=&r"(r.y), "=&r"(r.z), "=&r"(r.w) : "r"(addr), "r"(static_cast<uint32_t>(wanted)));
+  return r;
+}
+__device__ __forceinline__ void st_shared_vec(uint32_t addr, uint4 v) {
+  asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+
+// The next packed value where the element's bit is set, else zero: one test for the load and the count
+template <int DT>
+__device__ __forceinline__ uint32_t take_next(const void* __restrict__ values, uint32_t& rank, uint32_t bit) {
+  uint32_t r;
+  const unsigned char* src = static_cast<const unsigned char*>(values) + static_cast<size_t>(rank) * (DT == 0 ? 4 : 2);
+  if (DT == 0)
+    asm volatile("{.reg .pred q; setp.ne.u32 q, %3, 0; mov.u32 %0, 0; @q ld.global.nc.u32 %0, [%2]; @q add.u32 %1, %1, 1;}"
+                 : "=&r"(r), "+r"(rank) : "l"(src), "r"(bit));
+  else
+    asm volatile("{.reg .pred q; setp.ne.u32 q, %3, 0; mov.u32 %0, 0; @q ld.global.nc.u16 %0, [%2]; @q add.u32 %1, %1, 1;}"
+                 : "=&r"(r), "+r"(rank) : "l"(src), "r"(bit));
+  return r;
 }
 
 // A piece whose values are on their way: one predicated load per element (consecutive lanes have consecutive pieces of
@@ -65,23 +99,24 @@ __device__ __forceinline__ uint32_t pair(uint32_t lo, uint32_t hi) {
 // Into the row's phase planes.  The places of a piece are whole 16-byte vectors for strides 1 and 2; past the row's
 // end they are zeros like the elements there.
 template <int DT>
-__device__ __forceinline__ void place(const PieceValues& q, unsigned short* row, int stride, int plane, uint32_t inv_stride) {
+__device__ __forceinline__ void place(const PieceValues& q, uint32_t row, int stride, int plane, uint32_t inv_stride) {
   const uint32_t (&v)[kPiece] = q.v;
   if (stride == 1) {
-    uint4* to = reinterpret_cast<uint4*>(row + q.col);
-    to[0] = make_uint4(pair<DT>(v[0], v[1]), pair<DT>(v[2], v[3]), pair<DT>(v[4], v[5]), pair<DT>(v[6], v[7]));
-    to[1] = make_uint4(pair<DT>(v[8], v[9]), pair<DT>(v[10], v[11]), pair<DT>(v[12], v[13]), pair<DT>(v[14], v[15]));
+    const uint32_t to = row + 2 * q.col;
+    st_shared_vec(to, make_uint4(pair<DT>(v[0], v[1]), pair<DT>(v[2], v[3]), pair<DT>(v[4], v[5]), pair<DT>(v[6], v[7])));
+    st_shared_vec(to + 16, make_uint4(pair<DT>(v[8], v[9]), pair<DT>(v[10], v[11]), pair<DT>(v[12], v[13]), pair<DT>(v[14], v[15])));
   } else if (stride == 2) {
 #pragma unroll
     for (int ph = 0; ph < 2; ++ph)
-      *reinterpret_cast<uint4*>(row + ph * plane + (q.col >> 1)) =
-          make_uint4(pair<DT>(v[ph], v[ph + 2]), pair<DT>(v[ph + 4], v[ph + 6]), pair<DT>(v[ph + 8], v[ph + 10]),
-                     pair<DT>(v[ph + 12], v[ph + 14]));
+      st_shared_vec(row + 2 * ph * plane + q.col,
+                    make_uint4(pair<DT>(v[ph], v[ph + 2]), pair<DT>(v[ph + 4], v[ph + 6]), pair<DT>(v[ph + 8], v[ph + 10]),
+                               pair<DT>(v[ph + 12], v[ph + 14])));
   } else {
     uint32_t at = (q.col * inv_stride) >> 16, ph = q.col - at * stride;           // col / stride
 #pragma unroll
     for (int e = 0; e < kPiece; ++e) {
-      if (static_cast<uint32_t>(e) < q.len) row[ph * plane + at] = static_cast<unsigned short>(pair<DT>(v[e], 0u));
+      if (static_cast<uint32_t>(e) < q.len)
+        asm volatile("st.shared.u16 [%0], %1;" ::"r"(row + 2 * (ph * plane + at)), "h"(static_cast<unsigned short>(pair<DT>(v[e], 0u))) : "memory");
       if (++ph == static_cast<uint32_t>(stride)) { ph = 0; ++at; }
     }
   }
@@ -208,31 +243,34 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
     const int g = (warp - 2) / kGroupWarps;
     const int gtid = tid - 64 - g * kGroupThreads;
     unsigned char* patch = smem + p.stages * stage_bytes + g * p.patch_bytes;
-    unsigned short* patch16 = reinterpret_cast<unsigned short*>(patch);
-    const uint32_t patch_addr = smem_u32(patch);
+    const uint32_t smem_addr = smem_u32(smem), patch_addr = smem_u32(patch);
     const int c_first = nn0 / p.RS;
     const int c_last = (nn_end - 1) / p.RS;
     const int n_ch = c_last - c_first + 1;
-    const int row_len = p.stride * p.plane;        // elements of one input row in the patch
+    const int row_len = p.row_len;                 // elements of one input row in the patch, a multiple of 8
     // this thread's four operand rows and its chunk of 8 positions
     const int chunk = gtid & 7;
-    int row_base[4];                               // patch element of (channel, input row iy_lo, phase) and column offset
-    int row_r[4];                                  // kernel row, -1000000 past the last column
-    uint32_t dst_off[4];
+    // of row i: the 16 bytes of the patch that its column 0 of output row 0 begins in (with row_r input rows above the
+    // patch's first), how many elements in, and the kernel row, -1000000 past the last column
+    uint32_t row_addr[4], row_off[4], dst_off[4];
+    int row_r[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int row = (gtid >> 3) + 32 * i;
       const int nn = nn0 + row;
       dst_off[i] = tile_off(row, chunk);
-      row_base[i] = 0;
+      row_addr[i] = patch_addr;
+      row_off[i] = 0;
       row_r[i] = -1000000;
       if (nn < nn_end) {
         const int c = nn / p.RS, rs = nn - c * p.RS;
         const int r = rs / p.KW, s = rs - r * p.KW;
         const int d = s - p.pad;
         const int fd = d >= 0 ? d / p.stride : -((-d + p.stride - 1) / p.stride);
-        row_base[i] = (c - c_first) * p.patch_rows * row_len + (d - fd * p.stride) * p.plane + 8 + fd;
+        const int base = (c - c_first) * p.patch_rows * row_len + (d - fd * p.stride) * p.plane + 8 + fd;
         row_r[i] = r - p.pad;
+        row_off[i] = base & 7;
+        row_addr[i] = patch_addr + 2 * ((base & ~7) + row_r[i] * row_len);
       }
     }
     // Rows past the tile's share stay zero in every stage.
@@ -335,10 +373,7 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
         }
       } else {
 #pragma unroll
-        for (int e = 0; e < kPiece; ++e) {
-          v.v[e] = ld_packed<DT>(values, rank, bits & (1u << e));
-          if (bits & (1u << e)) ++rank;
-        }
+        for (int e = 0; e < kPiece; ++e) v.v[e] = take_next<DT>(values, rank, bits & (1u << e));
       }
       v.dst = r.dst; v.col = r.col; v.len = r.len; v.m = r.m;
     };
@@ -355,38 +390,52 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
       const int kt0 = q.kt0, n_t = q.n_t, iy_lo = q.iy_lo;
       // ---- the patch ----
       while (ready.m == m) {
-        const PieceValues now = ready;
+        place<DT>(ready, patch_addr + 2 * ready.dst, p.stride, p.plane, p.inv_stride);
         issue(raw, ready);
         raw = fetch_next();
-        place<DT>(now, patch16 + now.dst, p.stride, p.plane, p.inv_stride);
       }
       group_sync(g);
       // ---- the operand tiles ----
       for (int t = 0; t < n_t; ++t) {
         wait_stage();
         __syncwarp();
-        unsigned char* a_tile = smem + s * stage_bytes;
+        const uint32_t a_tile = smem_addr + s * stage_bytes;
         const int pos = (kt0 + t) * kTileK + 8 * chunk;
         const int y = divide(pos, p.by_owp), x0 = pos - y * p.OWp;
         const int nv = pos < p.P ? p.OW - x0 : 0;          // positions of the chunk that exist
         uint32_t keep[4];                                  // (the padding at the end of the row is zero)
 #pragma unroll
         for (int j = 0; j < 4; ++j) keep[j] = nv > 2 * j + 1 ? 0xFFFFFFFFu : (nv == 2 * j + 1 ? 0xFFFFu : 0u);
-        const int y_in = y * p.stride, e0 = x0 - iy_lo * row_len;
+        const int y_in = nv > 0 ? y * p.stride : -1000000;
+        const uint32_t from = 2 * (x0 + (y_in - iy_lo) * row_len);
+        // (all loads of two rows before the first store; rows at a whole vector's start need no second one; the patch
+        // begins with zeros, which stand for what lies outside)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          if (i >= n_mine) break;
-          const int iy = y_in + row_r[i];
-          const bool in = static_cast<uint32_t>(iy) < static_cast<uint32_t>(p.H) && nv > 0;
-          const uint32_t e = in ? static_cast<uint32_t>(row_base[i] + e0 + iy * row_len) : 8u;
-          const uint32_t addr = patch_addr + (e & ~1u) * 2u, shift = (e & 1u) * 16u, all = in ? 0xFFFFFFFFu : 0u;
-          uint32_t w[5];
+        for (int h = 0; h < 4; h += 2) {
+          if (h >= n_mine) break;
+          uint4 lo[2], hi[2];
 #pragma unroll
-          for (int j = 0; j < 5; ++j)
-            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w[j]) : "r"(addr + 4 * j) : "memory");
-          *reinterpret_cast<uint4*>(a_tile + dst_off[i]) =
-              make_uint4(__funnelshift_r(w[0], w[1], shift) & keep[0] & all, __funnelshift_r(w[1], w[2], shift) & keep[1] & all,
-                         __funnelshift_r(w[2], w[3], shift) & keep[2] & all, __funnelshift_r(w[3], w[4], shift) & keep[3] & all);
+          for (int k = 0; k < 2; ++k) {
+            const bool in = static_cast<uint32_t>(y_in + row_r[h + k]) < static_cast<uint32_t>(p.H);
+            const uint32_t addr = in ? row_addr[h + k] + from : patch_addr;
+            lo[k] = ld_shared_vec(addr);
+            hi[k] = ld_shared_vec_if(addr + 16, in && row_off[h + k] != 0);
+          }
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            if (h + k >= n_mine) break;
+            const uint32_t off = row_off[h + k];
+            const uint32_t w[8] = {lo[k].x, lo[k].y, lo[k].z, lo[k].w, hi[k].x, hi[k].y, hi[k].z, hi[k].w};
+            uint32_t q4[6], q2[5];
+#pragma unroll
+            for (int j = 0; j < 6; ++j) q4[j] = off & 4 ? w[j + 2] : w[j];
+#pragma unroll
+            for (int j = 0; j < 5; ++j) q2[j] = off & 2 ? q4[j + 1] : q4[j];
+            const uint32_t shift = (off & 1) * 16;
+            st_shared_vec(a_tile + dst_off[h + k],
+                          make_uint4(__funnelshift_r(q2[0], q2[1], shift) & keep[0], __funnelshift_r(q2[1], q2[2], shift) & keep[1],
+                                     __funnelshift_r(q2[2], q2[3], shift) & keep[2], __funnelshift_r(q2[3], q2[4], shift) & keep[3]));
+          }
         }
         fence_proxy_async();
         __syncwarp();
@@ -455,6 +504,19 @@ bool compute_plan_strided(const surgeon_layer_desc& d, StridedParams* out) {
   // 16-byte vectors
   const int pieces = (d.w + kPiece - 1) / kPiece * kPiece;
   p.plane = (std::max(p.OWp + 16, 8 + (pieces - 1) / d.stride + 1) + 7) / 8 * 8;
+  // Pitch of the patch's rows: eight lanes read the eight chunks of a K-tile at once, 16 bytes each, from one output row
+  // or several; of the four next multiples of 8 elements the one that leaves the fewest of them on the same banks.
+  // Where rows without padding allow a longer macro they have none.
+  int least = 1 << 30, pitch = 0;
+  for (int more = 0; more < 32; more += 8) {
+    const int len = d.stride * p.plane + more;
+    int clashes = 0, used[8] = {0};
+    for (int k = 0; k < 8; ++k) {
+      const int at = (8 * k / p.OWp) * d.stride * len + 8 * k % p.OWp;
+      clashes += used[at / 8 % 8]++;
+    }
+    if (clashes < least) { least = clashes; pitch = len; }
+  }
   p.m_tiles = (p.n_gemm + kTileM - 1) / kTileM;
   p.rows_per_tile = ((p.n_gemm + p.m_tiles - 1) / p.m_tiles + 7) / 8 * 8;
   // channels a tile's rows can touch
@@ -480,15 +542,18 @@ bool compute_plan_strided(const surgeon_layer_desc& d, StridedParams* out) {
         if (out_rows > p.OH) out_rows = p.OH;
         int rows = (out_rows - 1) * d.stride + d.kh;
         if (rows > d.h) rows = d.h;
-        const long long bytes = (static_cast<long long>(n_ch) * rows * d.stride * p.plane * 2 + 32 + 15) / 16 * 16;
-        if (bytes > kMaxPatchBytes) continue;
-        const int stage = kATileBytes + n_acc * p.acc_n * 128;
-        int stages = static_cast<int>((budget - kGroups * bytes) / stage);
-        if (stages > kMaxStages) stages = kMaxStages;
-        if (stages < want_stages || macro >= stages) continue;      // (macro < stages: see the producers' waits)
-        p.macro = macro; p.patch_rows = rows; p.patch_bytes = static_cast<int>(bytes); p.n_acc = n_acc;
-        p.stages = stages;
-        found = true;
+        for (int len : {pitch, d.stride * p.plane}) {
+          const long long bytes = (static_cast<long long>(n_ch) * rows * len * 2 + 32 + 15) / 16 * 16;
+          if (bytes > kMaxPatchBytes) continue;
+          const int stage = kATileBytes + n_acc * p.acc_n * 128;
+          int stages = static_cast<int>((budget - kGroups * bytes) / stage);
+          if (stages > kMaxStages) stages = kMaxStages;
+          if (stages < want_stages || macro >= stages) continue;    // (macro < stages: see the producers' waits)
+          p.macro = macro; p.patch_rows = rows; p.row_len = len; p.patch_bytes = static_cast<int>(bytes);
+          p.n_acc = n_acc; p.stages = stages;
+          found = true;
+          break;
+        }
       }
     }
   }

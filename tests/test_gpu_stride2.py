@@ -23,6 +23,8 @@ SHAPES = [
     W.conv("k3w32", 2, 40, 32, 48, 3, 2), W.conv("k3w40", 2, 24, 40, 32, 3, 2), W.conv("k3w23", 3, 20, 23, 72, 3, 2),
     W.conv("k3w6", 9, 40, 6, 48, 3, 2), W.conv("k5w48", 1, 20, 48, 32, 5, 2, 2), W.conv("k7w50", 1, 3, 50, 64, 7, 2, 3),
     W.conv("k4s4", 2, 24, 32, 64, 4, 4, 0), W.conv("k3s3w31", 2, 24, 31, 40, 3, 3, 1), W.conv("k3s1c12", 2, 12, 24, 40, 3),
+    # rows of the patch with and without padding between them
+    W.conv("k3w56", 1, 24, 56, 48, 3, 2), W.conv("k3w112", 1, 16, 112, 64, 3, 2), W.conv("k5w72", 1, 20, 72, 40, 5, 2, 2),
     W.Layer("k3h5w80", 1, 2, 20, 5, 80, 24, 3, 3, 2, 1),
 ]
 
