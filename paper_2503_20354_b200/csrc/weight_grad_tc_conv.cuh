@@ -52,7 +52,8 @@ struct StridedParams {
   int RS, n_gemm;           // KH * KW, C * RS
   int acc_n, n_acc;         // columns per accumulator, accumulators per CTA (1 or 2)
   int m_tiles, n_tiles, splits;
-  int rows_per_tile;        // im2col rows per row tile (a multiple of 8, at most 128)
+  int rows_per_tile;        // im2col rows per CTA (a multiple of 8, at most 128 m_acc)
+  int m_acc, a_bytes;       // row tiles of a CTA (1 or 2), operand bytes of a stage
   int tiles_per_img;        // K-tiles of 64 positions
   int macro;                // K-tiles per rebuilt patch
   int macros_per_img, total_macros, macros_per_split;

@@ -23,7 +23,8 @@
 // value costs one test for its load and its count, and a piece is put together in registers, not scattered bit by bit.
 // Calls, 70 % pruned, when bits were scattered, with 4-byte copies, and now: 128 -> 128 channels on 56x56, batch 64, bf16
 // 132, 94, 89 us; 256 -> 256 on 28x28 91, 73, 60; 512 -> 512 on 14x14 85, 68, 60; 160 -> 320 on 32x32, batch 200, fp32 179,
-// 148, 116; 320 -> 640 on 16x16 171, 126, 109; 7x7 stride 2 on 224x224, 3 -> 64, batch 64, bf16 192, 161, 160.
+// 148, 116; 320 -> 640 on 16x16 171, 126, 109; 7x7 stride 2 on 224x224, 3 -> 64, batch 64, bf16 192, 161, 142 (two
+// row tiles in a CTA).
 // Every wait is bounded and ends in SURGEON_ERR_TIMEOUT.
 #include <cuda.h>
 
@@ -131,7 +132,8 @@ struct PieceRaw {
   int m;                   // its macro
 };
 
-template <int DT>
+// MA: row tiles of a CTA, each an accumulator of 128 rows
+template <int DT, int MA>
 __global__ void __launch_bounds__(kThreads, 1)
 dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ values,
                   const uint32_t* __restrict__ offsets, const __grid_constant__ CUtensorMap grad_map,
@@ -140,7 +142,7 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   const int n_cols = p.acc_n * p.n_acc;
-  const int stage_bytes = kATileBytes + n_cols * 128;
+  const int a_bytes = MA == 1 ? kATileBytes : p.a_bytes, stage_bytes = a_bytes + n_cols * 128;
   __shared__ __align__(8) unsigned long long bars[2 * kMaxStages + 1];
   __shared__ uint32_t tmem_slot;
   __shared__ volatile uint32_t fail;
@@ -186,7 +188,7 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
     if (lane == 0) {
       const uint32_t idesc = make_idesc(kTileM, p.acc_n);
       const uint32_t smem0 = smem_u32(smem);
-      const uint64_t a_base = make_desc(smem0), b_base = make_desc(smem0 + kATileBytes);
+      const uint64_t a_base = make_desc(smem0), b_base = make_desc(smem0 + a_bytes);
       const uint64_t stage_inc = static_cast<uint64_t>(stage_bytes >> 4);
       const uint64_t acc_inc = static_cast<uint64_t>((p.acc_n * 128) >> 4);
       uint64_t da = a_base, db = b_base;
@@ -198,7 +200,10 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
           ok = mbar_wait_suspend(full_bar + 8 * s, parity);
           if (!ok) break;
           tc_fence_after();
-          if (n_acc_here == 1) umma_ktile<1, 2>(tmem_base, p.acc_n, da, db, acc_inc, idesc, accum);
+          if (MA == 2) {
+            umma_ktile<1, 2>(tmem_base, p.acc_n, da, db, acc_inc, idesc, accum);
+            umma_ktile<1, 2>(tmem_base + n_cols, p.acc_n, da + (kATileBytes >> 4), db, acc_inc, idesc, accum);
+          } else if (n_acc_here == 1) umma_ktile<1, 2>(tmem_base, p.acc_n, da, db, acc_inc, idesc, accum);
           else umma_ktile<2, 2>(tmem_base, p.acc_n, da, db, acc_inc, idesc, accum);
           umma_commit(empty_bar + 8 * s);
           accum = 1;
@@ -228,7 +233,7 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
             ok = false;
             break;
           }
-          const uint32_t b_addr = smem_u32(smem + s * stage_bytes + kATileBytes);
+          const uint32_t b_addr = smem_u32(smem + s * stage_bytes + a_bytes);
           mbar_arrive_expect_tx(full_bar + 8 * s, static_cast<uint32_t>(n_acc_here * p.acc_n) * 128u);
           for (int a = 0; a < n_acc_here; ++a)
             tma_load_3d(b_addr + a * p.acc_n * 128, &grad_map, (kt0 + t) * kTileK, o0 + a * p.acc_n, img,
@@ -248,17 +253,17 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
     const int c_last = (nn_end - 1) / p.RS;
     const int n_ch = c_last - c_first + 1;
     const int row_len = p.row_len;                 // elements of one input row in the patch, a multiple of 8
-    // this thread's four operand rows and its chunk of 8 positions
+    // this thread's operand rows, 32 apart, and its chunk of 8 positions
     const int chunk = gtid & 7;
     // of row i: the 16 bytes of the patch that its column 0 of output row 0 begins in (with row_r input rows above the
     // patch's first), how many elements in, and the kernel row, -1000000 past the last column
-    uint32_t row_addr[4], row_off[4], dst_off[4];
-    int row_r[4];
+    constexpr int kRows = 4 * MA;
+    uint32_t row_addr[kRows], row_off[kRows];
+    int row_r[kRows];
+    const uint32_t dst_off = tile_off(gtid >> 3, chunk);   // (32 rows are 4 KB)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int row = (gtid >> 3) + 32 * i;
-      const int nn = nn0 + row;
-      dst_off[i] = tile_off(row, chunk);
+    for (int i = 0; i < kRows; ++i) {
+      const int nn = nn0 + (gtid >> 3) + 32 * i;
       row_addr[i] = patch_addr;
       row_off[i] = 0;
       row_r[i] = -1000000;
@@ -273,12 +278,12 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
         row_addr[i] = patch_addr + 2 * ((base & ~7) + row_r[i] * row_len);
       }
     }
-    // Rows past the tile's share stay zero in every stage.
-    const int n_mine = max(0, min(4, (p.rows_per_tile - (gtid >> 3) + 31) / 32));
-    for (int st = 0; st < p.stages; ++st)
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (i >= n_mine) *reinterpret_cast<uint4*>(smem + st * stage_bytes + dst_off[i]) = make_uint4(0, 0, 0, 0);
+    // Rows past the tile's share stay zero in every stage; the second of two tiles ends with its share, and what the
+    // MMA reads past it goes to accumulator rows that nothing reads.
+    const int n_mine = max(0, min(kRows, (p.rows_per_tile - (gtid >> 3) + 31) / 32));
+    if (MA == 1)
+      for (int st = 0; st < p.stages; ++st)
+        for (int i = n_mine; i < kRows; ++i) st_shared_vec(smem_addr + st * stage_bytes + dst_off + i * 4096, make_uint4(0, 0, 0, 0));
     // A macro's pieces (channel, row, 16 columns), as many as its patch has; some rows may lie past the map.
     const uint32_t per_row = (p.W + kPiece - 1) / kPiece, per_ch = p.patch_rows * per_row, n_pieces = n_ch * per_ch;
     struct Macro { int kt0, n_t, iy_lo; uint32_t start; };
@@ -411,7 +416,7 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
         // (all loads of two rows before the first store; rows at a whole vector's start need no second one; the patch
         // begins with zeros, which stand for what lies outside)
 #pragma unroll
-        for (int h = 0; h < 4; h += 2) {
+        for (int h = 0; h < kRows; h += 2) {
           if (h >= n_mine) break;
           uint4 lo[2], hi[2];
 #pragma unroll
@@ -432,7 +437,7 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
 #pragma unroll
             for (int j = 0; j < 5; ++j) q2[j] = off & 2 ? q4[j + 1] : q4[j];
             const uint32_t shift = (off & 1) * 16;
-            st_shared_vec(a_tile + dst_off[h + k],
+            st_shared_vec(a_tile + dst_off + (h + k) * 4096,
                           make_uint4(__funnelshift_r(q2[0], q2[1], shift) & keep[0], __funnelshift_r(q2[1], q2[2], shift) & keep[1],
                                      __funnelshift_r(q2[2], q2[3], shift) & keep[2], __funnelshift_r(q2[3], q2[4], shift) & keep[3]));
           }
@@ -453,20 +458,24 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
     tc_fence_after();
     if (done && !fail) {
       const int lane_grp = warp & 3;              // TMEM lanes this warp may read
-      const int nn = nn0 + lane_grp * 32 + static_cast<int>(lane);
       float* out = partial + static_cast<long long>(split) * p.O * p.n_gemm;
       const int cols_here = n_acc_here * p.acc_n;
-      for (int col = 16 * ((warp - 2) >> 2); col < cols_here; col += 16 * (kGroups * kGroupWarps / 4)) {
-        uint32_t r[16];
-        tmem_ld16(tmem_base + (static_cast<uint32_t>(lane_grp * 32) << 16) + col, r);
-        if (nn < nn_end) {
 #pragma unroll
-          for (int e = 0; e < 16; ++e) {
-            const int o = o0 + col + e;
-            if (o < p.O && SURGEON_IN_BOUNDS(static_cast<long long>(split) * p.O * p.n_gemm +
-                                                 static_cast<long long>(o) * p.n_gemm + nn,
-                                             static_cast<long long>(p.splits) * p.O * p.n_gemm, status))
-              out[static_cast<long long>(o) * p.n_gemm + nn] = __uint_as_float(r[e]);
+      for (int m = 0; m < MA; ++m) {
+        const int nn = nn0 + m * kTileM + lane_grp * 32 + static_cast<int>(lane);
+        if (MA == 2 && nn - static_cast<int>(lane) >= nn_end) break;
+        for (int col = 16 * ((warp - 2) >> 2); col < cols_here; col += 16 * (kGroups * kGroupWarps / 4)) {
+          uint32_t r[16];
+          tmem_ld16(tmem_base + (static_cast<uint32_t>(lane_grp * 32) << 16) + m * n_cols + col, r);
+          if (nn < nn_end) {
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+              const int o = o0 + col + e;
+              if (o < p.O && SURGEON_IN_BOUNDS(static_cast<long long>(split) * p.O * p.n_gemm +
+                                                   static_cast<long long>(o) * p.n_gemm + nn,
+                                               static_cast<long long>(p.splits) * p.O * p.n_gemm, status))
+                out[static_cast<long long>(o) * p.n_gemm + nn] = __uint_as_float(r[e]);
+            }
           }
         }
       }
@@ -517,10 +526,6 @@ bool compute_plan_strided(const surgeon_layer_desc& d, StridedParams* out) {
     }
     if (clashes < least) { least = clashes; pitch = len; }
   }
-  p.m_tiles = (p.n_gemm + kTileM - 1) / kTileM;
-  p.rows_per_tile = ((p.n_gemm + p.m_tiles - 1) / p.m_tiles + 7) / 8 * 8;
-  // channels a tile's rows can touch
-  const int n_ch = p.rows_per_tile < 2 ? 1 : (p.C < (p.rows_per_tile - 2) / p.RS + 2 ? p.C : (p.rows_per_tile - 2) / p.RS + 2);
   p.tiles_per_img = (p.P + kTileK - 1) / kTileK;
   // columns: one or two accumulators of at most 256 columns, the fewest padded columns first
   int best_waste = -1;
@@ -533,26 +538,44 @@ bool compute_plan_strided(const surgeon_layer_desc& d, StridedParams* out) {
   // the longest macro (rows are rebuilt once per macro) whose patch fits, with three stages at least if possible
   const int budget = 226 * 1024 - 1024 - 256;
   bool found = false;
-  for (int want_stages = 3; want_stages >= 2 && !found; --want_stages) {
-    for (int n_acc = units >= 2 ? 2 : 1; n_acc >= 1 && !found; --n_acc) {
-      for (int macro = 8; macro >= 1 && !found; --macro) {
-        if (macro > p.tiles_per_img) continue;
-        // (where macros begin with a row, whole rows)
-        int out_rows = macro * kTileK % p.OWp == 0 ? macro * kTileK / p.OWp : (macro * kTileK + p.OWp - 2) / p.OWp + 1;
-        if (out_rows > p.OH) out_rows = p.OH;
-        int rows = (out_rows - 1) * d.stride + d.kh;
-        if (rows > d.h) rows = d.h;
-        for (int len : {pitch, d.stride * p.plane}) {
-          const long long bytes = (static_cast<long long>(n_ch) * rows * len * 2 + 32 + 15) / 16 * 16;
-          if (bytes > kMaxPatchBytes) continue;
-          const int stage = kATileBytes + n_acc * p.acc_n * 128;
-          int stages = static_cast<int>((budget - kGroups * bytes) / stage);
-          if (stages > kMaxStages) stages = kMaxStages;
-          if (stages < want_stages || macro >= stages) continue;    // (macro < stages: see the producers' waits)
-          p.macro = macro; p.patch_rows = rows; p.row_len = len; p.patch_bytes = static_cast<int>(bytes);
-          p.n_acc = n_acc; p.stages = stages;
-          found = true;
-          break;
+  // Between 129 and 256 rows one CTA takes them all, as two row tiles: one rebuild, one gradient tile, one round of
+  // waits for both, instead of two CTAs with halves that need the channels between them twice.  Its start and its
+  // epilogue are longer and there are twice the partial results, so only from 32 K-tiles an SM on: 3 -> 64 channels 7x7
+  // stride 2 on 224x224, batch 64 (85 an SM), 161 -> 142 us; 16 -> 64 3x3 on 56x56, batch 64 (21), 54 -> 52; 16 -> 160 3x3 on
+  // 32x32, batch 200 (22), 72.7 -> 74.8; the first at batch 4 (5) 25.6 -> 29.6.  Nor with 256 columns, where the copy is a smaller part of
+  // a K-tile: 16 -> 256 on 56x56, batch 110 (36), 148.5 -> 150.6; 3 -> 160 7x7 (64) 189 -> 175.
+  const bool pairs = p.n_gemm > kTileM && p.n_gemm <= 2 * kTileM && units == 1 && p.acc_n <= 192 &&
+                     static_cast<long long>(d.batch) * p.tiles_per_img >= 32LL * sm_count();
+  for (int m_acc = pairs ? 2 : 1; m_acc >= 1 && !found; --m_acc) {
+    p.m_acc = m_acc;
+    p.m_tiles = (p.n_gemm + m_acc * kTileM - 1) / (m_acc * kTileM);
+    p.rows_per_tile = ((p.n_gemm + p.m_tiles - 1) / p.m_tiles + 7) / 8 * 8;
+    p.a_bytes = m_acc == 1 ? kATileBytes : p.rows_per_tile * kTileK * 2;
+    // channels a tile's rows can touch
+    const int n_ch = p.rows_per_tile < 2 ? 1 : (p.C < (p.rows_per_tile - 2) / p.RS + 2 ? p.C : (p.rows_per_tile - 2) / p.RS + 2);
+    for (int want_stages = 3; want_stages >= 2 && !found; --want_stages) {
+      for (int n_acc = units >= 2 ? 2 : 1; n_acc >= 1 && !found; --n_acc) {
+        for (int macro = 8; macro >= 1 && !found; --macro) {
+          if (macro > p.tiles_per_img) continue;
+          // (where macros begin with a row, whole rows)
+          int out_rows = macro * kTileK % p.OWp == 0 ? macro * kTileK / p.OWp : (macro * kTileK + p.OWp - 2) / p.OWp + 1;
+          if (out_rows > p.OH) out_rows = p.OH;
+          int rows = (out_rows - 1) * d.stride + d.kh;
+          if (rows > d.h) rows = d.h;
+          for (int len : {pitch, d.stride * p.plane}) {
+            const long long bytes = (static_cast<long long>(n_ch) * rows * len * 2 + 32 + 15) / 16 * 16;
+            if (bytes > kMaxPatchBytes) continue;
+            const int stage = p.a_bytes + n_acc * p.acc_n * 128;
+            int stages = static_cast<int>((budget - kGroups * bytes) / stage);
+            if (stages > kMaxStages) stages = kMaxStages;
+            if (stages < want_stages || macro >= stages) continue;    // (macro < stages: see the producers' waits)
+            // (the MMAs read two whole row tiles of the last stage)
+            if (m_acc == 2 && stage + kGroups * bytes < 2 * kATileBytes) continue;
+            p.macro = macro; p.patch_rows = rows; p.row_len = len; p.patch_bytes = static_cast<int>(bytes);
+            p.n_acc = n_acc; p.stages = stages;
+            found = true;
+            break;
+          }
         }
       }
     }
@@ -579,8 +602,8 @@ bool compute_plan_strided(const surgeon_layer_desc& d, StridedParams* out) {
   p.macros_per_split = (p.total_macros + best - 1) / best;
   p.splits = (p.total_macros + p.macros_per_split - 1) / p.macros_per_split;
   p.tmem_cols = 32;
-  while (p.tmem_cols < p.acc_n * p.n_acc) p.tmem_cols *= 2;
-  p.smem_bytes = p.stages * (kATileBytes + p.n_acc * p.acc_n * 128) + kGroups * p.patch_bytes + 1024;
+  while (p.tmem_cols < p.acc_n * p.n_acc * p.m_acc) p.tmem_cols *= 2;
+  p.smem_bytes = p.stages * (p.a_bytes + p.n_acc * p.acc_n * 128) + kGroups * p.patch_bytes + 1024;
   *out = p;
   return true;
 }
@@ -631,7 +654,8 @@ cudaError_t launch_strided(const surgeon_compressed& act, const StridedParams& p
     return launch_kernel(kernel, grid, dim3(kThreads), static_cast<size_t>(p.smem_bytes), stream, true, act.bitmap,
                          static_cast<const void*>(act.values), act.block_offsets, map, partial, status, p);
   };
-  e = act.dt == 0 ? launch(dw_strided_kernel<0>) : launch(dw_strided_kernel<1>);
+  if (p.m_acc == 2) e = act.dt == 0 ? launch(dw_strided_kernel<0, 2>) : launch(dw_strided_kernel<1, 2>);
+  else e = act.dt == 0 ? launch(dw_strided_kernel<0, 1>) : launch(dw_strided_kernel<1, 1>);
   note_launches(1);
   return e;
 }

@@ -40,3 +40,11 @@ def test_against_the_oracle(layer, bf16, ratio):
     r = oracle.prune_compact(bits, ratio)
     ref = oracle_dw(layer, oracle.decompress(r["bitmap"], r["values"], bits.size), g.numpy())
     assert rel_frobenius(dw.cpu().numpy(), ref) <= 5e-3
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("layer", [W.conv("147 rows", 25, 3, 224, 8, 7, 2, 3), W.conv("245 rows", 112, 5, 97, 24, 7, 2, 3),
+                                   W.conv("144 rows", 80, 16, 64, 16, 3)], ids=lambda l: l.name)
+def test_two_row_tiles_in_a_cta(layer, bf16):
+    """129 to 256 operand rows and at least 32 K-tiles of 64 positions an SM: one CTA takes all rows."""
+    test_against_the_oracle(layer, bf16, 0.7)
