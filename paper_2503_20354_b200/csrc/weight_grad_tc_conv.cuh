@@ -61,7 +61,8 @@ struct StridedParams {
   int patch_bytes, stages, tmem_cols, smem_bytes;
   unsigned inv_stride;      // ix / stride = ix * inv_stride >> 16
   FastDiv by_row, by_ch;    // division by the pieces per row, and per channel of the patch,
-  FastDiv by_owp, by_macros;         // by OWp, and by the macros of an image
+  FastDiv by_owp, by_macros;         // by OWp, and by the macros of an image,
+  FastDiv by_rs, by_kw, by_stride;   // by RS, KW and the stride
   unsigned partial_blk;     // index of the bitmap's last block if it is partial, else 0xFFFFFFFF (launcher)
   long long n_words;        // words of the bitmap (filled by the launcher)
 };

@@ -19,11 +19,12 @@
 // One group rebuilds while the other copies; the words and the values of a macro's first pieces are
 // fetched while the macro before it is copied.  Bound by the instructions of the two steps, 430 for a warp's 32 pieces and
 // 200 for its part of a K-tile: with 16 warps an SM issues at 0.56 of its rate and each warp every 8 clocks, for no one
-// reason above a quarter; tensor pipe 17 %, DRAM 4 %.  So divisions are multiplications, the copy has no branches, a kept
-// value costs one test for its load and its count, and a piece is put together in registers, not scattered bit by bit.
+// reason above a quarter; tensor pipe 17 %, DRAM 4 %.  So divisions are multiplications (also the
+// sixteen of a thread's start: with them and branches in the fetch of a piece's words, a call of 15-21 us took 2 more), the
+// copy and the fetch have no branches, a kept value costs one test for its load and its count, and a piece is put together in registers, not scattered bit by bit.
 // Calls, 70 % pruned, when bits were scattered, with 4-byte copies, and now: 128 -> 128 channels on 56x56, batch 64, bf16
-// 132, 94, 89 us; 256 -> 256 on 28x28 91, 73, 60; 512 -> 512 on 14x14 85, 68, 60; 160 -> 320 on 32x32, batch 200, fp32 179,
-// 148, 116; 320 -> 640 on 16x16 171, 126, 109; 7x7 stride 2 on 224x224, 3 -> 64, batch 64, bf16 192, 161, 142 (two
+// 132, 94, 87 us; 256 -> 256 on 28x28 91, 73, 58; 512 -> 512 on 14x14 85, 68, 57; 160 -> 320 on 32x32, batch 200, fp32 179,
+// 148, 113; 320 -> 640 on 16x16 171, 126, 105; 7x7 stride 2 on 224x224, 3 -> 64, batch 64, bf16 192, 161, 141 (two
 // row tiles in a CTA).
 // Every wait is bounded and ends in SURGEON_ERR_TIMEOUT.
 #include <cuda.h>
@@ -268,10 +269,10 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
       row_off[i] = 0;
       row_r[i] = -1000000;
       if (nn < nn_end) {
-        const int c = nn / p.RS, rs = nn - c * p.RS;
-        const int r = rs / p.KW, s = rs - r * p.KW;
+        const int c = divide(nn, p.by_rs), rs = nn - c * p.RS;
+        const int r = divide(rs, p.by_kw), s = rs - r * p.KW;
         const int d = s - p.pad;
-        const int fd = d >= 0 ? d / p.stride : -((-d + p.stride - 1) / p.stride);
+        const int fd = static_cast<int>(divide(d + 8 * p.stride, p.by_stride)) - 8;     // rounded down; pad <= 8 stride
         const int base = (c - c_first) * p.patch_rows * row_len + (d - fd * p.stride) * p.plane + 8 + fd;
         row_r[i] = r - p.pad;
         row_off[i] = base & 7;
@@ -298,29 +299,26 @@ dw_strided_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ 
     };
     auto fetch = [&](const Macro& q, uint32_t t) {
       PieceRaw r;
-      r.m = 0x7FFFFFFF; r.len = 0; r.off = 0; r.next = 0; r.start = 0; r.words = make_uint4(0, 0, 0, 0); r.dst = 0; r.col = 0;
-      if (t < n_pieces) {
-        const uint32_t ci = divide(t, p.by_ch), rest = t - ci * per_ch, row = divide(rest, p.by_row);
-        r.col = (rest - row * per_row) * kPiece;
-        r.dst = (ci * p.patch_rows + row) * row_len + 8;
-        if (q.iy_lo + static_cast<int>(row) < p.H) {
-          r.start = q.start + ci * (p.H * p.W) + row * p.W + r.col;
-          r.len = min(static_cast<uint32_t>(kPiece), p.W - r.col);
-          const uint32_t blk = r.start >> kBlockShift;
-          r.off = __ldg(offsets + blk);
-          if (blk != p.partial_blk) {
-            r.words = __ldg(reinterpret_cast<const uint4*>(bitmap) + blk);
-          } else {                                 // the last, partial block of the bitmap
-            const uint32_t w0 = blk * kBlockWords;
-            r.words.x = __ldg(bitmap + w0);
-            r.words.y = (w0 + 1 < p.n_words) ? __ldg(bitmap + w0 + 1) : 0u;
-            r.words.z = (w0 + 2 < p.n_words) ? __ldg(bitmap + w0 + 2) : 0u;
-            r.words.w = (w0 + 3 < p.n_words) ? __ldg(bitmap + w0 + 3) : 0u;
-          }
-          const uint32_t wi = r.start >> 5;        // (within the block the next word is at hand)
-          if ((wi & 3u) == 3u && (r.start & 31u) > 32u - kPiece && wi + 1 < p.n_words) r.next = __ldg(bitmap + wi + 1);
-        }
+      const uint32_t ci = divide(t, p.by_ch), rest = t - ci * per_ch, row = divide(rest, p.by_row);
+      r.col = (rest - row * per_row) * kPiece;
+      r.dst = (ci * p.patch_rows + row) * row_len + 8;
+      const bool live = t < n_pieces && q.iy_lo + static_cast<int>(row) < p.H;   // (else nothing kept, at element 0)
+      r.start = live ? q.start + ci * (p.H * p.W) + row * p.W + r.col : 0u;
+      r.len = live ? min(static_cast<uint32_t>(kPiece), p.W - r.col) : 0u;
+      const uint32_t blk = r.start >> kBlockShift, wi = r.start >> 5;
+      r.off = __ldg(offsets + blk);
+      if (blk != p.partial_blk) {
+        r.words = __ldg(reinterpret_cast<const uint4*>(bitmap) + blk);
+      } else {                                     // the last, partial block of the bitmap
+        const uint32_t w0 = blk * kBlockWords;
+        r.words.x = __ldg(bitmap + w0);
+        r.words.y = (w0 + 1 < p.n_words) ? __ldg(bitmap + w0 + 1) : 0u;
+        r.words.z = (w0 + 2 < p.n_words) ? __ldg(bitmap + w0 + 2) : 0u;
+        r.words.w = (w0 + 3 < p.n_words) ? __ldg(bitmap + w0 + 3) : 0u;
       }
+      // (within the block the next word is at hand)
+      r.next = ld_packed<0>(bitmap, wi + 1, (wi & 3u) == 3u && (r.start & 31u) + r.len > 32u);
+      r.m = 0x7FFFFFFF;
       return r;
     };
     int s = 0;
@@ -585,6 +583,7 @@ bool compute_plan_strided(const surgeon_layer_desc& d, StridedParams* out) {
   p.macros_per_img = (p.tiles_per_img + p.macro - 1) / p.macro;
   const int per_row = (d.w + kPiece - 1) / kPiece;
   p.by_row = make_div(per_row); p.by_ch = make_div(per_row * p.patch_rows);
+  p.by_rs = make_div(p.RS); p.by_kw = make_div(d.kw); p.by_stride = make_div(d.stride);
   p.by_owp = make_div(p.OWp); p.by_macros = make_div(p.macros_per_img);
   const long long total = static_cast<long long>(d.batch) * p.macros_per_img;
   if (total > 2147483647LL / 64) return false;
