@@ -116,7 +116,7 @@ grad_split_kernel(const float* __restrict__ grad, unsigned char* __restrict__ ou
     if (g.vec) {                                 // (four columns from a multiple of 4 on are 16 bytes of one piece)
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const float4 v = col + 4 * h < len ? ld_once(reinterpret_cast<const float4*>(at)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        const float4 v = col + 4 * h < len ? __ldg(reinterpret_cast<const float4*>(at)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         x[4 * h] = v.x; x[4 * h + 1] = v.y; x[4 * h + 2] = v.z; x[4 * h + 3] = v.w;
         at += 4;
         q += 4;
@@ -139,9 +139,9 @@ grad_split_kernel(const float* __restrict__ grad, unsigned char* __restrict__ ou
     const int o = g.linear ? col : row, k = g.linear ? row : col, j = o / g.tile_n, n = o - j * g.tile_n;
     unsigned char* to = out + (static_cast<size_t>(k / kTileK) * g.nt + j) * 3 * plane +
                         (g.linear ? (n >> 6) * (kTileK * 128) + tile_off(k % kTileK, (n & 63) >> 3) : tile_off(n, (k % kTileK) >> 3));
-    st_kept(reinterpret_cast<uint4*>(to), make_uint4(a[0], a[1], a[2], a[3]));
-    st_kept(reinterpret_cast<uint4*>(to + plane), make_uint4(b[0], b[1], b[2], b[3]));
-    st_kept(reinterpret_cast<uint4*>(to + 2 * plane), make_uint4(c[0], c[1], c[2], c[3]));
+    *reinterpret_cast<uint4*>(to) = make_uint4(a[0], a[1], a[2], a[3]);
+    *reinterpret_cast<uint4*>(to + plane) = make_uint4(b[0], b[1], b[2], b[3]);
+    *reinterpret_cast<uint4*>(to + 2 * plane) = make_uint4(c[0], c[1], c[2], c[3]);
   }
   __shared__ uint32_t s_most;
   if (threadIdx.x == 0) s_most = 0;

@@ -20,12 +20,12 @@ grad_to_bf16_kernel(const float* __restrict__ g, long long n, unsigned short* __
   const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
   for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < n8;
        i += stride) {
-    const float4 a = ld_once(reinterpret_cast<const float4*>(g) + 2 * i);
-    const float4 b = ld_once(reinterpret_cast<const float4*>(g) + 2 * i + 1);
+    const float4 a = __ldg(reinterpret_cast<const float4*>(g) + 2 * i);
+    const float4 b = __ldg(reinterpret_cast<const float4*>(g) + 2 * i + 1);
     uint4 o;
     o.x = pack_bf16x2(a.x, a.y); o.y = pack_bf16x2(a.z, a.w);
     o.z = pack_bf16x2(b.x, b.y); o.w = pack_bf16x2(b.z, b.w);
-    st_kept(reinterpret_cast<uint4*>(out) + i, o);
+    reinterpret_cast<uint4*>(out)[i] = o;
   }
   if (blockIdx.x == 0)
     for (long long j = (n8 << 3) + threadIdx.x; j < n; j += blockDim.x)
@@ -47,8 +47,8 @@ grad_to_bf16_rows_kernel(const float* __restrict__ g, long long rows, int len, i
     const float* src = g + r * len + c0;
     float v[8];
     if ((len & 3) == 0 && c0 + 8 <= len) {         // rows start on 16-byte boundaries
-      const float4 a = ld_once(reinterpret_cast<const float4*>(src));
-      const float4 b = ld_once(reinterpret_cast<const float4*>(src) + 1);
+      const float4 a = __ldg(reinterpret_cast<const float4*>(src));
+      const float4 b = __ldg(reinterpret_cast<const float4*>(src) + 1);
       v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
       v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
     } else {
@@ -58,7 +58,7 @@ grad_to_bf16_rows_kernel(const float* __restrict__ g, long long rows, int len, i
     uint4 o;
     o.x = pack_bf16x2(v[0], v[1]); o.y = pack_bf16x2(v[2], v[3]);
     o.z = pack_bf16x2(v[4], v[5]); o.w = pack_bf16x2(v[6], v[7]);
-    st_kept(reinterpret_cast<uint4*>(out) + i, o);
+    reinterpret_cast<uint4*>(out)[i] = o;
   }
 }
 

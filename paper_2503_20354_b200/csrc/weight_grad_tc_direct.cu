@@ -1004,7 +1004,7 @@ grad_transpose_bf16_kernel(const float* __restrict__ g, unsigned short* __restri
         const float* src = g + (img * p.o_real + o) * hw + pos;
         float4 x = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         if (o < p.o_real) {
-          if ((hw & 3) == 0 && pos < hw) x = ld_once(reinterpret_cast<const float4*>(src));
+          if ((hw & 3) == 0 && pos < hw) x = __ldg(reinterpret_cast<const float4*>(src));
           else {
             x.x = pos < hw ? __ldg(src) : 0.0f;
             x.y = pos + 1 < hw ? __ldg(src + 1) : 0.0f;
@@ -1031,8 +1031,8 @@ grad_transpose_bf16_kernel(const float* __restrict__ g, unsigned short* __restri
       const int row = (threadIdx.x >> 3) + 32 * i, c8 = threadIdx.x & 7;
       const int at = pb * 64 + row, o = cb * 64 + 8 * c8;
       if (at < hw && o < p.o_real)
-        st_kept(reinterpret_cast<uint4*>(out + (img * hw + at) * p.o_real + o),
-                make_uint4(tile[row][4 * c8], tile[row][4 * c8 + 1], tile[row][4 * c8 + 2], tile[row][4 * c8 + 3]));
+        *reinterpret_cast<uint4*>(out + (img * hw + at) * p.o_real + o) =
+            make_uint4(tile[row][4 * c8], tile[row][4 * c8 + 1], tile[row][4 * c8 + 2], tile[row][4 * c8 + 3]);
     }
   }
 }
