@@ -44,8 +44,9 @@ import torch
 METRIC = "prune+compact GB/s and sparse-act dW TFLOP/s, as % of B200 HBM/tensor peak"
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 NOMINAL = {"hbm_gbs": 7700.0, "bf16_tflops": 2250.0}
-# fp32 CUDA-core peak for the fp32 path: 148 SMs x 128 FMA lanes x 2 flop x 1.965 GHz
-FP32_ALU_TFLOPS = 148 * 128 * 2 * 1.965e9 / 1e12
+# The fp32 path forms an fp32 product from six bf16 products on the tensor cores (three with bf16 activations, which
+# are counted as six here).
+FP32_PRODUCTS = 6
 HEADLINE = "vit"
 
 
@@ -389,9 +390,10 @@ def frac_entry(kind, achieved, peaks, path_tc=True, traffic=None, extra=None):
              "frac_sustained": round(achieved / sus, 4), "peak_sustained": round(sus, 1),
              "frac_nominal": round(achieved / NOMINAL["bf16_tflops"], 4)}
     else:
-        d = {"bound": "alu", "achieved": round(achieved, 3), "peak": round(FP32_ALU_TFLOPS, 1), "unit": "TFLOP/s",
-             "frac": round(achieved / FP32_ALU_TFLOPS, 4), "traffic": traffic,
-             "peak_source": "derived: 148 SMs x 128 fp32 FMA lanes x 2 x 1.965 GHz"}
+        peak = float(peaks["bf16_tflops"]) / FP32_PRODUCTS
+        d = {"bound": "tensor", "achieved": round(achieved, 3), "peak": round(peak, 1), "unit": "TFLOP/s",
+             "frac": round(achieved / peak, 4), "traffic": traffic,
+             "peak_source": "%s bf16 cuBLAS, burst / %d bf16 products" % (peaks["_source"], FP32_PRODUCTS)}
     if extra:
         d.update(extra)
     return d
@@ -464,7 +466,7 @@ def run_stack(key, args, rank, world, device, peaks, path, keep_stack=False, sam
     tc = path == B.PATH_TENSOR_CORE
     # per-layer roofline time of the weight gradient: the slower of the tensor cores on the
     # dense-equivalent flops and HBM on the least bytes (fp32 gradient + store + dW)
-    tpeak = float(peaks["bf16_tflops"]) * 1e12 if tc else FP32_ALU_TFLOPS * 1e12
+    tpeak = float(peaks["bf16_tflops"]) * 1e12 / (1 if tc else FP32_PRODUCTS)
     hpeak = float(peaks["hbm_gbs"]) * 1e9
     roof_us = [max(l.flops / tpeak, dw_min_bytes(l, s.sizes.n_keep) / hpeak) * 1e6
                for l, s in zip(layers, stack.store)]
