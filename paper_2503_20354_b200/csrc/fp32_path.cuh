@@ -6,6 +6,11 @@
 
 namespace surgeon {
 
+// Both operands are multiplied by 2^24 before they are cut: a subnormal number's last bit, 2^-149, then is 2^-125, so the
+// parts of every number are normal bf16 numbers, and a product that is lost (below 2^-126) is below 2^-174, of which
+// an fp32 sum keeps nothing.  The partial sums carry the factor of both operands, 2^48.
+constexpr int kSplitShift = 24;
+
 struct SplitGeom {
   int C, H, W, O, KW, RS, stride, pad, OH, OW;
   int P, K, N;              // positions per image (linear: 1), what the GEMM sums over, its columns (c, r, s)
@@ -23,7 +28,7 @@ struct SplitGeom {
 bool plan_split(const surgeon_layer_desc& d, SplitGeom* out);
 size_t split_planes_bytes(const SplitGeom& g);
 // partial: [chunks][O][N].  most: the largest magnitudes of the gradient (a word per block of the pre-pass) and then of the
-// activation (a word per CTA), as bf16 patterns; 0xFFFF from a CTA that gave up.
+// activation (a word per CTA), as bf16 patterns of the scaled numbers; 0xFFFF from a CTA that gave up.
 cudaError_t launch_split(const surgeon_compressed& act, const SplitGeom& g, const float* grad_out, void* planes,
                          float* partial, uint32_t* most, cudaStream_t stream);
 

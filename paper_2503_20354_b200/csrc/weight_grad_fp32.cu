@@ -46,18 +46,16 @@ struct Geom {
 // What the tensor cores (weight_grad_fp32_split.cu) left behind, where they ran first.
 struct SplitResult {
   const uint32_t* most;     // largest magnitudes: n_grad words of the gradient, n_act of the activation
-  int* n_parts;             // to be set: partial sums per output
+  int* n_parts;             // to be set: partial sums per output, and whether they carry the factor of both operands
   int n_grad, n_act, chunks;
 };
 
-// Whether the three bf16 parts held all of every operand, given the bit patterns of the largest magnitudes.  Infinities and
-// NaN have no parts.  A third part lies 2^-24 below its number and is lost below 2^-133, products below 2^-126: ranges
-// that end well above both, and below 2^127.
+// Whether the tensor cores' partial sums stand, given the bf16 patterns of the largest scaled magnitudes.  Infinities, NaN and
+// what the factor makes infinite have no parts; a chunk's 2048 products, each below 2^(ea + eb - 2 * 127 + 2), have to
+// stay below 2^127.  There is no lower limit: the factor gives every number its three parts (kSplitShift).
 __device__ __forceinline__ bool split_holds(uint32_t a, uint32_t b) {
   if (a >= 0x7F80u || b >= 0x7F80u) return false;
-  if (a == 0 || b == 0) return true;
-  const uint32_t ea = a >> 7, eb = b >> 7;       // exponents, 127 more than they are
-  return ea >= 127 - 80 && eb >= 127 - 80 && ea + eb >= 2 * 127 - 80 && ea + eb <= 2 * 127 + 100;
+  return (a >> 7) + (b >> 7) <= 2 * 127 + 127 - 11 - 2;    // (exponents, 127 more than they are)
 }
 
 Geom make_geom(const surgeon_layer_desc& d) {
@@ -191,7 +189,10 @@ dw_fp32_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ val
     }
     __syncthreads();
     const bool stands = split_holds(s_most[0], s_most[1]);
-    if (threadIdx.x == 0 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) *split.n_parts = stands ? split.chunks : g.chunks;
+    if (threadIdx.x == 0 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) {
+      split.n_parts[0] = stands ? split.chunks : g.chunks;
+      split.n_parts[1] = stands ? 1 : 0;
+    }
     pdl_trigger();
     if (stands) return;
   }
@@ -381,7 +382,8 @@ dw_fp32_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ val
   }
 }
 
-// The partial sums, in double, in a fixed order.  n_parts: how many there are (null: `chunks`).  V outputs a thread, or
+// The partial sums, in double, in a fixed order.  n_parts: how many there are (null: `chunks`), and whether the factor of
+// both operands is taken out again (exact in double: no number is rounded twice).  V outputs a thread, or
 // (V = 1, blocks of 32 x 8) one by eight threads, which take every eighth partial sum.
 template <int V, bool EIGHT>
 __global__ void __launch_bounds__(256)
@@ -389,7 +391,11 @@ reduce_chunks_kernel(const float* __restrict__ partial, long long mn, int chunks
                      float* __restrict__ dw, int accumulate) {
   static_assert(V == 1 || !EIGHT, "one output");
   pdl_wait();
-  if (n_parts) chunks = *n_parts;
+  double factor = 1.0;
+  if (n_parts) {
+    chunks = n_parts[0];
+    if (n_parts[1]) factor = 1.0 / static_cast<double>(1ull << (2 * kSplitShift));
+  }
   const long long i = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) * V;
   using Vec = typename std::conditional<V == 4, float4, float>::type;
   double s[V];
@@ -414,8 +420,10 @@ reduce_chunks_kernel(const float* __restrict__ partial, long long mn, int chunks
   if (i >= mn) return;
   float out[V];
 #pragma unroll
-  for (int e = 0; e < V; ++e)
+  for (int e = 0; e < V; ++e) {
+    s[e] *= factor;
     out[e] = accumulate ? static_cast<float>(static_cast<double>(dw[i + e]) + s[e]) : static_cast<float>(s[e]);
+  }
   *reinterpret_cast<Vec*>(dw + i) = *reinterpret_cast<const Vec*>(out);
 }
 

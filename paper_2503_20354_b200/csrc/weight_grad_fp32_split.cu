@@ -3,7 +3,9 @@
 // An fp32 number is the sum of three bf16 numbers, exactly: x1 = bf16(x), x2 = bf16(x - x1), x3 = x - x1 - x2 (24
 // significant bits in 3 x 8, both differences exact).  A product is then the sum of nine products of bf16 numbers, each
 // exact in fp32; six of them are formed (x1 y1, x1 y2, x2 y1, x2 y2, x1 y3, x3 y1), the other three are 2^-26 of it and
-// less.  For bf16 activations x = x1, and three products are all.
+// less.  For bf16 activations x = x1, and three products are all.  Both operands are first multiplied by 2^24 (exact), which
+// the reduction takes out: without it numbers below 2^-109 lost their low parts, however large others were (an output channel
+// of 1e-36 beside ordinary ones: 3e-5 of its row of dW, one of 1e-40 a quarter of it; now 1e-7).
 //
 // The tensor cores add with truncation, so no long chain of large terms runs in them: x1 y1 is summed over one K-tile of 64
 // positions, from zero, and leaves for fp32 registers, where it is added rounding to nearest.  The small products have an
@@ -26,8 +28,9 @@
 // what they wait for are the bound (store 750, asking for values 1300, sums 800, or 2000 beside MMAs).  MMAs issued by the
 // warps in turn instead of by a warp of their own: 7600 clocks a tile, since whoever issues is late for the next tile.
 //
-// What the planes cannot hold (infinities and NaN, magnitudes whose low parts or whose products leave the range of the
-// formats) sets the CTA's flag, as a wait that ran out does; the CUDA-core kernel then computes the whole call again.
+// Infinities and NaN, operands from 2^104 on and calls whose largest operands multiply to 2^64 and more (which the
+// factor could make infinite) are seen from the largest magnitudes, which every block records; a wait that ran out
+// records one too.  The CUDA-core kernel then computes the whole call again.
 #include <cuda.h>
 
 #include <algorithm>
@@ -51,9 +54,12 @@ static_assert(32 * kWarps * kRegsWork + 128 * kRegsIssue <= kThreads * 96, "regi
 constexpr int kMaxTileN = 160;                   // 40 sums a thread; two accumulators in 512 columns
 constexpr int kPlaneA = kTileM * kTileK * 2;     // 16 KB
 constexpr int kMaxTiles = 2048 / kTileK;         // K-tiles of one chunk at most
+constexpr float kSplitScale = static_cast<float>(1 << kSplitShift);
 
-// x0, x1 -> their three parts, two to a word.
+// x0, x1 times 2^kSplitShift -> their three parts, two to a word.
 __device__ __forceinline__ void split2(float x0, float x1, uint32_t& p1, uint32_t& p2, uint32_t& p3) {
+  x0 *= kSplitScale;
+  x1 *= kSplitScale;
   p1 = pack_bf16x2(x0, x1);
   x0 -= __uint_as_float(p1 << 16);
   x1 -= __uint_as_float(p1 & 0xFFFF0000u);
@@ -61,6 +67,12 @@ __device__ __forceinline__ void split2(float x0, float x1, uint32_t& p1, uint32_
   x0 -= __uint_as_float(p2 << 16);
   x1 -= __uint_as_float(p2 & 0xFFFF0000u);
   p3 = pack_bf16x2(x0, x1);
+}
+// Two bf16 numbers times 2^kSplitShift.
+__device__ __forceinline__ uint32_t scale_bf16x2(uint32_t x) {
+  uint32_t r;
+  asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(static_cast<uint32_t>((127 + kSplitShift) << 7) * 0x10001u));
+  return r;
 }
 // The packed value `idx` into r where `on`.
 template <int DT>
@@ -409,7 +421,7 @@ dw_split_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ va
           for (int e = 0; e < 4; ++e) {
             const uint32_t x0 = v[8 * h + 2 * e], x1 = v[8 * h + 2 * e + 1];
             if (DT == 0) split2(__uint_as_float(x0), __uint_as_float(x1), w[0][e], w[1][e], w[2][e]);
-            else w[0][e] = x0 | (x1 << 16);
+            else w[0][e] = scale_bf16x2(x0 | (x1 << 16));
             largest = __vmaxu2(largest, w[0][e] & 0x7FFF7FFFu);
           }
 #pragma unroll

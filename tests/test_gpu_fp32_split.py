@@ -62,6 +62,46 @@ def test_magnitudes_at_the_ends_of_the_range(scale_a, scale_g):
     assert np.linalg.norm(dw - ref) <= 1e-5 * np.linalg.norm(ref) + 2.0 ** -150 * 700 * np.sqrt(ref.size)
 
 
+ROWS = [replace(LINEAR, name="linear"), W.conv("k3", 2, 24, 12, 40, 3, dt=W.F32), W.conv("k3s2", 8, 40, 31, 96, 3, 2, dt=W.F32)]
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("layer", ROWS, ids=lambda l: l.name)
+def test_small_channels_beside_large_ones(layer, bf16):
+    """Output channels from 1e-30 down to the smallest subnormal numbers beside ordinary ones, and an input channel of each
+    size: every row of dW is as near to its own sum as an ordinary one (1e-6, and half of fp32's last bit, 2^-149)."""
+    layer = replace(layer, dt=W.BF16 if bf16 else W.F32)
+    a, g = W.activation(layer, 11), W.grad_out(layer, 11)
+    a, g = a.reshape(layer.act_shape), g.reshape(layer.grad_shape)
+    sizes = [1e-30, 1e-32, 1e-34, 1e-36, 1e-38, 1e-40, 1e-42, 1e-44]
+    for i, size in enumerate(sizes):
+        g[:, 3 + i] *= size / layer_scale(g)
+        a[:, 4 + i] = (a[:, 4 + i].float() * size).to(a.dtype)
+    a[:, 12:] = (a[:, 12:].float() * 1e6).to(a.dtype)          # (so that small rows are not all below fp32's range)
+    store = B.surgeon_prune_compact(a.cuda(), 0.0)
+    dw = B.surgeon_weight_grad(store, B.layer_desc(layer, B.PATH_FP32), g.cuda()).cpu().numpy().astype(np.float64)
+    ref = oracle_dw(layer, W.as_numpy_bits(a).reshape(-1), g.numpy()).astype(np.float64).reshape(dw.shape)
+    for rows, want in ((dw, ref), (dw.swapaxes(0, 1), ref.swapaxes(0, 1))):        # by output channel, by input channel
+        rows, want = rows.reshape(rows.shape[0], -1), want.reshape(rows.shape[0], -1)
+        far = np.linalg.norm(rows - want, axis=1) / (1e-6 * np.linalg.norm(want, axis=1) + 2.0 ** -150 * np.sqrt(want.shape[1]))
+        assert far.max() <= 1, (np.argmax(far), far.max())
+
+
+def layer_scale(g):
+    return float(g.abs().max())
+
+
+@pytest.mark.parametrize("small", ["activation", "gradient"])
+def test_subnormal_times_large(small):
+    """Every product is an ordinary number, one operand rounds to no bf16 number but zero."""
+    a, g = W.activation(LINEAR, 12), W.grad_out(LINEAR, 12)
+    a, g = (a * 4e-43, g * 1e30) if small == "activation" else (a * 1e30, g * 4e-43)
+    store = B.surgeon_prune_compact(a.cuda(), 0.0)
+    dw = B.surgeon_weight_grad(store, B.layer_desc(LINEAR, B.PATH_FP32), g.cuda()).cpu().numpy()
+    ref = g.numpy().astype(np.float64).T @ a.numpy().astype(np.float64).reshape(700, -1)
+    assert np.linalg.norm(ref) > 0 and rel_frobenius(dw, ref) <= 1e-6
+
+
 @pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
 @pytest.mark.parametrize("where", ["activation", "gradient"])
 def test_infinities_and_nan(where, value):
