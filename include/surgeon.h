@@ -235,7 +235,9 @@ typedef struct surgeon_layer_desc {
                     values of `path` run the same fp32 CUDA-core kernel for such a layer.       */
 } surgeon_layer_desc;
 
-/* Device scratch (bytes) surgeon_weight_grad needs for this layer and path; 0 on a bad desc. */
+/* Device scratch (bytes) surgeon_weight_grad needs for this layer and path; 0 on a bad desc.  Path 0: a bf16 copy of the
+ * gradient (half of its fp32 size) and partial sums.  Path 1: the bf16 parts of the gradient (1.5 times its fp32 size, more
+ * for channel counts that are padded; 128 MB, or half the fp32 size where that is more, at most) and partial sums. */
 size_t surgeon_weight_grad_workspace(const surgeon_layer_desc* d);
 
 /* ------------------------------------------------------------------------------------------

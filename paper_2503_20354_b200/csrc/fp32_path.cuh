@@ -23,11 +23,13 @@ struct SplitGeom {
   int tile_n, nt, mt;       // output channels per CTA, tiles of them, tiles of 128 columns
   int warp_cols, tmem_cols;
   int k_tiles, per_chunk, chunks, ctas;
+  int slabs, slab_chunks;   // the chunks are taken so many at a time, so that the gradient's planes stay small
+  int kt0, chunk0;          // (set for each launch) the slab's first K-tile and chunk
 };
 // False: the layer is not one for it.
 bool plan_split(const surgeon_layer_desc& d, SplitGeom* out);
 size_t split_planes_bytes(const SplitGeom& g);
-// partial: [chunks][O][N].  most: the largest magnitudes of the gradient (a word per block of the pre-pass) and then of the
+// partial: [chunks][O][N].  most: the largest magnitudes of the gradient (a word per block of the pre-passes) and then of the
 // activation (a word per CTA), as bf16 patterns of the scaled numbers; 0xFFFF from a CTA that gave up.
 cudaError_t launch_split(const surgeon_compressed& act, const SplitGeom& g, const float* grad_out, void* planes,
                          float* partial, uint32_t* most, cudaStream_t stream);

@@ -432,7 +432,7 @@ reduce_chunks_kernel(const float* __restrict__ partial, long long mn, int chunks
 // Scratch of a layer for the tensor cores: the count of partial sums per output and the largest magnitudes, the gradient's
 // planes, then the partial sums.
 static size_t split_head_bytes(const SplitGeom& s) {
-  return (16 + (static_cast<size_t>(s.grad_blocks) + s.ctas) * 4 + 255) & ~static_cast<size_t>(255);
+  return (16 + (static_cast<size_t>(s.slabs) * s.grad_blocks + s.ctas) * 4 + 255) & ~static_cast<size_t>(255);
 }
 
 size_t weight_grad_fp32_workspace(const surgeon_layer_desc& d) {
@@ -455,7 +455,7 @@ cudaError_t launch_weight_grad_fp32(const surgeon_compressed& act, const surgeon
     uint32_t* most = static_cast<uint32_t*>(workspace) + 4;
     char* planes = static_cast<char*>(workspace) + split_head_bytes(s);
     partial = reinterpret_cast<float*>(planes + split_planes_bytes(s));
-    result = {most, n_parts, s.grad_blocks, s.ctas, s.chunks};
+    result = {most, n_parts, s.slabs * s.grad_blocks, s.ctas, s.chunks};
     const cudaError_t e = launch_split(act, s, grad_out, planes, partial, most, stream);
     if (e != cudaSuccess) return e;
   }

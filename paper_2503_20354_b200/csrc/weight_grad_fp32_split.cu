@@ -54,6 +54,14 @@ static_assert(32 * kWarps * kRegsWork + 128 * kRegsIssue <= kThreads * 96, "regi
 constexpr int kMaxTileN = 160;                   // 40 sums a thread; two accumulators in 512 columns
 constexpr int kPlaneA = kTileM * kTileK * 2;     // 16 KB
 constexpr int kMaxTiles = 2048 / kTileK;         // K-tiles of one chunk at most
+// The planes take 1.5 times the gradient (more where columns are padded), so a large layer is done in slabs: as many chunks at
+// a time as 128 MB of planes hold, or half the fp32 gradient where that is more (what the bf16 path's copy of it takes).
+// 64 -> 256 channels 1x1 on 56x56, batch 64: 318 MB of scratch and 200 us in one piece, 117 and 218 in three slabs (8 MB of them
+// partial sums); with 64 MB at most it would be 97 and 228.  3x3, 160 -> 160 on 32x32, batch 200: 303 MB and 708 us, 172 and 739.
+constexpr long long kMaxPlanes = 128LL << 20;
+constexpr double kSlabCost = 4.0;                // of a further slab, in K-tiles
+constexpr int kLeastTiles = 20;                  // chunks of fewer K-tiles only while the partial sums are below
+constexpr double kMaxPartials = 32 << 20;
 constexpr float kSplitScale = static_cast<float>(1 << kSplitShift);
 
 // x0, x1 times 2^kSplitShift -> their three parts, two to a word.
@@ -103,21 +111,29 @@ __device__ __forceinline__ uint64_t make_desc_mn64(uint32_t saddr) {
          static_cast<uint64_t>(1024 >> 4) << 32 | static_cast<uint64_t>(1) << 46 | static_cast<uint64_t>(2) << 61;
 }
 
-// The gradient's planes, cut into the pieces that a CTA loads for a K-tile, byte for byte as they lie in its shared
-// memory: [K-tile][column tile][plane][tile_n x 64].  Eight columns a thread.  `most`: a word per block.
+__host__ __device__ __forceinline__ int slab_tiles(const SplitGeom& g) {        // K-tiles of the slab from kt0 on
+  const int all = g.slab_chunks * g.per_chunk, left = g.k_tiles - g.kt0;
+  return all < left ? all : left;
+}
+
+// The planes of a slab of the gradient, cut into the pieces that a CTA loads for a K-tile, byte for byte as they lie in its
+// shared memory: [K-tile][column tile][plane][tile_n x 64].  Eight columns a thread.  `most`: a word per block.
 __global__ void __launch_bounds__(256)
 grad_split_kernel(const float* __restrict__ grad, unsigned char* __restrict__ out, uint32_t* __restrict__ most, SplitGeom g) {
   pdl_wait();
   pdl_trigger();
   // a row is an output channel, its columns the positions of all images (linear: a row t, its columns channels)
   const int n_rows = g.linear ? g.K : g.O, n_cols = g.linear ? g.O : g.K;
-  const int rows = g.linear ? g.k_tiles * kTileK : g.nt * g.tile_n, per_row = (g.linear ? g.nt * g.tile_n : g.k_tiles * kTileK) >> 3;
+  const int k0 = g.kt0 * kTileK, k_here = slab_tiles(g) * kTileK;
+  const int rows = g.linear ? k_here : g.nt * g.tile_n, per_row = (g.linear ? g.nt * g.tile_n : k_here) >> 3;
   const long long items = static_cast<long long>(rows) * per_row;
   const size_t plane = static_cast<size_t>(g.tile_n) * kTileK * 2;
   uint32_t largest = 0;
   for (long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; i < items;
        i += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const int row = static_cast<int>(i / per_row), col = static_cast<int>(i - static_cast<long long>(row) * per_row) * 8;
+    int row = static_cast<int>(i / per_row), col = static_cast<int>(i - static_cast<long long>(row) * per_row) * 8;
+    if (g.linear) row += k0;
+    else col += k0;
     // a row's columns are in pieces of P, one per image (linear: in one piece)
     const uint32_t img = g.linear ? 0u : divide(col, g.by_p), p = col - img * g.P;
     const float* at = grad + (g.linear ? static_cast<size_t>(row) * g.O + col : (static_cast<size_t>(img) * g.O + row) * g.P + p);
@@ -148,7 +164,7 @@ grad_split_kernel(const float* __restrict__ grad, unsigned char* __restrict__ ou
       split2(x[2 * e], x[2 * e + 1], a[e], b[e], c[e]);
       largest = __vmaxu2(largest, a[e] & 0x7FFF7FFFu);
     }
-    const int o = g.linear ? col : row, k = g.linear ? row : col, j = o / g.tile_n, n = o - j * g.tile_n;
+    const int o = g.linear ? col : row, k = (g.linear ? row : col) - k0, j = o / g.tile_n, n = o - j * g.tile_n;
     unsigned char* to = out + (static_cast<size_t>(k / kTileK) * g.nt + j) * 3 * plane +
                         (g.linear ? (n >> 6) * (kTileK * 128) + tile_off(k % kTileK, (n & 63) >> 3) : tile_off(n, (k % kTileK) >> 3));
     *reinterpret_cast<uint4*>(to) = make_uint4(a[0], a[1], a[2], a[3]);
@@ -182,7 +198,7 @@ dw_split_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ va
   const int tid = threadIdx.x, warp = tid >> 5;
   const uint32_t lane = lane_id();
   const int n0 = blockIdx.x * kTileM, o0 = blockIdx.y * g.tile_n;
-  const int kt_begin = blockIdx.z * g.per_chunk, n_kt = min(g.per_chunk, g.k_tiles - kt_begin);
+  const int chunk = g.chunk0 + static_cast<int>(blockIdx.z), kt_begin = chunk * g.per_chunk, n_kt = min(g.per_chunk, g.k_tiles - kt_begin);
   const uint32_t full_a = smem_u32(bars), full_b = smem_u32(bars + 2), done = smem_u32(bars + 4);
   if (tid == 0) {
     for (int s = 0; s < 2; ++s) {
@@ -240,7 +256,7 @@ dw_split_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ va
         if (it >= 2 && (fail || !mbar_wait_suspend(done + 8 * s, ((it - 2) >> 1) & 1))) { fail = 1; break; }
         mbar_arrive_expect_tx(full_b + 8 * s, 3u * plane_b);
         bulk_load(smem_u32(smem) + s * stage_bytes + NA * kPlaneA,
-                  planes + (static_cast<size_t>(kt_begin + it) * gridDim.y + blockIdx.y) * (3u * plane_b), 3u * plane_b, full_b + 8 * s);
+                  planes + (static_cast<size_t>(kt_begin - g.kt0 + it) * gridDim.y + blockIdx.y) * (3u * plane_b), 3u * plane_b, full_b + 8 * s);
       }
       // (the loads under way write to shared memory)
       for (int i = max(0, it - 2); i < it; ++i) mbar_wait_suspend(full_b + 8 * (i & 1), (i >> 1) & 1);
@@ -448,7 +464,7 @@ dw_split_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ va
     if (lane == 0) atomicMax(&s_most, largest);
     // ---- the partial sums ----
     const int nn = n0 + 32 * (warp & 3) + static_cast<int>(lane);
-    float* out = partial + static_cast<size_t>(blockIdx.z) * g.O * g.N;
+    float* out = partial + static_cast<size_t>(chunk) * g.O * g.N;
     if (nn < g.N) {
 #pragma unroll
       for (int u = 0; u < 5; ++u) {
@@ -463,7 +479,7 @@ dw_split_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ va
   tc_fence_before();
   __syncthreads();
   if (warp == kWarps) tmem_dealloc(tmem_base, g.tmem_cols);
-  if (tid == 0) most[(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = fail ? 0xFFFFu : s_most;
+  if (tid == 0) most[(chunk * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = fail ? 0xFFFFu : s_most;
 }
 
 bool compute_plan_split(const surgeon_layer_desc& d, SplitGeom* out) {
@@ -503,22 +519,31 @@ bool compute_plan_split(const surgeon_layer_desc& d, SplitGeom* out) {
   g.tmem_cols = 32;
   while (g.tmem_cols < 3 * g.tile_n) g.tmem_cols *= 2;
   g.k_tiles = (g.K + kTileK - 1) / kTileK;
-  // K-tiles per chunk: as many rounds of CTAs (one per SM) as it takes, each as short as possible; a chunk costs about
-  // three K-tiles (start, epilogue, its part of the reduction) on top of its own.
+  // K-tiles per chunk and chunks per slab: as many rounds of CTAs (one per SM) as it takes, each as short as possible; a
+  // chunk costs about three K-tiles (start, epilogue, its part of the reduction) on top of its own, a slab kSlabCost.
   const long long tiles = static_cast<long long>(g.mt) * g.nt;
+  const long long room = std::max<long long>(std::max<long long>(kMaxPlanes, 2 * K * d.c_out) / (static_cast<long long>(g.nt) * 3 * g.tile_n * kTileK * 2), kMaxTiles);
   const int sms = sm_count();
+  const double chunk_cost = 0.6e-6 * g.O * g.N;  // written and read again, in K-tiles
   double best = 1e300;
   for (int per = 1; per <= kMaxTiles; ++per) {
     const long long chunks = (g.k_tiles + per - 1) / per;
     if (chunks > 65535) continue;                // (blockIdx.z)
-    const double cost = static_cast<double>((tiles * chunks + sms - 1) / sms) * (per + 3.0);
-    if (cost <= best) { best = cost; g.per_chunk = per; }
+    const long long least = (chunks + room / per - 1) / (room / per);
+    if (least > 1 && per < kLeastTiles && 4.0 * chunks * g.O * g.N > kMaxPartials) continue;
+    for (long long slabs = least; slabs <= (least == 1 ? 1 : least + 3) && slabs <= chunks; ++slabs) {
+      const long long each = (chunks + slabs - 1) / slabs, last = chunks - (slabs - 1) * each;
+      if (last < 1) continue;
+      const double cost = static_cast<double>((slabs - 1) * ((tiles * each + sms - 1) / sms) + (tiles * last + sms - 1) / sms) * (per + 3.0) +
+                          (slabs > 1 ? kSlabCost * (slabs - 1) + chunk_cost * chunks : 0.0);
+      if (cost <= best) { best = cost; g.per_chunk = per; g.slabs = static_cast<int>(slabs); g.slab_chunks = static_cast<int>(each); }
+    }
   }
   if (!g.per_chunk) return false;
   g.chunks = (g.k_tiles + g.per_chunk - 1) / g.per_chunk;
   if (tiles * g.chunks > (1LL << 30)) return false;
   g.ctas = static_cast<int>(tiles * g.chunks);
-  const long long items = static_cast<long long>(g.k_tiles) * kTileK * g.nt * g.tile_n / 8;
+  const long long items = static_cast<long long>(slab_tiles(g)) * kTileK * g.nt * g.tile_n / 8;
   g.grad_blocks = static_cast<int>(std::min<long long>((items + 255) / 256, 4LL * sms));
   *out = g;
   return true;
@@ -532,22 +557,28 @@ bool plan_split(const surgeon_layer_desc& d, SplitGeom* out) {
 }
 
 size_t split_planes_bytes(const SplitGeom& g) {
-  return static_cast<size_t>(g.k_tiles) * g.nt * 3 * g.tile_n * kTileK * 2;
+  return static_cast<size_t>(slab_tiles(g)) * g.nt * 3 * g.tile_n * kTileK * 2;
 }
 
-cudaError_t launch_split(const surgeon_compressed& act, const SplitGeom& g, const float* grad_out, void* planes,
+cudaError_t launch_split(const surgeon_compressed& act, const SplitGeom& plan, const float* grad_out, void* planes,
                          float* partial, uint32_t* most, cudaStream_t stream) {
-  note_launches(2);
-  const cudaError_t e = launch_kernel(grad_split_kernel, dim3(g.grad_blocks), dim3(256), 0, stream, true, grad_out,
-                                      static_cast<unsigned char*>(planes), most, g);
-  if (e != cudaSuccess) return e;
+  SplitGeom g = plan;
   const int smem = 2 * ((act.dt == 0 ? 3 : 1) * kPlaneA + 3 * g.tile_n * kTileK * 2) + 1024;
   auto launch = [&](auto kernel) -> cudaError_t {
-    const cudaError_t err = allow_dynamic_smem(reinterpret_cast<const void*>(kernel), smem);
-    if (err != cudaSuccess) return err;
-    return launch_kernel(kernel, dim3(g.mt, g.nt, g.chunks), dim3(kThreads), smem, stream, true, act.bitmap,
-                         static_cast<const void*>(act.values), act.block_offsets, static_cast<const unsigned char*>(planes),
-                         partial, most + g.grad_blocks, g);
+    cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void*>(kernel), smem);
+    for (int slab = 0; slab < g.slabs && e == cudaSuccess; ++slab) {
+      g.chunk0 = slab * g.slab_chunks;
+      g.kt0 = g.chunk0 * g.per_chunk;
+      const int chunks = std::min(g.slab_chunks, g.chunks - g.chunk0);
+      e = launch_kernel(grad_split_kernel, dim3(g.grad_blocks), dim3(256), 0, stream, true, grad_out,
+                        static_cast<unsigned char*>(planes), most + slab * g.grad_blocks, g);
+      if (e != cudaSuccess) break;
+      e = launch_kernel(kernel, dim3(g.mt, g.nt, chunks), dim3(kThreads), smem, stream, true, act.bitmap,
+                        static_cast<const void*>(act.values), act.block_offsets, static_cast<const unsigned char*>(planes),
+                        partial, most + g.slabs * g.grad_blocks, g);
+      note_launches(2);
+    }
+    return e;
   };
   if (g.linear) return act.dt == 0 ? launch(dw_split_kernel<0, 0>) : launch(dw_split_kernel<1, 0>);
   if (g.stride == 1) return act.dt == 0 ? launch(dw_split_kernel<0, 1>) : launch(dw_split_kernel<1, 1>);

@@ -117,6 +117,25 @@ def test_infinities_and_nan(where, value):
     assert ok.any() and rel_frobenius(dw[ok], ref[ok]) <= 1e-5
 
 
+# gradients whose planes are done in several slabs (154, 151 and 164 MB), the second one shorter
+SLABS = [W.linear("tokens", 400_003, 24, 40, dist="normal"), W.conv("k3", 48, 4, 128, 20, 3), W.conv("k3s2", 13, 3, 512, 24, 3, 2)]
+
+
+@pytest.mark.parametrize("layer", SLABS, ids=lambda l: l.name)
+def test_slabs(layer):
+    a, g = W.activation(layer, 13), W.grad_out(layer, 13)
+    store = B.surgeon_prune_compact(a.cuda(), 0.5)
+    dw = B.surgeon_weight_grad(store, B.layer_desc(layer, B.PATH_FP32), g.cuda()).cpu().numpy()
+    bits = W.as_numpy_bits(a).reshape(-1)
+    r = oracle.prune_compact(bits, 0.5)
+    ref = oracle_dw(layer, oracle.decompress(r["bitmap"], r["values"], bits.size), g.numpy())
+    assert rel_frobenius(dw, ref) <= 1e-6
+    # seen by the last slab alone
+    g.view(-1)[-1] = np.inf
+    again = B.surgeon_weight_grad(store, B.layer_desc(layer, B.PATH_FP32), g.cuda()).cpu().numpy().reshape(layer.c_out, -1)
+    assert not np.isfinite(again[-1]).all() and rel_frobenius(again[:-1], ref.reshape(layer.c_out, -1)[:-1]) <= 1e-5
+
+
 def test_an_exact_product_stays_exact():
     """One row of the gradient is one value: dW is that row of the activation, to the last bit."""
     a, g = W.activation(LINEAR, 9), torch.zeros(700, 96)

@@ -39,6 +39,19 @@ def test_struct_layouts_match_header():
     assert ctypes.sizeof(B.LayerDesc) == 48
 
 
+@pytest.mark.parametrize("layer", [
+    W.conv("shortcut", 200, 16, 32, 160, 1, 1, 0), W.conv("3x3", 200, 160, 32, 160, 3), W.conv("expand", 64, 64, 56, 256, 1, 1, 0),
+    W.conv("stem", 64, 3, 224, 64, 7, 2, 3), W.conv("head", 16, 64, 512, 19, 1, 1, 0), W.linear("fc1", 12608, 768, 3072),
+    W.linear("few columns", 1_000_000, 64, 10)], ids=lambda l: l.name)
+def test_scratch_of_the_fp32_path_is_bounded(layer):
+    """The bf16 parts of the gradient: 128 MB, or half the fp32 gradient where that is more; and the partial sums, one per
+    20 K-tiles of 64 (the number of weights each), or 64 MB of them."""
+    grad = 4 * int(np.prod(layer.grad_shape))
+    positions = grad // 4 // layer.c_out
+    partial = 4 * layer.n_weight * (positions // (20 * 64) + 2)
+    assert B.surgeon_weight_grad_workspace(B.layer_desc(layer, B.PATH_FP32)) <= max(128 << 20, grad // 2) + max(64 << 20, partial) + (1 << 20)
+
+
 def test_ratios_match_oracle_and_fixture():
     st, p = oracle.layer_ratios([2, 1, 4], [4, 2, 2])
     got = B.surgeon_layer_ratios([2, 1, 4], [4, 2, 2])
