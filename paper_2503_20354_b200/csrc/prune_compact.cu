@@ -98,6 +98,7 @@ struct PruneArgs {
   int n_chunks;                  // chunks in all
   int drop_zeros, stall;
   unsigned long long token;      // unlike any other call's
+  unsigned long long table_base; // unlike any other process's
   surgeon_header* hdr;
   uint32_t* bitmap;
   void* values;
@@ -138,6 +139,10 @@ __device__ __forceinline__ uint32_t hash_u32(uint32_t v) {
 // these reports where it asks for keys, off the chain (it has answered by then): it sees cleared words or this call's.
 // Where a CTA has more keys than it can report, the bin is narrowed and keys are reported once more, in the same words: the
 // tag names the phase.
+//
+// The table's words are not cleared (every CTA reads those of all others, so a fence would stand in every CTA's chain).
+// Their tag is 64 bits: the process's random number and how many executions of this kernel the GPU has begun, which CTA 0
+// counts up and tells the others with its first answer.  No two executions, replays included, have the same.
 __device__ __forceinline__ void word_store(ulonglong2* p, unsigned long long token, unsigned long long v) {
   asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}"
                ::"l"(p), "l"(token), "l"(v) : "memory");
@@ -163,9 +168,8 @@ __device__ __forceinline__ unsigned long long key_load_if(const unsigned long lo
                : "+l"(v) : "l"(p), "r"(static_cast<uint32_t>(wanted)) : "memory");
   return v;
 }
-__device__ __forceinline__ unsigned long long table_tag(unsigned long long token, unsigned long long nanoseconds) {
-  return token + nanoseconds * 0x9E3779B97F4A7C15ull;
-}
+// Executions of the kernel on this GPU so far (at most 2^64): part of the tags of the table, see below.
+__device__ unsigned long long g_executions;
 __device__ __forceinline__ uint32_t count_load(const uint32_t* p) {
   uint32_t v;
   asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -698,7 +702,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
   __shared__ uint32_t s_tot[4];                // keys above / inside the bracket, largest key inside, largest ~key inside
   __shared__ uint32_t s_over, s_fail, s_nkeys, s_list_n, s_list_lo;
   __shared__ unsigned long long s_ans[2];
-  __shared__ unsigned long long s_tag;         // of the table: unlike any other execution's, replays of this call included
+  __shared__ unsigned long long s_tag;         // of the table
   __shared__ uint32_t s_bin_key[kMaxKeys];      // the keys that this CTA reports at the last exchange,
   __shared__ int s_bin_chunk[kMaxKeys];        // and their chunks
 
@@ -964,8 +968,10 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
   for (int i = tid; i < kAuxBytes / 16; i += kThreads) reinterpret_cast<uint4*>(aux)[i] = make_uint4(0, 0, 0, 0);
   __syncthreads();
 
+  unsigned long long execution = 0;
   if (master) {                                  // meanwhile CTA 0 prepares the exchanges
     if (tid == 0) {                              // (no value yet: what reads the store trusts the count)
+      execution = atomicAdd(&g_executions, 1ull);
       a.hdr->status = SURGEON_OK;
       a.hdr->n_keep = 0;
     }
@@ -987,11 +993,9 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
   fly1 = start(false, 1);
   fly2 = start(false, 2);
   if (master && tid == 0) {                      // (by now its stores have arrived)
-    unsigned long long now;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-    s_tag = table_tag(a.token, now);
+    s_tag = a.table_base + execution;
     fence_gpu();
-    word_store(a.answer + (RES ? 0 : 1), a.token, now);      // phase 0: (RES) prepared
+    word_store(a.answer + (RES ? 0 : 1), a.token, execution);      // phase 0: (RES) prepared
   }
   // rank of the threshold inside the sample, and (RES) a margin of some standard deviations of a binomial count
   const float q = static_cast<float>(a.k) / static_cast<float>(a.n);
@@ -1108,7 +1112,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
         s_ans[tid] = w;
       }
       if (!__syncthreads_and(ok)) return kTimedOut;
-      if (tid == 0) s_tag = table_tag(a.token, s_ans[1]);
+      if (tid == 0) s_tag = a.table_base + s_ans[1];
       lo = static_cast<uint32_t>(s_ans[0]);
       hi = static_cast<uint32_t>(s_ans[0] >> 32);
     }
@@ -1279,7 +1283,7 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     }
     if (RES && round == 0 && tid == 0) {         // CTA 0 has zeroed the histograms
       if (prepared.x != a.token && !word_wait(a.answer, a.token, &prepared.y)) s_fail = 1;
-      if (!master) s_tag = table_tag(a.token, prepared.y);
+      if (!master) s_tag = a.table_base + prepared.y;
       fence_gpu();
     }
     __syncthreads();
@@ -1973,14 +1977,15 @@ bool make_row_map(const void* x, long long n_rows_full, CUtensorMap* map) {
                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+unsigned long long random_number() {
+  std::random_device rd;
+  const unsigned long long t = static_cast<unsigned long long>(
+      std::chrono::steady_clock::now().time_since_epoch().count());
+  return ((static_cast<unsigned long long>(rd()) << 32) | rd()) ^ (t << 20);
+}
 // A value that no other call of this or another process carries (see the grid-wide exchange).
 unsigned long long next_token() {
-  static std::atomic<unsigned long long> counter{[] {
-    std::random_device rd;
-    const unsigned long long t = static_cast<unsigned long long>(
-        std::chrono::steady_clock::now().time_since_epoch().count());
-    return ((static_cast<unsigned long long>(rd()) << 32) | rd()) ^ (t << 20);
-  }()};
+  static std::atomic<unsigned long long> counter{random_number()};
   return counter.fetch_add(1, std::memory_order_relaxed);
 }
 
@@ -2008,6 +2013,8 @@ cudaError_t run_prune_compact(const void* x, long long n, long long k, int drop_
   a.n_chunks = static_cast<int>(L.tiles);
   a.drop_zeros = drop_zeros; a.stall = stall;
   a.token = next_token();
+  static const unsigned long long table_base = random_number();
+  a.table_base = table_base;
   a.hdr = out.header; a.bitmap = out.bitmap; a.values = out.values; a.offsets = out.block_offsets;
   a.arrive = reinterpret_cast<ulonglong2*>(ws + L.arrive);
   a.answer = reinterpret_cast<ulonglong2*>(ws + L.answer);

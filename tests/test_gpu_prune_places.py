@@ -44,3 +44,23 @@ def test_replays_with_other_values(n, bf16):
         torch.cuda.synchronize()
         assert out.read_header().status == B.SURGEON_OK
         assert all(np.array_equal(u.view(np.uint8), v.view(np.uint8)) for u, v in zip(out.to_numpy()[:3], refs[i]))
+
+
+@pytest.mark.parametrize("n, bf16", [(1_500_001, False), (9 << 20, False), (1_500_001, True)])
+def test_every_execution_has_its_own_tag(n, bf16):
+    """What the CTAs show is told from an earlier replay's by a count of executions: words of the scratch that grow by one
+    from each replay to the next, at least one for each of dozens of CTAs."""
+    x = W.draw("relu_normal", n, seed=1, device="cuda")
+    x = x.to(torch.bfloat16) if bf16 else x
+    out = B.CompressedActivation(n, B.dtype_code(x.dtype), 0.6, "cuda")
+    ws = torch.zeros((out.sizes.workspace_bytes + 7) // 8, dtype=torch.int64, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        B.surgeon_prune_compact(x, 0.6, out=out, workspace=ws.view(torch.uint8))
+    seen = []
+    for _ in range(3):
+        graph.replay()
+        torch.cuda.synchronize()
+        seen.append(ws.clone())
+    grown = ((seen[1] - seen[0] == 1) & (seen[2] - seen[1] == 1)).sum().item()
+    assert grown >= 32, grown
