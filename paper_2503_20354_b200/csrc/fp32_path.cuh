@@ -10,6 +10,7 @@ namespace surgeon {
 // parts of every number are normal bf16 numbers, and a product that is lost (below 2^-126) is below 2^-174, of which
 // an fp32 sum keeps nothing.  The partial sums carry the factor of both operands, 2^48.
 constexpr int kSplitShift = 24;
+constexpr int kSplitTileK = 64;
 
 struct SplitGeom {
   int C, H, W, O, KW, RS, stride, pad, OH, OW;
@@ -25,10 +26,17 @@ struct SplitGeom {
   int k_tiles, per_chunk, chunks, ctas;
   int slabs, slab_chunks;   // the chunks are taken so many at a time, so that the gradient's planes stay small
   int kt0, chunk0;          // (set for each launch) the slab's first K-tile and chunk
+  uint32_t* status;         // (likewise) the store's status word, for checked builds
 };
 // False: the layer is not one for it.
 bool plan_split(const surgeon_layer_desc& d, SplitGeom* out);
-size_t split_planes_bytes(const SplitGeom& g);
+__host__ __device__ __forceinline__ int slab_tiles(const SplitGeom& g) {        // K-tiles of the slab from kt0 on
+  const int all = g.slab_chunks * g.per_chunk, left = g.k_tiles - g.kt0;
+  return all < left ? all : left;
+}
+__host__ __device__ __forceinline__ size_t split_planes_bytes(const SplitGeom& g) {      // of that slab; the first one's are the most
+  return static_cast<size_t>(slab_tiles(g)) * g.nt * 3 * g.tile_n * kSplitTileK * 2;
+}
 // partial: [chunks][O][N].  most: the largest magnitudes of the gradient (a word per block of the pre-passes) and then of the
 // activation (a word per CTA), as bf16 patterns of the scaled numbers; 0xFFFF from a CTA that gave up.
 cudaError_t launch_split(const surgeon_compressed& act, const SplitGeom& g, const float* grad_out, void* planes,

@@ -1308,11 +1308,13 @@ prune_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ P
     const bool shown = !spread && round == 0;
     auto show = [&]() {
       if (DT == 0) {
-        if (tid == 0) word_store(a.table + blockIdx.x, s_tag, (static_cast<unsigned long long>(s_tot[0]) << 32) | s_tot[1]);
+        if (tid == 0 && SURGEON_IN_BOUNDS(blockIdx.x, table_entries(a.n_chunks, DT), &a.hdr->status))
+          word_store(a.table + blockIdx.x, s_tag, (static_cast<unsigned long long>(s_tot[0]) << 32) | s_tot[1]);
       } else {
         uint32_t all;
         const uint32_t mine = my_bin(hist), bin = kSelBins - 1u - tid, up = count_above_mine(mine, s_warp, &all) + s_tot[0];
-        if (tid < kSelBins && bin < static_cast<uint32_t>(table_bins(DT)) && bin <= range >> shift)
+        if (tid < kSelBins && bin < static_cast<uint32_t>(table_bins(DT)) && bin <= range >> shift &&
+            SURGEON_IN_BOUNDS(blockIdx.x * table_bins(DT) + bin, table_entries(a.n_chunks, DT), &a.hdr->status))
           word_store(a.table + blockIdx.x * table_bins(DT) + bin, s_tag, (static_cast<unsigned long long>(up) << 32) | mine);
       }
     };

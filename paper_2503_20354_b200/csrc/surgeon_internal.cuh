@@ -41,6 +41,9 @@ constexpr int kSelPhases = 12;         // grid-wide exchanges of a call (3 in th
 constexpr int kSelMaxCtas = 256;
 constexpr int kClaimSets = 4, kClaimStride = 32;
 __host__ __device__ constexpr int table_bins(int dt) { return dt == 0 ? 1 : 256; }       // whose counts every CTA shows to the others
+__host__ __device__ constexpr size_t table_entries(int64_t chunks, int dt) {             // (a CTA has 16 chunks or all)
+  return static_cast<size_t>(chunks / 16 + 1 < kSelMaxCtas ? chunks / 16 + 1 : kSelMaxCtas) * table_bins(dt);
+}
 // Candidate slots: per chunk, room for 1/16 of its elements (fp32: 32-bit keys, bf16: 16-bit).
 __host__ __device__ constexpr int slot_entries(int dt) { return dt == 0 ? 64 : 128; }
 constexpr int slot_entry_bytes(int dt) { return dt == 0 ? 4 : 2; }
@@ -68,7 +71,7 @@ constexpr PruneLayout prune_layout(int64_t n, int dt) {
   L.cnt = off; off += t * 4;
   off = (off + 255) & ~static_cast<size_t>(255);
   L.table = off;
-  off += (t / 16 + 1 < kSelMaxCtas ? t / 16 + 1 : static_cast<size_t>(kSelMaxCtas)) * table_bins(dt) * 16;
+  off += table_entries(L.tiles, dt) * 16;
   L.slots = off;
   off += t * static_cast<size_t>(slot_entries(dt)) * slot_entry_bytes(dt);
   L.total = (off + 255) & ~static_cast<size_t>(255);

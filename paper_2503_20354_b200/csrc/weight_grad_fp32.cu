@@ -48,6 +48,7 @@ struct SplitResult {
   const uint32_t* most;     // largest magnitudes: n_grad words of the gradient, n_act of the activation
   int* n_parts;             // to be set: partial sums per output, and whether they carry the factor of both operands
   int n_grad, n_act, chunks;
+  uint32_t* status;         // the store's status word, for checked builds (set in either case)
 };
 
 // Whether the tensor cores' partial sums stand, given the bf16 patterns of the largest scaled magnitudes.  Infinities, NaN and
@@ -376,8 +377,9 @@ dw_fp32_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ val
       const long long nn = n0 + (b >> 1) * (TN / 2) + tx * 4 + (b & 1) * 2;
       const float lo = __uint_as_float(static_cast<uint32_t>(acc[a][b]));
       const float hi = __uint_as_float(static_cast<uint32_t>(acc[a][b] >> 32));
-      if (nn < g.N) out[m * g.N + nn] = lo;
-      if (nn + 1 < g.N) out[m * g.N + nn + 1] = hi;
+      const long long at = (blockIdx.z * g.M + m) * g.N + nn, all = g.chunks * g.M * g.N;
+      if (nn < g.N && SURGEON_IN_BOUNDS(at, all, split.status)) out[m * g.N + nn] = lo;
+      if (nn + 1 < g.N && SURGEON_IN_BOUNDS(at + 1, all, split.status)) out[m * g.N + nn + 1] = hi;
     }
   }
 }
@@ -388,7 +390,7 @@ dw_fp32_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ val
 template <int V, bool EIGHT>
 __global__ void __launch_bounds__(256)
 reduce_chunks_kernel(const float* __restrict__ partial, long long mn, int chunks, const int* n_parts,
-                     float* __restrict__ dw, int accumulate) {
+                     float* __restrict__ dw, int accumulate, uint32_t* status) {
   static_assert(V == 1 || !EIGHT, "one output");
   pdl_wait();
   double factor = 1.0;
@@ -417,7 +419,7 @@ reduce_chunks_kernel(const float* __restrict__ partial, long long mn, int chunks
 #pragma unroll
     for (int y = 1; y < 8; ++y) s[0] += part[y][threadIdx.x];
   }
-  if (i >= mn) return;
+  if (i >= mn || !SURGEON_IN_BOUNDS(i + V - 1, mn, status)) return;
   float out[V];
 #pragma unroll
   for (int e = 0; e < V; ++e) {
@@ -450,12 +452,13 @@ cudaError_t launch_weight_grad_fp32(const surgeon_compressed& act, const surgeon
   float* partial = static_cast<float*>(workspace);
   SplitGeom s;
   SplitResult result = {};
+  result.status = &act.header->status;
   if (g.chunks > 0 && plan_split(d, &s)) {
     int* n_parts = static_cast<int*>(workspace);
     uint32_t* most = static_cast<uint32_t*>(workspace) + 4;
     char* planes = static_cast<char*>(workspace) + split_head_bytes(s);
     partial = reinterpret_cast<float*>(planes + split_planes_bytes(s));
-    result = {most, n_parts, s.slabs * s.grad_blocks, s.ctas, s.chunks};
+    result = {most, n_parts, s.slabs * s.grad_blocks, s.ctas, s.chunks, result.status};
     const cudaError_t e = launch_split(act, s, grad_out, planes, partial, most, stream);
     if (e != cudaSuccess) return e;
   }
@@ -484,7 +487,7 @@ cudaError_t launch_weight_grad_fp32(const surgeon_compressed& act, const surgeon
   const int parts = result.most ? result.chunks : g.chunks;
   auto reduce = [&](auto kernel, int per_block, dim3 block) {
     launch_kernel(kernel, dim3(static_cast<unsigned>((mn + per_block - 1) / per_block)), block, 0, stream,
-                  result.most != nullptr, partial, mn, g.chunks, result.n_parts, dw, accumulate);
+                  result.most != nullptr, partial, mn, g.chunks, result.n_parts, dw, accumulate, &act.header->status);
   };
   // Few outputs of many partial sums: eight threads each (432 of 96: 14 us by one thread each).
   if (parts >= 16 && mn < 65536) reduce(reduce_chunks_kernel<1, true>, 32, dim3(32, 8));

@@ -45,7 +45,7 @@ namespace {
 
 using namespace tc;
 
-constexpr int kTileM = 128, kTileK = 64;
+constexpr int kTileM = 128, kTileK = kSplitTileK;
 // 16 warps work, one issues MMAs, one loads.  Five warpgroups are launched with 96 registers a thread; the last one gives
 // up 72 of them and the others take 16 more: 512 x 112 + 128 x 24 <= 640 x 96.
 constexpr int kWarps = 16, kThreads = 32 * (kWarps + 4);
@@ -111,11 +111,6 @@ __device__ __forceinline__ uint64_t make_desc_mn64(uint32_t saddr) {
          static_cast<uint64_t>(1024 >> 4) << 32 | static_cast<uint64_t>(1) << 46 | static_cast<uint64_t>(2) << 61;
 }
 
-__host__ __device__ __forceinline__ int slab_tiles(const SplitGeom& g) {        // K-tiles of the slab from kt0 on
-  const int all = g.slab_chunks * g.per_chunk, left = g.k_tiles - g.kt0;
-  return all < left ? all : left;
-}
-
 // The planes of a slab of the gradient, cut into the pieces that a CTA loads for a K-tile, byte for byte as they lie in its
 // shared memory: [K-tile][column tile][plane][tile_n x 64].  Eight columns a thread.  `most`: a word per block.
 __global__ void __launch_bounds__(256)
@@ -165,8 +160,10 @@ grad_split_kernel(const float* __restrict__ grad, unsigned char* __restrict__ ou
       largest = __vmaxu2(largest, a[e] & 0x7FFF7FFFu);
     }
     const int o = g.linear ? col : row, k = (g.linear ? row : col) - k0, j = o / g.tile_n, n = o - j * g.tile_n;
-    unsigned char* to = out + (static_cast<size_t>(k / kTileK) * g.nt + j) * 3 * plane +
-                        (g.linear ? (n >> 6) * (kTileK * 128) + tile_off(k % kTileK, (n & 63) >> 3) : tile_off(n, (k % kTileK) >> 3));
+    const size_t place = (static_cast<size_t>(k / kTileK) * g.nt + j) * 3 * plane +
+                         (g.linear ? (n >> 6) * (kTileK * 128) + tile_off(k % kTileK, (n & 63) >> 3) : tile_off(n, (k % kTileK) >> 3));
+    if (!SURGEON_IN_BOUNDS(place + 2 * plane + 15, split_planes_bytes(g), g.status)) continue;
+    unsigned char* to = out + place;
     *reinterpret_cast<uint4*>(to) = make_uint4(a[0], a[1], a[2], a[3]);
     *reinterpret_cast<uint4*>(to + plane) = make_uint4(b[0], b[1], b[2], b[3]);
     *reinterpret_cast<uint4*>(to + 2 * plane) = make_uint4(c[0], c[1], c[2], c[3]);
@@ -471,7 +468,9 @@ dw_split_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ va
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           const int o = o0 + col0 + 8 * u + i;
-          if (8 * u + i < n_cols && o < g.O) out[static_cast<size_t>(o) * g.N + nn] = acc[u][i];
+          if (8 * u + i < n_cols && o < g.O &&
+              SURGEON_IN_BOUNDS((static_cast<size_t>(chunk) * g.O + o) * g.N + nn, static_cast<size_t>(g.chunks) * g.O * g.N, g.status))
+            out[static_cast<size_t>(o) * g.N + nn] = acc[u][i];
         }
       }
     }
@@ -479,7 +478,8 @@ dw_split_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ va
   tc_fence_before();
   __syncthreads();
   if (warp == kWarps) tmem_dealloc(tmem_base, g.tmem_cols);
-  if (tid == 0) most[(chunk * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = fail ? 0xFFFFu : s_most;
+  const int cta = (chunk * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+  if (tid == 0 && SURGEON_IN_BOUNDS(cta, g.ctas, g.status)) most[cta] = fail ? 0xFFFFu : s_most;
 }
 
 bool compute_plan_split(const surgeon_layer_desc& d, SplitGeom* out) {
@@ -556,13 +556,10 @@ bool plan_split(const surgeon_layer_desc& d, SplitGeom* out) {
   return memo_plan<Tag>(d, 0, out, [&](SplitGeom* g) { return compute_plan_split(d, g); });
 }
 
-size_t split_planes_bytes(const SplitGeom& g) {
-  return static_cast<size_t>(slab_tiles(g)) * g.nt * 3 * g.tile_n * kTileK * 2;
-}
-
 cudaError_t launch_split(const surgeon_compressed& act, const SplitGeom& plan, const float* grad_out, void* planes,
                          float* partial, uint32_t* most, cudaStream_t stream) {
   SplitGeom g = plan;
+  g.status = &act.header->status;
   const int smem = 2 * ((act.dt == 0 ? 3 : 1) * kPlaneA + 3 * g.tile_n * kTileK * 2) + 1024;
   auto launch = [&](auto kernel) -> cudaError_t {
     cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void*>(kernel), smem);

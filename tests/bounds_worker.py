@@ -21,6 +21,7 @@ from gpu_util import assert_store_equals_oracle, oracle_dw, rel_frobenius
 def main():
     assert B.LIB_PATH.endswith("libsurgeon_bounds.so"), B.LIB_PATH
     shapes = [W.conv("c3x3", 3, 40, 16, 72, 3), W.conv("c3x3_s2", 3, 24, 16, 40, 3, 2),
+              W.conv("c3x3_s2_124mflop", 8, 40, 31, 96, 3, 2), W.conv("two_slabs", 44, 3, 128, 20, 3),
               W.conv("c1x1", 4, 40, 14, 96, 1, 1, 0), W.conv("c1x1_s2", 2, 72, 28, 136, 1, 2, 0),
               W.conv("stem", 2, 3, 32, 16, 7, 2, 3, dist="normal"), W.conv("c3x3_hw7", 5, 32, 7, 48, 3),
               W.linear("tokens", 2 * 197, 256, 200, dist="normal", dt=W.F32),
