@@ -494,6 +494,11 @@ bool compute_plan_split(const surgeon_layer_desc& d, SplitGeom* out) {
   // A small layer of stride 2 takes as long on the CUDA cores, which start sooner (0.06 GFLOP, fp32: 64 -> 64 channels,
   // 3x3 on 56x56 13.3 us and here 14.6, 256 -> 256 on 14x14 14.4 and 15.2; 0.15 GFLOP 14.9 and 13.9).
   if (d.stride > 1 && 2.0 * static_cast<double>(K) * d.c_out * static_cast<double>(N) < 1e8) return false;
+  // Strides of 7 and 8: pieces of five and four positions, a rank computation each.  With more than 64 outputs the CUDA
+  // cores rebuild them for every 64 (0.42-0.9 of their time here), with few inputs they lack columns (3-8: 0.76-1.0, 16-32: 0.96-1.05); else
+  // they are the faster ones: 64-128 inputs, 16-64 outputs, 0.1-4 GFLOP 1.02-1.19 of their time here in the mean, 1.48 at most
+  // (64 -> 64, 8x8 stride 8 on 56x56, batch 16, fp32: 33 us there, 44 here).  Strides 5 and 6: 0.97-1.0.
+  if (d.kind == 1 && d.stride >= 7 && d.c_out <= 64 && d.c_in >= 64) return false;
   g.C = d.c_in; g.H = d.h; g.W = d.w; g.O = d.c_out; g.KW = d.kw; g.RS = d.kh * d.kw;
   g.stride = d.stride; g.pad = d.pad; g.OH = OH; g.OW = OW;
   g.P = static_cast<int>(P); g.K = static_cast<int>(K); g.N = static_cast<int>(N);

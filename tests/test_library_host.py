@@ -52,6 +52,14 @@ def test_scratch_of_the_fp32_path_is_bounded(layer):
     assert B.surgeon_weight_grad_workspace(B.layer_desc(layer, B.PATH_FP32)) <= max(128 << 20, grad // 2) + max(64 << 20, partial) + (1 << 20)
 
 
+def test_strides_of_7_and_8_with_few_outputs_stay_on_cuda_cores():
+    """Their scratch is partial sums alone; layers of the other kernel have the gradient's parts in it too."""
+    for k, outputs, alone in ((8, 64, True), (7, 16, True), (8, 96, False), (6, 64, False)):
+        l = W.conv("k", 16, 64, 64, outputs, k, k, 0)
+        assert (B.surgeon_weight_grad_workspace(B.layer_desc(l, B.PATH_FP32)) % (4 * l.n_weight) == 0) == alone, (k, outputs)
+    assert B.surgeon_weight_grad_workspace(B.layer_desc(W.conv("k", 16, 32, 64, 64, 8, 8, 0), B.PATH_FP32)) % (4 * 64 * 32 * 64)
+
+
 def test_ratios_match_oracle_and_fixture():
     st, p = oracle.layer_ratios([2, 1, 4], [4, 2, 2])
     got = B.surgeon_layer_ratios([2, 1, 4], [4, 2, 2])
