@@ -1542,7 +1542,13 @@ cudaError_t launch_direct(const surgeon_compressed& act, const DirectParams& pla
     // From where on a warp's lanes share each run (70 % / 50 % / 0 % pruned; each lane its own run, and shared: 256 -> 512
     // channels on 56x56, batch 64, fp32 101, 142, 103 and 93, 97, 101 us; 512 -> 1024 on 28x28 79, 112, 126 and 95, 103,
     // 126; bf16 67, 89, 108 and 91, 93, 116, 60 % kept 155 and 101; 1024 -> 2048 on 14x14 54, 67, 77 and 83, 73, 77).
-    p.many_keep = static_cast<unsigned>(act.n * (p.slot_w >= 32 ? 35 : (act.dt == 0 ? 40 : 48)) / 100);
+    // Rows that fill two thirds of their slots or less leave a third of the shared lanes without an element: from 55 % kept on (bf16:
+    // 1024 -> 2048 on 33x33, batch 22, half pruned 114 us each its own and 207 shared, MODE 2 166; 20 % pruned 222 and 198) or 45 % (fp32:
+    // 256 -> 512 on 40x40, batch 61, half pruned 72 and 61); and with up to 64 channels, where half the runs are past the
+    // last one as well, never (64 -> 128 on 80x80, batch 61, bf16, 20 % pruned 58 and 77, MODE 2 71).
+    const bool padded = 3 * p.ow <= 2 * p.slot_w;
+    const int percent = padded ? (p.C <= 64 ? 100 : (act.dt == 0 ? 45 : 55)) : (p.slot_w >= 32 ? 35 : (act.dt == 0 ? 40 : 48));
+    p.many_keep = static_cast<unsigned>(act.n * percent / 100);
     e = act.dt ? launch(dw_direct_kernel<1, 3, 0, 1>) : launch(dw_direct_kernel<0, 3, 0, 1>);
     note_launches(1);
     return e;

@@ -17,6 +17,8 @@ SHAPES = [
     W.conv("w32", 2, 130, 32, 72, 1, 2, 0), W.conv("w33", 1, 19, 33, 48, 1, 2, 0), W.conv("w64", 1, 16, 64, 264, 1, 2, 0),
     W.conv("w65", 1, 9, 65, 48, 1, 2, 0), W.conv("w128", 1, 8, 128, 48, 1, 2, 0), W.conv("w1", 70, 32, 1, 48, 1, 2, 0),
     W.Layer("h3w56", 1, 2, 20, 3, 56, 48, 1, 1, 2, 0), W.Layer("h56w3", 1, 2, 20, 56, 3, 48, 1, 1, 2, 0),
+    # slots that are a third empty, with more than 64 channels: shared from 45 or 55 % kept on
+    W.conv("w17c72", 2, 72, 17, 64, 1, 2, 0), W.conv("w33c130", 1, 130, 33, 48, 1, 2, 0), W.conv("w65c72", 1, 72, 65, 48, 1, 2, 0),
     # what keeps the other kernel: wider maps, few output channels, channels no multiple of 8
     W.conv("w130", 1, 4, 130, 48, 1, 2, 0), W.conv("o40", 2, 24, 14, 40, 1, 2, 0), W.conv("o50", 2, 24, 14, 50, 1, 2, 0),
     # k x k: rows of whole pieces and not, macros that begin inside a row (20 and 12 positions), images shorter than a macro
