@@ -23,6 +23,7 @@ SHAPES = [
     W.conv("w130", 1, 4, 130, 48, 1, 2, 0), W.conv("o40", 2, 24, 14, 40, 1, 2, 0), W.conv("o50", 2, 24, 14, 50, 1, 2, 0),
     # k x k: rows of whole pieces and not, macros that begin inside a row (20 and 12 positions), images shorter than a macro
     W.conv("k3w32", 2, 40, 32, 48, 3, 2), W.conv("k3w40", 2, 24, 40, 32, 3, 2), W.conv("k3w23", 3, 20, 23, 72, 3, 2),
+    W.conv("k3w28", 2, 24, 28, 48, 3, 2), W.conv("k3w14s1", 2, 12, 14, 24, 3),
     W.conv("k3w6", 9, 40, 6, 48, 3, 2), W.conv("k5w48", 1, 20, 48, 32, 5, 2, 2), W.conv("k7w50", 1, 3, 50, 64, 7, 2, 3),
     W.conv("k4s4", 2, 24, 32, 64, 4, 4, 0), W.conv("k3s3w31", 2, 24, 31, 40, 3, 3, 1), W.conv("k3s1c12", 2, 12, 24, 40, 3),
     # rows of the patch with and without padding between them
