@@ -25,11 +25,22 @@ SHAPES = [
     # strides: pieces of 16, 11, 7 and 4 positions
     W.conv("s2", 6, 40, 30, 96, 3, 2), W.conv("s3", 8, 24, 40, 64, 5, 3, 1), W.conv("s5", 8, 16, 64, 96, 7, 5, 3),
     W.conv("s8", 12, 64, 64, 32, 8, 8, 0),
+    # (of these two the CUDA cores are the faster; the same kinds where the tensor cores are: even and odd maps with padding on the left)
+    W.conv("s2_b8", 8, 40, 30, 96, 3, 2), W.conv("s2_w31", 8, 40, 31, 96, 3, 2), W.conv("stem_w65", 12, 3, 65, 64, 7, 2, 3),
+    W.conv("s8_o96", 12, 24, 64, 96, 8, 8, 0),
     # linear: columns and channels around the tiles, channels that are no multiple of 4 or 16
     W.linear("t64", 64, 128, 64, dist="normal"), W.linear("t65", 65, 129, 65, dist="normal"),
     W.linear("t1000", 1000, 31, 127, dist="normal"), W.linear("t2049", 2049, 17, 130, dist="normal"),
     W.linear("t1", 1, 300, 10, dist="normal"),
 ]
+ON_CUDA_CORES = ("s2", "s8")
+
+
+def weight_grad(layer, store, g, **kw):
+    """The call, and how many kernels it launched: two on CUDA cores; with the tensor cores two more per slab."""
+    before = B.surgeon_launch_count()
+    dw = B.surgeon_weight_grad(store, B.layer_desc(layer, B.PATH_FP32), g, **kw)
+    return dw, B.surgeon_launch_count() - before
 
 
 @pytest.mark.parametrize("ratio", [0.0, 0.8])
@@ -39,7 +50,8 @@ def test_tile_edges(layer, bf16, ratio):
     layer = replace(layer, dt=W.BF16 if bf16 else W.F32)
     a, g = W.activation(layer, 5), W.grad_out(layer, 5)
     store = B.surgeon_prune_compact(a.cuda(), ratio)
-    dw = B.surgeon_weight_grad(store, B.layer_desc(layer, B.PATH_FP32), g.cuda())
+    dw, launches = weight_grad(layer, store, g.cuda())
+    assert launches == (2 if layer.name in ON_CUDA_CORES else 4)
     bits = W.as_numpy_bits(a).reshape(-1)
     r = oracle.prune_compact(bits, ratio)
     ref = oracle_dw(layer, oracle.decompress(r["bitmap"], r["values"], bits.size), g.numpy())
@@ -117,7 +129,41 @@ def test_infinities_and_nan(where, value):
     assert ok.any() and rel_frobenius(dw[ok], ref[ok]) <= 1e-5
 
 
-# gradients whose planes are done in several slabs (154, 151 and 164 MB), the second one shorter
+# 22, 313, 100, 64 and 210 partial sums on CUDA cores, 11, 105, 49, 32 and 69 before them on the tensor cores
+AGAIN = [LINEAR, W.linear("t20000", 20_000, 16, 16, dist="normal", dt=W.F32), W.conv("k3", 4, 24, 28, 40, 3, dt=W.F32),
+         W.conv("k3s2", 8, 40, 31, 96, 3, 2, dt=W.F32), W.conv("stem", 12, 3, 65, 64, 7, 2, 3, dt=W.F32)]
+
+
+@pytest.mark.parametrize("why", ["activation", "gradient", "large"])
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("layer", AGAIN, ids=lambda l: l.name)
+def test_calls_that_are_computed_again(layer, bf16, why):
+    """What the parts cannot hold: one infinity, or operands whose product the factor would make infinite.  The CUDA cores' sums take
+    the place of the others, in another number, also where dW is added to what is there."""
+    layer = replace(layer, dt=W.BF16 if bf16 else W.F32)
+    a, g = W.activation(layer, 14), W.grad_out(layer, 14)
+    if why == "large":
+        a, g = a * 2.0 ** 50, g * 2.0 ** 50
+    store = B.surgeon_prune_compact(a.cuda(), 0.0)
+    ref = oracle_dw(layer, W.as_numpy_bits(a).reshape(-1), g.numpy())
+    if why != "large":                             # the element in the middle of what dW's first or last channel is made of
+        t = (a if why == "activation" else g).view(layer.batch, -1)
+        t[layer.batch // 2, t.shape[1] // 2] = np.inf
+        store = B.surgeon_prune_compact(a.cuda(), 0.0)
+    dw, launches = weight_grad(layer, store, g.cuda())
+    assert launches == 4
+    dw = dw.cpu().numpy()
+    ok = np.isfinite(dw)
+    assert ok.all() == (why == "large") and ok.mean() >= 0.5
+    assert rel_frobenius(dw[ok], ref.reshape(dw.shape)[ok]) <= 1e-5
+    base = torch.full(dw.shape, 1.0, device="cuda")
+    added, _ = weight_grad(layer, store, g.cuda(), dw=base, accumulate=True)
+    added = added.cpu().numpy()
+    assert np.array_equal(np.isfinite(added), ok)
+    assert rel_frobenius(added[ok], 1.0 + ref.reshape(dw.shape)[ok]) <= 1e-5
+
+
+# gradients whose planes are done in two or three slabs (154, 151 and 164 MB), the last one shorter
 SLABS = [W.linear("tokens", 400_003, 24, 40, dist="normal"), W.conv("k3", 48, 4, 128, 20, 3), W.conv("k3s2", 13, 3, 512, 24, 3, 2)]
 
 
@@ -125,7 +171,9 @@ SLABS = [W.linear("tokens", 400_003, 24, 40, dist="normal"), W.conv("k3", 48, 4,
 def test_slabs(layer):
     a, g = W.activation(layer, 13), W.grad_out(layer, 13)
     store = B.surgeon_prune_compact(a.cuda(), 0.5)
-    dw = B.surgeon_weight_grad(store, B.layer_desc(layer, B.PATH_FP32), g.cuda()).cpu().numpy()
+    dw, launches = weight_grad(layer, store, g.cuda())
+    assert launches in (6, 8)
+    dw = dw.cpu().numpy()
     bits = W.as_numpy_bits(a).reshape(-1)
     r = oracle.prune_compact(bits, 0.5)
     ref = oracle_dw(layer, oracle.decompress(r["bitmap"], r["values"], bits.size), g.numpy())

@@ -1,6 +1,6 @@
 """GPU parity: surgeon_weight_grad through the C ABI vs the fp64 oracle.
 
-Tolerance (relative Frobenius error against the fp64 oracle): 1e-5 for the fp32 CUDA-core path,
+Tolerance (relative Frobenius error against the fp64 oracle): 1e-5 for the fp32 path,
 5e-3 for the tensor-core path (bf16 operands, fp32 accumulation)."""
 import numpy as np
 import pytest
