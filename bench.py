@@ -44,9 +44,18 @@ import torch
 METRIC = "prune+compact GB/s and sparse-act dW TFLOP/s, as % of B200 HBM/tensor peak"
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 NOMINAL = {"hbm_gbs": 7700.0, "bf16_tflops": 2250.0}
-# The fp32 path forms an fp32 product from six bf16 products on the tensor cores (three with bf16 activations, which
-# are counted as six here).
-FP32_PRODUCTS = 6
+# The fp32 path forms an fp32 product from six bf16 products on the tensor cores, three with bf16 activations; grouped layers are
+# on CUDA cores: 148 SMs x 128 FMA lanes x 2 flop x 1.965 GHz.  (So are a few others, small ones of stride 2 and more
+# among them, which are rated as if they were not.)
+FP32_ALU_TFLOPS = 148 * 128 * 2 * 1.965e9 / 1e12
+
+
+def fp32_path_tflops(layer, peaks):
+    if layer.groups > 1:
+        return FP32_ALU_TFLOPS
+    return float(peaks["bf16_tflops"]) / (3 if layer.dt == 1 else 6)
+
+
 HEADLINE = "vit"
 
 
@@ -371,7 +380,7 @@ class Stack:
         return out
 
 
-def frac_entry(kind, achieved, peaks, path_tc=True, traffic=None, extra=None):
+def frac_entry(kind, achieved, peaks, path_tc=True, traffic=None, extra=None, fp32_peak=None):
     """A roofline entry.  HBM: against the measured copy bandwidth.  Tensor: against the measured
     burst cuBLAS bf16 rate (a timed region of a fraction of a second runs at full clock, before
     the power cap settles), with the sustained and the nominal fractions beside it."""
@@ -390,10 +399,11 @@ def frac_entry(kind, achieved, peaks, path_tc=True, traffic=None, extra=None):
              "frac_sustained": round(achieved / sus, 4), "peak_sustained": round(sus, 1),
              "frac_nominal": round(achieved / NOMINAL["bf16_tflops"], 4)}
     else:
-        peak = float(peaks["bf16_tflops"]) / FP32_PRODUCTS
+        peak = fp32_peak
         d = {"bound": "tensor", "achieved": round(achieved, 3), "peak": round(peak, 1), "unit": "TFLOP/s",
              "frac": round(achieved / peak, 4), "traffic": traffic,
-             "peak_source": "%s bf16 cuBLAS, burst / %d bf16 products" % (peaks["_source"], FP32_PRODUCTS)}
+             "peak_source": peaks["_source"] + " bf16 cuBLAS, burst / 6 bf16 products (3 for bf16 activations); grouped layers: "
+                            "fp32 FMA lanes x clock; weighted by flops"}
     if extra:
         d.update(extra)
     return d
@@ -466,15 +476,16 @@ def run_stack(key, args, rank, world, device, peaks, path, keep_stack=False, sam
     tc = path == B.PATH_TENSOR_CORE
     # per-layer roofline time of the weight gradient: the slower of the tensor cores on the
     # dense-equivalent flops and HBM on the least bytes (fp32 gradient + store + dW)
-    tpeak = float(peaks["bf16_tflops"]) * 1e12 / (1 if tc else FP32_PRODUCTS)
+    tpeak = [1e12 * (float(peaks["bf16_tflops"]) if tc else fp32_path_tflops(l, peaks)) for l in layers]
     hpeak = float(peaks["hbm_gbs"]) * 1e9
-    roof_us = [max(l.flops / tpeak, dw_min_bytes(l, s.sizes.n_keep) / hpeak) * 1e6
-               for l, s in zip(layers, stack.store)]
+    roof_us = [max(l.flops / t, dw_min_bytes(l, s.sizes.n_keep) / hpeak) * 1e6
+               for l, s, t in zip(layers, stack.store, tpeak)]
     dw_entry = frac_entry("tensor", dw_tflops, peaks, tc,
                           recorded_traffic(key, "weight_grad") if (full and tc) else None,
                           {"kernel": "weight gradient (all layers of one step)", "ms": round(dw_ms, 4), "flops": flops,
                            "roofline_ms": round(sum(roof_us) / 1e3, 4),
-                           "frac_of_layer_rooflines": round(sum(roof_us) / 1e3 / dw_ms, 4)})
+                           "frac_of_layer_rooflines": round(sum(roof_us) / 1e3 / dw_ms, 4)},
+                          fp32_peak=flops / sum(l.flops / t for l, t in zip(layers, tpeak)) / 1e12)
     pc_entry = frac_entry("hbm", prune_gbs, peaks, True,
                           recorded_traffic(key, "prune_compact") if full else None,
                           {"kernel": "surgeon_prune_compact (all kernels of all layers of one step)",
