@@ -158,7 +158,8 @@ inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block
 #define SURGEON_IN_BOUNDS(idx, limit, status_word) true
 #endif
 
-// Division of numbers below 2^31 by one that the host knows: two instructions instead of some 35.
+// Division of numbers below 2^31 by one that the host knows: two instructions instead of some 35 (Granlund and Montgomery,
+// "Division by invariant integers using multiplication", 1994).
 struct FastDiv {
   uint32_t mul, shift;
 };

@@ -367,7 +367,6 @@ dw_fp32_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ val
     }
     __syncthreads();
   }
-  float* out = partial + static_cast<long long>(blockIdx.z) * g.M * g.N;
 #pragma unroll
   for (int a = 0; a < 8; ++a) {
     const long long m = m0 + ty * 8 + a;
@@ -377,9 +376,9 @@ dw_fp32_kernel(const uint32_t* __restrict__ bitmap, const void* __restrict__ val
       const long long nn = n0 + (b >> 1) * (TN / 2) + tx * 4 + (b & 1) * 2;
       const float lo = __uint_as_float(static_cast<uint32_t>(acc[a][b]));
       const float hi = __uint_as_float(static_cast<uint32_t>(acc[a][b] >> 32));
-      const long long at = (blockIdx.z * g.M + m) * g.N + nn, all = g.chunks * g.M * g.N;
-      if (nn < g.N && SURGEON_IN_BOUNDS(at, all, split.status)) out[m * g.N + nn] = lo;
-      if (nn + 1 < g.N && SURGEON_IN_BOUNDS(at + 1, all, split.status)) out[m * g.N + nn + 1] = hi;
+      const long long at = (blockIdx.z * g.M + m) * g.N + nn;
+      if (nn < g.N && SURGEON_IN_BOUNDS(at, g.chunks * g.M * g.N, split.status)) partial[at] = lo;
+      if (nn + 1 < g.N && SURGEON_IN_BOUNDS(at + 1, g.chunks * g.M * g.N, split.status)) partial[at + 1] = hi;
     }
   }
 }
