@@ -491,6 +491,10 @@ bool compute_plan_split(const surgeon_layer_desc& d, SplitGeom* out) {
   if (K < 1 || K > (1LL << 30) || N > (1LL << 30) || d.c_out > (1 << 30)) return false;
   // Rows of fewer than four positions: a rank computation for each piece costs more than the products save.
   if (d.kind == 1 && (OW < 4 || d.stride > 8)) return false;
+  // Linear layers of up to 16 rows: a quarter of a K-tile at most, and the CUDA cores launch two kernels less.  Time here over
+  // time there, fp32 and bf16, in replays of a graph: 1-4 rows 1.77 and 1.56 (10 instead of 5.6 us for 10 to 3072 outputs), 5-8 rows 1.64
+  // and 1.35, 9-16 rows 1.31 and 1.05; 17-23 rows 1.10 and 0.85, 24-32 rows 0.95 and 0.69.
+  if (d.kind != 1 && d.batch <= 16) return false;
   // A small layer of stride 2 takes as long on the CUDA cores, which start sooner (0.06 GFLOP, fp32: 64 -> 64 channels,
   // 3x3 on 56x56 13.3 us and here 14.6, 256 -> 256 on 14x14 14.4 and 15.2; 0.15 GFLOP 14.9 and 13.9).
   if (d.stride > 1 && 2.0 * static_cast<double>(K) * d.c_out * static_cast<double>(N) < 1e8) return false;

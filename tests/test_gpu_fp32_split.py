@@ -32,8 +32,10 @@ SHAPES = [
     W.linear("t64", 64, 128, 64, dist="normal"), W.linear("t65", 65, 129, 65, dist="normal"),
     W.linear("t1000", 1000, 31, 127, dist="normal"), W.linear("t2049", 2049, 17, 130, dist="normal"),
     W.linear("t1", 1, 300, 10, dist="normal"),
+    # the fewest rows of the tensor cores, and one less
+    W.linear("t17", 17, 300, 70, dist="normal"), W.linear("t16", 16, 300, 70, dist="normal"),
 ]
-ON_CUDA_CORES = ("s2", "s8")
+ON_CUDA_CORES = ("s2", "s8", "t1", "t16")
 
 
 def weight_grad(layer, store, g, **kw):

@@ -60,6 +60,14 @@ def test_strides_of_7_and_8_with_few_outputs_stay_on_cuda_cores():
     assert B.surgeon_weight_grad_workspace(B.layer_desc(W.conv("k", 16, 32, 64, 64, 8, 8, 0), B.PATH_FP32)) % (4 * 64 * 32 * 64)
 
 
+def test_linear_layers_of_up_to_16_rows_stay_on_cuda_cores():
+    for rows in (1, 2, 16, 17):
+        for c, o in ((320, 16), (2048, 1000)):
+            l = W.linear("few", rows, c, o)
+            alone = B.surgeon_weight_grad_workspace(B.layer_desc(l, B.PATH_FP32)) % (4 * l.n_weight) == 0
+            assert alone == (rows <= 16), (rows, c, o)
+
+
 def test_ratios_match_oracle_and_fixture():
     st, p = oracle.layer_ratios([2, 1, 4], [4, 2, 2])
     got = B.surgeon_layer_ratios([2, 1, 4], [4, 2, 2])
