@@ -225,7 +225,8 @@ typedef struct surgeon_layer_desc {
   int32_t c_out, kh, kw, stride, pad;
   int32_t path;  /* 0 = tensor-core path (bf16 x bf16 -> fp32, tcgen05/TMEM);
                     1 = fp32 path: products of fp32 numbers (as products of their three bf16 parts
-                        on the tensor cores where that loses nothing, else on CUDA cores)         */
+                        on the tensor cores, 2^-26 of a product left out; on CUDA cores where the
+                        parts cannot hold an operand, and for small layers)                       */
   int32_t groups; /* conv2d: channel groups (0 or 1 = an ordinary convolution).  groups > 1 (the
                     3x3 layers of ResNeXt, the network the paper adapts on CIFAR100-C in Section
                     5.1; groups = c_in = c_out is a depthwise convolution): c_in and c_out must

@@ -14,6 +14,10 @@
 // Error against 64 bits (320 -> 320 channels, 3x3 on 16x16, batch 16; relative 2-norm; the CUDA-core kernel's in brackets): nothing
 // pruned 1.0e-7 (3.4e-7), 90 % pruned 5.8e-8 (1.6e-7), 99 % 3.8e-8 (6.1e-8).  (With the small products first in the
 // same accumulator it was 1.1e-7, 1.05e-7 and more than before from 97 % on: every sum was cut off toward zero.)
+// 13 layers of all kinds, both types, seven pruning ratios, 182 calls: the 2-norm of the error is 0.49 of the CUDA cores' in the
+// geometric mean and above it in none.  Part of it has one sign, since what is cut off is cut off toward zero: unpruned, dW is 2.3e-8
+// to 6.1e-8 of itself too small, half pruned 0.8e-8 to 2.8e-8, from 70 % on within 6e-9 (CUDA cores: within 9e-9 at all ratios).  The
+// largest error of one element is above the CUDA cores' in 13 calls, most of them pruned by 97 % and more, by up to 1.22.
 //
 //   dW[m, nn] = sum_k G[k, m] * Acol[k, nn],  nn = (c, r, s) -> MMA M (128), m = output channel -> MMA N (up to 160),
 //   k = (b, y, x) over all images, or the row t of a linear layer -> MMA K, 64 per stage.
@@ -24,9 +28,10 @@
 // words of the one after it.  A pre-pass writes the gradient's planes as they lie in shared memory: one bulk copy a tile.
 //
 // Measured on 320 -> 320 channels, 3x3 on 16x16, batch 16 (7.5 GFLOP): 264 us on CUDA cores, 66-71 now, of which the pre-pass
-// takes 4, this kernel 55 and the reduction 4.  A K-tile takes 4700 clocks, its MMAs 2260: the warps' instructions and
-// what they wait for are the bound (store 750, asking for values 1300, sums 800, or 2000 beside MMAs).  MMAs issued by the
-// warps in turn instead of by a warp of their own: 7600 clocks a tile, since whoever issues is late for the next tile.
+// takes 4, this kernel 55 and the reduction 4.  70 % pruned, a K-tile takes 4000 clocks (start and epilogue included), its MMAs
+// 1920 at their nominal rate; tensor pipe 46 %, issue slots 64 %, DRAM 2 % busy: the warps' instructions and what they wait for are the bound.
+// (Clock stamps in a copy of the kernel: store 750, asking for values 1300, sums 800, or 2000 beside MMAs.)  MMAs issued by the
+// warps in turn instead of by a warp of their own took 1.6 times as long, since whoever issues is late for the next tile.
 //
 // Infinities and NaN, operands from 2^104 on and calls whose largest operands multiply to 2^64 and more (which the
 // factor could make infinite) are seen from the largest magnitudes, which every block records; a wait that ran out

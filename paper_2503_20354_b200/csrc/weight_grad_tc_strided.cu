@@ -18,8 +18,8 @@
 //      rows on the same banks, took 1440-2640 clocks a K-tile for what now takes 1040-1180).
 // One group rebuilds while the other copies; the words and the values of a macro's first pieces are
 // fetched while the macro before it is copied.  Bound by the instructions of the two steps, 430 for a warp's 32 pieces and
-// 200 for its part of a K-tile: with 16 warps an SM issues at 0.56 of its rate and each warp every 8 clocks, for no one
-// reason above a quarter; tensor pipe 17 %, DRAM 4 %.  So divisions are multiplications (also the
+// 200 for its part of a K-tile: with 16 warps an SM issues at 0.53-0.57 of its rate and each warp every 8 clocks, for no one
+// reason above a quarter; tensor pipe 11-15 %, DRAM 6-16 % busy (3x3 on 56x56 and the 7x7 stem, 70 % pruned).  So divisions are multiplications (also the
 // sixteen of a thread's start: with them and branches in the fetch of a piece's words, a call of 15-21 us took 2 more), the
 // copy and the fetch have no branches, a kept value costs one test for its load and its count, and a piece is put together in registers, not scattered bit by bit.
 // Calls, 70 % pruned, when bits were scattered, with 4-byte copies, and now: 128 -> 128 channels on 56x56, batch 64, bf16
