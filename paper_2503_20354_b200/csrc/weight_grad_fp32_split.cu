@@ -69,7 +69,8 @@ constexpr int kLeastTiles = 20;                  // chunks of fewer K-tiles only
 constexpr double kMaxPartials = 32 << 20;
 constexpr float kSplitScale = static_cast<float>(1 << kSplitShift);
 
-// x0, x1 times 2^kSplitShift -> their three parts, two to a word.
+// x0, x1 times 2^kSplitShift -> their three parts, two to a word.  (Multiplied before the first rounding: a subnormal number's first
+// part has fewer bits, and the products that are left out would be up to 2^-17 of the whole.)
 __device__ __forceinline__ void split2(float x0, float x1, uint32_t& p1, uint32_t& p2, uint32_t& p3) {
   x0 *= kSplitScale;
   x1 *= kSplitScale;
